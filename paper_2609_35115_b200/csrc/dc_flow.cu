@@ -191,7 +191,7 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   float* s_bias = reinterpret_cast<float*>(s_fail + 1);
   float* s_tau = s_bias + MAX_BN;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
   const int m0 = blockIdx.x * TILE_M, n0 = blockIdx.y * BN;
   const uint32_t pair_rank = PAIR ? ptx::cluster_ctarank() : 0u;   // 0: issues the UMMAs and owns the "full" barriers
   // Accumulator: BN columns, or 3 BN for a conv block, whose three taps are the column blocks of ONE
@@ -233,7 +233,6 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // The loops keep their state in registers (no division, no parameter reloads): a single thread
     // issues every copy, so its instruction count is what bounds the fill rate.
     {
-      const uint32_t on = lane == 0;   // the whole warp runs the loop, lane 0 issues
       const bool is_a = warp == 0;
       const int nkb = p.n_kblocks, taps = n_taps;
       const int ya = GUARD + m0;
@@ -262,29 +261,33 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           *s_fail = 1;
           break;
         }
-        if (PAIR) {
-          ptx::mbar_expect_tx_if(on && pair_rank == 0, &full[st], tx_bytes);
-          const uint32_t bar = full0 + (uint32_t)st * 8u;
-          if (is_a) {
-            ptx::tma_load_2d_pair_if(on, dst, &tmA, x, ya, bar);
+        if (ptx::elect_one()) {
+          if (PAIR) {
+            if (pair_rank == 0) ptx::mbar_expect_tx(&full[st], tx_bytes);
+            const uint32_t bar = full0 + (uint32_t)st * 8u;
+            if (is_a) {
+              ptx::tma_load_2d_pair(dst, &tmA, x, ya, bar);
+            } else {
+              ptx::tma_load_2d_pair(dst, &tmB, x + ux[0], uy[0], bar);
+              if (taps == 3) {
+                ptx::tma_load_2d_pair(dst + b_tile, &tmB, x + ux[1], uy[1], bar);
+                ptx::tma_load_2d_pair(dst + 2 * b_tile, &tmB, x + ux[2], uy[2], bar);
+              }
+            }
           } else {
-            ptx::tma_load_2d_pair_if(on, dst, &tmB, x + ux[0], uy[0], bar);
-            if (taps == 3) {
-              ptx::tma_load_2d_pair_if(on, dst + b_tile, &tmB, x + ux[1], uy[1], bar);
-              ptx::tma_load_2d_pair_if(on, dst + 2 * b_tile, &tmB, x + ux[2], uy[2], bar);
+            ptx::mbar_expect_tx(&full[st], tx_bytes);
+            if (is_a) {
+              ptx::tma_load_2d(dst, &tmA, x, ya, &full[st]);
+            } else {
+              ptx::tma_load_2d(dst, &tmB, x, n0, &full[st]);
+              if (taps == 3) {
+                ptx::tma_load_2d(dst + b_tile, &tmB, x + nkb * KBLK, n0, &full[st]);
+                ptx::tma_load_2d(dst + 2 * b_tile, &tmB, x + 2 * nkb * KBLK, n0, &full[st]);
+              }
             }
           }
-        } else if (is_a) {
-          ptx::mbar_expect_tx_if(on, &full[st], tx_bytes);
-          ptx::tma_load_2d_if(on, dst, &tmA, x, ya, &full[st]);
-        } else {
-          ptx::mbar_expect_tx_if(on, &full[st], tx_bytes);
-          ptx::tma_load_2d_if(on, dst, &tmB, x, n0, &full[st]);
-          if (taps == 3) {
-            ptx::tma_load_2d_if(on, dst + b_tile, &tmB, x + nkb * KBLK, n0, &full[st]);
-            ptx::tma_load_2d_if(on, dst + 2 * b_tile, &tmB, x + 2 * nkb * KBLK, n0, &full[st]);
-          }
         }
+        __syncwarp();
         x += KBLK;
         dst += stage_bytes;
         if (++st == STAGES) {
@@ -300,7 +303,6 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // of their own; the epilogue adds the two in a fixed order.
     const int me = warp >> 1;                     // 0 or 1
     if (me < n_iss && pair_rank == 0) {
-      const uint32_t on = lane == 0;
       // the weight tiles of the taps are adjacent in the stage (BN rows of 128 B each, BN a multiple of 8),
       // so together they are one K-major operand of taps * BN rows
       const uint32_t idesc = ptx::umma_idesc_bf16(PAIR ? 2 * TILE_M : TILE_M, n_taps * BN, 0, 0);
@@ -322,27 +324,33 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         ptx::tc_fence_after();
         const uint64_t da = d_a0 + (uint64_t)((uint32_t)st * stage16), db = da + ab16;
-        if (PAIR) {
-          ptx::umma_bf16_pair_if(on, d_acc, da, db, idesc, acc);
+        if (ptx::elect_one()) {
+          if (PAIR) {
+            ptx::umma_bf16_pair(d_acc, da, db, idesc, acc);
 #pragma unroll
-          for (int k = 1; k < 4; ++k) ptx::umma_bf16_pair_if(on, d_acc, da + 2 * k, db + 2 * k, idesc, 1);
-          ptx::umma_commit_pair_if(on, empty_mine + (uint32_t)st * 8u);
-          ptx::umma_commit_pair_if(on, empty_peer + (uint32_t)st * 8u);
-        } else {
-          ptx::umma_bf16_if(on, d_acc, da, db, idesc, acc);
+            for (int k = 1; k < 4; ++k) ptx::umma_bf16_pair(d_acc, da + 2 * k, db + 2 * k, idesc, 1);
+            ptx::umma_commit_pair(empty_mine + (uint32_t)st * 8u);
+            ptx::umma_commit_pair(empty_peer + (uint32_t)st * 8u);
+          } else {
+            ptx::umma_bf16(d_acc, da, db, idesc, acc);
 #pragma unroll
-          for (int k = 1; k < 4; ++k) ptx::umma_bf16_if(on, d_acc, da + 2 * k, db + 2 * k, idesc, 1);
-          ptx::umma_commit_if(on, &empty[st]);
+            for (int k = 1; k < 4; ++k) ptx::umma_bf16(d_acc, da + 2 * k, db + 2 * k, idesc, 1);
+            ptx::umma_commit(&empty[st]);
+          }
         }
+        __syncwarp();
         acc = 1;
       }
       // arrives when every UMMA above has finished (also on the failure path)
-      if (PAIR) {
-        ptx::umma_commit_pair_if(on, ptx::smem_u32(accum));
-        ptx::umma_commit_pair_if(on, ptx::map_to_cta(ptx::smem_u32(accum), 1u));
-      } else {
-        ptx::umma_commit_if(on, accum);
+      if (ptx::elect_one()) {
+        if (PAIR) {
+          ptx::umma_commit_pair(ptx::smem_u32(accum));
+          ptx::umma_commit_pair(ptx::map_to_cta(ptx::smem_u32(accum), 1u));
+        } else {
+          ptx::umma_commit(accum);
+        }
       }
+      __syncwarp();
     }
   } else {
     // ---------------- epilogue: 4 EPI_GROUPS warps; a thread owns one output row and every EPI_GROUPS-th 16-column chunk ----------------
@@ -833,7 +841,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_sfree + 2);
   float* s_x = reinterpret_cast<float*>(tmem_slot + 2);   // [2][64] exchange between the two column halves
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int slot = blockIdx.x, head = blockIdx.y;
   const int chunks = p.dh >> 3;             // 16-byte chunks per head row
 
@@ -904,7 +912,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         ptx::fence_proxy_async_smem();
         __syncwarp();
       }
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         int rr = row0 + b * ATT_KB;
         while (rr >= p.Rk) rr -= p.Rk;
         const int n1 = min(n, p.Rk - rr);
@@ -912,6 +920,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         ptx::bulk_load(dstb, src0 + (long long)rr * 64, (uint32_t)n1 * 128u, &full[st]);
         if (n1 < n) ptx::bulk_load(dstb + n1 * 128, src0, (uint32_t)(n - n1) * 128u, &full[st]);
       }
+      __syncwarp();
     };
     if (warp != 6)
       for (int b = 0; b < n_early; ++b) fetch(b);           // (b < ATT_STAGES: no stage to wait for)
@@ -1022,7 +1031,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     ptx::mbar_arrive(&full[(nkb - 1) % ATT_STAGES]);
   } else if (warp == 4) {
     // ---------------- UMMA issuer ----------------
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const uint32_t idesc_s = ptx::umma_idesc_bf16(128, ATT_KB, 0, 0);
       const uint32_t idesc_pv = ptx::umma_idesc_bf16(128, 64, 0, 1);   // B = V, MN-major
       const uint64_t dq = ptx::umma_desc_sw128(ptx::smem_u32(sQ));
