@@ -761,7 +761,7 @@ __global__ void flow_rmsnorm_kernel(const SlotInfo* slots, int n_slots, const bf
 constexpr int ATT_THREADS = 256;
 constexpr int ATT_KB = 128;             // keys per block
 constexpr int ATT_STAGES = 2;
-constexpr int ATT_TMEM_COLS = 256;      // S (128 columns) + O (64 columns); two CTAs share the SM's 512
+constexpr int ATT_TMEM_COLS = 256;      // S (128 columns) + the two O accumulators (64 columns each); two CTAs share the SM's 512
 constexpr int ATT_K_LOADERS = 64;       // warps 5 and 6: Q, then the K blocks
 constexpr int ATT_V_LOADERS = 32;       // warp 7: the V blocks
 constexpr int ATT_Q_BYTES = 128 * 128;  // 64 query rows, twice
@@ -798,6 +798,93 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Pairs of fp32 values in one instruction (each half is the ordinary rounded operation).
+__device__ __forceinline__ float2 pair2(uint32_t a, uint32_t b) { return make_float2(__uint_as_float(a), __uint_as_float(b)); }
+__device__ __forceinline__ float2 unpack2(uint32_t bf16x2) { return pair2(bf16x2 << 16, bf16x2 & 0xFFFF0000u); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n.reg .b64 x, y;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nadd.rn.f32x2 x, x, y;\nmov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n.reg .b64 x, y;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmul.rn.f32x2 x, x, y;\nmov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n.reg .b64 x, y, z;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmov.b64 z, {%6, %7};\nfma.rn.f32x2 x, x, y, z;\nmov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ float2 silu2(float2 z) {   // silu_f of both halves
+  const float2 h = mul2(z, make_float2(0.5f, 0.5f));
+  float2 t;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t.x) : "f"(h.x));
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(h.y));
+  return fma2(h, t, h);
+}
+
+// ---- the softmax of one key block, shared by both attention kernels (their results have to agree bit for bit) ----
+// A thread holds one query row and 64 of the block's 128 key columns.  Even and odd key blocks are two independent streams,
+// each with its own reference, row sum and output accumulator, combined at the end (att_combine): the products of a block need
+// not wait for the block before, and two groups of warps can work on them at once.
+
+// Masks the padding (columns >= valid; the first `skip` columns) and returns the largest score.
+__device__ __forceinline__ float att_mask_max(float (&v)[64], int valid, int skip) {
+  if (valid < 64) {                            // only the last block has padded key columns
+#pragma unroll
+    for (int i = 0; i < 64; ++i)
+      if (i >= valid) v[i] = -INFINITY;
+  }
+  if (skip > 0) {
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+      if (i < skip) v[i] = -INFINITY;
+  }
+  float m[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+  for (int i = 4; i < 64; ++i) m[i & 3] = fmaxf(m[i & 3], v[i]);
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+
+// e = exp2(scale v - m), P = bf16(e) into the row's swizzled 128-byte line; returns the sum of the unrounded e.
+__device__ __forceinline__ float att_exp_store(const float (&v)[64], float scale, float m, uint8_t* prow, int row) {
+  float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const float2 sc = make_float2(scale, scale), mm = make_float2(-m, -m);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 e = fma2(make_float2(v[8 * c + 2 * i], v[8 * c + 2 * i + 1]), sc, mm);
+      e.x = ex2_approx(e.x);
+      e.y = ex2_approx(e.y);
+      sum[i & 1] = add2(sum[i & 1], e);
+      const __nv_bfloat162 h = __floats2bfloat162_rn(e.x, e.y);
+      w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(prow + ((c ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  const float2 t = add2(sum[0], sum[1]);
+  return t.x + t.y;
+}
+
+// Weights of the two streams' accumulators: O = c0 O_0 + c1 O_1.
+__device__ __forceinline__ void att_combine(int nkb, float m0, float l0, float m1, float l1, float* c0, float* c1) {
+  if (nkb == 1) {
+    *c0 = 1.0f / l0;
+    *c1 = 0.f;
+  } else {
+    const float m = fmaxf(m0, m1), a0 = exp2f(m0 - m), a1 = exp2f(m1 - m);
+    const float inv = 1.0f / fmaf(a0, l0, a1 * l1);
+    *c0 = a0 * inv;
+    *c1 = a1 * inv;
+  }
 }
 
 // PROMPT = false: the carry is a plain window (no prompt rows); a separate instantiation, because this kernel sits at its
@@ -1065,16 +1152,15 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         const uint64_t dv = ptx::umma_desc_sw128(ptx::smem_u32(ring + st * ATT_STAGE_BYTES + ATT_KB * 128));
         const int valid = L - b * ATT_KB;
         const int ksteps = valid >= ATT_KB ? ATT_KB / 16 : (valid + 15) / 16;
-        // P tile k/4 (8 KB apart), 32-byte K steps; V: 16 key rows = 2 KB per step
+        // P tile k/4 (8 KB apart), 32-byte K steps; V: 16 key rows = 2 KB per step; even blocks into O_0, odd ones into O_1
+        const uint32_t d_o = tmem_base + ATT_KB + (uint32_t)(b & 1) * 64u;
         if (ksteps == ATT_KB / 16) {
 #pragma unroll
           for (int k = 0; k < ATT_KB / 16; ++k)
-            ptx::umma_bf16(tmem_base + ATT_KB, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)),
-                           idesc_pv, (b | k) != 0);
+            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
         } else {
           for (int k = 0; k < ksteps; ++k)
-            ptx::umma_bf16(tmem_base + ATT_KB, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)),
-                           idesc_pv, (b | k) != 0);
+            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
         }
         ptx::umma_commit(&empty_v[st]);
         ptx::umma_commit(&bar_pv[b & 1]);
@@ -1087,40 +1173,29 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     const int row = quarter * 32 + lane;        // query row
     const uint32_t lane_addr = tmem_base + ((uint32_t)(warp * 32) << 16);   // the lanes this warp may access
     bool ok = true;
-    float m_ref = -INFINITY, lsum = 0.f;
+    // reference and row sum of this block's stream and of the other one (they change places after every block)
+    float m_ref = -INFINITY, lsum = 0.f, m_oth = -INFINITY, l_oth = 0.f;
     for (int b = 0; b < nkb; ++b) {
       if (ok && !ptx::mbar_wait(bar_s, b & 1)) { ok = false; atomicExch(p.err, 7); }
       ptx::tc_fence_after();
-      const int valid = L - b * ATT_KB - half * 64;   // columns of this half that are real keys
       float v[64];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) ptx::tmem_ld16(lane_addr + (uint32_t)(half * 64 + c * 16), v + 16 * c);
+      ptx::tmem_ld64(lane_addr + (uint32_t)(half * 64), v);
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar_sfree);               // S(b) is in registers: the next block's scores may overwrite it
-      if (valid < 64) {                          // only the last block has padded key columns
-#pragma unroll
-        for (int i = 0; i < 64; ++i)
-          if (i >= valid) v[i] = -INFINITY;
-      }
-      if (BULK && b == 0 && half == 0) {         // the rows between the 8-row boundary and the attended interval
-#pragma unroll
-        for (int i = 0; i < 7; ++i)
-          if (i < phi) v[i] = -INFINITY;
-      }
-      float mx = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < 64; ++i) mx = fmaxf(mx, v[i]);
+      // (the first phi columns are the rows between the 8-row boundary and the attended interval)
+      float mx = att_mask_max(v, L - b * ATT_KB - half * 64, BULK && b == 0 && half == 0 ? phi : 0);
       s_x[half * 64 + row] = mx * p.scale_log2e;
       ptx::named_bar_sync(2, 128);
       mx = fmaxf(s_x[row], s_x[64 + row]);
       ptx::named_bar_sync(2, 128);   // all have read: the next block (or the row sums below) may overwrite the exchange
-      if (b == 0) {
+      if (b >= 2) {   // this block's P buffer was last read by P V of block b - 2, which also completes this stream's O
+        if (ok && !ptx::mbar_wait(&bar_pv[b & 1], ((b >> 1) - 1) & 1)) { ok = false; atomicExch(p.err, 15); }
+      }
+      if (b < 2) {
         m_ref = mx;
       } else {
         const bool need = mx > m_ref + ATT_RESCALE_LOG2;
         if (__any_sync(0xffffffffu, need)) {
-          // O must hold every earlier block and be quiescent before it is rescaled
-          if (ok && !ptx::mbar_wait(&bar_pv[(b - 1) & 1], ((b - 1) >> 1) & 1)) { ok = false; atomicExch(p.err, 8); }
           ptx::tc_fence_after();
           const float alpha = need ? exp2f(m_ref - mx) : 1.0f;
           if (need) m_ref = mx;
@@ -1128,7 +1203,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           if (half == 0) {                        // O rows 0..63 live in lanes 0..63
             for (int c = 0; c < p.dh; c += 16) {
               float o16[16];
-              const uint32_t addr = lane_addr + (uint32_t)(ATT_KB + c);
+              const uint32_t addr = lane_addr + (uint32_t)(ATT_KB + (b & 1) * 64 + c);
               ptx::tmem_ld16(addr, o16);
 #pragma unroll
               for (int i = 0; i < 16; ++i) o16[i] *= alpha;
@@ -1138,39 +1213,36 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           ptx::tc_fence_before();
         }
       }
-      if (b >= 2) {   // this block's P buffer was last read by P V of block b - 2
-        if (ok && !ptx::mbar_wait(&bar_pv[b & 1], ((b >> 1) - 1) & 1)) { ok = false; atomicExch(p.err, 15); }
-      }
-      uint8_t* prow = sP + (b & 1) * ATT_P_BYTES + half * 8192 + row * 128;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float e[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          e[i] = ex2_approx(fmaf(v[16 * c + i], p.scale_log2e, -m_ref));
-          lsum += e[i];
-        }
-        uint4 a, bq;
-        pack16_bf16(e, a, bq);
-        *reinterpret_cast<uint4*>(prow + (((2 * c) ^ (row & 7)) << 4)) = a;
-        *reinterpret_cast<uint4*>(prow + (((2 * c + 1) ^ (row & 7)) << 4)) = bq;
-      }
+      lsum += att_exp_store(v, p.scale_log2e, m_ref, sP + (b & 1) * ATT_P_BYTES + half * 8192 + row * 128, row);
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(&bar_p[b & 1]);
+      float t = m_ref; m_ref = m_oth; m_oth = t;
+      t = lsum; lsum = l_oth; l_oth = t;
     }
+    if (nkb & 1) {   // (m_ref, lsum): stream 0
+      float t = m_ref; m_ref = m_oth; m_oth = t;
+      t = lsum; lsum = l_oth; l_oth = t;
+    }
+    if (nkb >= 2 && ok && !ptx::mbar_wait(&bar_pv[nkb & 1], ((nkb - 2) >> 1) & 1)) { ok = false; atomicExch(p.err, 8); }
     if (ok && !ptx::mbar_wait(&bar_pv[(nkb - 1) & 1], ((nkb - 1) >> 1) & 1)) { ok = false; atomicExch(p.err, 9); }
     ptx::tc_fence_after();
     s_x[half * 64 + row] = lsum;
     ptx::named_bar_sync(2, 128);
-    const float inv = 1.0f / (s_x[row] + s_x[64 + row]);
+    const float l0 = s_x[row] + s_x[64 + row];
+    ptx::named_bar_sync(2, 128);
+    s_x[half * 64 + row] = l_oth;
+    ptx::named_bar_sync(2, 128);
+    float c0, c1;
+    att_combine(nkb, m_ref, l0, m_oth, s_x[row] + s_x[64 + row], &c0, &c1);
     bf16* orow = p.o + (long long)(GUARD + slot * SLOT_ROWS + HALO + row) * p.ld + head * p.dh;
     for (int c = 0; c < (half == 0 ? p.dh : 0); c += 16) {
-      float o16[16];
+      float o16[16], q16[16];
       ptx::tmem_ld16(lane_addr + (uint32_t)(ATT_KB + c), o16);
+      if (nkb > 1) ptx::tmem_ld16(lane_addr + (uint32_t)(ATT_KB + 64 + c), q16);
       if (row < T && ok) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) o16[i] *= inv;
+        for (int i = 0; i < 16; ++i) o16[i] = nkb > 1 ? fmaf(q16[i], c1, o16[i] * c0) : o16[i] * c0;
         uint4 a, bq;
         pack16_bf16(o16, a, bq);
         store16(orow + c, a, bq);
