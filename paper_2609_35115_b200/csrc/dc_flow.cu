@@ -261,6 +261,7 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           *s_fail = 1;
           break;
         }
+        __syncwarp();   // (lanes leave the polling loop one by one; as separate groups they would execute what follows several times)
         if (ptx::elect_one()) {
           if (PAIR) {
             if (pair_rank == 0) ptx::mbar_expect_tx(&full[st], tx_bytes);
@@ -322,6 +323,7 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           *s_fail = 1;
           break;
         }
+        __syncwarp();
         ptx::tc_fence_after();
         const uint64_t da = d_a0 + (uint64_t)((uint32_t)st * stage16), db = da + ab16;
         if (ptx::elect_one()) {
@@ -412,6 +414,7 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     ptx::named_bar_sync(1, EPI_THREADS);
 
     const bool got = ptx::mbar_wait_relaxed(accum, 0);
+    __syncwarp();
     if (PAIR) ptx::cluster_wait();   // (long complete; a thread waits once between its two arrivals)
     ptx::tc_fence_after();
     if (!got) atomicCAS(p.err, 0, 3 | (mode << 8));
@@ -933,6 +936,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
   const int chunks = p.dh >> 3;             // 16-byte chunks per head row
 
   if (tid == 0) {
+#pragma unroll 1
     for (int i = 0; i < ATT_STAGES; ++i) {
       ptx::mbar_init(&full_k[i], BULK ? 1 : ATT_K_LOADERS);
       ptx::mbar_init(&empty_k[i], 1);
@@ -940,6 +944,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       ptx::mbar_init(&empty_v[i], 1);
     }
     ptx::mbar_init(bar_s, 1);
+#pragma unroll 1
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&bar_p[i], 128);
       ptx::mbar_init(&bar_pv[i], 1);
@@ -990,17 +995,20 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         ok = false;
         atomicExch(p.err, 4);
       }
+      __syncwarp();
       uint8_t* dstb = ring + st * ATT_STAGE_BYTES + (is_k ? 0 : ATT_KB * 128);
       const int n = min(ATT_KB, L - b * ATT_KB);            // key rows of this block
       if (!is_k && n < ATT_KB) {
         // the P V product reads whole 16-row steps: the rows behind the last key must be finite (their weights are 0)
         const int n16 = min(ATT_KB, (n + 15) & ~15);
+#pragma unroll 1
         for (int i = lane; i < (n16 - n) * 8; i += 32) *reinterpret_cast<uint4*>(dstb + n * 128 + i * 16) = zero;
         ptx::fence_proxy_async_smem();
         __syncwarp();
       }
       if (ptx::elect_one()) {
         int rr = row0 + b * ATT_KB;
+#pragma unroll 1
         while (rr >= p.Rk) rr -= p.Rk;
         const int n1 = min(n, p.Rk - rr);
         ptx::mbar_expect_tx(&full[st], (uint32_t)n * 128u);
@@ -1010,11 +1018,13 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       __syncwarp();
     };
     if (warp != 6)
+#pragma unroll 1
       for (int b = 0; b < n_early; ++b) fetch(b);           // (b < ATT_STAGES: no stage to wait for)
     ptx::pdl_wait();                                        // Q and the chunk's own K / V rows are the projection's output
     if (is_k) {
       const int lt = (warp == 6 ? 32 : 0) + lane;
       const bf16* qbase = p.q + (long long)(GUARD + slot * SLOT_ROWS + HALO) * p.ld + head * 64;
+#pragma unroll 1
       for (int i = lt; i < 128 * 8; i += ATT_K_LOADERS) {
         const int row = i >> 3, j = i & 7, qrow = row & 63;   // rows 64.. repeat rows 0..
         uint8_t* dst = sQ + row * 128 + ((j ^ (row & 7)) << 4);
@@ -1026,6 +1036,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       ptx::mbar_arrive(bar_q);
     }
     if (warp != 6)
+#pragma unroll 1
       for (int b = n_early; b < nkb; ++b) fetch(b);
   } else if (warp >= 5) {
     // ---------------- loaders ----------------
@@ -1043,6 +1054,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     auto issue_block = [&](int b) {
       uint8_t* dstb = ring + (b % ATT_STAGES) * ATT_STAGE_BYTES + (is_k ? 0 : ATT_KB * 128);
       if (!PROMPT) {
+#pragma unroll 1
         for (int i = lt; i < ATT_KB * 8; i += nl) {
           const int row = i >> 3, j = i & 7;
           const int key = b * ATT_KB + row;
@@ -1057,6 +1069,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         }
       } else if ((b + 1) * ATT_KB <= n_prompt) {
         // a block of prompt rows only: row index = key
+#pragma unroll 1
         for (int i = lt; i < ATT_KB * 8; i += nl) {
           const int row = i >> 3, j = i & 7;
           const int off = row * 128 + ((j ^ (row & 7)) << 4);
@@ -1065,6 +1078,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         }
       } else {
         // the block where the prompt rows end and the ring behind them begins (or ring rows only)
+#pragma unroll 1
         for (int i = lt; i < ATT_KB * 8; i += nl) {
           const int row = i >> 3, j = i & 7;
           const int key = b * ATT_KB + row;
@@ -1087,10 +1101,12 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     // complete - the retained history behind them
     const int carried = PROMPT ? (n_prompt == si.n_prompt0 ? n_prompt + si.kv_len : si.n_prompt0) : si.kv_len;
     const int n_early = min(min(carried / ATT_KB, ATT_STAGES), nkb);
+#pragma unroll 1
     for (int b = 0; b < n_early; ++b) issue_block(b);
     ptx::pdl_wait();
     if (is_k) {
       const bf16* qbase = p.q + (long long)(GUARD + slot * SLOT_ROWS + HALO) * p.ld + head * p.dh;
+#pragma unroll 1
       for (int i = lt; i < 128 * 8; i += nl) {
         const int row = i >> 3, j = i & 7, qrow = row & 63;   // rows 64.. repeat rows 0..
         uint8_t* dst = sQ + row * 128 + ((j ^ (row & 7)) << 4);
@@ -1099,6 +1115,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       }
     }
     bool ok = true;
+#pragma unroll 1
     for (int b = 0; b < nkb; ++b) {
       const int st = b % ATT_STAGES;
       if (b >= 1) {   // the previous block has been issued a whole iteration ago: publish it (block 0 together with Q)
@@ -1139,6 +1156,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       };
       if (BULK && !ptx::mbar_wait(bar_q, 0)) { ok = false; atomicExch(p.err, 12); }
       issue_s(0);
+#pragma unroll 1
       for (int b = 0; b < nkb; ++b) {
         const int st = b % ATT_STAGES;
         if (b + 1 < nkb) {
@@ -1159,6 +1177,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           for (int k = 0; k < ATT_KB / 16; ++k)
             ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
         } else {
+#pragma unroll 1
           for (int k = 0; k < ksteps; ++k)
             ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
         }
@@ -1175,8 +1194,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     bool ok = true;
     // reference and row sum of this block's stream and of the other one (they change places after every block)
     float m_ref = -INFINITY, lsum = 0.f, m_oth = -INFINITY, l_oth = 0.f;
+#pragma unroll 1
     for (int b = 0; b < nkb; ++b) {
       if (ok && !ptx::mbar_wait(bar_s, b & 1)) { ok = false; atomicExch(p.err, 7); }
+      __syncwarp();
       ptx::tc_fence_after();
       float v[64];
       ptx::tmem_ld64(lane_addr + (uint32_t)(half * 64), v);
@@ -1190,6 +1211,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       ptx::named_bar_sync(2, 128);   // all have read: the next block (or the row sums below) may overwrite the exchange
       if (b >= 2) {   // this block's P buffer was last read by P V of block b - 2, which also completes this stream's O
         if (ok && !ptx::mbar_wait(&bar_pv[b & 1], ((b >> 1) - 1) & 1)) { ok = false; atomicExch(p.err, 15); }
+        __syncwarp();
       }
       if (b < 2) {
         m_ref = mx;
@@ -1201,6 +1223,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           if (need) m_ref = mx;
           lsum *= alpha;
           if (half == 0) {                        // O rows 0..63 live in lanes 0..63
+#pragma unroll 1
             for (int c = 0; c < p.dh; c += 16) {
               float o16[16];
               const uint32_t addr = lane_addr + (uint32_t)(ATT_KB + (b & 1) * 64 + c);
@@ -1226,6 +1249,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     }
     if (nkb >= 2 && ok && !ptx::mbar_wait(&bar_pv[nkb & 1], ((nkb - 2) >> 1) & 1)) { ok = false; atomicExch(p.err, 8); }
     if (ok && !ptx::mbar_wait(&bar_pv[(nkb - 1) & 1], ((nkb - 1) >> 1) & 1)) { ok = false; atomicExch(p.err, 9); }
+    __syncwarp();
     ptx::tc_fence_after();
     s_x[half * 64 + row] = lsum;
     ptx::named_bar_sync(2, 128);
@@ -1236,6 +1260,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     float c0, c1;
     att_combine(nkb, m_ref, l0, m_oth, s_x[row] + s_x[64 + row], &c0, &c1);
     bf16* orow = p.o + (long long)(GUARD + slot * SLOT_ROWS + HALO + row) * p.ld + head * p.dh;
+#pragma unroll 1
     for (int c = 0; c < (half == 0 ? p.dh : 0); c += 16) {
       float o16[16], q16[16];
       ptx::tmem_ld16(lane_addr + (uint32_t)(ATT_KB + c), o16);

@@ -44,6 +44,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // short, implementation-defined time), which is orders of magnitude beyond any legitimate wait here.
 constexpr uint32_t kMaxPolls = 4u << 20;
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, uint32_t max_polls) {
+#pragma unroll 1   // (waits are everywhere: unrolled they were a third of a kernel's code, and code comes through the instruction cache)
   for (uint32_t i = 0; i < max_polls; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
@@ -54,6 +55,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) { retu
 // main loop, so that their polling does not compete with the issuing warps for issue slots and
 // shared-memory bandwidth.
 __device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
   for (uint32_t i = 0; i < kMaxPolls; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     __nanosleep(100);
