@@ -99,7 +99,7 @@ struct GemmParams {
   long long    halo_off;        // element offset of the next conv's carry inside SlotInfo::halo, or -1
   bf16*        q_out;           // MODE_QKV
   long long    kv_off;          // element offset of this (step, layer)'s K ring inside SlotInfo::kv
-  int          kv_rs, kv_hs;    // K/V planes: elements between a head's consecutive rows / between heads
+  int          kv_hs;           // K/V planes: elements between heads (a head's rows are consecutive)
   int          dh_shift;        // log2(head_dim)
   int          Rk;              // ring rows
   int          P;               // prompt rows in front of the ring (0: none)
@@ -148,6 +148,11 @@ __device__ __forceinline__ void store16(bf16* p, const uint4& a, const uint4& b)
   *reinterpret_cast<uint4*>(p) = a;
   *reinterpret_cast<uint4*>(p + 8) = b;
 }
+
+// A head's K / V row is stored with its 16-byte chunks in the order of the swizzled shared-memory row that the attention kernels
+// copy it to: chunk c of plane row r at position c ^ kv_perm (128-byte rows in the 128-byte swizzle, 64-byte rows in the 64-byte
+// one).  A thread's two chunks of 16 columns stay inside their 32 bytes, swapped for odd kv_perm.
+__device__ __forceinline__ int kv_perm(int row, int dh_shift) { return dh_shift == 6 ? row & 7 : (row >> 1) & 3; }
 
 // PAIR: the CTAs of two adjacent row tiles (a cluster of two along x, one TPC) run ONE 256-row UMMA per
 // reduction step.  Each stages its own activation rows and only HALF of the weight tile (tmB then has boxes
@@ -585,12 +590,10 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               row += p.P;
             }
             const int hh = col >> p.dh_shift, wi = col - (hh << p.dh_shift);
-            // head_dim 64: a K / V row is stored with its 16-byte chunks in the order of the swizzled shared-memory row
-            // that the attention kernel copies it to, chunk c at position c ^ (row & 7).  The two chunks of this
-            // thread stay inside their 32 bytes, swapped for odd rows.
-            const int wp = p.dh_shift == 6 ? ((((wi >> 3) ^ (row & 7)) & ~1) << 3) : wi;
-            const bool swap = p.dh_shift == 6 && (row & 1);
-            store16(si.kv + p.kv_off + (long long)(which - 1) * (p.P + p.Rk) * p.C + (long long)hh * p.kv_hs + (long long)row * p.kv_rs + wp,
+            const int perm = kv_perm(row, p.dh_shift);
+            const int wp = (((wi >> 3) ^ perm) & ~1) << 3;
+            const bool swap = perm & 1;
+            store16(si.kv + p.kv_off + (long long)(which - 1) * (p.P + p.Rk) * p.C + (long long)hh * p.kv_hs + ((long long)row << p.dh_shift) + wp,
                     swap ? b : a, swap ? a : b);
           }
         }
@@ -746,10 +749,11 @@ __global__ void flow_rmsnorm_kernel(const SlotInfo* slots, int n_slots, const bf
 // in the 128 UMMA rows (row 64 + i repeats row i), so that S has a copy of every query row in both
 // halves of tensor memory: a warp can only read the 32 lanes of its own SM sub-partition, and with
 // the copy the softmax work spreads over all four sub-partitions (special-function throughput is
-// what bounds it) instead of the two that own lanes 0..63.  Keys/values: the kv_len carried frames
-// followed by the chunk's own T frames, streamed in place from the stream's ring in blocks of 128
-// keys with 128-bit cp.async loads (the ring may wrap; nothing is compacted or copied in global
-// memory) through a two-stage shared-memory ring.
+// what bounds it) instead of the two that own lanes 0..63.  Keys/values: prompt rows, carried
+// frames and the chunk's own, streamed in place from the stream's planes in blocks of 128 keys by
+// untiled bulk copies (see AttKeys) through a two-stage shared-memory ring.  Copies of 16 bytes per
+// thread instead took a loader warp about 2,800 cycles of issue per block: with prompt rows
+// 1,237 -> 1,115 us per chunk, head_dim 32 430 -> 409.
 //
 // Warp roles (8 warps): warps 0..3 = softmax (thread = (query row, half of the block's 128 key
 // columns); warps 0,1 read lanes 0..63 and own key columns 0..63, warps 2,3 read the copy in lanes
@@ -765,8 +769,7 @@ constexpr int ATT_THREADS = 256;
 constexpr int ATT_KB = 128;             // keys per block
 constexpr int ATT_STAGES = 2;
 constexpr int ATT_TMEM_COLS = 256;      // S (128 columns) + the two O accumulators (64 columns each); two CTAs share the SM's 512
-constexpr int ATT_K_LOADERS = 64;       // warps 5 and 6: Q, then the K blocks
-constexpr int ATT_V_LOADERS = 32;       // warp 7: the V blocks
+constexpr int ATT_K_LOADERS = 64;       // warps 5 and 6 copy Q
 constexpr int ATT_Q_BYTES = 128 * 128;  // 64 query rows, twice
 constexpr int ATT_P_BYTES = 2 * 64 * 128;   // one P buffer: 64 rows x 128 keys; there are two
 constexpr int ATT_STAGE_BYTES = 2 * ATT_KB * 128;   // K block + V block
@@ -783,9 +786,8 @@ struct AttnParams {
   const bf16*     q;          // [GUARD + rows][ld]
   bf16*           o;          // [GUARD + rows][ld]
   int             ld;
-  int             dh;         // 32 or 64 (smem rows are padded to 64 columns)
   long long       kv_off;     // element offset of this (step, layer)'s K ring inside SlotInfo::kv
-  int             kv_rs, kv_hs;   // K/V planes: elements between a head's consecutive rows / between heads
+  int             kv_hs;      // K/V planes: elements between heads (a head's rows are consecutive)
   int             Rk, C;
   int             P;          // prompt rows in front of the ring
   float           scale_log2e;  // log2(e) / sqrt(dh)
@@ -837,17 +839,17 @@ __device__ __forceinline__ float2 silu2(float2 z) {   // silu_f of both halves
 // each with its own reference, row sum and output accumulator, combined at the end (att_combine): the products of a block need
 // not wait for the block before, and two groups of warps can work on them at once.
 
-// Masks the padding (columns >= valid; the first `skip` columns) and returns the largest score.
-__device__ __forceinline__ float att_mask_max(float (&v)[64], int valid, int skip) {
+// Masks the padding (columns >= valid) and the gap (columns g0 .. g1 - 1) and returns the largest score.
+__device__ __forceinline__ float att_mask_max(float (&v)[64], int valid, int g0, int g1) {
   if (valid < 64) {                            // only the last block has padded key columns
 #pragma unroll
     for (int i = 0; i < 64; ++i)
       if (i >= valid) v[i] = -INFINITY;
   }
-  if (skip > 0) {
+  if (g1 > 0 && g0 < 64) {
 #pragma unroll
-    for (int i = 0; i < 7; ++i)
-      if (i < skip) v[i] = -INFINITY;
+    for (int i = 0; i < 64; ++i)
+      if (i >= g0 && i < g1) v[i] = -INFINITY;
   }
   float m[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
@@ -890,17 +892,57 @@ __device__ __forceinline__ void att_combine(int nkb, float m0, float l0, float m
   }
 }
 
-// PROMPT = false: the carry is a plain window (no prompt rows); a separate instantiation, because this kernel sits at its
-// register limit and the copy loops of its loader warps pace it.
-// BULK (no prompt rows, head_dim 64): a head's K / V rows are 128 contiguous bytes each, stored with their 16-byte
-// chunks already in the order of the swizzled shared-memory row they will occupy (chunk c of plane row r at
-// position c ^ (r & 7)), and the ring is walked from the 8-row boundary below the attended interval, so that a block
-// of 128 keys is one flat span of 16 KB (two at the ring's wrap) with shared-memory row == plane row (mod 8): ONE thread
-// fetches it with one or two untiled bulk copies that complete on the stage's barrier.  The up to seven keys in front
-// of the interval are masked like the padding behind it.  Without BULK the loader warps copy 16 bytes per thread and
-// instruction (about 2,800 cycles of issue per block and warp).
-template <bool PROMPT, bool BULK>
+// The keys of one head of one slot, as an axis of plane rows that bulk copies can fetch: prompt rows 0 .. n_prompt - 1 (with the
+// chunk's own prompt frames), then the circular interval of the history ring behind the P prompt rows (with the chunk's history
+// frames).  Every block of 128 keys consists of at most three flat spans whose plane rows are congruent (mod 8) to the
+// shared-memory rows they land in - the prompt rows are taken up to a multiple of 8, the ring is entered at the 8-row boundary below
+// the interval (it has a multiple of 8 rows), so that the stored chunk order is the swizzle.  The up to 14 keys between the two,
+// [g0, g1), are rows of something else: weight 0.
+struct AttKeys {
+  int L;            // keys on the axis
+  int nkb;          // blocks of ATT_KB keys
+  int g0, g1;       // the gap
+  int a8;           // keys [0, a8) are plane rows [0, a8); key a8 + i is ring row (row0 + i), wrapping at P + Rk to P
+  int row0;
+  int n_early;      // leading blocks that hold only rows of earlier chunks
+  __device__ __forceinline__ void set(const SlotInfo& si, int P, int Rk) {
+    const int tp = max(0, min(si.T, P - si.n_prompt0)), n_prompt = si.n_prompt0 + tp;   // tp frames of the chunk complete the prompt
+    const int hist = si.kv_len + si.T - tp;
+    int start = si.kv_head - si.kv_len;          // ring row of the oldest attended history frame
+    if (start < 0) start += Rk;
+    const int phi = (P + start) & 7;
+    row0 = P + start - phi;
+    a8 = hist > 0 ? (n_prompt + 7) & ~7 : n_prompt;
+    L = a8 + (hist > 0 ? phi + hist : 0);
+    g0 = n_prompt;
+    g1 = hist > 0 ? a8 + phi : n_prompt;
+    nkb = (L + ATT_KB - 1) / ATT_KB;
+    n_early = min((tp > 0 ? si.n_prompt0 : a8 + (hist > 0 ? phi + si.kv_len : 0)) / ATT_KB, nkb);
+  }
+  // Rows of block b (n of them) of one plane -> dst, completion on bar; one thread.
+  __device__ __forceinline__ void fetch(const bf16* plane, int b, int n, int P, int Rk, int dh_shift, uint8_t* dst, uint64_t* bar) const {
+    const int row_bytes = 2 << dh_shift, k0 = b * ATT_KB, na = min(n, max(0, a8 - k0));
+    ptx::mbar_expect_tx(bar, (uint32_t)(n * row_bytes));
+    if (na > 0) ptx::bulk_load(dst, plane + ((long long)k0 << dh_shift), (uint32_t)(na * row_bytes), bar);
+    if (n > na) {
+      int rr = row0 + max(0, k0 - a8);
+#pragma unroll 1
+      while (rr >= P + Rk) rr -= Rk;
+      const int n1 = min(n - na, P + Rk - rr);
+      ptx::bulk_load(dst + na * row_bytes, plane + ((long long)rr << dh_shift), (uint32_t)(n1 * row_bytes), bar);
+      if (na + n1 < n) ptx::bulk_load(dst + (na + n1) * row_bytes, plane + ((long long)P << dh_shift), (uint32_t)((n - na - n1) * row_bytes), bar);
+    }
+  }
+};
+
+template <int DH>
+__device__ __forceinline__ uint64_t att_kv_desc(uint32_t smem_addr) {
+  return DH == 64 ? ptx::umma_desc_sw128(smem_addr) : ptx::umma_desc_sw64(smem_addr);
+}
+
+template <int DH>
 __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnParams p) {
+  constexpr int DHS = DH == 64 ? 6 : 5;
   extern __shared__ __align__(1024) uint8_t att_smem_raw[];
   uint8_t* smem = att_smem_raw;
   if (p.empty) {
@@ -927,20 +969,19 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
   uint64_t* bar_p = bar_s + 1;          // [2]: all softmax threads have written P(b) into buffer b & 1
   uint64_t* bar_pv = bar_p + 2;         // [2]: P(b) V(b) has been accumulated: buffer b & 1 is free, O holds blocks <= b
   uint64_t* bar_sfree = bar_pv + 2;     // every softmax thread has copied its S columns to registers
-  uint64_t* bar_q = bar_sfree + 1;      // BULK: Q has landed (without BULK it is published with the first K block)
+  uint64_t* bar_q = bar_sfree + 1;      // Q has landed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_sfree + 2);
   float* s_x = reinterpret_cast<float*>(tmem_slot + 2);   // [2][64] exchange between the two column halves
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int slot = blockIdx.x, head = blockIdx.y;
-  const int chunks = p.dh >> 3;             // 16-byte chunks per head row
 
   if (tid == 0) {
 #pragma unroll 1
     for (int i = 0; i < ATT_STAGES; ++i) {
-      ptx::mbar_init(&full_k[i], BULK ? 1 : ATT_K_LOADERS);
+      ptx::mbar_init(&full_k[i], 1);
       ptx::mbar_init(&empty_k[i], 1);
-      ptx::mbar_init(&full_v[i], BULK ? 1 : ATT_V_LOADERS);
+      ptx::mbar_init(&full_v[i], 1);
       ptx::mbar_init(&empty_v[i], 1);
     }
     ptx::mbar_init(bar_s, 1);
@@ -965,31 +1006,24 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
   // and wait afterwards.
   if (warp < 5) ptx::pdl_wait();
   const SlotInfo si = p.slots[slot];
-  // attended keys, in this order: the prompt rows (with the chunk's own prompt frames, already appended), then
-  // the carried history and the chunk's history frames, a circular interval of the ring behind the prompt rows
   const int T = si.T;
-  const int n_prompt = PROMPT ? si.n_prompt0 + min(T, p.P - si.n_prompt0) : 0;
-  const int L0 = PROMPT ? n_prompt + si.kv_len + (T - (n_prompt - si.n_prompt0)) : si.kv_len + T;
-  int ring_start = si.kv_head - si.kv_len;      // ring row of the oldest attended history frame
-  if (ring_start < 0) ring_start += p.Rk;
-  const int phi = BULK ? (ring_start & 7) : 0;  // BULK: keys 0 .. phi - 1 are the rows between the 8-row boundary and the interval
-  const int L = L0 + phi;
-  const int nkb = (L + ATT_KB - 1) / ATT_KB;
+  AttKeys ak;
+  ak.set(si, p.P, p.Rk);
+  const int L = ak.L, nkb = ak.nkb;
 
   if (T == 0) {
     // a slot without frames (a hole in a wavefront): nothing to do but to release tensor memory below
-  } else if (BULK && warp >= 5) {
-    // ---------------- loaders, bulk copies: lane 0 of warp 5 fetches the K blocks, lane 0 of warp 7 the V blocks;
-    // warps 5 and 6 copy Q (64 rows of the projection's output, each held twice) ----------------
+  } else if (warp >= 5) {
+    // ---------------- loaders: one lane of warp 5 fetches the K blocks, one of warp 7 the V blocks; warps 5 and 6 copy Q (64
+    // rows of the projection's output, each held twice) ----------------
     const bool is_k = warp != 7;
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    const bf16* src0 = si.kv + p.kv_off + (long long)head * p.kv_hs + (is_k ? 0 : (long long)p.Rk * p.C);
+    const bf16* plane = si.kv + p.kv_off + (long long)head * p.kv_hs + (is_k ? 0 : (long long)(p.P + p.Rk) * p.C);
     uint64_t* full = is_k ? full_k : full_v;
     uint64_t* empty = is_k ? empty_k : empty_v;
-    const int row0 = ring_start - phi;                     // a multiple of 8 (the ring has a multiple of 8 rows)
-    const int n_early = min(min((si.kv_len + phi) / ATT_KB, ATT_STAGES), nkb);   // blocks of carried rows only (< nkb: the chunk's rows come last)
+    const int n_early = min(ak.n_early, ATT_STAGES);
     bool ok = true;
-    auto fetch = [&](int b) {                               // warps 5 and 7, all lanes (lane 0 issues)
+    auto fetch = [&](int b) {                               // warps 5 and 7, all lanes (one issues)
       const int st = b % ATT_STAGES;
       if (b >= ATT_STAGES && ok && !ptx::mbar_wait_relaxed(&empty[st], ((b / ATT_STAGES) - 1) & 1)) {
         ok = false;
@@ -1002,19 +1036,11 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         // the P V product reads whole 16-row steps: the rows behind the last key must be finite (their weights are 0)
         const int n16 = min(ATT_KB, (n + 15) & ~15);
 #pragma unroll 1
-        for (int i = lane; i < (n16 - n) * 8; i += 32) *reinterpret_cast<uint4*>(dstb + n * 128 + i * 16) = zero;
+        for (int i = lane; i < (n16 - n) * (DH / 8); i += 32) *reinterpret_cast<uint4*>(dstb + n * 2 * DH + i * 16) = zero;
         ptx::fence_proxy_async_smem();
         __syncwarp();
       }
-      if (ptx::elect_one()) {
-        int rr = row0 + b * ATT_KB;
-#pragma unroll 1
-        while (rr >= p.Rk) rr -= p.Rk;
-        const int n1 = min(n, p.Rk - rr);
-        ptx::mbar_expect_tx(&full[st], (uint32_t)n * 128u);
-        ptx::bulk_load(dstb, src0 + (long long)rr * 64, (uint32_t)n1 * 128u, &full[st]);
-        if (n1 < n) ptx::bulk_load(dstb + n1 * 128, src0, (uint32_t)(n - n1) * 128u, &full[st]);
-      }
+      if (ptx::elect_one()) ak.fetch(plane, b, n, p.P, p.Rk, DHS, dstb, &full[st]);
       __syncwarp();
     };
     if (warp != 6)
@@ -1023,10 +1049,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     ptx::pdl_wait();                                        // Q and the chunk's own K / V rows are the projection's output
     if (is_k) {
       const int lt = (warp == 6 ? 32 : 0) + lane;
-      const bf16* qbase = p.q + (long long)(GUARD + slot * SLOT_ROWS + HALO) * p.ld + head * 64;
-#pragma unroll 1
-      for (int i = lt; i < 128 * 8; i += ATT_K_LOADERS) {
-        const int row = i >> 3, j = i & 7, qrow = row & 63;   // rows 64.. repeat rows 0..
+      const bf16* qbase = p.q + (long long)(GUARD + slot * SLOT_ROWS + HALO) * p.ld + head * DH;
+#pragma unroll 4
+      for (int i = lt; i < 128 * (DH / 8); i += ATT_K_LOADERS) {
+        const int row = i / (DH / 8), j = i % (DH / 8), qrow = row & 63;   // rows 64.. repeat rows 0..
         uint8_t* dst = sQ + row * 128 + ((j ^ (row & 7)) << 4);
         if (qrow < T) cp_async16(dst, qbase + (long long)qrow * p.ld + j * 8);
         else *reinterpret_cast<uint4*>(dst) = zero;
@@ -1038,106 +1064,11 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     if (warp != 6)
 #pragma unroll 1
       for (int b = n_early; b < nkb; ++b) fetch(b);
-  } else if (warp >= 5) {
-    // ---------------- loaders ----------------
-    const bool is_k = warp != 7;
-    const int nl = is_k ? ATT_K_LOADERS : ATT_V_LOADERS;
-    const int lt = (warp == 6 ? 32 : 0) + lane;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    const bf16* src0 = si.kv + p.kv_off + (long long)head * p.kv_hs + (is_k ? 0 : (long long)((PROMPT ? p.P : 0) + p.Rk) * p.C);
-    const int rs = p.kv_rs;
-    uint64_t* full = is_k ? full_k : full_v;
-    uint64_t* empty = is_k ? empty_k : empty_v;
-    const int start = ring_start;
-    // head_dim 64: chunk j of plane row rr is stored at position j ^ (rr & 7) (see BULK); head_dim 32 rows are stored plainly
-    const int perm = p.dh == 64 ? 7 : 0;
-    auto issue_block = [&](int b) {
-      uint8_t* dstb = ring + (b % ATT_STAGES) * ATT_STAGE_BYTES + (is_k ? 0 : ATT_KB * 128);
-      if (!PROMPT) {
-#pragma unroll 1
-        for (int i = lt; i < ATT_KB * 8; i += nl) {
-          const int row = i >> 3, j = i & 7;
-          const int key = b * ATT_KB + row;
-          const int off = row * 128 + ((j ^ (row & 7)) << 4);
-          if (key < L && j < chunks) {
-            int rr = start + key;
-            if (rr >= p.Rk) rr -= p.Rk;
-            cp_async16(dstb + off, src0 + (long long)rr * rs + ((j ^ (rr & perm)) << 3));
-          } else {
-            *reinterpret_cast<uint4*>(dstb + off) = zero;   // for V: 0 * garbage must not poison O
-          }
-        }
-      } else if ((b + 1) * ATT_KB <= n_prompt) {
-        // a block of prompt rows only: row index = key
-#pragma unroll 1
-        for (int i = lt; i < ATT_KB * 8; i += nl) {
-          const int row = i >> 3, j = i & 7;
-          const int off = row * 128 + ((j ^ (row & 7)) << 4);
-          if (j < chunks) cp_async16(dstb + off, src0 + (long long)(b * ATT_KB + row) * rs + ((j ^ (row & perm)) << 3));
-          else *reinterpret_cast<uint4*>(dstb + off) = zero;
-        }
-      } else {
-        // the block where the prompt rows end and the ring behind them begins (or ring rows only)
-#pragma unroll 1
-        for (int i = lt; i < ATT_KB * 8; i += nl) {
-          const int row = i >> 3, j = i & 7;
-          const int key = b * ATT_KB + row;
-          const int off = row * 128 + ((j ^ (row & 7)) << 4);
-          if (key < L && j < chunks) {
-            int rr = key;                            // a prompt row, or ...
-            if (key >= n_prompt) {                   // ... a ring row behind the prompt rows
-              rr = start + key - n_prompt;
-              if (rr >= p.Rk) rr -= p.Rk;
-              rr += p.P;
-            }
-            cp_async16(dstb + off, src0 + (long long)rr * rs + ((j ^ (rr & perm)) << 3));
-          } else {
-            *reinterpret_cast<uint4*>(dstb + off) = zero;
-          }
-        }
-      }
-    };
-    // keys [0, carried) were appended by earlier steps: the prompt rows already there, and - once the prompt is
-    // complete - the retained history behind them
-    const int carried = PROMPT ? (n_prompt == si.n_prompt0 ? n_prompt + si.kv_len : si.n_prompt0) : si.kv_len;
-    const int n_early = min(min(carried / ATT_KB, ATT_STAGES), nkb);
-#pragma unroll 1
-    for (int b = 0; b < n_early; ++b) issue_block(b);
-    ptx::pdl_wait();
-    if (is_k) {
-      const bf16* qbase = p.q + (long long)(GUARD + slot * SLOT_ROWS + HALO) * p.ld + head * p.dh;
-#pragma unroll 1
-      for (int i = lt; i < 128 * 8; i += nl) {
-        const int row = i >> 3, j = i & 7, qrow = row & 63;   // rows 64.. repeat rows 0..
-        uint8_t* dst = sQ + row * 128 + ((j ^ (row & 7)) << 4);
-        if (qrow < T && j < chunks) cp_async16(dst, qbase + (long long)qrow * p.ld + j * 8);
-        else *reinterpret_cast<uint4*>(dst) = zero;
-      }
-    }
-    bool ok = true;
-#pragma unroll 1
-    for (int b = 0; b < nkb; ++b) {
-      const int st = b % ATT_STAGES;
-      if (b >= 1) {   // the previous block has been issued a whole iteration ago: publish it (block 0 together with Q)
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        ptx::fence_proxy_async_smem();
-        ptx::mbar_arrive(&full[(b - 1) % ATT_STAGES]);
-      }
-      if (b < n_early) continue;                                // already in flight
-      if (b >= ATT_STAGES && ok && !ptx::mbar_wait_relaxed(&empty[st], ((b / ATT_STAGES) - 1) & 1)) {
-        ok = false;
-        atomicExch(p.err, 4);
-      }
-      issue_block(b);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    ptx::fence_proxy_async_smem();
-    ptx::mbar_arrive(&full[(nkb - 1) % ATT_STAGES]);
   } else if (warp == 4) {
     // ---------------- UMMA issuer ----------------
     if (ptx::elect_one()) {
       const uint32_t idesc_s = ptx::umma_idesc_bf16(128, ATT_KB, 0, 0);
-      const uint32_t idesc_pv = ptx::umma_idesc_bf16(128, 64, 0, 1);   // B = V, MN-major
+      const uint32_t idesc_pv = ptx::umma_idesc_bf16(128, DH, 0, 1);   // B = V, MN-major
       const uint64_t dq = ptx::umma_desc_sw128(ptx::smem_u32(sQ));
       const uint64_t dp = ptx::umma_desc_sw128(ptx::smem_u32(sP));
       bool ok = true;
@@ -1148,13 +1079,13 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         const int st = b % ATT_STAGES;
         if (ok && !ptx::mbar_wait(&full_k[st], (b / ATT_STAGES) & 1)) { ok = false; atomicExch(p.err, 5); }
         ptx::tc_fence_after();
-        const uint64_t dk = ptx::umma_desc_sw128(ptx::smem_u32(ring + st * ATT_STAGE_BYTES));
+        const uint64_t dk = att_kv_desc<DH>(ptx::smem_u32(ring + st * ATT_STAGE_BYTES));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) ptx::umma_bf16(tmem_base, dq + 2 * k, dk + 2 * k, idesc_s, k != 0);
+        for (int k = 0; k < DH / 16; ++k) ptx::umma_bf16(tmem_base, dq + 2 * k, dk + 2 * k, idesc_s, k != 0);
         ptx::umma_commit(bar_s);
         ptx::umma_commit(&empty_k[st]);                  // the K stage is free once S(b) has been computed
       };
-      if (BULK && !ptx::mbar_wait(bar_q, 0)) { ok = false; atomicExch(p.err, 12); }
+      if (!ptx::mbar_wait(bar_q, 0)) { ok = false; atomicExch(p.err, 12); }
       issue_s(0);
 #pragma unroll 1
       for (int b = 0; b < nkb; ++b) {
@@ -1167,19 +1098,19 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         const uint64_t dpb = dp + (uint64_t)((b & 1) * (ATT_P_BYTES >> 4));
         if (ok && !ptx::mbar_wait(&full_v[st], (b / ATT_STAGES) & 1)) { ok = false; atomicExch(p.err, 11); }
         ptx::tc_fence_after();
-        const uint64_t dv = ptx::umma_desc_sw128(ptx::smem_u32(ring + st * ATT_STAGE_BYTES + ATT_KB * 128));
+        const uint64_t dv = att_kv_desc<DH>(ptx::smem_u32(ring + st * ATT_STAGE_BYTES + ATT_KB * 128));
         const int valid = L - b * ATT_KB;
         const int ksteps = valid >= ATT_KB ? ATT_KB / 16 : (valid + 15) / 16;
-        // P tile k/4 (8 KB apart), 32-byte K steps; V: 16 key rows = 2 KB per step; even blocks into O_0, odd ones into O_1
+        // P tile k/4 (8 KB apart), 32-byte K steps; V: 16 key rows per step; even blocks into O_0, odd ones into O_1
         const uint32_t d_o = tmem_base + ATT_KB + (uint32_t)(b & 1) * 64u;
         if (ksteps == ATT_KB / 16) {
 #pragma unroll
           for (int k = 0; k < ATT_KB / 16; ++k)
-            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
+            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2 * DH)), idesc_pv, (b >> 1 | k) != 0);
         } else {
 #pragma unroll 1
           for (int k = 0; k < ksteps; ++k)
-            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2048 >> 4)), idesc_pv, (b >> 1 | k) != 0);
+            ptx::umma_bf16(d_o, dpb + (uint64_t)((k >> 2) * (8192 >> 4) + (k & 3) * 2), dv + (uint64_t)(k * (2 * DH)), idesc_pv, (b >> 1 | k) != 0);
         }
         ptx::umma_commit(&empty_v[st]);
         ptx::umma_commit(&bar_pv[b & 1]);
@@ -1203,8 +1134,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
       ptx::tmem_ld64(lane_addr + (uint32_t)(half * 64), v);
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar_sfree);               // S(b) is in registers: the next block's scores may overwrite it
-      // (the first phi columns are the rows between the 8-row boundary and the attended interval)
-      float mx = att_mask_max(v, L - b * ATT_KB - half * 64, BULK && b == 0 && half == 0 ? phi : 0);
+      const int col0 = b * ATT_KB + half * 64;
+      float mx = att_mask_max(v, L - col0, ak.g0 - col0, ak.g1 - col0);
       s_x[half * 64 + row] = mx * p.scale_log2e;
       ptx::named_bar_sync(2, 128);
       mx = fmaxf(s_x[row], s_x[64 + row]);
@@ -1224,7 +1155,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           lsum *= alpha;
           if (half == 0) {                        // O rows 0..63 live in lanes 0..63
 #pragma unroll 1
-            for (int c = 0; c < p.dh; c += 16) {
+            for (int c = 0; c < DH; c += 16) {
               float o16[16];
               const uint32_t addr = lane_addr + (uint32_t)(ATT_KB + (b & 1) * 64 + c);
               ptx::tmem_ld16(addr, o16);
@@ -1259,9 +1190,9 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
     ptx::named_bar_sync(2, 128);
     float c0, c1;
     att_combine(nkb, m_ref, l0, m_oth, s_x[row] + s_x[64 + row], &c0, &c1);
-    bf16* orow = p.o + (long long)(GUARD + slot * SLOT_ROWS + HALO + row) * p.ld + head * p.dh;
+    bf16* orow = p.o + (long long)(GUARD + slot * SLOT_ROWS + HALO + row) * p.ld + head * DH;
 #pragma unroll 1
-    for (int c = 0; c < (half == 0 ? p.dh : 0); c += 16) {
+    for (int c = 0; c < (half == 0 ? DH : 0); c += 16) {
       float o16[16], q16[16];
       ptx::tmem_ld16(lane_addr + (uint32_t)(ATT_KB + c), o16);
       if (nkb > 1) ptx::tmem_ld16(lane_addr + (uint32_t)(ATT_KB + 64 + c), q16);
@@ -1369,7 +1300,7 @@ struct FlowModel {
   Profiler* prof = nullptr;
   // launch plumbing
   bool pdl = true;                       // programmatic dependent launch between the step's kernels
-  int  kv_rs = 0, kv_hs = 0, dh_shift = 0;   // K/V plane layout (see GemmParams)
+  int  kv_hs = 0, dh_shift = 0;   // K/V plane layout (see GemmParams)
   int  n_sm = 148;                       // SMs of the device (read at create)
   cudaStream_t cap_stream = nullptr;     // used only to capture graphs at create
   std::map<int, GraphEntry> graphs;      // batch size -> captured chunk step
@@ -1550,7 +1481,7 @@ dc_status flow_model_create(const dc_config& cfg, const float* w, FlowModel** ou
   if (e == cudaSuccess)
     chk(cudaFuncSetAttribute(flow_gemm_kernel<true, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM_MAX_PAIR));
   if (e == cudaSuccess && cfg.n_attn > 0)
-    chk(cudaFuncSetAttribute(m->P > 0 ? flow_attn_kernel<true, false> : (cfg.head_dim == 64 ? flow_attn_kernel<false, true> : flow_attn_kernel<false, false>),
+    chk(cudaFuncSetAttribute(cfg.head_dim == 64 ? flow_attn_kernel<64> : flow_attn_kernel<32>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ATT_SMEM));
   if (e != cudaSuccess) {
     set_error("flow model allocation failed: %s", cudaGetErrorString(e));
@@ -1587,7 +1518,6 @@ dc_status flow_model_create(const dc_config& cfg, const float* w, FlowModel** ou
     m->pdl = !(cfg.options & DC_OPT_NO_PDL);
     // K/V planes are head-major: the rows one attention CTA streams are contiguous
     m->dh_shift = m->cfg.head_dim == 64 ? 6 : 5;
-    m->kv_rs = m->cfg.head_dim;
     m->kv_hs = (m->P + m->Rk) * m->cfg.head_dim;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
@@ -1832,14 +1762,14 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
   };
   auto attention = [&](int step, int layer) {
     AttnParams p{};
-    p.slots = m->d_slots; p.q = m->Q; p.o = m->O; p.ld = C; p.dh = c.head_dim;
+    p.slots = m->d_slots; p.q = m->Q; p.o = m->O; p.ld = C;
     p.kv_off = ((long long)step * c.n_attn + layer) * 2 * (m->P + m->Rk) * C;
     p.Rk = m->Rk; p.C = C; p.P = m->P;
-    p.kv_rs = m->kv_rs; p.kv_hs = m->kv_hs;
+    p.kv_hs = m->kv_hs;
     p.scale_log2e = (float)(1.4426950408889634 / sqrt((double)c.head_dim));
     p.err = m->d_err;
     p.empty = (c.options & DC_OPT_EMPTY_KERNELS) ? 1 : 0;
-    launch(lc, m->P > 0 ? flow_attn_kernel<true, false> : (c.head_dim == 64 ? flow_attn_kernel<false, true> : flow_attn_kernel<false, false>),
+    launch(lc, c.head_dim == 64 ? flow_attn_kernel<64> : flow_attn_kernel<32>,
            dim3(n, c.n_heads), dim3(ATT_THREADS), ATT_SMEM, true, 2, p);
   };
   const float* fc = m->fconst;
@@ -1881,7 +1811,7 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
           p.mode = MODE_QKV; p.BN = bq; p.n_kblocks = C / KBLK; p.taps = 1;
           p.bias = fc + m->o_bqkv[g]; p.q_out = m->Q; p.halo_off = -1;
           p.kv_off = ((long long)s * c.n_attn + g) * 2 * (m->P + m->Rk) * C;
-          p.kv_rs = m->kv_rs; p.kv_hs = m->kv_hs; p.dh_shift = m->dh_shift;
+          p.kv_hs = m->kv_hs; p.dh_shift = m->dh_shift;
           if (rounded_norm) {
             rmsnorm(X);
             gemm(m->tmU, m->tmWqkv[v][g], p, 3 * C, &m->tmWqkv[1][g]);
