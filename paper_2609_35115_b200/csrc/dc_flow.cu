@@ -683,7 +683,8 @@ __global__ void set_slots_kernel(const SlotSet set, SlotInfo* dst) {
 // input-projection operand [x_0 | mu].  Device noise: the draw of (frame t, channels 4g..4g+3) is Philox at
 // counter (t, g, stream) under the model's seed - the offset is the stream's frame clock, so a replayed graph
 // draws what direct launches would, and a look-ahead frame draws the same noise when it is presented again.
-__global__ void flow_prep_kernel(const SlotInfo* slots, int mel, float* xstate, bf16* ain, int ld_ain, uint32_t seed_lo, uint32_t seed_hi) {
+// panel: the operand goes to the one-kernel step, in its block layout (dc_flow_cluster.cuh), instead of a row-major matrix.
+__global__ void flow_prep_kernel(const SlotInfo* slots, int mel, float* xstate, bf16* ain, int ld_ain, uint32_t seed_lo, uint32_t seed_hi, int panel) {
   ptx::pdl_launch();
   ptx::pdl_wait();
   const SlotInfo si = slots[blockIdx.x];
@@ -708,8 +709,13 @@ __global__ void flow_prep_kernel(const SlotInfo* slots, int mel, float* xstate, 
       const int c = 4 * g + j;
       const float mu = si.pass == 0 ? si.feats[(long long)f * fw + c] : 0.f;
       xstate[r * mel + c] = x0[j];
-      ain[(GUARD + r) * ld_ain + c] = __float2bfloat16_rn(x0[j]);
-      ain[(GUARD + r) * ld_ain + mel + c] = __float2bfloat16_rn(mu);
+      auto at = [&](int col) -> long long {
+        if (!panel) return (GUARD + r) * ld_ain + col;
+        const int rho = HALO + f;
+        return ((long long)blockIdx.x * (ld_ain >> 6) + (col >> 6)) * (SLOT_ROWS * KBLK) + rho * KBLK + ((((col >> 3) & 7) ^ (rho & 7)) << 3) + (col & 7);
+      };
+      ain[at(c)] = __float2bfloat16_rn(x0[j]);
+      ain[at(mel + c)] = __float2bfloat16_rn(mu);
     }
   }
 }
@@ -879,6 +885,19 @@ __device__ __forceinline__ float att_exp_store(const float (&v)[64], float scale
   return t.x + t.y;
 }
 
+// O rows of this thread's lane scaled by alpha.  Rare (a block whose largest score exceeds the reference by 2^8), hence a call: inlined
+// beside the 64 live scores it costs registers that every block would pay for.
+__device__ __noinline__ void att_rescale(uint32_t addr, float alpha, int cols) {
+#pragma unroll 1
+  for (int c = 0; c < cols; c += 16) {
+    float o16[16];
+    ptx::tmem_ld16(addr + (uint32_t)c, o16);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) o16[i] *= alpha;
+    ptx::tmem_st16(addr + (uint32_t)c, o16);
+  }
+}
+
 // Weights of the two streams' accumulators: O = c0 O_0 + c1 O_1.
 __device__ __forceinline__ void att_combine(int nkb, float m0, float l0, float m1, float l1, float* c0, float* c1) {
   if (nkb == 1) {
@@ -918,6 +937,19 @@ struct AttKeys {
     g1 = hist > 0 ? a8 + phi : n_prompt;
     nkb = (L + ATT_KB - 1) / ATT_KB;
     n_early = min((tp > 0 ? si.n_prompt0 : a8 + (hist > 0 ? phi + si.kv_len : 0)) / ATT_KB, nkb);
+  }
+  // Asks a block of carried rows into L2; one thread.
+  __device__ __forceinline__ void prefetch(const bf16* plane, int b, int P, int Rk, int dh_shift) const {
+    const int row_bytes = 2 << dh_shift, k0 = b * ATT_KB, na = min(ATT_KB, max(0, a8 - k0));
+    if (na > 0) ptx::bulk_prefetch(plane + ((long long)k0 << dh_shift), (uint32_t)(na * row_bytes));
+    if (ATT_KB > na) {
+      int rr = row0 + max(0, k0 - a8);
+#pragma unroll 1
+      while (rr >= P + Rk) rr -= Rk;
+      const int n1 = min(ATT_KB - na, P + Rk - rr);
+      ptx::bulk_prefetch(plane + ((long long)rr << dh_shift), (uint32_t)(n1 * row_bytes));
+      if (na + n1 < ATT_KB) ptx::bulk_prefetch(plane + ((long long)P << dh_shift), (uint32_t)((ATT_KB - na - n1) * row_bytes));
+    }
   }
   // Rows of block b (n of them) of one plane -> dst, completion on bar; one thread.
   __device__ __forceinline__ void fetch(const bf16* plane, int b, int n, int P, int Rk, int dh_shift, uint8_t* dst, uint64_t* bar) const {
@@ -1153,17 +1185,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
           const float alpha = need ? exp2f(m_ref - mx) : 1.0f;
           if (need) m_ref = mx;
           lsum *= alpha;
-          if (half == 0) {                        // O rows 0..63 live in lanes 0..63
-#pragma unroll 1
-            for (int c = 0; c < DH; c += 16) {
-              float o16[16];
-              const uint32_t addr = lane_addr + (uint32_t)(ATT_KB + (b & 1) * 64 + c);
-              ptx::tmem_ld16(addr, o16);
-#pragma unroll
-              for (int i = 0; i < 16; ++i) o16[i] *= alpha;
-              ptx::tmem_st16(addr, o16);
-            }
-          }
+          if (half == 0) att_rescale(lane_addr + (uint32_t)(ATT_KB + (b & 1) * 64), alpha, DH);   // O rows 0..63 live in lanes 0..63
           ptx::tc_fence_before();
         }
       }
@@ -1209,6 +1231,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
   __syncthreads();
   if (warp == 4) ptx::tmem_dealloc(tmem_base, ATT_TMEM_COLS);
 }
+
+#include "dc_flow_cluster.cuh"
 
 // ---- host helpers ----------------------------------------------------------------------------
 
@@ -1306,6 +1330,11 @@ struct FlowModel {
   std::map<int, GraphEntry> graphs;      // batch size -> captured chunk step
   uint64_t graph_launches = 0;           // graph launches issued by decode calls
   std::vector<SlotSet> sets;
+  // one-kernel chunk steps (flow_cluster_kernel): resident clusters (0: not for this model) and the packed weights
+  int       max_clusters = 0;
+  uint8_t*  clu_stream = nullptr;
+  long long clu_stream_bytes = 0;
+  bf16* AinP = nullptr;      // the input-projection operand in the layout of the one-kernel step
 };
 
 struct FlowState {
@@ -1337,6 +1366,8 @@ void pack_wt(std::vector<uint16_t>& dst, size_t off, const float* W, int K, int 
 
 namespace {
 bool build_graph(FlowModel* m, int n, bool tick = false);
+cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>& w_conv, const std::vector<size_t>& w_qkv,
+                           const std::vector<size_t>& w_o, size_t w_out);
 }
 
 void flow_model_destroy(FlowModel* m) {
@@ -1513,6 +1544,12 @@ dc_status flow_model_create(const dc_config& cfg, const float* w, FlowModel** ou
     flow_model_destroy(m);
     return DC_ERR_CUDA;
   }
+  e = cluster_create(m, w_in, w_conv, w_qkv, w_o, w_out);
+  if (e != cudaSuccess) {
+    set_error("flow model allocation failed: %s", cudaGetErrorString(e));
+    flow_model_destroy(m);
+    return e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;
+  }
   m->sets.resize((size_t)(m->S + MAX_SLOTS_PER_SET - 1) / MAX_SLOTS_PER_SET);
   {
     m->pdl = !(cfg.options & DC_OPT_NO_PDL);
@@ -1664,6 +1701,108 @@ void launch(LaunchCtx& lc, void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   ++lc.launches;
 }
 
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int CL, int n_clusters, cudaStream_t st, bool pdl) {
+  cfg = cudaLaunchConfig_t{};
+  cfg.gridDim = dim3((unsigned)(CL * n_clusters));
+  cfg.blockDim = dim3(CLU_THREADS);
+  cfg.dynamicSmemBytes = CLU_SMEM;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.numAttrs = 1;
+  if (pdl) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
+}
+
+// Which models the one-kernel step serves: hidden 64 .. 512 in powers of two (the activation panel of two slots is 128 rows of
+// `hidden` bf16 in shared memory, a cluster has at most 16 CTAs of 32 columns).  The measurement options and the CTA-pair option ask
+// for the kernels of their own.
+cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>& w_conv, const std::vector<size_t>& w_qkv,
+                           const std::vector<size_t>& w_o, size_t w_out) {
+  const dc_config& c = m->cfg;
+  const int C = m->C, CL = C / CLU_BN, nL = c.n_conv, nA = c.n_attn;
+  const uint32_t apart = DC_OPT_SKIP_CONV_GEMM | DC_OPT_SKIP_ATTENTION | DC_OPT_EMPTY_KERNELS | DC_OPT_CTA_PAIRS;
+  if ((c.options & apart) || (C != 64 && C != 128 && C != 256 && C != 512)) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(flow_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
+  if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(flow_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  int n_cl = 0;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  cluster_config(cfg, attr, CL, 1, nullptr, false);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, flow_cluster_kernel, &cfg);
+  cudaFuncAttributes fa{};
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, flow_cluster_kernel);
+  // (the kernel redistributes the registers that it was launched with: they have to cover the split)
+  if (e == cudaSuccess && fa.numRegs * CLU_THREADS < 128 * CLU_REGS_CTRL + CLU_EPI * CLU_REGS_EPI) n_cl = 0;
+  if (e != cudaSuccess || n_cl < 1) {   // the kernels of their own serve the model
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  const int n_out = m->mel / 16, nch = (n_out + CL - 1) / CL, nkb_c = C / KBLK, nkb_in = m->Kin / KBLK;
+  const long long conv_b = (long long)nkb_c * CLU_SLOT, proj_b = conv_b / 3;
+  m->clu_stream_bytes = (long long)nkb_in * CLU_BN * 128 + nL * conv_b + nA * (conv_b + proj_b) + (long long)nkb_c * nch * 2048;
+  e = dalloc(m, &m->AinP, (size_t)m->S * SLOT_ROWS * m->Kin);
+  if (e == cudaSuccess) e = dalloc(m, &m->clu_stream, (size_t)m->clu_stream_bytes * CL, false);
+  if (e != cudaSuccess) return e;
+  long long off = 0;
+  auto pack = [&](size_t w, int ldk, int nkb, int J, int RJ, int rs_rank, int rs_j, int cs_j, int n_valid, long long bytes) {
+    const CluPack pk{m->wts + w, off, ldk, J, RJ, rs_rank, rs_j, cs_j, n_valid};
+    clu_pack_kernel<<<dim3(4, CL, nkb), 128>>>(pk, m->clu_stream, m->clu_stream_bytes);
+    off += bytes;
+  };
+  pack(w_in, m->Kin, nkb_in, 1, CLU_BN, CLU_BN, 0, 0, C, (long long)nkb_in * CLU_BN * 128);
+  for (int g = 0, l = 0; g < (nA > 0 ? nA : 1); ++g) {
+    for (int j = 0; j < m->cpa; ++j, ++l) pack(w_conv[l], 3 * C, nkb_c, 3, CLU_BN, CLU_BN, 0, C, C, conv_b);
+    if (nA > 0) {
+      pack(w_qkv[g], C, nkb_c, 3, CLU_BN, CLU_BN, C, 0, 3 * C, conv_b);
+      pack(w_o[g], C, nkb_c, 1, CLU_BN, CLU_BN, 0, 0, C, proj_b);
+    }
+  }
+  pack(w_out, C, nkb_c, nch, 16, 16, 16 * CL, 0, m->mel, (long long)nkb_c * nch * 2048);
+  e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) m->max_clusters = n_cl;
+  return e;
+}
+
+// Slots per cluster of the one-kernel step for a batch of n slots, 0 if its clusters would not all be resident at once (a second
+// wave doubles the step: the kernels of their own serve the batch).  One slot per cluster where that fits, else two; the two passes
+// of a guided stream share a cluster.
+int cluster_slots(const FlowModel* m, int n) {
+  for (int spc = m->n_pass; spc <= 2; ++spc)
+    if ((n + spc - 1) / spc <= m->max_clusters) return spc;
+  return 0;
+}
+
+void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick) {
+  const dc_config& c = m->cfg;
+  CluParams p{};
+  p.slots = m->d_slots; p.n_slots = n; p.spc = spc; p.CL = m->C / CLU_BN;
+  p.C = m->C; p.mel = m->mel; p.Kin = m->Kin; p.n_heads = c.n_heads;
+  p.n_conv = c.n_conv; p.n_attn = c.n_attn; p.cpa = m->cpa; p.n_steps = tick ? 1 : c.n_steps; p.tick = tick;
+  for (int l = 0; l < c.n_conv; ++l) p.dil[l] = c.dilations[l];
+  p.fc = m->fconst; p.o_bout = (int)m->o_bout; p.o_tau = (int)m->o_tau;
+  p.wstream = m->clu_stream; p.wstream_bytes = m->clu_stream_bytes;
+  p.X[0] = m->Xa; p.X[1] = m->Xb; p.Q = m->Q; p.O = m->O; p.Ain = m->AinP;
+  p.xstate = m->xstate; p.ssq = m->ssq;
+  p.inv_C = 1.0f / (float)m->C; p.eps = c.rms_eps; p.inv_n = 1.0f / c.n_steps; p.cfg_w = c.cfg_scale;
+  p.rounded = m->U != nullptr;
+  p.P = m->P; p.Rk = m->Rk; p.kv_hs = m->kv_hs; p.dh_shift = m->dh_shift;
+  p.scale_log2e = c.n_attn > 0 ? (float)(1.4426950408889634 / sqrt((double)c.head_dim)) : 0.f;
+  p.err = m->d_err;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  cluster_config(cfg, attr, p.CL, (n + spc - 1) / spc, lc.st, lc.pdl);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, flow_cluster_kernel, p);
+  if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+  ++lc.launches;
+}
+
 // Issues every kernel of one chunk step for n slots (the slot table is uploaded by the first
 // kernel(s) from `sets`).
 // tick = false: the n slots' chunks, all Euler steps.  tick = true: ONE pass of the network, every slot at the Euler step
@@ -1673,8 +1812,14 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
   const int C = m->C, mel = m->mel;
   for (int i = 0; i < n_sets; ++i)   // not a programmatic launch: it overwrites the table the previous chunk still reads
     launch(lc, set_slots_kernel, dim3(1), dim3(MAX_SLOTS_PER_SET), 0, false, 4, sets[i], m->d_slots);
-  launch(lc, flow_prep_kernel, dim3(n), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, m->Ain, m->Kin,
-         (uint32_t)c.noise_seed_lo, (uint32_t)c.noise_seed_hi);
+  // (a profiled call keeps the kernels apart: its figures are per kernel class; the bytes are the same)
+  const int spc = lc.prof == nullptr || !lc.prof->on ? cluster_slots(m, n) : 0;
+  launch(lc, flow_prep_kernel, dim3(n), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, spc > 0 ? m->AinP : m->Ain, m->Kin,
+         (uint32_t)c.noise_seed_lo, (uint32_t)c.noise_seed_hi, (int)(spc > 0));
+  if (spc > 0) {
+    enqueue_cluster(m, n, spc, lc, tick);
+    return;
+  }
 
   const int m_tiles = (n * SLOT_ROWS + TILE_M - 1) / TILE_M;
   // N-tile variant: the narrowest whose C-wide GEMMs still fit ONE wave (a GEMM CTA has an SM to itself);
@@ -1699,9 +1844,8 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
     p.empty = (c.options & DC_OPT_EMPTY_KERNELS) ? 1 : 0;
     const int stage_bytes = A_BYTES + p.taps * ((p.BN * 128 + 1023) & ~1023);
     // the issuer count fixes the summation order, so it depends on the GEMM's role only, never on the tile
-    // width chosen for the batch size (batched and single-stream results must agree bit for bit);
-    // the QKV and output projections keep one issuer (their wide tiles would not fit two accumulators)
-    p.n_issuers = (p.mode != MODE_QKV && p.mode != MODE_OUT && p.n_kblocks >= 2) ? 2 : 1;
+    // width chosen for the batch size (batched and single-stream results must agree bit for bit)
+    p.n_issuers = p.n_kblocks >= 2 ? 2 : 1;
     // Stage count.  With two issuers the count must be EVEN: issuer i takes
     // the reduction blocks kb = i (mod 2), and only with an even ring does every stage always belong
     // to the same issuer - a parity wait cannot tell "my block has landed" from "the other issuer's
