@@ -43,7 +43,6 @@ constexpr int HALO = 8;         // carried frames per (step, conv block); dilati
 constexpr int TILE_M = 128;
 constexpr int KBLK = 64;        // bf16 elements per 128-byte swizzled smem row
 constexpr int MAX_STAGES = 8;
-constexpr int GEMM_TILE_SMEM = 88 * 1024;    // operand stages of the single-issuer GEMMs (a short reduction needs no deeper ring)
 constexpr int A_ROWS = TILE_M;         // rows of an A box = rows of the output tile (the conv taps are shifted in the epilogue)
 constexpr int A_BYTES = A_ROWS * 128;
 constexpr int MAX_BN = 192;
@@ -85,7 +84,7 @@ struct GemmParams {
   int          mode;
   int          BN;              // output columns per CTA (multiple of 16, <= 128)
   int          n_issuers;       // 1 or 2 UMMA-issuing threads (2: even / odd reduction blocks, own accumulators)
-  int          n_stages;        // TMA pipeline depth (<= MAX_STAGES, n_stages * stage bytes <= GEMM_TILE_SMEM)
+  int          n_stages;        // TMA pipeline depth (<= MAX_STAGES)
   int          n_slots;
   int          n_kblocks;       // 64-wide channel blocks of the A matrix (one pipeline stage each)
   int          taps;            // 1, or 3 for the conv blocks (weights: K index = tap * 64 * n_kblocks + channel)
@@ -1850,13 +1849,9 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
     // the reduction blocks kb = i (mod 2), and only with an even ring does every stage always belong
     // to the same issuer - a parity wait cannot tell "my block has landed" from "the other issuer's
     // earlier block has landed" on a stage that both use.
-    if (p.n_issuers == 2) {
-      p.n_stages = (p.n_kblocks >= 4 && (4 * stage_bytes <= 104 * 1024 || stage_bytes > 32 * 1024)) ? 4 : 2;
-    } else {
-      p.n_stages = std::max(1, std::min(std::min(MAX_STAGES, GEMM_TILE_SMEM / stage_bytes), p.n_kblocks));
-      // the wide QKV tiles fill the GPU with one CTA per SM anyway: a deeper ring hides the load latency
-      if (p.mode == MODE_QKV && stage_bytes > 32 * 1024 && p.n_kblocks >= 4) p.n_stages = 4;
-    }
+    // Four stages wherever there are four blocks: with two, 32-column conv tiles waited for their operands (16 streams 1,714 us per
+    // step against 1,461).
+    p.n_stages = p.n_kblocks >= 4 ? 4 : (p.n_issuers == 2 ? 2 : 1);
     if (pairs_ok && tBh != nullptr) {
       const int pair_stage = A_BYTES + p.taps * (p.BN * 64);
       int ns = p.n_kblocks < MAX_STAGES ? p.n_kblocks : MAX_STAGES;
