@@ -126,6 +126,7 @@ struct F32Layer {
   size_t w_off, b_off;  // float offsets in the blob
   int    ring_cap;    // rows of its input ring
   int    excite;      // the random excitation is added to this layer's output
+  TapConvTc tc;       // conv / transposed conv: the packed weights
 };
 
 }  // namespace dc
@@ -137,6 +138,8 @@ struct dc_model {
   dc_config cfg;
   int       device = 0;
   float*    d_w = nullptr;   // fp32 pipelines: the blob on the device
+  uint8_t*  d_wp = nullptr;  // ... and the conv weights as packed bf16 planes
+  int*      f32_err = nullptr;   // ... and the device word that a bounded wait sets when it gives up
   // flow pipeline: staging of dc_decode_batch_host (pinned host + device, max_batch chunks each way)
   float *h_in = nullptr, *h_out = nullptr, *d_in = nullptr, *d_out = nullptr;
   bool   zero_copy = true;   // dc_decode_batch_host: kernels access page-locked caller buffers directly
@@ -356,6 +359,52 @@ static void build_f32_layers(dc_model* m) {
 static void build_f32_graph(dc_stream* s);
 static void build_f32_batch_graph(dc_model* m);
 
+// What of a conv layer's launch does not depend on the call.
+static dc::TapConvF32 tapconv_layer(const dc_model* m, int l) {
+  const F32Layer& L = m->layers[l];
+  dc::TapConvF32 p{};
+  p.in_mask = L.ring_cap - 1; p.C_in = L.C_in;
+  p.first_layer = l == 0; p.last_layer = l + 1 == (int)m->layers.size(); p.rate_in = L.rate_in;
+  if (L.kind == 0) {
+    p.n_taps = 3; p.shift[0] = 2 * L.dil; p.shift[1] = L.dil; p.shift[2] = 0; p.n_phase = 1;
+    p.w_tap_stride = (long long)L.C_in * L.C_out; p.w_phase_stride = 0;
+  } else {
+    p.n_taps = 2; p.shift[0] = 0; p.shift[1] = 1; p.shift[2] = 0; p.n_phase = L.stride;
+    p.w_tap_stride = (long long)L.stride * L.C_in * L.C_out; p.w_phase_stride = (long long)L.C_in * L.C_out;
+  }
+  p.W = m->d_w + L.w_off; p.bias = m->d_w + L.b_off; p.C_out = L.C_out;
+  p.residual_silu = L.residual_silu; p.post_silu = L.post_silu;
+  if (l == 0) p.save_rows = L.halo;
+  if (l + 1 < (int)m->layers.size()) p.out_mask = m->layers[l + 1].ring_cap - 1;
+  if (L.excite) {
+    p.exc_std = m->cfg.excitation_std; p.exc_seed_lo = m->cfg.excitation_seed_lo; p.exc_seed_hi = m->cfg.excitation_seed_hi;
+  }
+  return p;
+}
+
+// Splits and packs the conv weights (once, at create).
+static cudaError_t pack_f32_weights(dc_model* m) {
+  size_t bytes = 0;
+  for (int l = 0; l < (int)m->layers.size(); ++l)
+    if (m->layers[l].kind != 2) bytes += dc::tapconv_pack_bytes(tapconv_layer(m, l));
+  cudaError_t e = dc::dev_alloc(&m->d_wp, bytes);
+  if (e == cudaSuccess) e = dc::dev_alloc(&m->f32_err, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&m->h_err, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(m->f32_err, 0, sizeof(int));
+  if (e == cudaSuccess) e = dc::prepare_tapconv();
+  if (e != cudaSuccess) return e;
+  size_t off = 0;
+  for (int l = 0; l < (int)m->layers.size(); ++l) {
+    F32Layer& L = m->layers[l];
+    if (L.kind == 2) continue;
+    const dc::TapConvF32 p = tapconv_layer(m, l);
+    dc::pack_tapconv(p, m->d_wp + off, &L.tc);
+    L.tc.err = m->f32_err;
+    off += dc::tapconv_pack_bytes(p);
+  }
+  return cudaDeviceSynchronize();
+}
+
 // ---------------------------------------------------------------------------------------------
 // lifetime
 // ---------------------------------------------------------------------------------------------
@@ -419,6 +468,7 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
     build_f32_layers(m);
     cudaError_t e = dc::dev_alloc(&m->d_w, n_floats * sizeof(float));
     if (e == cudaSuccess) e = cudaMemcpy(m->d_w, w, n_floats * sizeof(float), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = pack_f32_weights(m);
     if (e == cudaSuccess) e = dc::prepare_f32_constants();
     if (e == cudaSuccess && cfg->max_batch > 1) {
       e = dc::dev_alloc(&m->d_batch, sizeof(dc::F32Batch));
@@ -450,6 +500,8 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
     if (m->sub_voc) dc_destroy(m->sub_voc);
     free_batch_graph(m);
     if (m->d_w) dc::dev_free(m->d_w);
+    if (m->d_wp) dc::dev_free(m->d_wp);
+    if (m->f32_err) dc::dev_free(m->f32_err);
     if (m->flow) dc::flow_model_destroy(m->flow);
     if (m->h_in) cudaFreeHost(m->h_in);
     if (m->h_out) cudaFreeHost(m->h_out);
@@ -474,6 +526,8 @@ extern "C" dc_status dc_destroy(dc_model* m) {
   free_batch_graph(m);
   if (m->flow) dc::flow_model_destroy(m->flow);
   if (m->d_w) dc::dev_free(m->d_w);
+  if (m->d_wp) dc::dev_free(m->d_wp);
+  if (m->f32_err) dc::dev_free(m->f32_err);
   if (m->h_in) cudaFreeHost(m->h_in);
   if (m->h_out) cudaFreeHost(m->h_out);
   if (m->h_err) cudaFreeHost(m->h_err);
@@ -792,36 +846,23 @@ static void enqueue_f32(dc_stream* s, bool use_call, const float* feats, int T, 
       dc::ProfScope ps(&m->prof, 6, cs);
       dc::launch_head_istft_f32(h, cs, Tgrid, pdl);
     } else {
-      dc::TapConvF32 p{};
-      p.in_ring = ring; p.in_mask = L.ring_cap - 1; p.C_in = L.C_in;
-      p.first_layer = l == 0; p.last_layer = l + 1 == nL; p.rate_in = L.rate_in;
+      dc::TapConvF32 p = tapconv_layer(m, l);
+      p.in_ring = ring;
       if (use_call) {
         p.call = s->d_call;
       } else {
         p.pos_in = pos; p.T_in = Tin;
         if (l == 0) p.in_direct = feats;
       }
-      if (l == 0) { p.save_ring = ring; p.save_rows = L.halo; }
-      if (L.kind == 0) {
-        p.n_taps = 3; p.shift[0] = 2 * L.dil; p.shift[1] = L.dil; p.shift[2] = 0; p.n_phase = 1;
-        p.w_tap_stride = (long long)L.C_in * L.C_out; p.w_phase_stride = 0;
-      } else {
-        p.n_taps = 2; p.shift[0] = 0; p.shift[1] = 1; p.shift[2] = 0; p.n_phase = L.stride;
-        p.w_tap_stride = (long long)L.stride * L.C_in * L.C_out; p.w_phase_stride = (long long)L.C_in * L.C_out;
-      }
-      p.W = m->d_w + L.w_off; p.bias = m->d_w + L.b_off; p.C_out = L.C_out;
-      p.residual_silu = L.residual_silu; p.post_silu = L.post_silu;
-      if (L.excite) {
-        p.exc_std = m->cfg.excitation_std; p.exc_seed_lo = m->cfg.excitation_seed_lo; p.exc_seed_hi = m->cfg.excitation_seed_hi;
-        p.exc_rng_id = s->rng_id;
-      }
+      if (l == 0) p.save_ring = ring;
+      p.exc_rng_id = s->rng_id;
       if (l + 1 < nL) {
-        p.out_ring = (float*)s->f32_rings[l + 1].p; p.out_mask = m->layers[l + 1].ring_cap - 1;
+        p.out_ring = (float*)s->f32_rings[l + 1].p;
       } else if (!use_call) {
         p.out_direct = out; p.pos_out = pos * p.n_phase;
       }
       dc::ProfScope ps(&m->prof, 5, cs);
-      dc::launch_tapconv_f32(p, cs, Tgrid, pdl);
+      dc::launch_tapconv_tc(p, L.tc, cs, Tgrid);
     }
     ++*launches;
   }
@@ -884,26 +925,10 @@ static void enqueue_f32_batch(dc_model* m, cudaStream_t cs, int* launches) {
       dc::ProfScope ps(&m->prof, 6, cs);
       dc::launch_head_istft_f32(h, cs, Tgrid, false, nb);
     } else {
-      dc::TapConvF32 p{};
+      dc::TapConvF32 p = tapconv_layer(m, l);
       p.batch = m->d_batch; p.layer = l;
-      p.in_mask = L.ring_cap - 1; p.C_in = L.C_in;
-      p.first_layer = l == 0; p.last_layer = l + 1 == nL; p.rate_in = L.rate_in;
-      if (l == 0) p.save_rows = L.halo;
-      if (L.kind == 0) {
-        p.n_taps = 3; p.shift[0] = 2 * L.dil; p.shift[1] = L.dil; p.shift[2] = 0; p.n_phase = 1;
-        p.w_tap_stride = (long long)L.C_in * L.C_out; p.w_phase_stride = 0;
-      } else {
-        p.n_taps = 2; p.shift[0] = 0; p.shift[1] = 1; p.shift[2] = 0; p.n_phase = L.stride;
-        p.w_tap_stride = (long long)L.stride * L.C_in * L.C_out; p.w_phase_stride = (long long)L.C_in * L.C_out;
-      }
-      p.W = m->d_w + L.w_off; p.bias = m->d_w + L.b_off; p.C_out = L.C_out;
-      p.residual_silu = L.residual_silu; p.post_silu = L.post_silu;
-      if (L.excite) {
-        p.exc_std = m->cfg.excitation_std; p.exc_seed_lo = m->cfg.excitation_seed_lo; p.exc_seed_hi = m->cfg.excitation_seed_hi;
-      }
-      if (l + 1 < nL) p.out_mask = m->layers[l + 1].ring_cap - 1;
       dc::ProfScope ps(&m->prof, 5, cs);
-      dc::launch_tapconv_f32(p, cs, Tgrid, false, nb);
+      dc::launch_tapconv_tc(p, L.tc, cs, Tgrid, nb);
     }
     ++*launches;
   }
@@ -1250,6 +1275,36 @@ extern "C" dc_status dc_decode_batch(dc_model* m, int n, dc_stream* const* strea
   return DC_OK;
 }
 
+namespace {
+// The device error words that a decode call of m may set (flow decoder, fp32 kernels): their copies are enqueued behind the call ...
+dc_status enqueue_error_words(dc_model* m, cudaStream_t cs) {
+  for (dc_model* q : {m, m->sub_flow, m->sub_voc}) {
+    if (!q || !q->h_err) continue;
+    DC_CUDA(cudaMemcpyAsync(q->h_err, q->flow ? dc::flow_error_word(q->flow) : q->f32_err, sizeof(int), cudaMemcpyDeviceToHost, cs));
+  }
+  return DC_OK;
+}
+// Reads and clears the word of one model (synchronous); 0: no timeout.
+int take_error(dc_model* q) {
+  if (q->flow) return dc::flow_take_device_error(q->flow);
+  int v = 0;
+  if (!q->f32_err || cudaMemcpy(&v, q->f32_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return 0;
+  if (v != 0) cudaMemset(q->f32_err, 0, sizeof(int));
+  return v;
+}
+// ... and looked at once the stream has been synchronised.
+dc_status check_error_words(dc_model* m, int n, dc_stream* const* streams) {
+  int code = 0;
+  for (dc_model* q : {m, m->sub_flow, m->sub_voc})
+    if (q && q->h_err && *q->h_err != 0) code = take_error(q);
+  if (code == 0) return DC_OK;
+  m->counters[4]++;
+  for (int i = 0; i < n; ++i) streams[i]->poisoned = true;
+  dc::set_error("device-side wait timed out (code %d)", code);
+  return DC_ERR_TIMEOUT;
+}
+}  // namespace
+
 extern "C" dc_status dc_decode_chunk_host(dc_stream* s, const float* feats_host, int T, float* out_host, int* n_out,
                                           void* cuda_stream) {
   dc_status st = admit(s, feats_host, T, out_host, false);
@@ -1276,16 +1331,11 @@ extern "C" dc_status dc_decode_chunk_host(dc_stream* s, const float* feats_host,
   st = dc_decode_chunk(s, fin, T, fout, &n, cuda_stream);
   if (st != DC_OK) return st;
   if (fout == s->stage_out) DC_CUDA(cudaMemcpyAsync(out_host, s->stage_out, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, cs));
-  dc_model* fmod = m->flow ? m : m->sub_flow;   // the model that owns the flow decoder, if any
-  if (fmod && fmod->h_err) DC_CUDA(cudaMemcpyAsync(fmod->h_err, dc::flow_error_word(fmod->flow), sizeof(int), cudaMemcpyDeviceToHost, cs));
+  st = enqueue_error_words(m, cs);
+  if (st != DC_OK) return st;
   DC_CUDA(cudaStreamSynchronize(cs));
-  if (fmod && fmod->h_err && *fmod->h_err != 0) {   // a bounded device-side wait gave up: the chunk's result is not valid
-    const int code = dc::flow_take_device_error(fmod->flow);   // reads and clears the word
-    m->counters[4]++;
-    s->poisoned = true;
-    dc::set_error("device-side wait timed out (code %d)", code);
-    return DC_ERR_TIMEOUT;
-  }
+  st = check_error_words(m, 1, &s);   // a bounded device-side wait gave up: the chunk's result is not valid
+  if (st != DC_OK) return st;
   if (n_out) *n_out = n;
   return DC_OK;
 }
@@ -1299,7 +1349,6 @@ extern "C" dc_status dc_decode_batch_host(dc_model* m, int n, dc_stream* const* 
   }
   if (n < 1 || n > m->cfg.max_batch) return DC_ERR_ARG;
   cudaStream_t cs = (cudaStream_t)cuda_stream;
-  dc_model* fmod = m->flow ? m : m->sub_flow;   // the model that owns a flow decoder (and its device error word), if any
   const size_t in_stride = (size_t)(m->cfg.f_chunk + m->cfg.f_lookahead) * m->in_dim, out_stride = (size_t)m->cfg.f_chunk * m->out_per_frame;
   std::vector<const float*> fin((size_t)n);
   std::vector<float*> fout((size_t)n);
@@ -1347,16 +1396,11 @@ extern "C" dc_status dc_decode_batch_host(dc_model* m, int n, dc_stream* const* 
   dc_status st = dc_decode_batch(m, n, streams, fin.data(), n_frames, fout.data(), cuda_stream);
   if (st != DC_OK) return st;
   if (!out_direct) DC_CUDA(cudaMemcpyAsync(m->h_out, m->d_out, (size_t)n * out_stride * sizeof(float), cudaMemcpyDeviceToHost, cs));
-  if (fmod) DC_CUDA(cudaMemcpyAsync(fmod->h_err, dc::flow_error_word(fmod->flow), sizeof(int), cudaMemcpyDeviceToHost, cs));
+  st = enqueue_error_words(m, cs);
+  if (st != DC_OK) return st;
   DC_CUDA(cudaStreamSynchronize(cs));
-  if (fmod && *fmod->h_err != 0) {   // a bounded device-side wait gave up: the results are not valid
-    const int code = *fmod->h_err;
-    dc::flow_take_device_error(fmod->flow);
-    m->counters[4]++;
-    for (int i = 0; i < n; ++i) streams[i]->poisoned = true;
-    dc::set_error("device-side wait timed out (code %d)", code);
-    return DC_ERR_TIMEOUT;
-  }
+  st = check_error_words(m, n, streams);   // a bounded device-side wait gave up: the results are not valid
+  if (st != DC_OK) return st;
   if (!out_direct)
     for (int i = 0; i < n; ++i)
       memcpy(out_host[i], m->h_out + (size_t)i * out_stride,
@@ -1414,8 +1458,8 @@ extern "C" dc_status dc_profile_end(dc_model* m, double ms[8], uint64_t launches
 
 extern "C" dc_status dc_get_counters(const dc_model* m, uint64_t counters[8]) {
   if (!m || !counters) return DC_ERR_ARG;
-  if (m->flow) {   // synchronous read of the device error word (asynchronous decode calls cannot see it)
-    const int code = dc::flow_take_device_error(m->flow);
+  if (m->flow || m->f32_err) {   // synchronous read of the device error word (asynchronous decode calls cannot see it)
+    const int code = take_error(const_cast<dc_model*>(m));
     if (code > 0) const_cast<dc_model*>(m)->counters[4]++;
   }
   for (int i = 0; i < 8; ++i) counters[i] = m->counters[i].load();

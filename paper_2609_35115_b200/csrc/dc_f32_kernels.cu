@@ -1,7 +1,7 @@
-// fp32 kernels of the conv pipeline and the vocoder tail: a tiled FFMA "tap GEMM" over ring
-// buffers (causal conv k=3 with dilation, and the phases of the causal transposed conv), and the
-// fused head conv + inverse STFT + overlap-add kernel.  fp32 parity (max err <= 1e-4 of RMS) rules
-// out single-pass TF32, so these run on the FP32 pipe.
+// fp32 kernels of the conv pipeline and the vocoder tail: the tap convolution over ring buffers (causal conv k=3 with
+// dilation, and the phases of the causal transposed conv) on the tensor cores with operands split into three bf16 planes
+// (dc_f32_tapconv.cuh), the same on the FP32 pipe for weights that are not packed, and the fused head conv + inverse STFT +
+// overlap-add kernel.
 #include "dc_internal.h"
 #include "dc_ptx.cuh"
 #include "dc_rng.cuh"
@@ -58,39 +58,13 @@ struct TapTile {
 template <int BM, int BN>
 __global__ void __launch_bounds__(512) tapconv_f32_kernel(const TapConvF32 p, const int KS) {
   using TT = TapTile<BM, BN>;
-  ptx::pdl_launch();
-  ptx::pdl_wait();          // the call record and the input ring come from earlier kernels
-  // per-call values: by value, or from the device-side call record (captured graphs)
-  int T_in = p.T_in;
-  long long pos_in = p.pos_in, pos_out = p.pos_out;
+  const int T_in = p.T_in;
+  const long long pos_in = p.pos_in, pos_out = p.pos_out;
   const float* in_direct = p.in_direct;
   float* out_direct = p.out_direct;
-  int exc_rng_id = p.exc_rng_id;
   const float* in_ring = p.in_ring;
   float* out_ring = p.out_ring;
-  float* save_ring = p.save_ring;
-  int phase = blockIdx.z;
-  const F32Call* callp = p.call;
-  if (p.batch != nullptr) {
-    const int slot = blockIdx.z / p.n_phase;
-    phase = blockIdx.z - slot * p.n_phase;
-    if (slot >= p.batch->n) return;
-    const F32BatchSlot& bs = p.batch->s[slot];
-    callp = &bs.call;
-    in_ring = bs.ptrs->ring[p.layer];
-    out_ring = p.last_layer ? nullptr : bs.ptrs->ring[p.layer + 1];
-    save_ring = p.first_layer ? bs.ptrs->ring[p.layer] : nullptr;
-  }
-  if (callp != nullptr) {
-    const F32Call c = *callp;
-    exc_rng_id = c.rng_id;
-    T_in = c.T * p.rate_in;
-    pos_in = c.frames * p.rate_in;
-    pos_out = pos_in * p.n_phase;
-    in_direct = p.first_layer ? c.feats : nullptr;
-    out_direct = p.last_layer ? c.out : nullptr;
-  }
-  if ((int)blockIdx.x * BM >= T_in) return;   // the grid is sized for the longest chunk
+  const int phase = blockIdx.z;
   const int in_mask = p.in_mask, C_in = p.C_in, C_out = p.C_out;
   const int sh0 = p.shift[0], sh1 = p.shift[1], sh2 = p.shift[2];
   constexpr int NTG = TT::NTG;
@@ -237,34 +211,15 @@ __global__ void __launch_bounds__(512) tapconv_f32_kernel(const TapConvF32 p, co
       }
       if (p.post_silu) v = make_float4(silu_f(v.x), silu_f(v.y), silu_f(v.z), silu_f(v.w));
       const long long t_out = (long long)p.n_phase * t_in + phase;
-      if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
-        uint32_t w[4];
-        float z[4];
-        philox4x32_10((uint32_t)(unsigned long long)t_out, (uint32_t)((unsigned long long)t_out >> 32), (uint32_t)(n >> 2),
-                      0x80000000u + (uint32_t)exc_rng_id, p.exc_seed_lo, p.exc_seed_hi, w);
-        normals4(w, z);
-        v.x = fmaf(p.exc_std, z[0], v.x); v.y = fmaf(p.exc_std, z[1], v.y); v.z = fmaf(p.exc_std, z[2], v.z); v.w = fmaf(p.exc_std, z[3], v.w);
-      }
       float* dst = (out_direct != nullptr)
                        ? out_direct + (t_out - pos_out) * C_out + n
                        : out_ring + (long long)((int)(t_out & (long long)p.out_mask)) * C_out + n;
       *reinterpret_cast<float4*>(dst) = v;
     }
   }
-
-  // Carry update of the first layer: its left context for the next chunk is the tail of the
-  // caller's chunk, written into ring rows that no CTA of this launch reads (distinct logical
-  // frames map to distinct rows because the ring holds f_chunk + halo frames).
-  if (save_ring != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && phase == 0) {
-    const int first = T_in > p.save_rows ? T_in - p.save_rows : 0;
-    const int c4 = C_in >> 2;
-    for (int i = tid; i < (T_in - first) * c4; i += NTG) {
-      const int r = first + i / c4, c = (i - (i / c4) * c4) * 4;
-      const float4 v = *reinterpret_cast<const float4*>(in_direct + (long long)r * C_in + c);
-      *reinterpret_cast<float4*>(save_ring + (long long)((int)((pos_in + r) & (long long)in_mask)) * C_in + c) = v;
-    }
-  }
 }
+
+#include "dc_f32_tapconv.cuh"
 
 // ---------------------------------------------------------------------------------------------
 
@@ -428,7 +383,7 @@ void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cud
 }
 
 template <int BM, int BN>
-void launch_tile(const TapConvF32& p, int KS, int T_grid, cudaStream_t st, bool pdl, int n_batch) {
+void launch_tile(const TapConvF32& p, int KS, cudaStream_t st) {
   using TT = TapTile<BM, BN>;
   static bool attr_set[64] = {false};
   int dev = 0;
@@ -438,9 +393,13 @@ void launch_tile(const TapConvF32& p, int KS, int T_grid, cudaStream_t st, bool 
     cudaFuncSetAttribute(tapconv_f32_kernel<BM, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, want > 227 * 1024 ? 227 * 1024 : want);
     attr_set[dev] = true;
   }
-  dim3 grid((T_grid + BM - 1) / BM, (p.C_out + BN - 1) / BN, p.n_phase * (n_batch > 0 ? n_batch : 1));
-  launch_ex(tapconv_f32_kernel<BM, BN>, grid, dim3(KS * TT::NTG), (size_t)KS * TT::GROUP_FLOATS * sizeof(float), st, pdl, p, KS);
+  dim3 grid((p.T_in + BM - 1) / BM, (p.C_out + BN - 1) / BN, p.n_phase);
+  launch_ex(tapconv_f32_kernel<BM, BN>, grid, dim3(KS * TT::NTG), (size_t)KS * TT::GROUP_FLOATS * sizeof(float), st, false, p, KS);
 }
+
+constexpr size_t tc_smem_bytes(int BN, int n_a, int n_b) { return (size_t)n_a * TC_PANEL + (size_t)n_b * 3 * BN * 128 + TC_BARS; }
+static_assert(tc_smem_bytes(64, 1, 2) <= 113 * 1024 && tc_smem_bytes(32, 1, TC_MAX_B) <= 113 * 1024, "a single panel: two CTAs per SM");
+static_assert(tc_smem_bytes(64, 2, 3) <= 227 * 1024 && tc_smem_bytes(32, 2, TC_MAX_B) <= 227 * 1024, "several panels: one");
 }  // namespace
 
 const void* set_f32_call_func() { return (const void*)set_f32_call_kernel; }
@@ -454,19 +413,55 @@ void launch_set_f32_batch(const F32Batch& v, F32Batch* dst, cudaStream_t st) {
 }
 const void* set_f32_batch_func() { return (const void*)set_f32_batch_kernel; }
 
-void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st, int T_grid, bool pdl, int n_batch) {
-  if (T_grid < 0) T_grid = p.T_in;
+size_t tapconv_pack_bytes(const TapConvF32& p) {
+  return (size_t)p.n_phase * ((p.C_in + 63) / 64) * p.n_taps * 3 * ((p.C_out + 31) / 32 * 32) * 128;
+}
+
+void pack_tapconv(const TapConvF32& p, uint8_t* dst, TapConvTc* tc) {
+  *tc = TapConvTc{};
+  tc->W = dst;
+  tc->C_pad = (p.C_out + 31) / 32 * 32;
+  tc->n_blocks = (p.C_in + 63) / 64;
+  for (int j = 0; j < p.n_taps; ++j) tc->per_tap |= p.shift[j] > TC_H;
+  tapconv_pack_kernel<<<dim3(8, tc->n_blocks, p.n_taps * p.n_phase), 256>>>(p.W, p.w_phase_stride, p.w_tap_stride, p.C_in, p.C_out, tc->C_pad, tc->n_blocks,
+                                                                           p.n_taps, dst);
+}
+
+cudaError_t prepare_tapconv() {
+  cudaError_t e = cudaSuccess;
+  for (auto fn : {tapconv_tc_kernel<32, false>, tapconv_tc_kernel<64, false>, tapconv_tc_kernel<32, true>, tapconv_tc_kernel<64, true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  return e;
+}
+
+void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc_in, cudaStream_t st, int T_grid, int n_batch) {
+  TapConvTc tc = tc_in;
+  const int planes = p.n_phase * (n_batch > 0 ? n_batch : 1), m_tiles = (T_grid + TC_M - 1) / TC_M;
+  const bool drain = tc.n_blocks * (tc.per_tap ? p.n_taps : 1) > 1;   // (of the layer, not of the batch: it decides the order of the sum)
+  // 64 columns per CTA once that fills the GPU (a reduction step costs 209 cycles of the tensor pipe at 64 columns, 134 at 32), else 32
+  // over twice the SMs.  A column's sum is the same either way.  A single panel leaves room for two CTAs per SM, which overlap one's
+  // conversion and epilogue with the other's products; several panels overlap inside the CTA.
+  const bool wide = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= 148;
+  tc.n_a = drain ? 2 : 1;
+  tc.n_b = wide ? (drain ? 3 : 2) : TC_MAX_B;
+  const int bn = wide ? 64 : 32;
+  const dim3 grid(m_tiles, tc.C_pad / bn, planes);
+  auto fn = wide ? (drain ? tapconv_tc_kernel<64, true> : tapconv_tc_kernel<64, false>) : (drain ? tapconv_tc_kernel<32, true> : tapconv_tc_kernel<32, false>);
+  launch_ex(fn, grid, dim3(TC_THREADS), tc_smem_bytes(bn, tc.n_a, tc.n_b), st, false, p, tc);
+}
+
+void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st) {
   const int nkb = p.n_taps * ((p.C_in + BK - 1) / BK);
-  const long long ctas64 = (long long)((T_grid + 63) / 64) * ((p.C_out + 63) / 64) * p.n_phase;
+  const long long ctas64 = (long long)((p.T_in + 63) / 64) * ((p.C_out + 63) / 64) * p.n_phase;
   if (ctas64 >= 296) {
-    launch_tile<64, 64>(p, 1, T_grid, st, pdl, n_batch);
+    launch_tile<64, 64>(p, 1, st);
   } else {
     // few tiles: small tiles, and split the reduction inside the CTA until the GPU holds about
     // 1200 warps (8 per SM), keeping at least 4 steps per group; at most 8 groups (512 threads)
-    const long long ctas32 = (long long)((T_grid + 31) / 32) * ((p.C_out + 31) / 32) * p.n_phase;
+    const long long ctas32 = (long long)((p.T_in + 31) / 32) * ((p.C_out + 31) / 32) * p.n_phase;
     int KS = 1;
     while (KS < 8 && ctas32 * 2 * KS < 1200 && nkb / (2 * KS) >= 4) KS *= 2;
-    launch_tile<32, 32>(p, KS, T_grid, st, pdl, n_batch);
+    launch_tile<32, 32>(p, KS, st);
   }
 }
 

@@ -1,0 +1,375 @@
+// fp32 tap convolution on the tensor cores.  Included by dc_f32_kernels.cu inside its anonymous namespace.
+//
+// An fp32 number is the exact sum of three bf16 numbers (8 + 8 + 8 bits of significand): x = h + m + l with h = bf16(x),
+// m = bf16(x - h), l = x - h - m.  The product of two such sums keeps the six terms down to 2^-16 of the leading one,
+//   a b = ah bh + (ah bm + am bh) + (ah bl + am bm + al bh),
+// and drops three below 2^-24, the size of an fp32 rounding.  tcgen05 multiplies bf16 exactly and accumulates in fp32; the three
+// magnitudes have accumulators of their own, so that the small terms are not rounded to the large one's grid, and the epilogue adds
+// them smallest first.  Six bf16 products still run at several times the rate of the FP32 pipe: the batched 64-channel residual
+// block of the vocoder (192,000 frames) went from 213 us, 22 TFLOP/s, on FFMA tiles (4 x 4 per thread, bound by shared-memory
+// operand latency) to what the conversion and the fp32 rows' traffic cost.
+//
+// One CTA: 128 frames x BN channels of one phase.  Ten warps: 0..7 read the fp32 input rows (ring, or the caller's chunk), split
+// them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue (a thread owns one output row and every
+// second 16-column chunk); 8 issues the products; 9 streams the weights, split and packed as swizzled tiles at create.
+// A panel holds 64 channels of the 128 frames and of the up to 8 in front of them: a tap is a row offset of the operand
+// descriptor, so a row is read and split once for all its taps.  (Dilations above 4 fill the panel once per tap.)
+// Per 64 channels and tap: 4 reduction steps of ah x [bh bm bl], am x [bh bm], al x bh.
+
+constexpr int TC_M = 128, TC_H = 8;               // frames per tile; left-context rows in front of them
+constexpr int TC_ROWS = TC_M + TC_H;
+constexpr int TC_PLANE = TC_ROWS * 128;            // bytes of one bf16 plane of a panel (64 channels)
+constexpr int TC_PANEL = 3 * TC_PLANE;
+constexpr int TC_THREADS = 320, TC_CONV = 256;     // converting / epilogue threads
+constexpr int TC_ITEMS = (TC_ROWS * 8 + TC_CONV - 1) / TC_CONV;   // 8-channel pieces per thread and panel
+constexpr int TC_MAX_A = 2, TC_MAX_B = 4;
+constexpr int TC_BARS = 1024;                      // barriers (and alignment slack: the base is declared 1024-byte aligned)
+
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* s_fail, int* err, int code) {
+  const uint32_t a = ptx::smem_u32(bar);
+#pragma unroll 1
+  for (uint32_t i = 0; i < (1u << 20); ++i) {
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait_s(a, parity))) return true;
+    if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0)) return false;
+  }
+  *reinterpret_cast<volatile int*>(s_fail) = 1;
+  atomicCAS(err, 0, code);
+  __syncwarp();
+  return false;
+}
+
+// Two fp32 values -> their h, m and l parts as bf16 pairs.
+__device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+  __nv_bfloat162 b = __floats2bfloat162_rn(x, y);
+  h = *reinterpret_cast<const uint32_t*>(&b);
+  x -= __uint_as_float(h << 16);
+  y -= __uint_as_float(h & 0xFFFF0000u);
+  b = __floats2bfloat162_rn(x, y);
+  m = *reinterpret_cast<const uint32_t*>(&b);
+  x -= __uint_as_float(m << 16);
+  y -= __uint_as_float(m & 0xFFFF0000u);
+  b = __floats2bfloat162_rn(x, y);
+  l = *reinterpret_cast<const uint32_t*>(&b);
+}
+
+// DRAIN (inputs of more than one panel): the tensor cores truncate when they add to an accumulator, which over a long reduction
+// is a bias (7.6e-5 of RMS at the vocoder's end with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel,
+// tap) - four additions - has an accumulator of its own, two panels' worth in turn, which the epilogue threads add up in registers,
+// rounded to nearest, while the next panel is multiplied.
+template <int BN, bool DRAIN>
+__global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(const __grid_constant__ TapConvF32 p, const __grid_constant__ TapConvTc tc) {
+  // per-call values: from the device-side call record of the stream or of the slot (captured graphs), or by value
+  int T_in = p.T_in;
+  long long pos_in = p.pos_in, pos_out = p.pos_out;
+  const float* in_direct = p.in_direct;
+  float* out_direct = p.out_direct;
+  int exc_rng_id = p.exc_rng_id;
+  const float* in_ring = p.in_ring;
+  float* out_ring = p.out_ring;
+  float* save_ring = p.save_ring;
+  int phase = blockIdx.z;
+  const F32Call* callp = p.call;
+  if (p.batch != nullptr) {
+    const int slot = blockIdx.z / p.n_phase;
+    phase = blockIdx.z - slot * p.n_phase;
+    if (slot >= p.batch->n) return;
+    const F32BatchSlot& bs = p.batch->s[slot];
+    callp = &bs.call;
+    in_ring = bs.ptrs->ring[p.layer];
+    out_ring = p.last_layer ? nullptr : bs.ptrs->ring[p.layer + 1];
+    save_ring = p.first_layer ? bs.ptrs->ring[p.layer] : nullptr;
+  }
+  if (callp != nullptr) {
+    const F32Call c = *callp;
+    exc_rng_id = c.rng_id;
+    T_in = c.T * p.rate_in;
+    pos_in = c.frames * p.rate_in;
+    pos_out = pos_in * p.n_phase;
+    in_direct = p.first_layer ? c.feats : nullptr;
+    out_direct = p.last_layer ? c.out : nullptr;
+  }
+  const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * BN;
+  if (m0 >= T_in) return;   // the grid is sized for the longest chunk
+
+  extern __shared__ __align__(1024) uint8_t tc_smem[];
+  constexpr int B_TILE = 3 * BN * 128;
+  uint8_t* sA = tc_smem;
+  uint8_t* sB = sA + tc.n_a * TC_PANEL;
+  uint64_t* full_a = reinterpret_cast<uint64_t*>(sB + tc.n_b * B_TILE);
+  uint64_t* empty_a = full_a + TC_MAX_A;
+  uint64_t* full_b = empty_a + TC_MAX_A;
+  uint64_t* empty_b = full_b + TC_MAX_B;
+  uint64_t* accum = empty_b + TC_MAX_B;           // [2]: products of a panel done (without DRAIN: [0], all products)
+  uint64_t* drained = accum + 2;                  // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 2);
+  int* s_fail = reinterpret_cast<int*>(tmem_slot + 1);
+
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  if ((ptx::smem_u32(tc_smem) & 1023u) != 0u) {   // would corrupt the swizzled tiles: refuse (uniform)
+    if (tid == 0) atomicExch(tc.err, 14);
+    return;
+  }
+  if (tid == 0) {
+#pragma unroll 1
+    for (int i = 0; i < TC_MAX_A; ++i) {
+      ptx::mbar_init(&full_a[i], TC_CONV);
+      ptx::mbar_init(&empty_a[i], 1);
+    }
+#pragma unroll 1
+    for (int i = 0; i < TC_MAX_B; ++i) {
+      ptx::mbar_init(&full_b[i], 1);
+      ptx::mbar_init(&empty_b[i], 1);
+    }
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&accum[i], 1);
+      ptx::mbar_init(&drained[i], TC_CONV);
+    }
+    *s_fail = 0;
+    ptx::fence_barrier_init();
+  }
+  // columns: leading term (two sets of three with DRAIN), then the 2^-8 and the 2^-16 terms
+  constexpr uint32_t S_COL = DRAIN ? 6 * BN : BN;
+  constexpr uint32_t TMEM_COLS = S_COL + 2 * BN <= 128 ? 128 : (S_COL + 2 * BN <= 256 ? 256 : 512);
+  if (warp == 8) ptx::tmem_alloc(tmem_slot, TMEM_COLS);
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+  const int n_units = tc.n_blocks * (tc.per_tap ? p.n_taps : 1), taps_u = tc.per_tap ? 1 : p.n_taps;
+
+  if (warp == 9) {
+    // ---------------- weight stream: one tile of three planes per (block, tap) ----------------
+    const size_t plane = (size_t)tc.C_pad * 128;
+    const uint8_t* src = tc.W + (size_t)phase * tc.n_blocks * p.n_taps * 3 * plane + (size_t)n0 * 128;
+    const int n = tc.n_blocks * p.n_taps;
+    int st = 0;
+    uint32_t ph = 1;
+    bool ok = true;
+#pragma unroll 1
+    for (int i = 0; i < n && ok; ++i, src += 3 * plane) {
+      if (i >= tc.n_b) ok = tc_wait(&empty_b[st], ph, s_fail, tc.err, 0x201);
+      if (ok && ptx::elect_one()) {
+        ptx::mbar_expect_tx(&full_b[st], B_TILE);
+#pragma unroll 1
+        for (int q = 0; q < 3; ++q) ptx::bulk_load(sB + st * B_TILE + q * BN * 128, src + q * plane, BN * 128, &full_b[st]);
+      }
+      __syncwarp();
+      if (++st == tc.n_b) { st = 0; ph ^= 1u; }
+    }
+  } else if (warp == 8) {
+    // ---------------- products ----------------
+    const uint32_t id3 = ptx::umma_idesc_bf16(TC_M, 3 * BN, 0, 0), id2 = ptx::umma_idesc_bf16(TC_M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(TC_M, BN, 0, 0);
+    const uint64_t dA = ptx::umma_desc_sw128(ptx::smem_u32(sA)), dB = ptx::umma_desc_sw128(ptx::smem_u32(sB));
+    int sa = 0, sb = 0;
+    uint32_t pa = 0, pb = 0, acc = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int u = 0; u < n_units && ok; ++u) {
+      if (DRAIN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
+      if (ok) ok = tc_wait(&full_a[sa], pa, s_fail, tc.err, 0x202);
+#pragma unroll 1
+      for (int j = 0; j < taps_u && ok; ++j) {
+        ok = tc_wait(&full_b[sb], pb, s_fail, tc.err, 0x203);
+        ptx::tc_fence_after();
+        const int off = tc.per_tap ? TC_H : TC_H - p.shift[j];   // (a panel filled for one tap has its rows at TC_H)
+        const uint64_t ah = dA + (uint64_t)(uint32_t)((sa * TC_PANEL + off * 128) >> 4), am = ah + (TC_PLANE >> 4), al = am + (TC_PLANE >> 4);
+        const uint64_t b = dB + (uint64_t)(uint32_t)(sb * (B_TILE >> 4));
+        if (ok && ptx::elect_one()) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (DRAIN) {
+              ptx::umma_bf16(tmem_base + (uint32_t)((u & 1) * 3 + j) * BN, ah + 2 * k, b + 2 * k, id1, k != 0);
+              ptx::umma_bf16(tmem_base + S_COL, ah + 2 * k, b + (BN * 128 >> 4) + 2 * k, id2, k == 0 ? (uint32_t)((u | j) != 0) : 1u);
+            } else {
+              ptx::umma_bf16(tmem_base, ah + 2 * k, b + 2 * k, id3, k == 0 ? acc : 1u);
+            }
+            ptx::umma_bf16(tmem_base + S_COL, am + 2 * k, b + 2 * k, id2, 1);
+            ptx::umma_bf16(tmem_base + S_COL + BN, al + 2 * k, b + 2 * k, id1, 1);
+          }
+          ptx::umma_commit(&empty_b[sb]);
+          if (j + 1 == taps_u) {
+            ptx::umma_commit(&empty_a[sa]);
+            if (DRAIN) ptx::umma_commit(&accum[u & 1]);
+          }
+        }
+        __syncwarp();
+        acc = 1;
+        if (++sb == tc.n_b) { sb = 0; pb ^= 1u; }
+      }
+      if (++sa == tc.n_a) { sa = 0; pa ^= 1u; }
+    }
+    if (!DRAIN && ptx::elect_one()) ptx::umma_commit(accum);
+    __syncwarp();
+  } else {
+    // ---------------- input rows -> bf16 planes ----------------
+    const int C_in = p.C_in, in_mask = p.in_mask;
+    const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
+    float4 xa[TC_ITEMS], xb[TC_ITEMS];
+    auto load = [&](int u) {
+      const int blk = tc.per_tap ? u / p.n_taps : u, tap = tc.per_tap ? u - blk * p.n_taps : 0;
+      const int c = blk * 64 + c8;
+      const long long t0 = pos_in + m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
+#pragma unroll
+      for (int i = 0; i < TC_ITEMS; ++i) {
+        const int row = row0 + 32 * i;
+        xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        xb[i] = xa[i];
+        if (row < TC_ROWS && m0 + row - TC_H < T_in && c < C_in) {
+          const float* src = in_row_ptr(in_direct, pos_in, in_ring, in_mask, C_in, t0 + row) + c;
+          xa[i] = *reinterpret_cast<const float4*>(src);
+          if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
+        }
+      }
+    };
+    const int q = warp & 3, half = warp >> 2;      // epilogue: TMEM lane quarter; 16-column chunks half, half + 2, ...
+    const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
+    constexpr int NC = BN / 32;
+    float sum[NC][16];
+    if (DRAIN) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sum[c][i] = 0.f;
+    }
+    auto drain = [&](int u) {
+      const bool got = tc_wait(&accum[u & 1], (u >> 1) & 1, s_fail, tc.err, 0x205);
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const uint32_t col = lanes + (uint32_t)((u & 1) * 3 * BN + 16 * (half + 2 * c));
+        float z[16], y[16];
+        if (taps_u == 1) {
+          ptx::tmem_ld16(col, z);
+        } else {
+          ptx::tmem_ld16x2(col, col + BN, z, y);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) z[i] += y[i];
+          if (taps_u == 3) {
+            ptx::tmem_ld16(col + 2 * BN, y);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) z[i] += y[i];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sum[c][i] += z[i];
+      }
+      ptx::tc_fence_before();
+      ptx::mbar_arrive(&drained[u & 1]);
+      return got;
+    };
+    load(0);
+    int sa = 0;
+    uint32_t ph = 1;
+    bool ok = true;
+#pragma unroll 1
+    for (int u = 0; u < n_units; ++u) {
+      if (u >= tc.n_a) ok &= tc_wait(&empty_a[sa], ph, s_fail, tc.err, 0x204);
+      uint8_t* dst = sA + sa * TC_PANEL;
+#pragma unroll
+      for (int i = 0; i < TC_ITEMS; ++i) {
+        const int row = row0 + 32 * i;
+        if (row < TC_ROWS) {
+          uint4 h, m, l;
+          split2(xa[i].x, xa[i].y, h.x, m.x, l.x);
+          split2(xa[i].z, xa[i].w, h.y, m.y, l.y);
+          split2(xb[i].x, xb[i].y, h.z, m.z, l.z);
+          split2(xb[i].z, xb[i].w, h.w, m.w, l.w);
+          uint8_t* d = dst + row * 128 + (((tid & 7) ^ (row & 7)) << 4);
+          *reinterpret_cast<uint4*>(d) = h;
+          *reinterpret_cast<uint4*>(d + TC_PLANE) = m;
+          *reinterpret_cast<uint4*>(d + 2 * TC_PLANE) = l;
+        }
+      }
+      ptx::fence_proxy_async_smem();
+      ptx::mbar_arrive(&full_a[sa]);
+      if (++sa == tc.n_a) { sa = 0; ph ^= 1u; }
+      if (u + 1 < n_units) load(u + 1);
+      if (DRAIN && u > 0) ok &= drain(u - 1);
+    }
+
+    // Carry update of the first layer: its left context for the next chunk is the tail of the caller's chunk, written into ring
+    // rows that no CTA of this launch reads (distinct logical frames map to distinct rows: the ring holds f_chunk + halo frames).
+    if (save_ring != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && phase == 0) {
+      const int first = T_in > p.save_rows ? T_in - p.save_rows : 0;
+      const int c4 = C_in >> 2;
+#pragma unroll 1
+      for (int i = tid; i < (T_in - first) * c4; i += TC_CONV) {
+        const int r = first + i / c4, c = (i - (i / c4) * c4) * 4;
+        const float4 v = *reinterpret_cast<const float4*>(in_direct + (long long)r * C_in + c);
+        *reinterpret_cast<float4*>(save_ring + (long long)((int)((pos_in + r) & (long long)in_mask)) * C_in + c) = v;
+      }
+    }
+
+    // ---------------- epilogue ----------------
+    const int row = m0 + q * 32 + lane;
+    const long long t_in = pos_in + row, t_out = (long long)p.n_phase * t_in + phase;
+    const float* xrow = p.residual_silu ? in_row_ptr(in_direct, pos_in, in_ring, in_mask, C_in, t_in) : nullptr;
+    float* dst = out_direct != nullptr ? out_direct + (t_out - pos_out) * p.C_out : out_ring + (long long)((int)(t_out & (long long)p.out_mask)) * p.C_out;
+    const bool valid = row < T_in;
+    float4 x[NC][4];                               // the residual row, fetched under the products
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const int n = n0 + 16 * (half + 2 * c) + 4 * g;
+        x[c][g] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.residual_silu && valid && n < p.C_out) x[c][g] = *reinterpret_cast<const float4*>(xrow + n);
+      }
+    if (DRAIN) ok &= drain(n_units - 1);
+    else ok &= tc_wait(accum, 0, s_fail, tc.err, 0x205);
+    ptx::tc_fence_after();
+    ok = ok && *reinterpret_cast<volatile int*>(s_fail) == 0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int c0 = 16 * (half + 2 * c);
+      float z0[16], z1[16], z2[16];
+      ptx::tmem_ld16x2(lanes + (uint32_t)(S_COL + c0), lanes + (uint32_t)(S_COL + BN + c0), z1, z2);
+      if (!DRAIN) ptx::tmem_ld16(lanes + (uint32_t)c0, z0);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) z0[i] = (DRAIN ? sum[c][i] : z0[i]) + (z1[i] + z2[i]);
+      if (!valid || !ok) continue;
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const int n = n0 + c0 + 4 * g;
+        if (n >= p.C_out) continue;
+        const float4 bias = *reinterpret_cast<const float4*>(p.bias + n);
+        float4 v = make_float4(z0[4 * g] + bias.x, z0[4 * g + 1] + bias.y, z0[4 * g + 2] + bias.z, z0[4 * g + 3] + bias.w);
+        if (p.residual_silu) v = make_float4(x[c][g].x + silu_f(v.x), x[c][g].y + silu_f(v.y), x[c][g].z + silu_f(v.z), x[c][g].w + silu_f(v.w));
+        if (p.post_silu) v = make_float4(silu_f(v.x), silu_f(v.y), silu_f(v.z), silu_f(v.w));
+        if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
+          uint32_t w[4];
+          float e[4];
+          philox4x32_10((uint32_t)(unsigned long long)t_out, (uint32_t)((unsigned long long)t_out >> 32), (uint32_t)(n >> 2),
+                        0x80000000u + (uint32_t)exc_rng_id, p.exc_seed_lo, p.exc_seed_hi, w);
+          normals4(w, e);
+          v.x = fmaf(p.exc_std, e[0], v.x); v.y = fmaf(p.exc_std, e[1], v.y); v.z = fmaf(p.exc_std, e[2], v.z); v.w = fmaf(p.exc_std, e[3], v.w);
+        }
+        *reinterpret_cast<float4*>(dst + n) = v;
+      }
+    }
+    ptx::tc_fence_before();
+  }
+  __syncthreads();
+  // (a wait that gave up may have left copies in flight: they land before the shared memory is given back)
+  if (*reinterpret_cast<volatile int*>(s_fail) != 0) __nanosleep(1000000);
+  if (warp == 8) ptx::tmem_dealloc(tmem_base, TMEM_COLS);
+}
+
+// W of (phase, tap), [C_in][C_out] fp32 -> planes of swizzled tiles (see TapConvTc::W).
+__global__ void tapconv_pack_kernel(const float* W, long long w_phase_stride, long long w_tap_stride, int C_in, int C_out, int C_pad, int n_blocks, int n_taps,
+                                    uint8_t* dst) {
+  const int blk = blockIdx.y, tap = blockIdx.z % n_taps, phase = blockIdx.z / n_taps;
+  const float* w = W + phase * w_phase_stride + tap * w_tap_stride;
+  uint8_t* d = dst + ((size_t)(phase * n_blocks + blk) * n_taps + tap) * 3 * C_pad * 128;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < C_pad * 32; i += gridDim.x * blockDim.x) {
+    const int n = i % C_pad, k = 2 * (i / C_pad), c = blk * 64 + k;   // two input channels of one output channel
+    const float x = n < C_out && c < C_in ? w[(size_t)c * C_out + n] : 0.f, y = n < C_out && c + 1 < C_in ? w[(size_t)(c + 1) * C_out + n] : 0.f;
+    uint32_t s[3];
+    split2(x, y, s[0], s[1], s[2]);
+    for (int q = 0; q < 3; ++q)
+      *reinterpret_cast<uint32_t*>(d + (size_t)q * C_pad * 128 + (size_t)n * 128 + (((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2) = s[q];
+  }
+}

@@ -83,10 +83,25 @@ struct TapConvF32 {
   int          exc_rng_id;    // by value, or from *call
 };
 
+// The tensor-core form of a tap convolution (dc_f32_tapconv.cuh): weights split into bf16 planes and packed as swizzled tiles.
+struct TapConvTc {
+  const uint8_t* W;          // [phase][64-channel block][tap][plane][C_pad][128 B]
+  int            C_pad;      // output channels, rounded up to a multiple of 32
+  int            n_blocks;   // 64-channel blocks of the input
+  int            per_tap;    // a panel serves one tap only (a tap reaches more than 8 frames back)
+  int            n_a, n_b;   // panels and weight tiles in shared memory (chosen by the launch)
+  int*           err;        // device word that a bounded wait sets when it gives up
+};
+size_t      tapconv_pack_bytes(const TapConvF32& p);
+// Fills tc (but for err) and enqueues the packing of p's weights into dst (tapconv_pack_bytes).
+void        pack_tapconv(const TapConvF32& p, uint8_t* dst, TapConvTc* tc);
+cudaError_t prepare_tapconv();   // function attributes; once per model
+
 // T_grid: frames the grid is sized for (p.T_in, or the largest T_in when p.call is set).
-// n_batch > 0: the launch carries that many slots (p.batch set); tile shape and reduction split are those of the
-// single-stream launch of the same layer, so that a slot's result has the single-stream bytes.
-void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st, int T_grid = -1, bool pdl = false, int n_batch = 0);
+// n_batch > 0: the launch carries that many slots (p.batch set).
+void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc, cudaStream_t st, int T_grid, int n_batch = 0);
+// The FP32-pipe form, for weights that are not packed (dc_conv_stack_noalloc).
+void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st);
 void launch_set_f32_call(const F32Call& v, F32Call* dst, cudaStream_t st);
 const void* set_f32_call_func();
 void launch_set_f32_batch(const F32Batch& v, F32Batch* dst, cudaStream_t st);
