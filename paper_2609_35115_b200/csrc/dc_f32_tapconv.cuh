@@ -10,8 +10,7 @@
 // operand latency) to what the conversion and the fp32 rows' traffic cost.
 //
 // One CTA: 128 frames x BN channels of one phase.  Ten warps: 0..7 read the fp32 input rows (ring, or the caller's chunk), split
-// them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue (a thread owns one output row and every
-// second 16-column chunk); 8 issues the products; 9 streams the weights, split and packed as swizzled tiles at create.
+// them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue; 8 issues the products; 9 streams the weights, split and packed as swizzled tiles at create.
 // A panel holds 64 channels of the 128 frames and of the up to 8 in front of them: a tap is a row offset of the operand
 // descriptor, so a row is read and split once for all its taps.  (Dilations above 4 fill the panel once per tap.)
 // Per 64 channels and tap: 4 reduction steps of ah x [bh bm bl], am x [bh bm], al x bh.
@@ -52,6 +51,17 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& 
   l = *reinterpret_cast<const uint32_t*>(&b);
 }
 
+// The random excitation of four channels of one output frame.  A call: inlined into the epilogue's unrolled loop the generator and its
+// logarithms and sines are most of the kernel's code, which every CTA then fetches past.
+__device__ __noinline__ float4 excite4(float4 v, long long t, int n, int rng_id, float std_dev, uint32_t seed_lo, uint32_t seed_hi) {
+  uint32_t w[4];
+  float e[4];
+  philox4x32_10((uint32_t)(unsigned long long)t, (uint32_t)((unsigned long long)t >> 32), (uint32_t)(n >> 2), 0x80000000u + (uint32_t)rng_id, seed_lo,
+                seed_hi, w);
+  normals4(w, e);
+  return make_float4(fmaf(std_dev, e[0], v.x), fmaf(std_dev, e[1], v.y), fmaf(std_dev, e[2], v.z), fmaf(std_dev, e[3], v.w));
+}
+
 // DRAIN (inputs of more than one panel): the tensor cores truncate when they add to an accumulator, which over a long reduction
 // is a bias (7.6e-5 of RMS at the vocoder's end with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel,
 // tap) - four additions - has an accumulator of its own, two panels' worth in turn, which the epilogue threads add up in registers,
@@ -60,7 +70,7 @@ template <int BN, bool DRAIN>
 __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(const __grid_constant__ TapConvF32 p, const __grid_constant__ TapConvTc tc) {
   // per-call values: from the device-side call record of the stream or of the slot (captured graphs), or by value
   int T_in = p.T_in;
-  long long pos_in = p.pos_in, pos_out = p.pos_out;
+  long long pos_in = p.pos_in;
   const float* in_direct = p.in_direct;
   float* out_direct = p.out_direct;
   int exc_rng_id = p.exc_rng_id;
@@ -84,7 +94,6 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     exc_rng_id = c.rng_id;
     T_in = c.T * p.rate_in;
     pos_in = c.frames * p.rate_in;
-    pos_out = pos_in * p.n_phase;
     in_direct = p.first_layer ? c.feats : nullptr;
     out_direct = p.last_layer ? c.out : nullptr;
   }
@@ -161,70 +170,93 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
   } else if (warp == 8) {
     // ---------------- products ----------------
+    // One (panel, tap) after the other; the loop is a chain of one thread's instructions, so addresses advance on 32-bit values and
+    // the next barriers are polled ahead of this step's products (with a wait in front of every step it took 1,700 cycles, the
+    // products alone 900).
     const uint32_t id3 = ptx::umma_idesc_bf16(TC_M, 3 * BN, 0, 0), id2 = ptx::umma_idesc_bf16(TC_M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(TC_M, BN, 0, 0);
-    const uint64_t dA = ptx::umma_desc_sw128(ptx::smem_u32(sA)), dB = ptx::umma_desc_sw128(ptx::smem_u32(sB));
-    int sa = 0, sb = 0;
-    uint32_t pa = 0, pb = 0, acc = 0;
-    bool ok = true;
+    constexpr uint32_t DESC_HI = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61)) >> 32);
+    const uint32_t a_lo = ((ptx::smem_u32(sA) & 0x3FFFF) >> 4) | (1u << 16), b_lo = ((ptx::smem_u32(sB) & 0x3FFFF) >> 4) | (1u << 16);
+    const uint32_t bar_b = ptx::smem_u32(full_b), bar_eb = ptx::smem_u32(empty_b), bar_a = ptx::smem_u32(full_a), bar_ea = ptx::smem_u32(empty_a);
+    const uint32_t off0 = (uint32_t)(tc.per_tap ? TC_H : TC_H - p.shift[0]) * 8u, off1 = (uint32_t)(TC_H - p.shift[1]) * 8u, off2 = (uint32_t)(TC_H - p.shift[2]) * 8u;
+    uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
+    bool ok = true, ready_a = ptx::mbar_try_wait_s(bar_a, 0), ready_b = ptx::mbar_try_wait_s(bar_b, 0);
+    int u = 0, j = 0;
 #pragma unroll 1
-    for (int u = 0; u < n_units && ok; ++u) {
-      if (DRAIN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
-      if (ok) ok = tc_wait(&full_a[sa], pa, s_fail, tc.err, 0x202);
-#pragma unroll 1
-      for (int j = 0; j < taps_u && ok; ++j) {
-        ok = tc_wait(&full_b[sb], pb, s_fail, tc.err, 0x203);
-        ptx::tc_fence_after();
-        const int off = tc.per_tap ? TC_H : TC_H - p.shift[j];   // (a panel filled for one tap has its rows at TC_H)
-        const uint64_t ah = dA + (uint64_t)(uint32_t)((sa * TC_PANEL + off * 128) >> 4), am = ah + (TC_PLANE >> 4), al = am + (TC_PLANE >> 4);
-        const uint64_t b = dB + (uint64_t)(uint32_t)(sb * (B_TILE >> 4));
-        if (ok && ptx::elect_one()) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (DRAIN) {
-              ptx::umma_bf16(tmem_base + (uint32_t)((u & 1) * 3 + j) * BN, ah + 2 * k, b + 2 * k, id1, k != 0);
-              ptx::umma_bf16(tmem_base + S_COL, ah + 2 * k, b + (BN * 128 >> 4) + 2 * k, id2, k == 0 ? (uint32_t)((u | j) != 0) : 1u);
-            } else {
-              ptx::umma_bf16(tmem_base, ah + 2 * k, b + 2 * k, id3, k == 0 ? acc : 1u);
-            }
-            ptx::umma_bf16(tmem_base + S_COL, am + 2 * k, b + 2 * k, id2, 1);
-            ptx::umma_bf16(tmem_base + S_COL + BN, al + 2 * k, b + 2 * k, id1, 1);
-          }
-          ptx::umma_commit(&empty_b[sb]);
-          if (j + 1 == taps_u) {
-            ptx::umma_commit(&empty_a[sa]);
-            if (DRAIN) ptx::umma_commit(&accum[u & 1]);
-          }
-        }
-        __syncwarp();
-        acc = 1;
-        if (++sb == tc.n_b) { sb = 0; pb ^= 1u; }
+    while (u < n_units && ok) {
+      if (j == 0) {
+        if (DRAIN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
+        if (!__all_sync(0xffffffffu, ready_a)) ok &= tc_wait(&full_a[sa], pa, s_fail, tc.err, 0x202);
       }
-      if (++sa == tc.n_a) { sa = 0; pa ^= 1u; }
+      if (!__all_sync(0xffffffffu, ready_b)) ok &= tc_wait(&full_b[sb], pb, s_fail, tc.err, 0x203);
+      if (!ok) break;
+      ptx::tc_fence_after();
+      const bool last = j + 1 == taps_u, first = u == 0 && j == 0;
+      const uint32_t al0 = a_lo + sa * (uint32_t)(TC_PANEL >> 4) + (j == 0 ? off0 : (j == 1 ? off1 : off2)), bl0 = b_lo + sb * (uint32_t)(B_TILE >> 4);
+      const uint64_t ah = ((uint64_t)DESC_HI << 32) | al0, am = ah + (TC_PLANE >> 4), al = am + (TC_PLANE >> 4), b = ((uint64_t)DESC_HI << 32) | bl0;
+      const uint32_t eb = bar_eb + 8u * sb, ea = bar_ea + 8u * sa, d_main = tmem_base + (uint32_t)((u & 1) * 3 + j) * BN;
+      uint64_t* done_u = &accum[u & 1];
+      if (++sb == (uint32_t)tc.n_b) { sb = 0; pb ^= 1u; }
+      if (last) {
+        if (++sa == (uint32_t)tc.n_a) { sa = 0; pa ^= 1u; }
+        ++u;
+        j = 0;
+        ready_a = u < n_units && ptx::mbar_try_wait_s(bar_a + 8u * sa, pa);
+      } else {
+        ++j;
+      }
+      ready_b = u < n_units && ptx::mbar_try_wait_s(bar_b + 8u * sb, pb);
+      if (ptx::elect_one()) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (DRAIN) {
+            ptx::umma_bf16(d_main, ah + 2 * k, b + 2 * k, id1, k != 0);
+            ptx::umma_bf16(tmem_base + S_COL, ah + 2 * k, b + (BN * 128 >> 4) + 2 * k, id2, k == 0 ? (uint32_t)!first : 1u);
+          } else {
+            ptx::umma_bf16(tmem_base, ah + 2 * k, b + 2 * k, id3, k == 0 ? (uint32_t)!first : 1u);
+          }
+          ptx::umma_bf16(tmem_base + S_COL, am + 2 * k, b + 2 * k, id2, 1);
+          ptx::umma_bf16(tmem_base + S_COL + BN, al + 2 * k, b + 2 * k, id1, 1);
+        }
+        ptx::umma_commit_s(eb);
+        if (last) {
+          ptx::umma_commit_s(ea);
+          if (DRAIN) ptx::umma_commit(done_u);
+        }
+      }
+      __syncwarp();
     }
     if (!DRAIN && ptx::elect_one()) ptx::umma_commit(accum);
     __syncwarp();
   } else {
     // ---------------- input rows -> bf16 planes ----------------
+    // Row addresses in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
+    // address of a row cost more instructions than its arithmetic): frame m0 + i, i possibly negative.
     const int C_in = p.C_in, in_mask = p.in_mask;
+    const uint32_t pos32 = (uint32_t)pos_in;
+    auto in_row = [&](int i) -> const float* {
+      const bool direct = in_direct != nullptr && i >= 0;
+      const uint32_t r = direct ? (uint32_t)i : (pos32 + (uint32_t)i) & (uint32_t)in_mask;
+      return (direct ? in_direct : in_ring) + (size_t)(r * (uint32_t)C_in);
+    };
     const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
     float4 xa[TC_ITEMS], xb[TC_ITEMS];
     auto load = [&](int u) {
       const int blk = tc.per_tap ? u / p.n_taps : u, tap = tc.per_tap ? u - blk * p.n_taps : 0;
       const int c = blk * 64 + c8;
-      const long long t0 = pos_in + m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
+      const int i0 = m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
 #pragma unroll
       for (int i = 0; i < TC_ITEMS; ++i) {
         const int row = row0 + 32 * i;
         xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         xb[i] = xa[i];
         if (row < TC_ROWS && m0 + row - TC_H < T_in && c < C_in) {
-          const float* src = in_row_ptr(in_direct, pos_in, in_ring, in_mask, C_in, t0 + row) + c;
+          const float* src = in_row(i0 + row) + c;
           xa[i] = *reinterpret_cast<const float4*>(src);
           if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
         }
       }
     };
-    const int q = warp & 3, half = warp >> 2;      // epilogue: TMEM lane quarter; 16-column chunks half, half + 2, ...
+    const int q = warp & 3, col0 = (warp >> 2) * (BN / 2);   // epilogue: TMEM lane quarter; columns col0 .. col0 + BN / 2 - 1
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
     constexpr int NC = BN / 32;
     float sum[NC][16];
@@ -239,7 +271,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       ptx::tc_fence_after();
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const uint32_t col = lanes + (uint32_t)((u & 1) * 3 * BN + 16 * (half + 2 * c));
+        const uint32_t col = lanes + (uint32_t)((u & 1) * 3 * BN + col0 + 16 * c);
         float z[16], y[16];
         if (taps_u == 1) {
           ptx::tmem_ld16(col, z);
@@ -304,50 +336,69 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
 
     // ---------------- epilogue ----------------
-    const int row = m0 + q * 32 + lane;
-    const long long t_in = pos_in + row, t_out = (long long)p.n_phase * t_in + phase;
-    const float* xrow = p.residual_silu ? in_row_ptr(in_direct, pos_in, in_ring, in_mask, C_in, t_in) : nullptr;
-    float* dst = out_direct != nullptr ? out_direct + (t_out - pos_out) * p.C_out : out_ring + (long long)((int)(t_out & (long long)p.out_mask)) * p.C_out;
-    const bool valid = row < T_in;
-    float4 x[NC][4];                               // the residual row, fetched under the products
+    // A thread's accumulator row crosses to row-wise order through shared memory (the panel is idle by then), so that a warp reads the
+    // residual and writes the result in whole 64- or 128-byte pieces of rows: a thread per row took 32 wavefronts per access, half
+    // of the load/store pipe's time.
+    constexpr int LPR = BN / 8;                    // lanes that share a row, 4 channels each
+    constexpr int LD = BN / 2 + 4;                 // floats between rows of the staging tile (no bank conflicts)
+    float* stage = reinterpret_cast<float*>(sA) + warp * 32 * LD;
+    const int g = lane % LPR, rr = lane / LPR, n = n0 + col0 + 4 * g;
+    const bool n_ok = n < p.C_out;
+    float* const out = out_direct != nullptr ? out_direct : out_ring;
+    const uint32_t out0 = out_direct != nullptr ? 0u : (uint32_t)(p.n_phase * pos_in), out_mask = out_direct != nullptr ? ~0u : (uint32_t)p.out_mask;
+    float4 x[LPR];                                 // the residual rows, fetched under the products
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int n = n0 + 16 * (half + 2 * c) + 4 * g;
-        x[c][g] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p.residual_silu && valid && n < p.C_out) x[c][g] = *reinterpret_cast<const float4*>(xrow + n);
-      }
+    for (int i = 0; i < LPR; ++i) {
+      const int row = m0 + q * 32 + rr + i * (32 / LPR);
+      x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (p.residual_silu && row < T_in && n_ok)
+        x[i] = *reinterpret_cast<const float4*>(in_row(row) + n);
+    }
+    const float4 bias = n_ok ? *reinterpret_cast<const float4*>(p.bias + n) : make_float4(0.f, 0.f, 0.f, 0.f);
     if (DRAIN) ok &= drain(n_units - 1);
     else ok &= tc_wait(accum, 0, s_fail, tc.err, 0x205);
     ptx::tc_fence_after();
     ok = ok && *reinterpret_cast<volatile int*>(s_fail) == 0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const int c0 = 16 * (half + 2 * c);
       float z0[16], z1[16], z2[16];
-      ptx::tmem_ld16x2(lanes + (uint32_t)(S_COL + c0), lanes + (uint32_t)(S_COL + BN + c0), z1, z2);
-      if (!DRAIN) ptx::tmem_ld16(lanes + (uint32_t)c0, z0);
+      ptx::tmem_ld16x2(lanes + (uint32_t)(S_COL + col0 + 16 * c), lanes + (uint32_t)(S_COL + BN + col0 + 16 * c), z1, z2);
+      if (!DRAIN) ptx::tmem_ld16(lanes + (uint32_t)(col0 + 16 * c), z0);
 #pragma unroll
       for (int i = 0; i < 16; ++i) z0[i] = (DRAIN ? sum[c][i] : z0[i]) + (z1[i] + z2[i]);
-      if (!valid || !ok) continue;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int n = n0 + c0 + 4 * g;
-        if (n >= p.C_out) continue;
-        const float4 bias = *reinterpret_cast<const float4*>(p.bias + n);
-        float4 v = make_float4(z0[4 * g] + bias.x, z0[4 * g + 1] + bias.y, z0[4 * g + 2] + bias.z, z0[4 * g + 3] + bias.w);
-        if (p.residual_silu) v = make_float4(x[c][g].x + silu_f(v.x), x[c][g].y + silu_f(v.y), x[c][g].z + silu_f(v.z), x[c][g].w + silu_f(v.w));
-        if (p.post_silu) v = make_float4(silu_f(v.x), silu_f(v.y), silu_f(v.z), silu_f(v.w));
-        if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
-          uint32_t w[4];
-          float e[4];
-          philox4x32_10((uint32_t)(unsigned long long)t_out, (uint32_t)((unsigned long long)t_out >> 32), (uint32_t)(n >> 2),
-                        0x80000000u + (uint32_t)exc_rng_id, p.exc_seed_lo, p.exc_seed_hi, w);
-          normals4(w, e);
-          v.x = fmaf(p.exc_std, e[0], v.x); v.y = fmaf(p.exc_std, e[1], v.y); v.z = fmaf(p.exc_std, e[2], v.z); v.w = fmaf(p.exc_std, e[3], v.w);
-        }
-        *reinterpret_cast<float4*>(dst + n) = v;
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(stage + lane * LD + 16 * c + 4 * i) = make_float4(z0[4 * i], z0[4 * i + 1], z0[4 * i + 2], z0[4 * i + 3]);
+    }
+    __syncwarp();
+    // (one pass per step over all of the thread's pieces: the options cost one branch each, and the pieces' latencies overlap)
+    float4 v[LPR];
+#pragma unroll
+    for (int i = 0; i < LPR; ++i) {
+      v[i] = *reinterpret_cast<const float4*>(stage + (rr + i * (32 / LPR)) * LD + 4 * g);
+      v[i] = make_float4(v[i].x + bias.x, v[i].y + bias.y, v[i].z + bias.z, v[i].w + bias.w);
+    }
+    if (p.residual_silu) {
+#pragma unroll
+      for (int i = 0; i < LPR; ++i)
+        v[i] = make_float4(x[i].x + silu_f(v[i].x), x[i].y + silu_f(v[i].y), x[i].z + silu_f(v[i].z), x[i].w + silu_f(v[i].w));
+    }
+    if (p.post_silu) {
+#pragma unroll
+      for (int i = 0; i < LPR; ++i) v[i] = make_float4(silu_f(v[i].x), silu_f(v[i].y), silu_f(v[i].z), silu_f(v[i].w));
+    }
+    const int first = m0 + q * 32 + rr;
+    if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
+#pragma unroll
+      for (int i = 0; i < LPR; ++i)
+        v[i] = excite4(v[i], (long long)p.n_phase * (pos_in + first + i * (32 / LPR)) + phase, n, exc_rng_id, p.exc_std, p.exc_seed_lo, p.exc_seed_hi);
+    }
+    if (n_ok && ok) {
+#pragma unroll
+      for (int i = 0; i < LPR; ++i) {
+        const int row = first + i * (32 / LPR);
+        const uint32_t ro = (out0 + (uint32_t)(p.n_phase * row + phase)) & out_mask;
+        if (row < T_in) *reinterpret_cast<float4*>(out + (size_t)(ro * (uint32_t)p.C_out) + n) = v[i];
       }
     }
     ptx::tc_fence_before();
