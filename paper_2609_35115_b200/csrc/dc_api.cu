@@ -154,10 +154,13 @@ struct dc_model {
   // fp32 pipelines: dc_decode_batch runs every layer ONCE for all the streams of the batch (slot = grid plane); the slot
   // records live here and are rewritten per call by the first node of the captured batch step
   dc::F32Batch*   d_batch = nullptr;
-  cudaGraph_t     gb_graph = nullptr;
-  cudaGraphExec_t gb_exec = nullptr;
-  cudaGraphNode_t gb_set_node = nullptr;
-  int             gb_launches = 0;
+  struct BatchGraph {
+    cudaGraph_t     graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaGraphNode_t set_node = nullptr;
+    int             launches = 0;
+  };
+  std::map<int, BatchGraph> gb;   // batch size -> captured chunk step
   std::atomic<uint64_t> counters[8];
   std::atomic<int> open_streams{0};
   int    streams_opened = 0;   // so far: the next fp32 stream's random-stream index (streams of a model are opened one at a time)
@@ -167,11 +170,12 @@ struct dc_model {
 };
 
 static void free_batch_graph(dc_model* m) {
-  if (m->gb_exec) cudaGraphExecDestroy(m->gb_exec);
-  if (m->gb_graph) cudaGraphDestroy(m->gb_graph);
+  for (auto& kv : m->gb) {
+    if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+    if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
+  }
+  m->gb.clear();
   if (m->d_batch) dc::dev_free(m->d_batch);
-  m->gb_exec = nullptr;
-  m->gb_graph = nullptr;
   m->d_batch = nullptr;
 }
 
@@ -357,7 +361,7 @@ static void build_f32_layers(dc_model* m) {
 }
 
 static void build_f32_graph(dc_stream* s);
-static void build_f32_batch_graph(dc_model* m);
+static void build_f32_batch_graph(dc_model* m, int nb);
 
 // What of a conv layer's launch does not depend on the call.
 static dc::TapConvF32 tapconv_layer(const dc_model* m, int l) {
@@ -478,7 +482,7 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
       dc::set_error("weight upload failed: %s", cudaGetErrorString(e));
       st = e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;
     }
-    if (st == DC_OK && m->d_batch) build_f32_batch_graph(m);
+    if (st == DC_OK && m->d_batch) build_f32_batch_graph(m, m->cfg.max_batch);
   }
   if (st == DC_OK && !m->flow && m->h_in == nullptr) {
     // bounce buffers of dc_decode_batch_host for the pipelines whose kernels do not read host memory themselves
@@ -909,11 +913,11 @@ static void build_f32_graph(dc_stream* s) {
   cudaStreamDestroy(cap);
 }
 
-// The layers of one fp32 chunk step for up to max_batch streams at once: every layer is ONE launch whose grid planes
+// The layers of one fp32 chunk step for nb streams at once: every layer is ONE launch whose grid planes
 // are the slots of the batch record (stream, frames, pointers); per slot the tiles, the reduction split and the
 // arithmetic are those of the single-stream step, so a stream's bytes do not depend on who shares its launch.
-static void enqueue_f32_batch(dc_model* m, cudaStream_t cs, int* launches) {
-  const int nL = (int)m->layers.size(), nb = m->cfg.max_batch;
+static void enqueue_f32_batch(dc_model* m, int nb, cudaStream_t cs, int* launches) {
+  const int nL = (int)m->layers.size();
   for (int l = 0; l < nL; ++l) {
     const F32Layer& L = m->layers[l];
     const int Tgrid = m->cfg.f_chunk * L.rate_in;
@@ -934,8 +938,10 @@ static void enqueue_f32_batch(dc_model* m, cudaStream_t cs, int* launches) {
   }
 }
 
-// Captured once per model (at dc_create): the batch step is one graph launch, only the slot records change.
-static void build_f32_batch_graph(dc_model* m) {
+// One graph per batch size, kept for the model's lifetime (max_batch at dc_create, another size at its first call): the
+// batch step is one graph launch, only the slot records change.  A grid captured for the largest batch alone made a smaller
+// call wait for the empty CTAs of the slots it does not have.
+static void build_f32_batch_graph(dc_model* m, int nb) {
   if (m->cfg.options & DC_OPT_NO_GRAPH) return;
   cudaStream_t cap = nullptr;
   if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return; }
@@ -944,7 +950,8 @@ static void build_f32_batch_graph(dc_model* m) {
     static const dc::F32Batch empty{};
     dc::launch_set_f32_batch(empty, m->d_batch, cap);
     int n = 1;
-    enqueue_f32_batch(m, cap, &n);
+    dc_model::BatchGraph bg;
+    enqueue_f32_batch(m, nb, cap, &n);
     if (cudaStreamEndCapture(cap, &graph) == cudaSuccess && graph != nullptr) {
       size_t n_nodes = 0;
       cudaGraphGetNodes(graph, nullptr, &n_nodes);
@@ -955,14 +962,13 @@ static void build_f32_batch_graph(dc_model* m) {
         cudaKernelNodeParams kp{};
         if (cudaGraphNodeGetType(nd, &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel &&
             cudaGraphKernelNodeGetParams(nd, &kp) == cudaSuccess && kp.func == dc::set_f32_batch_func())
-          m->gb_set_node = nd;
+          bg.set_node = nd;
       }
-      if (m->gb_set_node != nullptr && cudaGraphInstantiate(&m->gb_exec, graph, 0) == cudaSuccess) {
-        m->gb_graph = graph;
-        m->gb_launches = n;
+      if (bg.set_node != nullptr && cudaGraphInstantiate(&bg.exec, graph, 0) == cudaSuccess) {
+        bg.graph = graph;
+        bg.launches = n;
+        m->gb[nb] = bg;
         graph = nullptr;
-      } else {
-        m->gb_exec = nullptr;
       }
     }
   }
@@ -981,7 +987,12 @@ static dc_status decode_f32_batch(dc_model* m, int n, dc_stream* const* streams,
     hb.s[i].call = dc::F32Call{s->frames_total, T[i], (int)(s->chunks & 1), feats[i], out[i], s->rng_id};
     hb.s[i].ptrs = s->d_ptrs;
   }
-  if (m->gb_exec != nullptr && !m->prof.on) {
+  auto it = m->gb.find(n);
+  if (it == m->gb.end() && !m->prof.on) {
+    build_f32_batch_graph(m, n);
+    it = m->gb.find(n);
+  }
+  if (it != m->gb.end() && !m->prof.on) {
     dc::F32Batch* dst = m->d_batch;
     void* args[2] = {&hb, &dst};
     cudaKernelNodeParams kp{};
@@ -989,15 +1000,15 @@ static dc_status decode_f32_batch(dc_model* m, int n, dc_stream* const* streams,
     kp.gridDim = dim3(1);
     kp.blockDim = dim3(dc::F32_MAX_BATCH);
     kp.kernelParams = args;
-    DC_CUDA(cudaGraphExecKernelNodeSetParams(m->gb_exec, m->gb_set_node, &kp));
-    DC_CUDA(cudaGraphLaunch(m->gb_exec, cs));
-    *launches += m->gb_launches;
+    DC_CUDA(cudaGraphExecKernelNodeSetParams(it->second.exec, it->second.set_node, &kp));
+    DC_CUDA(cudaGraphLaunch(it->second.exec, cs));
+    *launches += it->second.launches;
     m->counters[7]++;
     return DC_OK;
   }
   dc::launch_set_f32_batch(hb, m->d_batch, cs);
   ++*launches;
-  enqueue_f32_batch(m, cs, launches);
+  enqueue_f32_batch(m, n, cs, launches);
   DC_CUDA(cudaGetLastError());
   return DC_OK;
 }

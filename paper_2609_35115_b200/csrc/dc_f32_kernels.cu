@@ -225,19 +225,24 @@ __global__ void __launch_bounds__(512) tapconv_f32_kernel(const TapConvF32 p, co
 
 constexpr int HFR = 64;         // frames per CTA of the head kernel: 3 recomputed frames of overlap + 61 new ones
 constexpr int HF = HFR - 3;     // new frames per CTA
-constexpr int HQ = 4;           // threads per frame: each reduces a quarter of the channels, then a quarter of the DFT outputs
+constexpr int HQ = 4;           // threads per frame once the channels are reduced: each produces a quarter of the DFT outputs
+constexpr int HG = 4;           // consecutive frames whose reduction 16 lanes share, four channels of every 64 each
 constexpr int HT = HFR * HQ;    // threads per CTA
+constexpr int HWP = 4 * 18 + 2; // shared-memory words of the weights of four channels: 16 lanes hit 16 different pairs of banks
 constexpr int NFFT = 16, NB = 9, NH = 18, HOP = 4, TAIL = NFFT - HOP;
 
 __constant__ float c_cos16[16];  // cos(2 pi j / 16)
 __constant__ float c_sin16[16];
 __constant__ float c_hann16[16];
 
-// One thread per frame left a 3 x C x 18 reduction (3,456 dependent multiply-adds at C = 64) on two warps per CTA:
-// 23 us for 6,000 frames.  Four adjacent lanes share a frame: lane q reduces the channels c = q (mod 4) blocks of
-// four, the partial sums are added across the four lanes in a fixed butterfly (every lane ends with the same
-// bits), and lane q then produces DFT outputs 4q .. 4q + 3 of the frame.
-__global__ void __launch_bounds__(HT) head_istft_f32_kernel(const HeadIstftF32 p_in) {
+// Bound by the fp32 units (3 x C x 18 multiply-adds a frame, 36 k cycles for 32 streams of 6,000 frames).  A thread that
+// reduced one frame read a weight from shared memory for every two multiply-adds and computed every exponential and
+// sine of its frame although three other lanes had the same ones: 114 us for 32 streams of 6,000 frames, 69 like this.  Sixteen lanes now reduce four
+// consecutive frames together: a lane takes four channels, reads each of the six rows once, and a weight serves four
+// frames.  The partial sums are then handed out so that each frame ends up with four lanes (the halves of the frames
+// are exchanged at distances 8 and 4, the sums added at distances 2 and 1: a fixed order, every lane of a frame
+// has the same bits), which share the nine bins and the sixteen outputs of the inverse transform.
+__global__ void __launch_bounds__(HT, 2) head_istft_f32_kernel(const HeadIstftF32 p_in) {
   extern __shared__ __align__(16) float smem[];
   ptx::pdl_launch();
   ptx::pdl_wait();
@@ -258,94 +263,153 @@ __global__ void __launch_bounds__(HT) head_istft_f32_kernel(const HeadIstftF32 p
     p.pcm = c.out;
   }
   if ((int)blockIdx.x * HF >= p.T) return;
-  float* Ws = smem;                              // [3*C][NH]
-  float* g = smem + 3 * p.C * NH;                // [HFR][NFFT] windowed frame signals
+  float* Ws = smem;                              // [3][C / 4] blocks of four channels
+  float* g = smem + 3 * (p.C / 4) * HWP;         // [HFR][NFFT] windowed frame signals
   const int tid = threadIdx.x;
-  for (int i = tid; i < 3 * p.C * NH; i += HT) Ws[i] = p.W[i];
+  const int l16 = tid & 15;
+  for (int i = tid; i < 3 * p.C * NH / 4; i += HT) {   // 72 floats of a block are whole float4s; its padding breaks their alignment
+    const float4 w = reinterpret_cast<const float4*>(p.W)[i];
+    float2* d = reinterpret_cast<float2*>(Ws + (i / 18) * HWP + (i % 18) * 4);
+    d[0] = make_float2(w.x, w.y);
+    d[1] = make_float2(w.z, w.w);
+  }
   __syncthreads();
-
-  const int fr = tid / HQ, q = tid % HQ;          // frame slot of the CTA, quarter
-  const int f_local = blockIdx.x * HF + fr - 3;   // frame index within the chunk (may be < 0)
-  const bool compute = f_local >= 0 && f_local < p.T;   // frames of earlier chunks come from the tail
-  // (all four lanes of a frame take the same branch, and a warp holds whole frames: the shuffles below are
-  // executed by complete groups)
-  float z[NH];
+  // a CTA takes every gridDim.x-th run of HF frames: the weights are laid out once for all of them
+#pragma unroll 1
+  for (int tile = blockIdx.x; tile * HF < p.T; tile += gridDim.x) {
+    const int f_base = tile * HF - 3 + (tid >> 4) * HG;   // first of the four frames (may be < 0)
+    const int t32 = (int)((p.pos + f_base) & (long long)p.in_mask);
+    unsigned long long z2[HG][NH / 2];             // pairs of neighbouring outputs
 #pragma unroll
-  for (int o = 0; o < NH; ++o) z[o] = 0.f;
-  if (compute) {
-    const long long t = p.pos + f_local;
-    for (int tap = 0; tap < 3; ++tap) {
-      const float* x = p.in_ring + (long long)((int)((t - (2 - tap)) & (long long)p.in_mask)) * p.C;
-      const float* w = Ws + tap * p.C * NH;
-      for (int c = 4 * q; c < p.C; c += 4 * HQ) {
-        const float4 xv = *reinterpret_cast<const float4*>(x + c);
-        const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+    for (int f = 0; f < HG; ++f)
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+      for (int o = 0; o < NH / 2; ++o) z2[f][o] = 0;
+#pragma unroll 1
+    for (int c = 4 * l16; c < p.C; c += 64) {
+      float4 x[HG + 2];                            // rows f_base - 2 .. f_base + 3: those outside the chunk are read and not used
 #pragma unroll
-          for (int o = 0; o < NH; ++o) z[o] = fmaf(xs[u], w[(c + u) * NH + o], z[o]);
+      for (int r = 0; r < HG + 2; ++r)
+        x[r] = *reinterpret_cast<const float4*>(p.in_ring + (long long)((t32 + r - 2) & p.in_mask) * p.C + c);
+#pragma unroll
+      for (int tap = 0; tap < 3; ++tap) {
+        const float* w = Ws + (tap * (p.C / 4) + c / 4) * HWP;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          unsigned long long xx[HG];
+#pragma unroll
+          for (int f = 0; f < HG; ++f) {
+            const float4 xr = x[f + tap];
+            const float xv = u == 0 ? xr.x : u == 1 ? xr.y : u == 2 ? xr.z : xr.w;
+            asm("mov.b64 %0, {%1, %1};" : "=l"(xx[f]) : "f"(xv));
+          }
+#pragma unroll
+          for (int o = 0; o < NH / 2; ++o) {
+            const unsigned long long wv = *reinterpret_cast<const unsigned long long*>(w + u * NH + 2 * o);
+#pragma unroll
+            for (int f = 0; f < HG; ++f) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(z2[f][o]) : "l"(xx[f]), "l"(wv));
+          }
+        }
       }
     }
-  }
+    float z[HG][NH];
 #pragma unroll
-  for (int o = 0; o < NH; ++o) {
-    z[o] += __shfl_xor_sync(0xffffffffu, z[o], 1);
-    z[o] += __shfl_xor_sync(0xffffffffu, z[o], 2);
-  }
-  float gv[NFFT / HQ];
+    for (int f = 0; f < HG; ++f)
 #pragma unroll
-  for (int k = 0; k < NFFT / HQ; ++k) gv[k] = 0.f;
-  if (compute) {
-    float re[NB], im[NB];
+      for (int o = 0; o < NH / 2; ++o) asm("mov.b64 {%0, %1}, %2;" : "=f"(z[f][2 * o]), "=f"(z[f][2 * o + 1]) : "l"(z2[f][o]));
+    // lane bits 3 and 2 select the frame, bits 1 and 0 are the quarter
+    const int q = l16 & 3, sel = l16 >> 2;
+    const int fr = (tid >> 4) * HG + sel;           // frame slot of the CTA
+    const int f_local = f_base + sel;               // frame index within the chunk
+    const bool compute = f_local >= 0 && f_local < p.T;   // frames of earlier chunks come from the tail
+    const bool up8 = (sel & 2) != 0, up4 = (sel & 1) != 0;
+    float zf[NH];
 #pragma unroll
-    for (int f = 0; f < NB; ++f) {
-      const float mag = expf(fminf(z[f] + p.bias[f], p.clamp));
-      float sn, cs;
-      sincosf(z[NB + f] + p.bias[NB + f], &sn, &cs);
-      re[f] = mag * cs;
-      im[f] = mag * sn;
+    for (int o = 0; o < NH; ++o) {
+      const float k0 = up8 ? z[2][o] : z[0][o], k1 = up8 ? z[3][o] : z[1][o];
+      const float s0 = up8 ? z[0][o] : z[2][o], s1 = up8 ? z[1][o] : z[3][o];
+      const float a0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 8), a1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 8);
+      zf[o] = (up4 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up4 ? a0 : a1, 4);
+      zf[o] += __shfl_xor_sync(0xffffffffu, zf[o], 2);
+      zf[o] += __shfl_xor_sync(0xffffffffu, zf[o], 1);
     }
+    // bins q, q + 4 and (for all four lanes alike) 8
+    float re[NB], im[NB];
+    {
+      float rq[3], iq[3];
 #pragma unroll
-    for (int kk = 0; kk < NFFT / HQ; ++kk) {
-      const int k = q * (NFFT / HQ) + kk;
-      float a = re[0] + ((k & 1) ? -re[NB - 1] : re[NB - 1]);
+      for (int i = 0; i < 3; ++i) {
+        const int f = i < 2 ? 4 * i + q : NB - 1;
+        const float zm = i == 2 ? zf[NB - 1] : q == 0 ? zf[4 * i] : q == 1 ? zf[4 * i + 1] : q == 2 ? zf[4 * i + 2] : zf[4 * i + 3];
+        const float zp = i == 2 ? zf[NH - 1] : q == 0 ? zf[NB + 4 * i] : q == 1 ? zf[NB + 4 * i + 1] : q == 2 ? zf[NB + 4 * i + 2] : zf[NB + 4 * i + 3];
+        const float mag = expf(fminf(zm + p.bias[f], p.clamp));
+        float sn, cs;
+        sincosf(zp + p.bias[NB + f], &sn, &cs);
+        rq[i] = mag * cs;
+        iq[i] = mag * sn;
+      }
+#pragma unroll
+      for (int f = 0; f < NB; ++f) {
+        re[f] = f == NB - 1 ? rq[2] : __shfl_sync(0xffffffffu, rq[f >> 2], f & 3, 4);
+        im[f] = f == NB - 1 ? iq[2] : __shfl_sync(0xffffffffu, iq[f >> 2], f & 3, 4);
+      }
+    }
+    float gv[NFFT / HQ];
+#pragma unroll
+    for (int k = 0; k < NFFT / HQ; ++k) gv[k] = 0.f;
+    if (compute) {
+      // sample k = 4 q + kk: the angle f k 2 pi / 16 is f kk 2 pi / 16 and f q quarter turns.  The turns are taken by
+      // exchanging re and im, so that the table is indexed by constants alone: lanes with indices of their own made the
+      // constant cache serve them one after another, which alone was most of the kernel.
 #pragma unroll
       for (int f = 1; f < NB - 1; ++f) {
-        const int j = (f * k) & 15;
-        a += 2.0f * (re[f] * c_cos16[j] - im[f] * c_sin16[j]);
+        const int turn = (f * q) & 3;
+        const float r = (turn & 1) ? im[f] : re[f], i = (turn & 1) ? re[f] : im[f];
+        re[f] = turn == 1 || turn == 2 ? -r : r;
+        im[f] = turn >= 2 ? -i : i;
       }
-      gv[kk] = c_hann16[k] * a * (1.0f / NFFT);
-    }
-  }
 #pragma unroll
-  for (int kk = 0; kk < NFFT / HQ; ++kk) g[fr * NFFT + q * (NFFT / HQ) + kk] = gv[kk];
-  __syncthreads();
+      for (int kk = 0; kk < NFFT / HQ; ++kk) {
+        float a = re[0] + ((kk & 1) ? -re[NB - 1] : re[NB - 1]);
+#pragma unroll
+        for (int f = 1; f < NB - 1; ++f) {
+          const int j = (f * kk) & 15;
+          a += 2.0f * (re[f] * c_cos16[j] - im[f] * c_sin16[j]);
+        }
+        const float hann = q == 0 ? c_hann16[kk] : q == 1 ? c_hann16[4 + kk] : q == 2 ? c_hann16[8 + kk] : c_hann16[12 + kk];
+        gv[kk] = hann * a * (1.0f / NFFT);
+      }
+    }
+#pragma unroll
+    for (int kk = 0; kk < NFFT / HQ; ++kk) g[fr * NFFT + q * (NFFT / HQ) + kk] = gv[kk];
+    __syncthreads();
 
-  // overlap-add: one thread per new frame
-  const int fo = tid;                              // frame slot
-  const int fo_local = blockIdx.x * HF + fo - 3;
-  if (tid < HFR && fo >= 3 && fo_local < p.T) {
-    const float inv_norm = 1.0f / 1.5f;   // sum of the four overlapping squared Hann windows
-    float out[HOP];
+    // overlap-add: one thread per new frame
+    const int fo = tid;                              // frame slot
+    const int fo_local = tile * HF + fo - 3;
+    if (tid < HFR && fo >= 3 && fo_local < p.T) {
+      const float inv_norm = 1.0f / 1.5f;   // sum of the four overlapping squared Hann windows
+      float out[HOP];
 #pragma unroll
-    for (int j = 0; j < HOP; ++j) {
-      // sample 4 f + j: contributions of frames f, f-1, f-2, f-3 at offsets j, 4+j, 8+j, 12+j;
-      // the part that frames of earlier chunks contribute is the carried tail
-      float a = (fo_local < 3 && 4 * fo_local + j < TAIL) ? p.tail_in[4 * fo_local + j] : 0.f;
+      for (int j = 0; j < HOP; ++j) {
+        // sample 4 f + j: contributions of frames f, f-1, f-2, f-3 at offsets j, 4+j, 8+j, 12+j;
+        // the part that frames of earlier chunks contribute is the carried tail
+        float a = (fo_local < 3 && 4 * fo_local + j < TAIL) ? p.tail_in[4 * fo_local + j] : 0.f;
 #pragma unroll
-      for (int i = 3; i >= 0; --i) a += g[(fo - i) * NFFT + 4 * i + j];
-      out[j] = a * inv_norm;
-    }
-    *reinterpret_cast<float4*>(p.pcm + 4ll * fo_local) = make_float4(out[0], out[1], out[2], out[3]);
-    if (fo_local == p.T - 1) {
-      // tail for the next chunk: samples 4T + q, q in [0,12), from the last three frames
-      for (int qq = 0; qq < TAIL; ++qq) {
-        float a = 0.f;
-        for (int i = 2; i >= 0; --i)
-          if (4 * (i + 1) + qq < NFFT) a += g[(fo - i) * NFFT + 4 * (i + 1) + qq];
-        p.tail_out[qq] = a;
+        for (int i = 3; i >= 0; --i) a += g[(fo - i) * NFFT + 4 * i + j];
+        out[j] = a * inv_norm;
+      }
+      *reinterpret_cast<float4*>(p.pcm + 4ll * fo_local) = make_float4(out[0], out[1], out[2], out[3]);
+      if (fo_local == p.T - 1) {
+        // tail for the next chunk: samples 4T + q, q in [0,12), from the last three frames
+        for (int qq = 0; qq < TAIL; ++qq) {
+          float a = 0.f;
+          for (int i = 2; i >= 0; --i)
+            if (4 * (i + 1) + qq < NFFT) a += g[(fo - i) * NFFT + 4 * (i + 1) + qq];
+          p.tail_out[qq] = a;
+        }
       }
     }
+    __syncthreads();
   }
 }
 
@@ -431,6 +495,7 @@ cudaError_t prepare_tapconv() {
   cudaError_t e = cudaSuccess;
   for (auto fn : {tapconv_tc_kernel<32, false>, tapconv_tc_kernel<64, false>, tapconv_tc_kernel<32, true>, tapconv_tc_kernel<64, true>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(head_istft_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
 }
 
@@ -526,9 +591,10 @@ cudaError_t prepare_f32_constants() {
 
 void launch_head_istft_f32(const HeadIstftF32& p, cudaStream_t st, int T_grid, bool pdl, int n_batch) {
   if (T_grid < 0) T_grid = p.T;
-  const size_t smem = (size_t)(3 * p.C * NH + HFR * NFFT) * sizeof(float);
-  const int grid = (T_grid + HF - 1) / HF;
-  launch_ex(head_istft_f32_kernel, dim3(grid, n_batch > 0 ? n_batch : 1), dim3(HT), smem, st, pdl, p);
+  const size_t smem = (size_t)(3 * (p.C / 4) * HWP + HFR * NFFT) * sizeof(float);
+  // as many CTAs as are resident at once, two per SM: each lays out the weights once and takes several runs of frames
+  const int planes = n_batch > 0 ? n_batch : 1, grid = (T_grid + HF - 1) / HF, most = planes < 2 * 148 ? 2 * 148 / planes : 1;
+  launch_ex(head_istft_f32_kernel, dim3(grid < most ? grid : most, planes), dim3(HT), smem, st, pdl, p);
 }
 
 }  // namespace dc
