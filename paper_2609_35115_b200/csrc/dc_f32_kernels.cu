@@ -493,7 +493,8 @@ void pack_tapconv(const TapConvF32& p, uint8_t* dst, TapConvTc* tc) {
 
 cudaError_t prepare_tapconv() {
   cudaError_t e = cudaSuccess;
-  for (auto fn : {tapconv_tc_kernel<32, false>, tapconv_tc_kernel<64, false>, tapconv_tc_kernel<32, true>, tapconv_tc_kernel<64, true>})
+  for (auto fn : {tapconv_tc_kernel<32, false, false>, tapconv_tc_kernel<64, false, false>, tapconv_tc_kernel<32, true, false>, tapconv_tc_kernel<64, true, false>,
+                  tapconv_tc_kernel<64, true, true>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(head_istft_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
@@ -506,12 +507,17 @@ void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc_in, cudaStream_t
   // 64 columns per CTA once that fills the GPU (a reduction step costs 209 cycles of the tensor pipe at 64 columns, 134 at 32), else 32
   // over twice the SMs.  A column's sum is the same either way.  A single panel leaves room for two CTAs per SM, which overlap one's
   // conversion and epilogue with the other's products; several panels overlap inside the CTA.
-  const bool wide = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= 148;
+  const bool wide0 = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= 148;
+  // two slots per tile where that saves a wave: several panels (one CTA per SM), chunks of at most half a tile
+  const bool pack = drain && n_batch > 1 && T_grid <= TC_PACK && tc.C_pad % 64 == 0 && (long long)(tc.C_pad / (wide0 ? 64 : 32)) * planes > 148;
+  const bool wide = wide0 || pack;
   tc.n_a = drain ? 2 : 1;
   tc.n_b = wide ? (drain ? 3 : 2) : TC_MAX_B;
   const int bn = wide ? 64 : 32;
-  const dim3 grid(m_tiles, tc.C_pad / bn, planes);
-  auto fn = wide ? (drain ? tapconv_tc_kernel<64, true> : tapconv_tc_kernel<64, false>) : (drain ? tapconv_tc_kernel<32, true> : tapconv_tc_kernel<32, false>);
+  const dim3 grid(m_tiles, tc.C_pad / bn, pack ? p.n_phase * ((n_batch + 1) / 2) : planes);
+  auto fn = pack ? tapconv_tc_kernel<64, true, true>
+                 : wide ? (drain ? tapconv_tc_kernel<64, true, false> : tapconv_tc_kernel<64, false, false>)
+                        : (drain ? tapconv_tc_kernel<32, true, false> : tapconv_tc_kernel<32, false, false>);
   launch_ex(fn, grid, dim3(TC_THREADS), tc_smem_bytes(bn, tc.n_a, tc.n_b), st, false, p, tc);
 }
 

@@ -66,39 +66,55 @@ __device__ __noinline__ float4 excite4(float4 v, long long t, int n, int rng_id,
 // is a bias (7.6e-5 of RMS at the vocoder's end with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel,
 // tap) - four additions - has an accumulator of its own, two panels' worth in turn, which the epilogue threads add up in registers,
 // rounded to nearest, while the next panel is multiplied.
-template <int BN, bool DRAIN>
+//
+// PACK (batches; chunks of up to TC_PACK frames at the layer's rate): a tile holds two slots, the second one's rows 64 behind the
+// first one's, so that the panel's rows 64 .. 71 are its left context.  Alone, a chunk of 50 frames at the vocoder's first rate left 61 %
+// of every product to padding.
+constexpr int TC_SEG = 64, TC_PACK = TC_SEG - TC_H;
+struct TcSlot {       // one stream's share of a launch
+  int          T;     // frames at the layer's rate
+  long long    pos;
+  const float* in_direct;
+  float*       out_direct;
+  const float* in_ring;
+  float*       out_ring;
+  float*       save_ring;
+  int          rng_id;
+};
+
+template <int BN, bool DRAIN, bool PACK>
 __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(const __grid_constant__ TapConvF32 p, const __grid_constant__ TapConvTc tc) {
   // per-call values: from the device-side call record of the stream or of the slot (captured graphs), or by value
-  int T_in = p.T_in;
-  long long pos_in = p.pos_in;
-  const float* in_direct = p.in_direct;
-  float* out_direct = p.out_direct;
-  int exc_rng_id = p.exc_rng_id;
-  const float* in_ring = p.in_ring;
-  float* out_ring = p.out_ring;
-  float* save_ring = p.save_ring;
-  int phase = blockIdx.z;
-  const F32Call* callp = p.call;
-  if (p.batch != nullptr) {
-    const int slot = blockIdx.z / p.n_phase;
-    phase = blockIdx.z - slot * p.n_phase;
-    if (slot >= p.batch->n) return;
-    const F32BatchSlot& bs = p.batch->s[slot];
-    callp = &bs.call;
-    in_ring = bs.ptrs->ring[p.layer];
-    out_ring = p.last_layer ? nullptr : bs.ptrs->ring[p.layer + 1];
-    save_ring = p.first_layer ? bs.ptrs->ring[p.layer] : nullptr;
-  }
-  if (callp != nullptr) {
-    const F32Call c = *callp;
-    exc_rng_id = c.rng_id;
-    T_in = c.T * p.rate_in;
-    pos_in = c.frames * p.rate_in;
-    in_direct = p.first_layer ? c.feats : nullptr;
-    out_direct = p.last_layer ? c.out : nullptr;
-  }
-  const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * BN;
-  if (m0 >= T_in) return;   // the grid is sized for the longest chunk
+  const int plane = (p.batch != nullptr ? blockIdx.z / p.n_phase : 0), phase = blockIdx.z - plane * p.n_phase;
+  auto record = [&](int slot) {
+    TcSlot a{p.T_in, p.pos_in, p.in_direct, p.out_direct, p.in_ring, p.out_ring, p.save_ring, p.exc_rng_id};
+    const F32Call* callp = p.call;
+    if (p.batch != nullptr) {
+      if (slot >= p.batch->n) {
+        a.T = 0;
+        return a;
+      }
+      const F32BatchSlot& bs = p.batch->s[slot];
+      callp = &bs.call;
+      a.in_ring = bs.ptrs->ring[p.layer];
+      a.out_ring = p.last_layer ? nullptr : bs.ptrs->ring[p.layer + 1];
+      a.save_ring = p.first_layer ? bs.ptrs->ring[p.layer] : nullptr;
+    }
+    if (callp != nullptr) {
+      const F32Call c = *callp;
+      a.rng_id = c.rng_id;
+      a.T = c.T * p.rate_in;
+      a.pos = c.frames * p.rate_in;
+      a.in_direct = p.first_layer ? c.feats : nullptr;
+      a.out_direct = p.last_layer ? c.out : nullptr;
+    }
+    return a;
+  };
+  const TcSlot s0 = record(PACK ? 2 * plane : plane);
+  TcSlot s1 = s0;
+  if (PACK) s1 = record(2 * plane + 1);
+  const int m0 = PACK ? 0 : blockIdx.x * TC_M, n0 = blockIdx.y * BN;
+  if (PACK ? s0.T <= 0 : m0 >= s0.T) return;   // the grid is sized for the longest chunk
 
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   constexpr int B_TILE = 3 * BN * 128;
@@ -232,11 +248,10 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     // Row addresses in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
     // address of a row cost more instructions than its arithmetic): frame m0 + i, i possibly negative.
     const int C_in = p.C_in, in_mask = p.in_mask;
-    const uint32_t pos32 = (uint32_t)pos_in;
-    auto in_row = [&](int i) -> const float* {
-      const bool direct = in_direct != nullptr && i >= 0;
-      const uint32_t r = direct ? (uint32_t)i : (pos32 + (uint32_t)i) & (uint32_t)in_mask;
-      return (direct ? in_direct : in_ring) + (size_t)(r * (uint32_t)C_in);
+    auto in_row = [&](const TcSlot& a, int i) -> const float* {
+      const bool direct = a.in_direct != nullptr && i >= 0;
+      const uint32_t r = direct ? (uint32_t)i : ((uint32_t)a.pos + (uint32_t)i) & (uint32_t)in_mask;
+      return (direct ? a.in_direct : a.in_ring) + (size_t)(r * (uint32_t)C_in);
     };
     const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
     float4 xa[TC_ITEMS], xb[TC_ITEMS];
@@ -246,11 +261,12 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       const int i0 = m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
 #pragma unroll
       for (int i = 0; i < TC_ITEMS; ++i) {
-        const int row = row0 + 32 * i;
+        const int row = row0 + 32 * i, seg = PACK && i >= TC_SEG / 32 ? TC_SEG : 0;   // (with PACK the tile starts at frame 0)
+        const TcSlot& a = seg ? s1 : s0;
         xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         xb[i] = xa[i];
-        if (row < TC_ROWS && m0 + row - TC_H < T_in && c < C_in) {
-          const float* src = in_row(i0 + row) + c;
+        if (row < TC_ROWS && m0 + row - seg - TC_H < a.T && c < C_in && (!PACK || a.T > 0)) {   // (an odd batch's last tile has no second slot)
+          const float* src = in_row(a, i0 + row - seg) + c;
           xa[i] = *reinterpret_cast<const float4*>(src);
           if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
         }
@@ -324,15 +340,19 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
 
     // Carry update of the first layer: its left context for the next chunk is the tail of the caller's chunk, written into ring
     // rows that no CTA of this launch reads (distinct logical frames map to distinct rows: the ring holds f_chunk + halo frames).
-    if (save_ring != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && phase == 0) {
-      const int first = T_in > p.save_rows ? T_in - p.save_rows : 0;
+    auto save = [&](const TcSlot& a) {
+      const int first = a.T > p.save_rows ? a.T - p.save_rows : 0;
       const int c4 = C_in >> 2;
 #pragma unroll 1
-      for (int i = tid; i < (T_in - first) * c4; i += TC_CONV) {
+      for (int i = tid; i < (a.T - first) * c4; i += TC_CONV) {
         const int r = first + i / c4, c = (i - (i / c4) * c4) * 4;
-        const float4 v = *reinterpret_cast<const float4*>(in_direct + (long long)r * C_in + c);
-        *reinterpret_cast<float4*>(save_ring + (long long)((int)((pos_in + r) & (long long)in_mask)) * C_in + c) = v;
+        const float4 v = *reinterpret_cast<const float4*>(a.in_direct + (long long)r * C_in + c);
+        *reinterpret_cast<float4*>(a.save_ring + (long long)((int)((a.pos + r) & (long long)in_mask)) * C_in + c) = v;
       }
+    };
+    if (p.first_layer && blockIdx.x == 0 && blockIdx.y == 0 && phase == 0) {
+      if (s0.save_ring != nullptr) save(s0);
+      if (PACK && s1.T > 0) save(s1);
     }
 
     // ---------------- epilogue ----------------
@@ -344,15 +364,20 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     float* stage = reinterpret_cast<float*>(sA) + warp * 32 * LD;
     const int g = lane % LPR, rr = lane / LPR, n = n0 + col0 + 4 * g;
     const bool n_ok = n < p.C_out;
-    float* const out = out_direct != nullptr ? out_direct : out_ring;
-    const uint32_t out0 = out_direct != nullptr ? 0u : (uint32_t)(p.n_phase * pos_in), out_mask = out_direct != nullptr ? ~0u : (uint32_t)p.out_mask;
+    // the warp's slot and its first frame there
+    const TcSlot& a = PACK && q >= TC_SEG / 32 ? s1 : s0;
+    const int first = m0 + q * 32 + rr - (PACK && q >= TC_SEG / 32 ? TC_SEG : 0);
+    const bool direct = a.out_direct != nullptr;
+    float* const out = direct ? a.out_direct : a.out_ring;
+    const uint32_t out0 = direct ? 0u : (uint32_t)(p.n_phase * a.pos), out_mask = direct ? ~0u : (uint32_t)p.out_mask;
+    const int T_out = PACK ? min(a.T, TC_SEG) : a.T;
     float4 x[LPR];                                 // the residual rows, fetched under the products
 #pragma unroll
     for (int i = 0; i < LPR; ++i) {
-      const int row = m0 + q * 32 + rr + i * (32 / LPR);
+      const int row = first + i * (32 / LPR);
       x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (p.residual_silu && row < T_in && n_ok)
-        x[i] = *reinterpret_cast<const float4*>(in_row(row) + n);
+      if (p.residual_silu && row < T_out && n_ok)
+        x[i] = *reinterpret_cast<const float4*>(in_row(a, row) + n);
     }
     const float4 bias = n_ok ? *reinterpret_cast<const float4*>(p.bias + n) : make_float4(0.f, 0.f, 0.f, 0.f);
     if (DRAIN) ok &= drain(n_units - 1);
@@ -387,18 +412,17 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
 #pragma unroll
       for (int i = 0; i < LPR; ++i) v[i] = make_float4(silu_f(v[i].x), silu_f(v[i].y), silu_f(v[i].z), silu_f(v[i].w));
     }
-    const int first = m0 + q * 32 + rr;
     if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
 #pragma unroll
       for (int i = 0; i < LPR; ++i)
-        v[i] = excite4(v[i], (long long)p.n_phase * (pos_in + first + i * (32 / LPR)) + phase, n, exc_rng_id, p.exc_std, p.exc_seed_lo, p.exc_seed_hi);
+        v[i] = excite4(v[i], (long long)p.n_phase * (a.pos + first + i * (32 / LPR)) + phase, n, a.rng_id, p.exc_std, p.exc_seed_lo, p.exc_seed_hi);
     }
     if (n_ok && ok) {
 #pragma unroll
       for (int i = 0; i < LPR; ++i) {
         const int row = first + i * (32 / LPR);
         const uint32_t ro = (out0 + (uint32_t)(p.n_phase * row + phase)) & out_mask;
-        if (row < T_in) *reinterpret_cast<float4*>(out + (size_t)(ro * (uint32_t)p.C_out) + n) = v[i];
+        if (row < T_out) *reinterpret_cast<float4*>(out + (size_t)(ro * (uint32_t)p.C_out) + n) = v[i];
       }
     }
     ptx::tc_fence_before();
