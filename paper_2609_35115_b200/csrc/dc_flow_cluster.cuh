@@ -51,7 +51,7 @@ struct CluParams {
   long long       wstream_bytes;
   bf16 *          X[2], *Q, *O, *Ain;  // activations in block layout (CLU_SLOT_KB)
   float*          xstate;
-  float*          ssq;                 // [row][C / 16] partial sums of squares of the rows that feed an RMS norm
+  float*          ssq;                 // [slot][C / 16][SLOT_ROWS] partial sums of squares of the rows that feed an RMS norm
   float           inv_C, eps, inv_n, cfg_w;
   int             rounded;             // DC_OPT_ROUNDED_NORM
   int             P, Rk, kv_hs, dh_shift;
@@ -626,10 +626,11 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       // ---- what does not depend on the accumulator, under the main loop ----
       float4 part[8];                                // partial sums of squares of the row, 16 channels each (first: their loads take longest)
       if (norm && chunk_row) {
-        const float4* src = reinterpret_cast<const float4*>(p.ssq + (long long)r * (p.C >> 4));
+        const float* src = p.ssq + (long long)slot * (p.C >> 4) * SLOT_ROWS + rho;
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          if (j < p.C >> 6) part[j] = __ldcg(src + j);
+          if (j < p.C >> 6)
+            part[j] = make_float4(__ldcg(src + 4 * j * SLOT_ROWS), __ldcg(src + (4 * j + 1) * SLOT_ROWS), __ldcg(src + (4 * j + 2) * SLOT_ROWS), __ldcg(src + (4 * j + 3) * SLOT_ROWS));
       }
       {
         const int gbase = p.C + st.g * (p.cpa + 4) * p.C;     // biases in blob order: input, then per group conv..., Q, K, V, O
@@ -867,7 +868,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               ss = fmaf(hi, hi, ss);
             }
           }
-          p.ssq[(long long)r * (p.C >> 4) + (n >> 4)] = ss;
+          p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
         }
         ptx::tc_fence_before();
         clu_arrive_release(warp);
