@@ -1,0 +1,83 @@
+"""The edges of the kernels' tiles: sizes one below, at and one above what a tile, a panel, a cluster or a launch holds."""
+import numpy as np
+import pytest
+import torch
+
+import dc_workloads as wl
+from oracle import dc_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dc():
+    import paper_2609_35115_b200 as dc
+    dc.load_library()
+    return dc
+
+
+def _util():
+    from tests import gpu_util
+    return gpu_util
+
+
+def _batch_equals_single(dc, cfg, n, chunks=3, max_batch=None, ragged=True):
+    """Every stream of n batched calls gives the bytes of its own calls; returns a stream's input and output."""
+    w = wl.make_workload(cfg)
+    m = dc.Model(cfg, w.weights, max_batch=max_batch or n)
+    streams = [m.open_stream() for _ in range(n)]
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    feats, outs = [], []
+    for c in range(chunks):
+        T = [cfg.f_chunk if not ragged or c == 0 else 1 + (7 * i + 5 * c) % cfg.f_chunk for i in range(n)]
+        feats.append([torch.randn(t, cfg.in_dim, generator=gen, device="cuda") for t in T])
+        outs.append([torch.zeros(t, cfg.out_per_frame, device="cuda") for t in T])
+        dc.decode_batch(m, streams, feats[-1], outs[-1])
+    torch.cuda.synchronize()
+    for i, s in enumerate(streams):
+        s.reset()
+        for c in range(chunks):
+            assert torch.equal(s.decode_chunk(feats[c][i]).flatten(), outs[c][i].flatten()), (n, i, c)
+    assert m.counters()[4] == 0
+    for s in streams:
+        s.close()
+    m.destroy()
+    x = torch.cat([f[-1] for f in feats]).cpu().numpy()
+    bounds = np.cumsum([0] + [f[-1].shape[0] for f in feats]).tolist()
+    return w.weights, x, bounds, torch.cat([o[-1].flatten() for o in outs]).cpu().numpy()
+
+
+# channels: one panel of 64 and more, remainders of 4; frames around the 128-row tile; dilations that share a panel (<= 4) and not
+@pytest.mark.parametrize("hidden,dilations,T", [(4, (1, 4), 127), (64, (4, 5), 128), (68, (2, 1), 129), (60, (9, 1), 1), (132, (1, 64), 257)])
+def test_tap_convolution_tiles(dc, hidden, dilations, T):
+    gu = _util()
+    cfg = wl.CONFIGS["cfg1"].replace(name="tiles", hidden=hidden, dilations=dilations, f_chunk=T, n_chunks=3, seed=31, bias_std=0.3)
+    bounds = [0, T, T + 1, 2 * T + 1]
+    w = wl.make_workload(cfg, boundaries=[bounds])
+    m = dc.Model(cfg, w.weights)
+    got = gu.run_gpu_stream(m, w.streams[0].feats, bounds)
+    assert gu.rel_err(got, orc.run_offline(cfg, w.weights, w.streams[0].feats, bounds)) <= 1e-4
+    m.destroy()
+
+
+# the head's runs of 61 frames and 64 channels, and the batches whose short first layers share tiles (up to 56 frames): even and odd
+@pytest.mark.parametrize("mel,channels,f_chunk,n", [(8, (264, 128, 4), 56, 33), (8, (264, 128, 68), 57, 33), (80, (512, 64, 64), 56, 20), (80, (256, 128, 132), 1, 50),
+                                                    (8, (128, 256, 8), 61, 2), (8, (16, 8, 8), 5, 64)])
+def test_vocoder_batch_tiles(dc, mel, channels, f_chunk, n):
+    gu = _util()
+    cfg = wl.tiny_vocoder(mel_dim=mel, up_channels=channels, f_chunk=f_chunk, n_chunks=3, seed=32)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n)
+    assert gu.rel_err(got, orc.run_offline(cfg, weights, x, bounds).reshape(-1)) <= 1e-4
+
+
+# batches on both sides of one and two slots per cluster and of the kernels of their own; every cluster size; keys with a gap between
+# prompt and history, one block and several
+@pytest.mark.parametrize("hidden,heads,n,kw", [
+    (512, 8, 7, {}), (512, 8, 8, {}), (512, 16, 15, {}), (256, 4, 3, dict(f_prompt=13, kv_cap=150)), (128, 4, 2, dict(cfg_scale=0.7)),
+    (64, 1, 5, dict(kv_cap=300, f_lookahead=6)), (192, 3, 3, dict(f_prompt=130)), (64, 2, 64, dict(f_prompt=9, f_chunk=56))])
+def test_flow_cluster_edges(dc, hidden, heads, n, kw):
+    gu = _util()
+    cfg = wl.tiny_flow(hidden=hidden, n_heads=heads, head_dim=hidden // heads, n_steps=2, seed=33, **kw)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n, max_batch=2 * n)
+    if not cfg.f_lookahead:      # (a call's look-ahead frames are presented again by the next one: other tests compare those)
+        assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
