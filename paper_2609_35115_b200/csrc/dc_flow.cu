@@ -692,33 +692,37 @@ __global__ void flow_prep_kernel(const SlotInfo* slots, int mel, float* xstate, 
   if (!(si.flags & SLOT_FIRST)) return;      // (wavefront: this slot's chunk is past its first Euler step)
   const bool draw = (seed_lo | seed_hi) != 0u;
   const int fw = draw ? mel : 2 * mel;       // width of a row of feats
-  for (int i = threadIdx.x; i < si.T * (mel / 4); i += blockDim.x) {
-    const int f = i / (mel / 4), g = i - f * (mel / 4);
-    const long long r = (long long)blockIdx.x * SLOT_ROWS + HALO + f;
-    float x0[4];
-    if (draw) {
-      const unsigned long long t = (unsigned long long)(si.frame0 + f);
-      uint32_t w[4];
-      philox4x32_10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, (uint32_t)si.rng_id, seed_lo, seed_hi, w);
-      normals4(w, x0);
-    } else {
-      const float4 v = *reinterpret_cast<const float4*>(si.feats + (long long)f * fw + mel + 4 * g);
-      x0[0] = v.x; x0[1] = v.y; x0[2] = v.z; x0[3] = v.w;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = 4 * g + j;
-      const float mu = si.pass == 0 ? si.feats[(long long)f * fw + c] : 0.f;
-      xstate[r * mel + c] = x0[j];
-      auto at = [&](int col) -> long long {
-        if (!panel) return (GUARD + r) * ld_ain + col;
-        const int rho = HALO + f;
-        return ((long long)blockIdx.x * (ld_ain >> 6) + (col >> 6)) * (SLOT_ROWS * KBLK) + rho * KBLK + ((((col >> 3) & 7) ^ (rho & 7)) << 3) + (col & 7);
-      };
-      ain[at(c)] = __float2bfloat16_rn(x0[j]);
-      ain[at(mel + c)] = __float2bfloat16_rn(mu);
-    }
+  // four channels of a frame per thread, the frames over several CTAs: a kernel of one latency (128 threads that went over a slot's
+  // 1,000 pieces took eight of them one after the other, each across the bus when the features are in host memory)
+  const int i = blockIdx.y * blockDim.x + threadIdx.x;
+  if (i >= si.T * (mel / 4)) return;
+  const int f = i / (mel / 4), g = i - f * (mel / 4), c = 4 * g;
+  const long long r = (long long)blockIdx.x * SLOT_ROWS + HALO + f;
+  const float* row = si.feats + (long long)f * fw;
+  float4 mu = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (si.pass == 0) mu = *reinterpret_cast<const float4*>(row + c);
+  float x0[4];
+  if (draw) {
+    const unsigned long long t = (unsigned long long)(si.frame0 + f);
+    uint32_t w[4];
+    philox4x32_10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, (uint32_t)si.rng_id, seed_lo, seed_hi, w);
+    normals4(w, x0);
+  } else {
+    const float4 v = *reinterpret_cast<const float4*>(row + mel + c);
+    x0[0] = v.x; x0[1] = v.y; x0[2] = v.z; x0[3] = v.w;
   }
+  *reinterpret_cast<float4*>(xstate + r * mel + c) = make_float4(x0[0], x0[1], x0[2], x0[3]);
+  auto put = [&](int col, float a, float b, float d, float e) {   // four adjacent columns lie in one 16-byte chunk of either layout
+    long long at = (GUARD + r) * ld_ain + col;
+    if (panel) {
+      const int rho = HALO + f;
+      at = ((long long)blockIdx.x * (ld_ain >> 6) + (col >> 6)) * (SLOT_ROWS * KBLK) + rho * KBLK + ((((col >> 3) & 7) ^ (rho & 7)) << 3) + (col & 7);
+    }
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(d, e);
+    *reinterpret_cast<uint2*>(ain + at) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  };
+  put(c, x0[0], x0[1], x0[2], x0[3]);
+  put(mel + c, mu.x, mu.y, mu.z, mu.w);
 }
 
 // u = bf16(x * rsqrt(mean(x^2) + eps)), one warp per chunk row: the normalised activation as a stored, rounded
@@ -1815,7 +1819,7 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
     launch(lc, set_slots_kernel, dim3(1), dim3(MAX_SLOTS_PER_SET), 0, false, 4, sets[i], m->d_slots);
   // (a profiled call keeps the kernels apart: its figures are per kernel class; the bytes are the same)
   const int spc = lc.prof == nullptr || !lc.prof->on ? cluster_slots(m, n) : 0;
-  launch(lc, flow_prep_kernel, dim3(n), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, spc > 0 ? m->AinP : m->Ain, m->Kin,
+  launch(lc, flow_prep_kernel, dim3(n, ((c.f_chunk + c.f_lookahead) * (mel / 4) + 127) / 128), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, spc > 0 ? m->AinP : m->Ain, m->Kin,
          (uint32_t)c.noise_seed_lo, (uint32_t)c.noise_seed_hi, (int)(spc > 0));
   if (spc > 0) {
     enqueue_cluster(m, n, spc, lc, tick);
