@@ -13,7 +13,7 @@
 // them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue; 8 issues the products; 9 streams the weights, split and packed as swizzled tiles at create.
 // A panel holds 64 channels of the 128 frames and of the up to 8 in front of them: a tap is a row offset of the operand
 // descriptor, so a row is read and split once for all its taps.  (Dilations above 4 fill the panel once per tap.)
-// Per 64 channels and tap: 4 reduction steps of ah x [bh bm bl], am x [bh bm], al x bh.
+// Per 64 channels and tap: 4 reduction steps of ah x bh, ah x [bm bl], am x [bh bm], al x bh.
 
 constexpr int TC_M = 128, TC_H = 8;               // frames per tile; left-context rows in front of them
 constexpr int TC_ROWS = TC_M + TC_H;
@@ -62,10 +62,12 @@ __device__ __noinline__ float4 excite4(float4 v, long long t, int n, int rng_id,
   return make_float4(fmaf(std_dev, e[0], v.x), fmaf(std_dev, e[1], v.y), fmaf(std_dev, e[2], v.z), fmaf(std_dev, e[3], v.w));
 }
 
-// DRAIN (inputs of more than one panel): the tensor cores truncate when they add to an accumulator, which over a long reduction
-// is a bias (7.6e-5 of RMS at the vocoder's end with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel,
-// tap) - four additions - has an accumulator of its own, two panels' worth in turn, which the epilogue threads add up in registers,
-// rounded to nearest, while the next panel is multiplied.
+// The tensor cores truncate when they add to an accumulator, which over a long reduction is a bias (7.6e-5 of RMS at the vocoder's end
+// with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel, tap) - four additions - has an accumulator of
+// its own, which the epilogue threads add up in registers, rounded to nearest.  DRAIN (inputs of more than one panel): two sets of three, a
+// panel's taps each, one set added up while the next panel is multiplied.  One panel: one set; at 64 columns, where two CTAs share the SM's
+// tensor memory, two accumulators that the taps take in turn (TURN).  (A single one for the three taps, twelve additions: ten layers of 64 channels
+// end at 4.3e-6 of their norm, against 2.0e-6 for sums of the FP32 pipe.)
 //
 // PACK (batches; chunks of up to TC_PACK frames at the layer's rate): a tile holds two slots, the second one's rows 64 behind the
 // first one's, so that the panel's rows 64 .. 71 are its left context.  Alone, a chunk of 50 frames at the vocoder's first rate left 61 %
@@ -124,7 +126,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
   uint64_t* empty_a = full_a + TC_MAX_A;
   uint64_t* full_b = empty_a + TC_MAX_A;
   uint64_t* empty_b = full_b + TC_MAX_B;
-  uint64_t* accum = empty_b + TC_MAX_B;           // [2]: products of a panel done (without DRAIN: [0], all products)
+  uint64_t* accum = empty_b + TC_MAX_B;           // [2]: products of a panel (with TURN: of a tap) done
   uint64_t* drained = accum + 2;                  // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 2);
   int* s_fail = reinterpret_cast<int*>(tmem_slot + 1);
@@ -154,8 +156,9 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     *s_fail = 0;
     ptx::fence_barrier_init();
   }
-  // columns: leading term (two sets of three with DRAIN), then the 2^-8 and the 2^-16 terms
-  constexpr uint32_t S_COL = DRAIN ? 6 * BN : BN;
+  // columns: leading term (see above), then the 2^-8 and the 2^-16 terms
+  constexpr bool TURN = !DRAIN && BN > 32;
+  constexpr uint32_t S_COL = DRAIN ? 6 * BN : (TURN ? 2 * BN : 3 * BN);
   constexpr uint32_t TMEM_COLS = S_COL + 2 * BN <= 128 ? 128 : (S_COL + 2 * BN <= 256 ? 256 : 512);
   if (warp == 8) ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   ptx::tc_fence_before();
@@ -189,7 +192,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     // One (panel, tap) after the other; the loop is a chain of one thread's instructions, so addresses advance on 32-bit values and
     // the next barriers are polled ahead of this step's products (with a wait in front of every step it took 1,700 cycles, the
     // products alone 900).
-    const uint32_t id3 = ptx::umma_idesc_bf16(TC_M, 3 * BN, 0, 0), id2 = ptx::umma_idesc_bf16(TC_M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(TC_M, BN, 0, 0);
+    const uint32_t id2 = ptx::umma_idesc_bf16(TC_M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(TC_M, BN, 0, 0);
     constexpr uint32_t DESC_HI = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61)) >> 32);
     const uint32_t a_lo = ((ptx::smem_u32(sA) & 0x3FFFF) >> 4) | (1u << 16), b_lo = ((ptx::smem_u32(sB) & 0x3FFFF) >> 4) | (1u << 16);
     const uint32_t bar_b = ptx::smem_u32(full_b), bar_eb = ptx::smem_u32(empty_b), bar_a = ptx::smem_u32(full_a), bar_ea = ptx::smem_u32(empty_a);
@@ -203,14 +206,15 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
         if (DRAIN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
         if (!__all_sync(0xffffffffu, ready_a)) ok &= tc_wait(&full_a[sa], pa, s_fail, tc.err, 0x202);
       }
+      if (TURN && j >= 2) ok = tc_wait(&drained[j & 1], ((j >> 1) - 1) & 1, s_fail, tc.err, 0x206);
       if (!__all_sync(0xffffffffu, ready_b)) ok &= tc_wait(&full_b[sb], pb, s_fail, tc.err, 0x203);
       if (!ok) break;
       ptx::tc_fence_after();
       const bool last = j + 1 == taps_u, first = u == 0 && j == 0;
       const uint32_t al0 = a_lo + sa * (uint32_t)(TC_PANEL >> 4) + (j == 0 ? off0 : (j == 1 ? off1 : off2)), bl0 = b_lo + sb * (uint32_t)(B_TILE >> 4);
       const uint64_t ah = ((uint64_t)DESC_HI << 32) | al0, am = ah + (TC_PLANE >> 4), al = am + (TC_PLANE >> 4), b = ((uint64_t)DESC_HI << 32) | bl0;
-      const uint32_t eb = bar_eb + 8u * sb, ea = bar_ea + 8u * sa, d_main = tmem_base + (uint32_t)((u & 1) * 3 + j) * BN;
-      uint64_t* done_u = &accum[u & 1];
+      const uint32_t eb = bar_eb + 8u * sb, ea = bar_ea + 8u * sa, d_main = tmem_base + (uint32_t)(TURN ? j & 1 : (u & 1) * 3 + j) * BN;
+      uint64_t* done = &accum[(TURN ? j : u) & 1];
       if (++sb == (uint32_t)tc.n_b) { sb = 0; pb ^= 1u; }
       if (last) {
         if (++sa == (uint32_t)tc.n_a) { sa = 0; pa ^= 1u; }
@@ -224,25 +228,17 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       if (ptx::elect_one()) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if (DRAIN) {
-            ptx::umma_bf16(d_main, ah + 2 * k, b + 2 * k, id1, k != 0);
-            ptx::umma_bf16(tmem_base + S_COL, ah + 2 * k, b + (BN * 128 >> 4) + 2 * k, id2, k == 0 ? (uint32_t)!first : 1u);
-          } else {
-            ptx::umma_bf16(tmem_base, ah + 2 * k, b + 2 * k, id3, k == 0 ? (uint32_t)!first : 1u);
-          }
+          ptx::umma_bf16(d_main, ah + 2 * k, b + 2 * k, id1, k != 0);
+          ptx::umma_bf16(tmem_base + S_COL, ah + 2 * k, b + (BN * 128 >> 4) + 2 * k, id2, k == 0 ? (uint32_t)!first : 1u);
           ptx::umma_bf16(tmem_base + S_COL, am + 2 * k, b + 2 * k, id2, 1);
           ptx::umma_bf16(tmem_base + S_COL + BN, al + 2 * k, b + 2 * k, id1, 1);
         }
         ptx::umma_commit_s(eb);
-        if (last) {
-          ptx::umma_commit_s(ea);
-          if (DRAIN) ptx::umma_commit(done_u);
-        }
+        if (last) ptx::umma_commit_s(ea);
+        if (TURN || last) ptx::umma_commit(done);
       }
       __syncwarp();
     }
-    if (!DRAIN && ptx::elect_one()) ptx::umma_commit(accum);
-    __syncwarp();
   } else {
     // ---------------- input rows -> bf16 planes ----------------
     // Row addresses in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
@@ -276,20 +272,18 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
     constexpr int NC = BN / 32;
     float sum[NC][16];
-    if (DRAIN) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c)
+    for (int c = 0; c < NC; ++c)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum[c][i] = 0.f;
-    }
-    auto drain = [&](int u) {
+      for (int i = 0; i < 16; ++i) sum[c][i] = 0.f;
+    auto drain = [&](int u) {                                // panel u (with TURN: tap u)
       const bool got = tc_wait(&accum[u & 1], (u >> 1) & 1, s_fail, tc.err, 0x205);
       ptx::tc_fence_after();
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const uint32_t col = lanes + (uint32_t)((u & 1) * 3 * BN + col0 + 16 * c);
+        const uint32_t col = lanes + (uint32_t)((u & 1) * (TURN ? 1 : 3) * BN + col0 + 16 * c);
         float z[16], y[16];
-        if (taps_u == 1) {
+        if (TURN || taps_u == 1) {
           ptx::tmem_ld16(col, z);
         } else {
           ptx::tmem_ld16x2(col, col + BN, z, y);
@@ -371,30 +365,35 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     float* const out = direct ? a.out_direct : a.out_ring;
     const uint32_t out0 = direct ? 0u : (uint32_t)(p.n_phase * a.pos), out_mask = direct ? ~0u : (uint32_t)p.out_mask;
     const int T_out = PACK ? min(a.T, TC_SEG) : a.T;
-    float4 x[LPR];                                 // the residual rows, fetched under the products
-#pragma unroll
-    for (int i = 0; i < LPR; ++i) {
+    const int n_sums = TURN ? p.n_taps : n_units;
+    if (TURN) {
+#pragma unroll 1
+      for (int j = 0; j + 1 < n_sums; ++j) ok &= drain(j);
+    }
+    float4 x[LPR];                                 // the residual rows, fetched under the products (with TURN half of them: registers)
+    auto residual = [&](int i) {
       const int row = first + i * (32 / LPR);
       x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (p.residual_silu && row < T_out && n_ok)
-        x[i] = *reinterpret_cast<const float4*>(in_row(a, row) + n);
-    }
+      if (p.residual_silu && row < T_out && n_ok) x[i] = *reinterpret_cast<const float4*>(in_row(a, row) + n);
+    };
+    constexpr int X_EARLY = TURN ? LPR / 2 : LPR;
+#pragma unroll
+    for (int i = 0; i < X_EARLY; ++i) residual(i);
     const float4 bias = n_ok ? *reinterpret_cast<const float4*>(p.bias + n) : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (DRAIN) ok &= drain(n_units - 1);
-    else ok &= tc_wait(accum, 0, s_fail, tc.err, 0x205);
-    ptx::tc_fence_after();
+    ok &= drain(n_sums - 1);
     ok = ok && *reinterpret_cast<volatile int*>(s_fail) == 0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       float z0[16], z1[16], z2[16];
       ptx::tmem_ld16x2(lanes + (uint32_t)(S_COL + col0 + 16 * c), lanes + (uint32_t)(S_COL + BN + col0 + 16 * c), z1, z2);
-      if (!DRAIN) ptx::tmem_ld16(lanes + (uint32_t)(col0 + 16 * c), z0);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) z0[i] = (DRAIN ? sum[c][i] : z0[i]) + (z1[i] + z2[i]);
+      for (int i = 0; i < 16; ++i) z0[i] = sum[c][i] + (z1[i] + z2[i]);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         *reinterpret_cast<float4*>(stage + lane * LD + 16 * c + 4 * i) = make_float4(z0[4 * i], z0[4 * i + 1], z0[4 * i + 2], z0[4 * i + 3]);
     }
+#pragma unroll
+    for (int i = X_EARLY; i < LPR; ++i) residual(i);
     __syncwarp();
     // (one pass per step over all of the thread's pieces: the options cost one branch each, and the pieces' latencies overlap)
     float4 v[LPR];

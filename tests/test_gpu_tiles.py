@@ -81,3 +81,27 @@ def test_flow_cluster_edges(dc, hidden, heads, n, kw):
     weights, x, bounds, got = _batch_equals_single(dc, cfg, n, max_batch=2 * n)
     if not cfg.f_lookahead:      # (a call's look-ahead frames are presented again by the next one: other tests compare those)
         assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
+
+
+def test_single_panel_sums_keep_fp32_precision(dc):
+    """Ten layers of 64 channels (one panel each): the taps' sums are added rounded to nearest.  Sums of the FP32 pipe end at 1.8e-6 to 2.1e-6 of
+    the output's norm over six seeds, one truncating accumulator for all taps at 3.5e-6 to 5.0e-6; the bound lies between.  Four streams
+    fill the 64-column tiles, one the 32-column ones: the same bytes."""
+    gu = _util()
+    cfg = wl.CONFIGS["cfg4"].replace(name="single_panel", mel_dim=64, up_channels=(64, 64, 64, 64), n_streams=4, n_chunks=2)
+    bounds = [0, cfg.f_chunk, 2 * cfg.f_chunk]
+    w = wl.make_workload(cfg, boundaries=[bounds] * 4)
+    m = dc.Model(cfg, w.weights, max_batch=4)
+    streams = [m.open_stream() for _ in range(4)]
+    feats = torch.stack([torch.from_numpy(s.feats) for s in w.streams]).cuda()
+    outs = [torch.zeros(4, cfg.f_chunk, cfg.out_per_frame, device="cuda") for _ in range(2)]
+    for c in range(2):
+        dc.decode_batch(m, streams, feats[:, bounds[c]:bounds[c + 1]].contiguous(), outs[c])
+    got = torch.cat(outs, dim=1).reshape(4, -1).cpu().numpy()
+    ref = np.stack([orc.run_offline(cfg, w.weights, s.feats, bounds).reshape(-1) for s in w.streams]).astype(np.float64)
+    err = np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.mean() <= 3e-6, err
+    assert np.array_equal(gu.run_gpu_stream(m, w.streams[0].feats, bounds).reshape(-1), got[0])
+    for s in streams:
+        s.close()
+    m.destroy()
