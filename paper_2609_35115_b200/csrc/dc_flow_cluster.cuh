@@ -276,12 +276,13 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         } else if (warp == 0) {
           ptx::fence_proxy_async_global();         // what the cluster wrote before the barrier, visible to the copies below
           const bf16* src = (st.kind == CLU_IN ? p.Ain : (st.kind == CLU_OPROJ ? p.O : p.X[xi])) + (long long)slot0 * nkb * CLU_SLOT_KB;
+          const bool two = p.spc == 2 && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
           if (ptx::elect_one()) {
 #pragma unroll 1
             for (int kb = 0; kb < nkb; ++kb) {
-              ptx::mbar_expect_tx(&full_a[kb], (uint32_t)kb_bytes);
+              ptx::mbar_expect_tx(&full_a[kb], two ? 16384u : 8192u);
               ptx::bulk_load(panel + kb * kb_bytes, src + kb * CLU_SLOT_KB, 8192u, &full_a[kb]);
-              if (p.spc == 2) ptx::bulk_load(panel + kb * kb_bytes + 8192, src + (nkb + kb) * CLU_SLOT_KB, 8192u, &full_a[kb]);
+              if (two) ptx::bulk_load(panel + kb * kb_bytes + 8192, src + (nkb + kb) * CLU_SLOT_KB, 8192u, &full_a[kb]);
             }
           }
           __syncwarp();

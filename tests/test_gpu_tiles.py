@@ -105,3 +105,12 @@ def test_single_panel_sums_keep_fp32_precision(dc):
     for s in streams:
         s.close()
     m.destroy()
+
+
+# full batches of an odd number of slots, two per cluster: the last cluster's second slot does not exist, in no buffer
+@pytest.mark.parametrize("hidden,n", [(512, 9), (512, 13), (256, 17), (128, 35)])
+def test_flow_cluster_odd_full_batch(dc, hidden, n):
+    gu = _util()
+    cfg = wl.tiny_flow(hidden=hidden, n_heads=hidden // 64, head_dim=64, mel_dim=80, n_steps=2, seed=34)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n)
+    assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
