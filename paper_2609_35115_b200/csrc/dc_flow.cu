@@ -1285,6 +1285,7 @@ bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, u
 
 constexpr size_t GEMM_SMEM_EXTRA = 1024 + 2 * MAX_STAGES * 8 + 8 + 8 + 2 * MAX_BN * 4 + 64;   // alignment slack + barriers + constants
 constexpr size_t GEMM_SMEM_MAX = 200 * 1024;
+constexpr int CONV_XCHG = 2 * 4 * TILE_M * 16;      // exchange area of 16 columns in a conv epilogue: two taps, [4 float4 columns][128 rows] each
 constexpr int SPECIALISE_FROM_TILES = 8;   // row tiles of a batch from which the GEMMs run as one kernel per role
 constexpr size_t GEMM_SMEM_MAX_PAIR = 227 * 1024;   // the opt-in limit of the device: eight 28 KB stages of a CTA pair
 
@@ -1858,6 +1859,9 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
     // Four stages wherever there are four blocks: with two, 32-column conv tiles waited for their operands (16 streams 1,714 us per
     // step against 1,461).
     p.n_stages = p.n_kblocks >= 4 ? 4 : (p.n_issuers == 2 ? 2 : 1);
+    // A conv epilogue exchanges shifted rows through the ring, 16 KB per 16 columns: one reduction block (hidden 64) has two stages for
+    // that from 32 columns on.
+    while (p.mode == MODE_CONV && p.n_stages * stage_bytes < (p.BN >> 4) * CONV_XCHG) ++p.n_stages;
     if (pairs_ok && tBh != nullptr) {
       const int pair_stage = A_BYTES + p.taps * (p.BN * 64);
       int ns = p.n_kblocks < MAX_STAGES ? p.n_kblocks : MAX_STAGES;

@@ -21,10 +21,10 @@ def _util():
     return gpu_util
 
 
-def _batch_equals_single(dc, cfg, n, chunks=3, max_batch=None, ragged=True):
+def _batch_equals_single(dc, cfg, n, chunks=3, max_batch=None, ragged=True, options=0):
     """Every stream of n batched calls gives the bytes of its own calls; returns a stream's input and output."""
     w = wl.make_workload(cfg)
-    m = dc.Model(cfg, w.weights, max_batch=max_batch or n)
+    m = dc.Model(cfg, w.weights, max_batch=max_batch or n, options=options)
     streams = [m.open_stream() for _ in range(n)]
     gen = torch.Generator(device="cuda").manual_seed(n)
     feats, outs = [], []
@@ -113,4 +113,13 @@ def test_flow_cluster_odd_full_batch(dc, hidden, n):
     gu = _util()
     cfg = wl.tiny_flow(hidden=hidden, n_heads=hidden // 64, head_dim=64, mel_dim=80, n_steps=2, seed=34)
     weights, x, bounds, got = _batch_equals_single(dc, cfg, n)
+    assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
+
+
+# one reduction block per conv product (hidden 64): 32- and 64-column tiles, whose epilogue exchanges more rows than one pipeline stage holds
+@pytest.mark.parametrize("n", [76, 150])
+def test_conv_exchange_of_one_reduction_block(dc, n):
+    gu = _util()
+    cfg = wl.tiny_flow(n_steps=2, seed=35)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n, options=dc.OPT_CTA_PAIRS)    # (the option keeps the kernels apart)
     assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
