@@ -758,6 +758,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             }
           }
         }
+        if (p.cfg_w > 0.f) ptx::fence_proxy_async_smem();   // (the exchange above: the next stage's bulk copies overwrite it)
         ptx::tc_fence_before();
         clu_arrive_release(warp);
       } else if (kind == CLU_QKV) {
@@ -871,6 +872,9 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           }
           p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
         }
+        // The next stage's bulk copies overwrite the exchange of the taps: the writers' fence.  (One stream 909 -> 919 us; right behind the writes
+        // 925, behind the barrier of clu_arrive_release 918.)
+        if (kind == CLU_CONV) ptx::fence_proxy_async_smem();
         ptx::tc_fence_before();
         clu_arrive_release(warp);
         // shift the carry by the committed frames: nobody in this launch reads it again

@@ -123,3 +123,24 @@ def test_conv_exchange_of_one_reduction_block(dc, n):
     cfg = wl.tiny_flow(n_steps=2, seed=35)
     weights, x, bounds, got = _batch_equals_single(dc, cfg, n, options=dc.OPT_CTA_PAIRS)    # (the option keeps the kernels apart)
     assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
+
+
+# the row exchanges of the cluster step's epilogues lie where the next stage's activations land: one and two slots per cluster, guided passes
+@pytest.mark.parametrize("n,kw", [(1, {}), (9, {}), (2, dict(cfg_scale=0.7))])
+def test_flow_cluster_exchange_repeats(dc, n, kw):
+    cfg = wl.tiny_flow(hidden=512, n_heads=8, head_dim=64, mel_dim=80, n_steps=8, f_chunk=50, seed=36, **kw)
+    w = wl.make_workload(cfg)
+    m = dc.Model(cfg, w.weights, max_batch=2 * n)
+    streams = [m.open_stream() for _ in range(n)]
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.randn(n, cfg.f_chunk, cfg.in_dim, generator=gen, device="cuda")
+    outs = torch.zeros(40, n, cfg.f_chunk, cfg.mel_dim, device="cuda")
+    for out in outs:
+        for s in streams:
+            s.reset()
+        dc.decode_batch(m, streams, x, out)
+    assert m.counters()[4] == 0
+    assert torch.equal(outs, outs[:1].expand_as(outs))
+    for s in streams:
+        s.close()
+    m.destroy()
