@@ -1617,9 +1617,16 @@ void flow_state_set_frames(FlowState* s, long long frames) { s->frames = frames;
 int flow_state_rng_id(const FlowState* s) { return s->rng_id; }
 void flow_state_set_rng_id(FlowState* s, int id) { s->rng_id = id; }
 
-dc_status flow_state_reset(FlowModel*, FlowState* s, cudaStream_t st) {
-  // base state: zero left context, empty K/V carry (stale ring rows are never attended)
+dc_status flow_state_reset(FlowModel* m, FlowState* s, cudaStream_t st) {
+  // base state: zero left context, empty K/V carry.  Stale rows are not attended, but the attention kernels take the prompt rows up to a
+  // multiple of 8 (AttKeys): until the new history has reached them, the first ring rows go through P V with weight 0, and
+  // 0 x NaN would carry an earlier session's NaN over.  So those rows of every plane are cleared.
   if (cudaMemsetAsync(s->halo, 0, s->halo_bytes, st) != cudaSuccess) return DC_ERR_CUDA;
+  const int pad = -m->P & 7;
+  if (s->kv != nullptr && pad != 0) {
+    const size_t row = (size_t)m->cfg.head_dim * sizeof(bf16), plane = (size_t)(m->P + m->Rk) * row;   // one head's K or V
+    if (cudaMemset2DAsync(reinterpret_cast<uint8_t*>(s->kv) + m->P * row, plane, 0, pad * row, s->kv_bytes / plane, st) != cudaSuccess) return DC_ERR_CUDA;
+  }
   s->frames = 0;
   return DC_OK;
 }

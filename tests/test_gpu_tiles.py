@@ -144,3 +144,31 @@ def test_flow_cluster_exchange_repeats(dc, n, kw):
     for s in streams:
         s.close()
     m.destroy()
+
+
+# a stream that has held NaN is reset: its new session's history does not fill the gap behind the prompt rows yet.  One kernel per chunk and
+# kernels of their own, both head widths, wavefront
+@pytest.mark.parametrize("kw", [dict(hidden=128, head_dim=64), dict(hidden=128, head_dim=32), dict(hidden=192, head_dim=64), dict(hidden=192, head_dim=32)])
+@pytest.mark.parametrize("f_prompt", [13, 17])
+def test_reset_leaves_nothing_of_the_session_before(dc, kw, f_prompt):
+    cfg = wl.tiny_flow(f_prompt=f_prompt, n_heads=kw["hidden"] // kw["head_dim"], n_steps=2, seed=37, **kw)
+    w = wl.make_workload(cfg)
+    m = dc.Model(cfg, w.weights, max_batch=cfg.n_steps)
+    gen = torch.Generator(device="cuda").manual_seed(f_prompt)
+    x = torch.randn(f_prompt + 21, cfg.in_dim, generator=gen, device="cuda")
+    cuts = list(range(0, f_prompt, cfg.f_chunk)) + [f_prompt, f_prompt + 1, f_prompt + 2, f_prompt + 11, f_prompt + 21]
+    fresh, used = m.open_stream(), m.open_stream()
+    for _ in range(8):
+        assert used.decode_chunk(torch.full((cfg.f_chunk, cfg.in_dim), float("nan"), device="cuda")).isnan().all()
+    used.reset()
+    for a, b in zip(cuts, cuts[1:]):
+        got = used.decode_chunk(x[a:b].contiguous())
+        assert torch.equal(got, fresh.decode_chunk(x[a:b].contiguous())) and got.isfinite().all(), (a, b)
+    for s in (fresh, used):
+        s.reset()
+    used.decode_wavefront(torch.full((8 * cfg.f_chunk, cfg.in_dim), float("nan"), device="cuda"))
+    used.reset()
+    assert torch.equal(used.decode_wavefront(x), fresh.decode_wavefront(x))
+    for s in (fresh, used):
+        s.close()
+    m.destroy()
