@@ -241,13 +241,13 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
   } else {
     // ---------------- input rows -> bf16 planes ----------------
-    // Row addresses in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
-    // address of a row cost more instructions than its arithmetic): frame m0 + i, i possibly negative.
+    // Row numbers in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
+    // address of a row cost more instructions than its arithmetic), the element offset widened: frame m0 + i, i possibly negative.
     const int C_in = p.C_in, in_mask = p.in_mask;
     auto in_row = [&](const TcSlot& a, int i) -> const float* {
       const bool direct = a.in_direct != nullptr && i >= 0;
       const uint32_t r = direct ? (uint32_t)i : ((uint32_t)a.pos + (uint32_t)i) & (uint32_t)in_mask;
-      return (direct ? a.in_direct : a.in_ring) + (size_t)(r * (uint32_t)C_in);
+      return (direct ? a.in_direct : a.in_ring) + (size_t)r * (uint32_t)C_in;
     };
     const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
     float4 xa[TC_ITEMS], xb[TC_ITEMS];
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       for (int i = 0; i < LPR; ++i) {
         const int row = first + i * (32 / LPR);
         const uint32_t ro = (out0 + (uint32_t)(p.n_phase * row + phase)) & out_mask;
-        if (row < T_out) *reinterpret_cast<float4*>(out + (size_t)(ro * (uint32_t)p.C_out) + n) = v[i];
+        if (row < T_out) *reinterpret_cast<float4*>(out + (size_t)ro * (uint32_t)p.C_out + n) = v[i];
       }
     }
     ptx::tc_fence_before();

@@ -172,3 +172,19 @@ def test_reset_leaves_nothing_of_the_session_before(dc, kw, f_prompt):
     for s in (fresh, used):
         s.close()
     m.destroy()
+
+
+def test_ring_of_more_than_2_to_32_elements(dc):
+    """A vocoder ring of 2^20 rows of 4,100 channels (34 GB): element offsets beyond 32 bits.  The same frames in short chunks, whose rings are small, give
+    the same bytes."""
+    cfg = wl.tiny_vocoder(mel_dim=4, up_strides=(16, 16, 1), up_channels=(4, 4, 4100, 4), res_dilations=(), f_chunk=4096, seed=38)
+    w = wl.make_workload(cfg.replace(n_chunks=1))
+    x = torch.from_numpy(w.streams[0].feats).cuda()
+    big, small = dc.Model(cfg, w.weights), dc.Model(cfg.replace(f_chunk=64), w.weights)
+    a, b = big.open_stream(), small.open_stream()
+    got = a.decode_chunk(x).flatten()
+    want = torch.cat([b.decode_chunk(x[t:t + 64].contiguous()).flatten() for t in range(0, 4096, 64)])
+    assert torch.equal(got, want) and got.isfinite().all()
+    for s, m in ((a, big), (b, small)):
+        s.close()
+        m.destroy()
