@@ -427,8 +427,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     ptx::tc_fence_before();
   }
   __syncthreads();
-  // (a wait that gave up may have left copies in flight: they land before the shared memory is given back)
-  if (*reinterpret_cast<volatile int*>(s_fail) != 0) __nanosleep(1000000);
+  if (*reinterpret_cast<volatile int*>(s_fail) != 0) ptx::pause_for_copies();
   if (warp == 8) ptx::tmem_dealloc(tmem_base, TMEM_COLS);
 }
 

@@ -94,8 +94,8 @@ __device__ __forceinline__ void clu_arrive_release(int warp) {
   ptx::cluster_arrive_relaxed();
 }
 
-// Bounded wait of a whole warp that gives up at once after any wait of this CTA has given up (the step then runs through without
-// waiting).  The vote keeps the warp together: lanes that leave a polling loop one by one go on as separate groups, and everything
+// Bounded wait of a whole warp that gives up at once after any wait of this CTA has given up: the step then runs through without
+// waiting, the copying warps request nothing more, and the CTA pauses before it exits.  The vote keeps the warp together: lanes that leave a polling loop one by one go on as separate groups, and everything
 // up to the next warp-wide instruction is then executed several times (an issue loop took 600 cycles per block instead of 260).
 __device__ __forceinline__ bool clu_wait(uint64_t* bar, uint32_t parity, int* s_fail, int* err, int code) {
   const uint32_t a = ptx::smem_u32(bar);
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           continue;
         }
         const uint32_t bytes = w.kind == CLU_CONV || w.kind == CLU_QKV ? 3u * BN * 128u : (w.kind == CLU_OUT ? (uint32_t)nch_out * 2048u : BN * 128u);
-        if (t >= RS) clu_wait(&empty_w[slot], ph, s_fail, p.err, 0x101);
+        if (t >= RS && !clu_wait(&empty_w[slot], ph, s_fail, p.err, 0x101)) break;
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full_w[slot], bytes);
           ptx::bulk_load(wring + slot * CLU_SLOT, src0 + off, bytes, &full_w[slot]);
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         // one slot per cluster: the K/V ring is its own, the next attention's carried blocks are requested in the first conv block
         // (s_job is there from the second stage on); two: the panel is free once the projection's products are done
         fetch = p.n_attn > 0 && (p.spc == 1 ? st.kind == CLU_CONV : st.kind == CLU_QKV);
-        if (fetch && warp == 0 && p.spc == 2) clu_wait(accum, n_g & 1u, s_fail, p.err, 0x106);
+        if (fetch && warp == 0 && p.spc == 2 && !clu_wait(accum, n_g & 1u, s_fail, p.err, 0x106)) fetch = false;
         ++n_g;
         if (st.kind == CLU_IN) { ++n_gi; xi = 0; } else if (!skip) ++n_gc;
         if (!skip && (st.kind == CLU_QKV || st.kind == CLU_OUT)) ++n_norm;
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           if (att) {
             // S of the previous job's last block has been computed when its K slot is released (the slot's earlier phases
             // have all been waited for when it was filled)
-            if (!first) clu_wait(&empty_kv[last_k % CLU_KVS], (last_k / CLU_KVS) & 1u, s_fail, p.err, 0x107);
+            if (!first && !clu_wait(&empty_kv[last_k % CLU_KVS], (last_k / CLU_KVS) & 1u, s_fail, p.err, 0x107)) break;
             // the slot's 56 chunk rows of the head's 64-column block (rows T.. are never stored; with head_dim 32 the block
             // holds two heads), twice: see flow_attn_kernel
             if (ptx::elect_one()) {
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             clu_item(item, jb.k.nkb, &is_v, &b);
             if (!att && (item == (int)CLU_KVS || b >= jb.k.n_early)) break;
             const uint32_t gi = it0 + (uint32_t)item, ks = gi % CLU_KVS, k = gi / CLU_KVS;
-            if (k > 0) clu_wait(&empty_kv[ks], (k - 1) & 1u, s_fail, p.err, 0x102);
+            if (k > 0 && !clu_wait(&empty_kv[ks], (k - 1) & 1u, s_fail, p.err, 0x102)) break;
             uint8_t* dst = kvring + ks * CLU_KV_BYTES;
             const int n = min(ATT_KB, jb.k.L - b * ATT_KB);   // key rows of this block
             if (is_v && n < ATT_KB) {              // rows behind the last key must be finite up to the next UMMA step
@@ -492,7 +492,17 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         }
       }
       ptx::cluster_arrive_relaxed();
+      // (read here, where nobody waits for it: a wait takes so long to give up that what it left behind one stage earlier has landed)
+      const bool failed = warp == 0 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0);
       ptx::cluster_wait();
+      if (failed) {
+#pragma unroll 1
+        for (st.next(p); st.s < p.n_steps; st.next(p)) {
+          ptx::cluster_arrive_relaxed();
+          ptx::cluster_wait();
+        }
+        break;
+      }
     }
   } else {
     // ---------------- epilogue: a thread owns one row and 16 columns; attention: warps 4..7 even, 8..11 odd key blocks ----------------
@@ -888,6 +898,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   }
   ptx::tc_fence_before();
   __syncthreads();
+  if (*reinterpret_cast<volatile int*>(s_fail) != 0) ptx::pause_for_copies();
   if (warp == 1) ptx::tmem_dealloc(tmem_base, 512);
 }
 

@@ -77,6 +77,14 @@ __device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// A CTA in which a wait has given up leaves copies and products in flight: it keeps its shared memory and its tensor memory
+// for 2 M cycles more (a millisecond; a copy takes microseconds), in which they land.
+__device__ __forceinline__ void pause_for_copies() {
+  const long long t0 = clock64();
+#pragma unroll 1
+  for (int i = 0; i < (1 << 16) && clock64() - t0 < 2000000; ++i) __nanosleep(1000);
+}
+
 // ---- programmatic dependent launch --------------------------------------------------------------
 // pdl_wait: blocks until every grid this one depends on has completed and its writes are visible
 // (a no-op for a launch without the programmatic attribute).  pdl_launch: lets the next grid of
