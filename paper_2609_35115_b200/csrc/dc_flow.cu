@@ -1077,7 +1077,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
         ptx::fence_proxy_async_smem();
         __syncwarp();
       }
-      if (ptx::elect_one()) ak.fetch(plane, b, n, p.P, p.Rk, DHS, dstb, &full[st]);
+      if (ptx::elect_one() && ok) ak.fetch(plane, b, n, p.P, p.Rk, DHS, dstb, &full[st]);   // (nothing more behind a wait that gave up)
       __syncwarp();
     };
     if (warp != 6)

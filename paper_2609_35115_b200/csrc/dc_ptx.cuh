@@ -55,7 +55,8 @@ __device__ __forceinline__ bool mbar_try_wait_s(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 // Bounded wait.  Returns false after kMaxPolls failed polls (each poll blocks in hardware for a
-// short, implementation-defined time), which is orders of magnitude beyond any legitimate wait here.
+// short, implementation-defined time), which is orders of magnitude beyond any legitimate wait here: whatever was in flight when
+// the wait began has landed when it gives up.
 constexpr uint32_t kMaxPolls = 4u << 20;
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, uint32_t max_polls) {
 #pragma unroll 1   // (waits are everywhere: unrolled they were a third of a kernel's code, and code comes through the instruction cache)
