@@ -480,6 +480,10 @@ def main():
         roof = {"kernel": "flow_gemm_kernel (conv blocks)" if dom == "gemm_conv" else "flow_gemm_kernel<PAIR> (conv blocks and QKV projections on CTA pairs)", "bound": "tensor", "achieved": fl / avg_s / 1e12,
                 "peak": tensor_peak, "unit": "TFLOP/s", "peak_kind": tensor_kind,
                 "frac_of_sustained_peak": fl / avg_s / 1e12 / pk["bf16_tflops_sustained"]}
+    elif dom == "flow_cluster":                      # the whole chunk step in one launch
+        fl, _ = flow_step_work(cfg, S)
+        roof = {"kernel": "flow_cluster_kernel (every Euler step and layer of a chunk)", "bound": "latency of the dependent stages", "achieved": fl * nprof / (1e-3 * ms[dom]) / 1e12,
+                "peak": tensor_peak, "unit": "TFLOP/s", "peak_kind": tensor_kind}
     elif dom == "attention":
         by = attention_bytes_per_launch(cfg, S)
         roof = {"kernel": "flow_attn_kernel", "bound": "hbm", "achieved": by / avg_s / 1e9, "peak": pk["hbm_gbs"],

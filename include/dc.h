@@ -315,10 +315,11 @@ dc_status dc_decode_batch_host(dc_model* model, int n, dc_stream* const* streams
  * bracketed by CUDA events on the launching stream (this slows the step down: never report
  * throughput from a profiled pass).  dc_profile_end synchronises the device and returns, per
  * class, the summed milliseconds and the launch count.  Classes: 0 conv GEMM, 1 other GEMMs
- * (input/QKV/output projections), 2 attention, 3 unused (the RMS norm is folded into the GEMMs),
- * 4 slot table + input prep,
- * 5 fp32 tap convolution, 6 fp32 head + inverse STFT, 7 conv / QKV GEMMs launched as CTA pairs
- * (DC_OPT_CTA_PAIRS; they then do not count in classes 0 and 1).
+ * (input/QKV/output projections), 2 attention, 3 RMS norm (DC_OPT_ROUNDED_NORM; otherwise it is folded into
+ * the GEMMs), 4 slot table + input prep,
+ * 5 fp32 tap convolution, 6 fp32 head + inverse STFT, 7 kernels of CTA clusters: the flow decoder's whole chunk step
+ * (one launch, for batches whose slots fit the resident clusters), or with DC_OPT_CTA_PAIRS the conv / QKV GEMMs
+ * launched as CTA pairs (they then do not count in classes 0 and 1).
  * max_launches bounds the event pool allocated by dc_profile_begin. */
 dc_status dc_profile_begin(dc_model* model, int max_launches);
 dc_status dc_profile_end(dc_model* model, double ms[8], uint64_t launches[8]);

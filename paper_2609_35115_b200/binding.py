@@ -191,8 +191,10 @@ class Model:
         ms = (C.c_double * 8)()
         n = (C.c_uint64 * 8)()
         _check(self.lib.dc_profile_end(self.handle, ms, n), "dc_profile_end")
-        names = ["gemm_conv", "gemm_proj", "attention", "rmsnorm", "prep", "tapconv_f32", "head_istft_f32", "gemm_pair"]
-        return ({k: ms[i] for i, k in enumerate(names)}, {k: n[i] for i, k in enumerate(names)})
+        names = ["gemm_conv", "gemm_proj", "attention", "rmsnorm", "prep", "tapconv_f32", "head_istft_f32"]
+        pairs = bool(self.c_cfg.options & OPT_CTA_PAIRS)      # class 7 is one or the other
+        names += ["gemm_pair", "flow_cluster"] if pairs else ["flow_cluster", "gemm_pair"]
+        return ({k: ms[i] if i < 8 else 0.0 for i, k in enumerate(names)}, {k: n[i] if i < 8 else 0 for i, k in enumerate(names)})
 
     def destroy(self):
         if self.handle:

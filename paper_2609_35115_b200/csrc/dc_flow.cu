@@ -1811,6 +1811,7 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, p.CL, (n + spc - 1) / spc, lc.st, lc.pdl);
+  ProfScope ps(lc.prof, 7, lc.st);
   cudaError_t e = cudaLaunchKernelEx(&cfg, flow_cluster_kernel, p);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
   ++lc.launches;
@@ -1825,8 +1826,7 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
   const int C = m->C, mel = m->mel;
   for (int i = 0; i < n_sets; ++i)   // not a programmatic launch: it overwrites the table the previous chunk still reads
     launch(lc, set_slots_kernel, dim3(1), dim3(MAX_SLOTS_PER_SET), 0, false, 4, sets[i], m->d_slots);
-  // (a profiled call keeps the kernels apart: its figures are per kernel class; the bytes are the same)
-  const int spc = lc.prof == nullptr || !lc.prof->on ? cluster_slots(m, n) : 0;
+  const int spc = cluster_slots(m, n);
   launch(lc, flow_prep_kernel, dim3(n, ((c.f_chunk + c.f_lookahead) * (mel / 4) + 127) / 128), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, spc > 0 ? m->AinP : m->Ain, m->Kin,
          (uint32_t)c.noise_seed_lo, (uint32_t)c.noise_seed_hi, (int)(spc > 0));
   if (spc > 0) {

@@ -188,3 +188,23 @@ def test_ring_of_more_than_2_to_32_elements(dc):
     for s, m in ((a, big), (b, small)):
         s.close()
         m.destroy()
+
+
+# one kernel of clusters (1, 14 streams), kernels of their own (15): a profiled call launches what the same call launches otherwise
+@pytest.mark.parametrize("n,cluster", [(1, 1), (14, 1), (15, 0)])
+def test_profile_brackets_the_launches_of_a_call(dc, n, cluster):
+    cfg = wl.CONFIGS["cfg3"].replace(n_steps=2)
+    m = dc.Model(cfg, wl.make_weights(cfg, np.random.default_rng(39)), max_batch=n, options=dc.OPT_NO_GRAPH)
+    streams = [m.open_stream() for _ in range(n)]
+    x, out = torch.randn(n, cfg.f_chunk, cfg.in_dim, device="cuda"), torch.zeros(n, cfg.f_chunk, cfg.mel_dim, device="cuda")
+    before = m.counters()[5]
+    dc.decode_batch(m, streams, x, out)
+    launched = m.counters()[5] - before
+    m.profile_begin()
+    dc.decode_batch(m, streams, x, out)
+    ms, count = m.profile_end()
+    assert sum(count.values()) == launched and count["flow_cluster"] == cluster
+    assert all(ms[k] > 0 for k in count if count[k])
+    for s in streams:
+        s.close()
+    m.destroy()
