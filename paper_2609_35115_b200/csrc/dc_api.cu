@@ -136,7 +136,7 @@ using dc::F32Layer;
 
 struct dc_model {
   dc_config cfg;
-  int       device = 0;
+  int       device = 0, n_sm = 0;
   float*    d_w = nullptr;   // fp32 pipelines: the blob on the device
   uint8_t*  d_wp = nullptr;  // ... and the conv weights as packed bf16 planes
   int*      f32_err = nullptr;   // ... and the device word that a bounded wait sets when it gives up
@@ -404,6 +404,7 @@ static cudaError_t pack_f32_weights(dc_model* m) {
     const dc::TapConvF32 p = tapconv_layer(m, l);
     dc::pack_tapconv(p, m->d_wp + off, &L.tc);
     L.tc.err = m->f32_err;
+    L.tc.n_sm = m->n_sm;
     off += dc::tapconv_pack_bytes(p);
   }
   return cudaDeviceSynchronize();
@@ -437,6 +438,7 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
   if (!m) return DC_ERR_OOM;
   m->cfg = *cfg;
   m->device = dev;
+  m->n_sm = prop.multiProcessorCount;
   for (auto& c : m->counters) c = 0;
   dc_status st = DC_OK;
   if (cfg->pipeline == DC_PIPE_TOKEN2WAV) {
@@ -838,7 +840,7 @@ static void enqueue_f32(dc_stream* s, bool use_call, const float* feats, int T, 
     if (L.kind == 2) {
       dc::HeadIstftF32 h{};
       h.in_ring = ring; h.in_mask = L.ring_cap - 1; h.C = L.C_in;
-      h.W = m->d_w + L.w_off; h.bias = m->d_w + L.b_off; h.clamp = m->cfg.logmag_clamp;
+      h.W = m->d_w + L.w_off; h.bias = m->d_w + L.b_off; h.clamp = m->cfg.logmag_clamp; h.n_sm = m->n_sm;
       if (use_call) {
         h.call = s->d_call; h.rate_in = L.rate_in; h.tails = s->tails;
       } else {
@@ -925,7 +927,7 @@ static void enqueue_f32_batch(dc_model* m, int nb, cudaStream_t cs, int* launche
       dc::HeadIstftF32 h{};
       h.batch = m->d_batch; h.layer = l; h.rate_in = L.rate_in;
       h.in_mask = L.ring_cap - 1; h.C = L.C_in;
-      h.W = m->d_w + L.w_off; h.bias = m->d_w + L.b_off; h.clamp = m->cfg.logmag_clamp;
+      h.W = m->d_w + L.w_off; h.bias = m->d_w + L.b_off; h.clamp = m->cfg.logmag_clamp; h.n_sm = m->n_sm;
       dc::ProfScope ps(&m->prof, 6, cs);
       dc::launch_head_istft_f32(h, cs, Tgrid, false, nb);
     } else {

@@ -507,9 +507,9 @@ void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc_in, cudaStream_t
   // 64 columns per CTA once that fills the GPU (a reduction step costs 209 cycles of the tensor pipe at 64 columns, 134 at 32), else 32
   // over twice the SMs.  A column's sum is the same either way.  A single panel leaves room for two CTAs per SM, which overlap one's
   // conversion and epilogue with the other's products; several panels overlap inside the CTA.
-  const bool wide0 = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= 148;
+  const bool wide0 = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= tc.n_sm;
   // two slots per tile where that saves a wave: several panels (one CTA per SM), chunks of at most half a tile
-  const bool pack = drain && n_batch > 1 && T_grid <= TC_PACK && tc.C_pad % 64 == 0 && (long long)(tc.C_pad / (wide0 ? 64 : 32)) * planes > 148;
+  const bool pack = drain && n_batch > 1 && T_grid <= TC_PACK && tc.C_pad % 64 == 0 && (long long)(tc.C_pad / (wide0 ? 64 : 32)) * planes > tc.n_sm;
   const bool wide = wide0 || pack;
   tc.n_a = drain ? 2 : 1;
   tc.n_b = wide ? (drain ? 3 : 2) : TC_MAX_B;
@@ -599,7 +599,7 @@ void launch_head_istft_f32(const HeadIstftF32& p, cudaStream_t st, int T_grid, b
   if (T_grid < 0) T_grid = p.T;
   const size_t smem = (size_t)(3 * (p.C / 4) * HWP + HFR * NFFT) * sizeof(float);
   // as many CTAs as are resident at once, two per SM: each lays out the weights once and takes several runs of frames
-  const int planes = n_batch > 0 ? n_batch : 1, grid = (T_grid + HF - 1) / HF, most = planes < 2 * 148 ? 2 * 148 / planes : 1;
+  const int planes = n_batch > 0 ? n_batch : 1, grid = (T_grid + HF - 1) / HF, most = planes < 2 * p.n_sm ? 2 * p.n_sm / planes : 1;
   launch_ex(head_istft_f32_kernel, dim3(grid < most ? grid : most, planes), dim3(HT), smem, st, pdl, p);
 }
 

@@ -90,10 +90,11 @@ struct TapConvTc {
   int            n_blocks;   // 64-channel blocks of the input
   int            per_tap;    // a panel serves one tap only (a tap reaches more than 8 frames back)
   int            n_a, n_b;   // panels and weight tiles in shared memory (chosen by the launch)
+  int            n_sm;       // SMs of the device
   int*           err;        // device word that a bounded wait sets when it gives up
 };
 size_t      tapconv_pack_bytes(const TapConvF32& p);
-// Fills tc (but for err) and enqueues the packing of p's weights into dst (tapconv_pack_bytes).
+// Fills tc (but for err and n_sm) and enqueues the packing of p's weights into dst (tapconv_pack_bytes).
 void        pack_tapconv(const TapConvF32& p, uint8_t* dst, TapConvTc* tc);
 cudaError_t prepare_tapconv();   // function attributes; once per model
 
@@ -126,6 +127,7 @@ struct HeadIstftF32 {
   const float* tail_in;       // [12] unnormalised partial sums of samples hop*pos .. +11
   float*       tail_out;      // [12] the same for the next chunk (a different buffer)
   float*       pcm;           // [4*T]
+  int          n_sm;          // SMs of the device
 };
 
 void launch_head_istft_f32(const HeadIstftF32& p, cudaStream_t st, int T_grid = -1, bool pdl = false, int n_batch = 0);
