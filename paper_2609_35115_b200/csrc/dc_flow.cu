@@ -435,9 +435,8 @@ flow_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // to the cluster barrier as soon as it has happened; the barrier's latency (about 1500 cycles) then runs
     // under the arithmetic and the stores that follow, and the freeing warp finds it complete.
     const int last_kk = (BN - 16 * cg - 1) / (16 * EPI_GROUPS);   // (BN > 16 cg for every chunk group of a paired GEMM)
-    // (in the generic kernel, the one of small batches, the loop stays a loop: three unrolled copies of the epilogue
-    // body are code that has to come through the instruction cache at every one of their short launches - cfg3 1.371 ->
-    // 1.359 ms per chunk; the kernels of a role keep them: a QKV thread overlaps its three chunks, 1.911 against 1.926)
+    // (the kernels of a role unroll it: a QKV thread overlaps its three chunks, 1.911 against 1.926 ms per step; in the generic kernel it
+    // stays a loop)
 #pragma unroll(MODE_T >= 0 ? MAX_BN / (16 * EPI_GROUPS) : 1)
     for (int kk = 0; kk < MAX_BN / (16 * EPI_GROUPS); ++kk) {
       const int ch = EPI_GROUPS * kk + cg;
@@ -1286,7 +1285,6 @@ bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, u
 constexpr size_t GEMM_SMEM_EXTRA = 1024 + 2 * MAX_STAGES * 8 + 8 + 8 + 2 * MAX_BN * 4 + 64;   // alignment slack + barriers + constants
 constexpr size_t GEMM_SMEM_MAX = 200 * 1024;
 constexpr int CONV_XCHG = 2 * 4 * TILE_M * 16;      // exchange area of 16 columns in a conv epilogue: two taps, [4 float4 columns][128 rows] each
-constexpr int SPECIALISE_FROM_TILES = 8;   // row tiles of a batch from which the GEMMs run as one kernel per role
 constexpr size_t GEMM_SMEM_MAX_PAIR = 227 * 1024;   // the opt-in limit of the device: eight 28 KB stages of a CTA pair
 
 }  // namespace
@@ -1836,8 +1834,8 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
 
   const int m_tiles = (n * SLOT_ROWS + TILE_M - 1) / TILE_M;
   // N-tile variant: the narrowest whose C-wide GEMMs still fit ONE wave (a GEMM CTA has an SM to itself);
-  // a second, part-filled wave costs more than wider tiles do (measured with 5 and 10 row tiles: 160 CTAs
-  // of 16 columns 0.26 ms per pass, 80 CTAs of 32 columns 0.20 ms)
+  // a second, part-filled wave costs more than wider tiles do (hidden 768, 8 streams: 192 CTAs of 16 columns 2,581 us per
+  // step, 96 of 32 columns 1,640; hidden 448, 12 streams 1,964 against 1,307)
   int v = 2;
   while (v > 0 && m_tiles * (C / (64 >> v)) > m->n_sm) --v;
   // the output projection always uses 16-column tiles: mel/16 CTAs per row tile instead of one, and a
@@ -1884,25 +1882,23 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
       }
     }
     const size_t smem = GEMM_SMEM_EXTRA + (size_t)p.n_stages * stage_bytes;
-    // One instantiation per role for batches of eight row tiles or more: the other roles' epilogues and the slot
-    // fields only they read then cost neither registers nor instructions (32 streams: 2.01 -> 1.94 ms per step).
-    // Small batches keep the one generic kernel for every role: their launches are so short that five alternating
-    // kernel images cost more in instruction-cache misses than the leaner code saves (1 stream: 1.37 -> 1.46 ms
-    // with the specialised forms; the two break even between 4 and 8 row tiles).
+    // One instantiation per role: the other roles' epilogues and the slot fields only they read then cost neither
+    // registers nor instructions.  (hidden 512, 32 streams: 2.01 -> 1.94 ms per step.  The widths that do not run as one kernel of
+    // clusters, with few streams, against the generic kernel for every role: hidden 192 984 -> 949 us with one stream, 1,054 -> 988 with 14; hidden 768
+    // 1,337 -> 1,280 and 1,880 -> 1,792; hidden 1024 1,651 -> 1,597 and 2,181 -> 2,095.)
     const dim3 grid(m_tiles, N / p.BN);
     const int cls = p.mode == MODE_CONV ? 0 : 1;
-    if (m_tiles < SPECIALISE_FROM_TILES) launch(lc, flow_gemm_kernel<false, -1>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     // (a conv block's widest tile, that of a full batch, also has its width fixed at compile time - the epilogue's chunk
     // loop unrolls away: 1.94 -> 1.91 ms per step; the same for the other roles, or a second conv image per kind of
     // tail - carried rows / row statistics - measured nothing or cost what another kernel image costs)
-    else if (p.mode == MODE_CONV && p.n_issuers == 2 && p.BN == 64)
+    if (p.mode == MODE_CONV && p.n_issuers == 2 && p.BN == 64)
       launch(lc, flow_gemm_kernel<false, MODE_CONV, 64>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     else if (p.mode == MODE_CONV && p.n_issuers == 2) launch(lc, flow_gemm_kernel<false, MODE_CONV>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     else if (p.mode == MODE_QKV) launch(lc, flow_gemm_kernel<false, MODE_QKV>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     else if (p.mode == MODE_OPROJ) launch(lc, flow_gemm_kernel<false, MODE_OPROJ>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     else if (p.mode == MODE_INPROJ) launch(lc, flow_gemm_kernel<false, MODE_INPROJ>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
     else if (p.mode == MODE_OUT) launch(lc, flow_gemm_kernel<false, MODE_OUT>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
-    else launch(lc, flow_gemm_kernel<false, -1>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);
+    else launch(lc, flow_gemm_kernel<false, -1>, grid, dim3(GEMM_THREADS), smem, true, cls, tA, tB, p);   // a conv of one reduction block
   };
   // the GEMM whose output feeds an RMS norm leaves the row statistics; the GEMM after the norm applies them
   auto feeds_norm = [&](GemmParams& p) { p.ssq_out = m->ssq; p.ssq_ld = m->rows; };
