@@ -246,8 +246,8 @@ dc_status dc_decode_chunk(dc_stream* stream, const float* feats_dev, int n_frame
  * dc_create, for any other n at the first call that carries n streams (that one call also pays the
  * capture; the graphs form the finite catalog of Section 3.3, Eq. 5) - and only the slot table
  * passed by value changes from call to call.  All four pipelines: the fp32 pipelines run every layer
- * once for the whole batch (a slot of the batch is a plane of the layer's grid, with the tiles and the
- * reduction split of the single-stream step; at most 64 streams), and the token2wav composite batches
+ * once for the whole batch (a slot of the batch is a plane of the layer's grid or half of one's tiles; the order
+ * of every sum is that of the single-stream step; at most 64 streams), and the token2wav composite batches
  * the flow decoder and then the vocoder tails in the same way - a serving round of n sessions is two
  * graph launches. */
 dc_status dc_decode_batch(dc_model* model, int n, dc_stream* const* streams,

@@ -916,8 +916,8 @@ static void build_f32_graph(dc_stream* s) {
 }
 
 // The layers of one fp32 chunk step for nb streams at once: every layer is ONE launch whose grid planes
-// are the slots of the batch record (stream, frames, pointers); per slot the tiles, the reduction split and the
-// arithmetic are those of the single-stream step, so a stream's bytes do not depend on who shares its launch.
+// are the slots of the batch record (stream, frames, pointers).  Tile width and slots per tile depend on the batch, the order in which
+// an output element is summed only on the layer, so a stream's bytes do not depend on who shares its launch.
 static void enqueue_f32_batch(dc_model* m, int nb, cudaStream_t cs, int* launches) {
   const int nL = (int)m->layers.size();
   for (int l = 0; l < nL; ++l) {

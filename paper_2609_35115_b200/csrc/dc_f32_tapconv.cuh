@@ -10,7 +10,8 @@
 // operand latency) to what the conversion and the fp32 rows' traffic cost.
 //
 // One CTA: 128 frames x BN channels of one phase.  Ten warps: 0..7 read the fp32 input rows (ring, or the caller's chunk), split
-// them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue; 8 issues the products; 9 streams the weights, split and packed as swizzled tiles at create.
+// them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue; 8 issues the products; 9 streams the
+// weights, split and packed as swizzled tiles at create.
 // A panel holds 64 channels of the 128 frames and of the up to 8 in front of them: a tap is a row offset of the operand
 // descriptor, so a row is read and split once for all its taps.  (Dilations above 4 fill the panel once per tap.)
 // Per 64 channels and tap: 4 reduction steps of ah x bh, ah x [bm bl], am x [bh bm], al x bh.
