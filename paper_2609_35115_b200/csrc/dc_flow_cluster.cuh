@@ -33,7 +33,10 @@ constexpr int CLU_CONST_FLOATS = 3 * 64 + 128 + 256;
 // own wherever 32 do not fit: 16 streams 1,822 us against 1,667.)
 constexpr int CLU_BN = 32;
 constexpr int CLU_SLOT = 3 * CLU_BN * 128;           // bytes of the largest weight tile (three taps / Q, K, V)
-constexpr int CLU_RS = 6;                            // weight ring (even: within a stage a ring slot belongs to one issuer)
+// Weight ring: the tiles of a whole stage, so that a stage's last products do not wait for slots that its first ones free, 1,000 cycles of
+// latency later.  (Six slots: 2,325 cycles from a conv stage's first product to its last one's end, eight: 2,000.  One stream 916 -> 895 us per
+// chunk, seven 960 -> 911, fourteen 1,097 -> 1,032.)  Even: within a stage a ring slot belongs to one issuer.
+constexpr int CLU_RS = 8;
 constexpr size_t CLU_SMEM = (size_t)CLU_PANEL + CLU_RS * CLU_SLOT + CLU_TAIL;
 static_assert(CLU_SMEM <= 227 * 1024, "one CTA's shared memory");
 
