@@ -91,20 +91,22 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
   const int plane = (p.batch != nullptr ? blockIdx.z / p.n_phase : 0), phase = blockIdx.z - plane * p.n_phase;
   auto record = [&](int slot) {
     TcSlot a{p.T_in, p.pos_in, p.in_direct, p.out_direct, p.in_ring, p.out_ring, p.save_ring, p.exc_rng_id};
-    const F32Call* callp = p.call;
-    if (p.batch != nullptr) {
+    F32Call c{};
+    if (p.batch != nullptr) {   // (the count, the call and the stream's table are requested together: an L2 latency less in front of the rows)
+      const F32BatchSlot& bs = p.batch->s[slot];
+      const F32StreamPtrs* ptrs = bs.ptrs;
+      c = bs.call;
       if (slot >= p.batch->n) {
         a.T = 0;
         return a;
       }
-      const F32BatchSlot& bs = p.batch->s[slot];
-      callp = &bs.call;
-      a.in_ring = bs.ptrs->ring[p.layer];
-      a.out_ring = p.last_layer ? nullptr : bs.ptrs->ring[p.layer + 1];
-      a.save_ring = p.first_layer ? bs.ptrs->ring[p.layer] : nullptr;
+      a.in_ring = ptrs->ring[p.layer];
+      a.out_ring = p.last_layer ? nullptr : ptrs->ring[p.layer + 1];
+      a.save_ring = p.first_layer ? ptrs->ring[p.layer] : nullptr;
+    } else if (p.call != nullptr) {
+      c = *p.call;
     }
-    if (callp != nullptr) {
-      const F32Call c = *callp;
+    if (p.batch != nullptr || p.call != nullptr) {
       a.rng_id = c.rng_id;
       a.T = c.T * p.rate_in;
       a.pos = c.frames * p.rate_in;
@@ -138,25 +140,72 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     if (tid == 0) atomicExch(tc.err, 14);
     return;
   }
-  if (tid == 0) {
-#pragma unroll 1
-    for (int i = 0; i < TC_MAX_A; ++i) {
-      ptx::mbar_init(&full_a[i], TC_CONV);
-      ptx::mbar_init(&empty_a[i], 1);
+  // Row numbers in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
+  // address of a row cost more instructions than its arithmetic), the element offset widened: frame m0 + i, i possibly negative.
+  const int C_in = p.C_in, in_mask = p.in_mask;
+  auto in_row = [&](const TcSlot& a, int i) -> const float* {
+    const bool direct = a.in_direct != nullptr && i >= 0;
+    const uint32_t r = direct ? (uint32_t)i : ((uint32_t)a.pos + (uint32_t)i) & (uint32_t)in_mask;
+    return (direct ? a.in_direct : a.in_ring) + (size_t)r * (uint32_t)C_in;
+  };
+  const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
+  float4 xa[TC_ITEMS], xb[TC_ITEMS];
+  auto load = [&](int u) {
+    const int blk = tc.per_tap ? u / p.n_taps : u, tap = tc.per_tap ? u - blk * p.n_taps : 0;
+    const int c = blk * 64 + c8;
+    const int i0 = m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
+#pragma unroll
+    for (int i = 0; i < TC_ITEMS; ++i) {
+      const int row = row0 + 32 * i, seg = PACK && i >= TC_SEG / 32 ? TC_SEG : 0;   // (with PACK the tile starts at frame 0)
+      const TcSlot& a = seg ? s1 : s0;
+      xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      xb[i] = xa[i];
+      if (row < TC_ROWS && m0 + row - seg - TC_H < a.T && c < C_in && (!PACK || a.T > 0)) {   // (an odd batch's last tile has no second slot)
+        const float* src = in_row(a, i0 + row - seg) + c;
+        xa[i] = *reinterpret_cast<const float4*>(src);
+        if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
+      }
     }
+  };
+  // The set-up beside the first latencies: the converting warps request their rows, warp 9 the first weights, warp 8 does the rest.
+  // (Behind the block's barrier both came one latency later: one stream of the vocoder 107.0 -> 99.6 us per chunk, 8 streams 234 -> 220, 32 streams 698 -> 645.)
+  auto weights = [&](int i, int st) {             // tile i of n_blocks x n_taps: three planes
+    const uint8_t* src = tc.W + ((size_t)((phase * tc.n_blocks * p.n_taps + i) * 3) * tc.C_pad + (size_t)n0) * 128;
+    ptx::mbar_expect_tx(&full_b[st], B_TILE);
 #pragma unroll 1
-    for (int i = 0; i < TC_MAX_B; ++i) {
-      ptx::mbar_init(&full_b[i], 1);
-      ptx::mbar_init(&empty_b[i], 1);
-    }
+    for (int q = 0; q < 3; ++q) ptx::bulk_load(sB + st * B_TILE + q * BN * 128, src + (size_t)q * tc.C_pad * 128, BN * 128, &full_b[st]);
+  };
+  if (warp < 8) {
+    load(0);
+  } else if (lane == 0) {
+    if (warp == 9) {
 #pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
-      ptx::mbar_init(&accum[i], 1);
-      ptx::mbar_init(&drained[i], TC_CONV);
+      for (int i = 0; i < TC_MAX_B; ++i) {
+        ptx::mbar_init(&full_b[i], 1);
+        ptx::mbar_init(&empty_b[i], 1);
+      }
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < TC_MAX_A; ++i) {
+        ptx::mbar_init(&full_a[i], TC_CONV);
+        ptx::mbar_init(&empty_a[i], 1);
+      }
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {
+        ptx::mbar_init(&accum[i], 1);
+        ptx::mbar_init(&drained[i], TC_CONV);
+      }
+      *s_fail = 0;
     }
-    *s_fail = 0;
     ptx::fence_barrier_init();
+    ptx::fence_proxy_async_smem();
   }
+  __syncwarp();
+  if (warp == 9 && ptx::elect_one()) {
+#pragma unroll 1
+    for (int i = 0; i < tc.n_b && i < tc.n_blocks * p.n_taps; ++i) weights(i, i);
+  }
+  __syncwarp();
   // columns: leading term (see above), then the 2^-8 and the 2^-16 terms
   constexpr bool TURN = !DRAIN && BN > 32;
   constexpr uint32_t S_COL = DRAIN ? 6 * BN : (TURN ? 2 * BN : 3 * BN);
@@ -171,20 +220,13 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
 
   if (warp == 9) {
     // ---------------- weight stream: one tile of three planes per (block, tap) ----------------
-    const size_t plane = (size_t)tc.C_pad * 128;
-    const uint8_t* src = tc.W + (size_t)phase * tc.n_blocks * p.n_taps * 3 * plane + (size_t)n0 * 128;
-    const int n = tc.n_blocks * p.n_taps;
     int st = 0;
-    uint32_t ph = 1;
+    uint32_t ph = 0;
     bool ok = true;
 #pragma unroll 1
-    for (int i = 0; i < n && ok; ++i, src += 3 * plane) {
-      if (i >= tc.n_b) ok = tc_wait(&empty_b[st], ph, s_fail, tc.err, 0x201);
-      if (ok && ptx::elect_one()) {
-        ptx::mbar_expect_tx(&full_b[st], B_TILE);
-#pragma unroll 1
-        for (int q = 0; q < 3; ++q) ptx::bulk_load(sB + st * B_TILE + q * BN * 128, src + q * plane, BN * 128, &full_b[st]);
-      }
+    for (int i = tc.n_b; i < tc.n_blocks * p.n_taps && ok; ++i) {   // (the first n_b have been requested)
+      ok = tc_wait(&empty_b[st], ph, s_fail, tc.err, 0x201);
+      if (ok && ptx::elect_one()) weights(i, st);
       __syncwarp();
       if (++st == tc.n_b) { st = 0; ph ^= 1u; }
     }
@@ -242,33 +284,6 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
   } else {
     // ---------------- input rows -> bf16 planes ----------------
-    // Row numbers in 32-bit arithmetic (a ring index needs only the low bits of the clock; in 64 bits, with its branches, the
-    // address of a row cost more instructions than its arithmetic), the element offset widened: frame m0 + i, i possibly negative.
-    const int C_in = p.C_in, in_mask = p.in_mask;
-    auto in_row = [&](const TcSlot& a, int i) -> const float* {
-      const bool direct = a.in_direct != nullptr && i >= 0;
-      const uint32_t r = direct ? (uint32_t)i : ((uint32_t)a.pos + (uint32_t)i) & (uint32_t)in_mask;
-      return (direct ? a.in_direct : a.in_ring) + (size_t)r * (uint32_t)C_in;
-    };
-    const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
-    float4 xa[TC_ITEMS], xb[TC_ITEMS];
-    auto load = [&](int u) {
-      const int blk = tc.per_tap ? u / p.n_taps : u, tap = tc.per_tap ? u - blk * p.n_taps : 0;
-      const int c = blk * 64 + c8;
-      const int i0 = m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
-#pragma unroll
-      for (int i = 0; i < TC_ITEMS; ++i) {
-        const int row = row0 + 32 * i, seg = PACK && i >= TC_SEG / 32 ? TC_SEG : 0;   // (with PACK the tile starts at frame 0)
-        const TcSlot& a = seg ? s1 : s0;
-        xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        xb[i] = xa[i];
-        if (row < TC_ROWS && m0 + row - seg - TC_H < a.T && c < C_in && (!PACK || a.T > 0)) {   // (an odd batch's last tile has no second slot)
-          const float* src = in_row(a, i0 + row - seg) + c;
-          xa[i] = *reinterpret_cast<const float4*>(src);
-          if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
-        }
-      }
-    };
     const int q = warp & 3, col0 = (warp >> 2) * (BN / 2);   // epilogue: TMEM lane quarter; columns col0 .. col0 + BN / 2 - 1
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
     constexpr int NC = BN / 32;
@@ -303,7 +318,6 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       ptx::mbar_arrive(&drained[u & 1]);
       return got;
     };
-    load(0);
     int sa = 0;
     uint32_t ph = 1;
     bool ok = true;
