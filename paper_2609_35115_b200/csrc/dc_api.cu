@@ -477,8 +477,12 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
     if (e == cudaSuccess) e = pack_f32_weights(m);
     if (e == cudaSuccess) e = dc::prepare_f32_constants();
     if (e == cudaSuccess && cfg->max_batch > 1) {
-      e = dc::dev_alloc(&m->d_batch, sizeof(dc::F32Batch));
-      if (e == cudaSuccess) e = cudaMemset(m->d_batch, 0, sizeof(dc::F32Batch));
+      dc::F32BatchTable* table = nullptr;
+      e = dc::dev_alloc(&table, sizeof(dc::F32BatchTable));
+      if (e == cudaSuccess) {
+        m->d_batch = &table->b;
+        e = cudaMemset(table, 0, sizeof(dc::F32BatchTable));
+      }
     }
     if (e != cudaSuccess) {
       dc::set_error("weight upload failed: %s", cudaGetErrorString(e));

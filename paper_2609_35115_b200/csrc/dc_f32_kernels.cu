@@ -251,8 +251,9 @@ __global__ void __launch_bounds__(HT, 2) head_istft_f32_kernel(const HeadIstftF3
     if ((int)blockIdx.y >= p.batch->n) return;
     const F32BatchSlot& bs = p.batch->s[blockIdx.y];
     p.call = &bs.call;
-    p.in_ring = bs.ptrs->ring[p.layer];
-    p.tails = bs.ptrs->tails;
+    const F32StreamPtrs& ptrs = reinterpret_cast<const F32BatchTable*>(p.batch)->ptrs[blockIdx.y];
+    p.in_ring = ptrs.ring[p.layer];
+    p.tails = ptrs.tails;
   }
   if (p.call != nullptr) {
     const F32Call c = *p.call;
@@ -426,7 +427,10 @@ __global__ void set_f32_batch_kernel(const __grid_constant__ F32Batch v, F32Batc
     dst->n = v.n;
     dst->pad = 0;
   }
-  if ((int)threadIdx.x < v.n) dst->s[threadIdx.x] = v.s[threadIdx.x];
+  if ((int)threadIdx.x < v.n) {
+    dst->s[threadIdx.x] = v.s[threadIdx.x];
+    reinterpret_cast<F32BatchTable*>(dst)->ptrs[threadIdx.x] = *v.s[threadIdx.x].ptrs;
+  }
 }
 
 template <typename... KArgs, typename... Args>

@@ -47,6 +47,12 @@ struct F32Batch {
   int          n, pad;
   F32BatchSlot s[F32_MAX_BATCH];
 };
+// The record in device memory: the setter kernel copies the streams' tables behind it, so that a layer's CTAs find the rings' addresses
+// beside the call and not one latency behind it.
+struct F32BatchTable {
+  F32Batch      b;
+  F32StreamPtrs ptrs[F32_MAX_BATCH];
+};
 
 struct TapConvF32 {
   const F32Batch* batch;   // if set: slot = blockIdx.z / n_phase; per-call values and ring addresses come from batch->s[slot]
