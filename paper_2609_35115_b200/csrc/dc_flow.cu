@@ -71,7 +71,7 @@ struct SlotInfo {
   // is folded into its halo / kv pointers by the host; what remains per slot is the timestep-bias row and two flags.
   int          tau_off;   // float offset of the slot's Euler step inside the timestep-bias table (0 when the launch's own step applies)
   int          flags;     // SLOT_FIRST: the prep kernel loads x_0 and mu; SLOT_LAST: the output projection also writes `out`
-  int          pad;
+  int          pad;       // slot 0, wavefront: where the live slots begin (flow_cluster_kernel)
 };
 constexpr int SLOT_FIRST = 1, SLOT_LAST = 2;
 
@@ -1369,7 +1369,9 @@ void pack_wt(std::vector<uint16_t>& dst, size_t off, const float* W, int K, int 
 }  // namespace
 
 namespace {
-bool build_graph(FlowModel* m, int n, bool tick = false);
+bool build_graph(FlowModel* m, int n, bool tick = false, bool ring = false);
+int cluster_slots(const FlowModel* m, int n);
+bool wave_ring(const FlowModel* m, int n);
 cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>& w_conv, const std::vector<size_t>& w_qkv,
                            const std::vector<size_t>& w_o, size_t w_out);
 }
@@ -1570,7 +1572,10 @@ dc_status flow_model_create(const dc_config& cfg, const float* w, FlowModel** ou
       const bool gs = m->S > m->n_pass ? build_graph(m, m->S) : g1;
       // ... and one pass of the network over n_steps chunks (wavefront decoding), where the model has room for it
       const int n_wave = cfg.n_steps * m->n_pass;
-      if (n_wave <= m->S && n_wave <= MAX_SLOTS_PER_SET) build_graph(m, n_wave, true);
+      if (n_wave <= m->S && n_wave <= MAX_SLOTS_PER_SET) {
+        build_graph(m, n_wave, true);
+        if (wave_ring(m, n_wave)) build_graph(m, n_wave, true, true);
+      }
       (void)gs;
     }
     cudaGetLastError();
@@ -1740,17 +1745,22 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   const int C = m->C, CL = C / CLU_BN, nL = c.n_conv, nA = c.n_attn;
   const uint32_t apart = DC_OPT_SKIP_CONV_GEMM | DC_OPT_SKIP_ATTENTION | DC_OPT_EMPTY_KERNELS | DC_OPT_CTA_PAIRS;
   if ((c.options & apart) || (C != 64 && C != 128 && C != 256 && C != 512)) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(flow_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
-  if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(flow_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaSuccess;
+  cudaFuncAttributes fa{};
+  int regs = 1 << 16;
+  for (auto fn : {flow_cluster_kernel<false>, flow_cluster_kernel<true>}) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
+    if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+    regs = std::min(regs, fa.numRegs);
+  }
   int n_cl = 0;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, CL, 1, nullptr, false);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, flow_cluster_kernel, &cfg);
-  cudaFuncAttributes fa{};
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, flow_cluster_kernel);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, flow_cluster_kernel<false>, &cfg);
   // (the kernel redistributes the registers that it was launched with: they have to cover the split)
-  if (e == cudaSuccess && fa.numRegs * CLU_THREADS < 128 * CLU_REGS_CTRL + CLU_EPI * CLU_REGS_EPI) n_cl = 0;
+  if (e == cudaSuccess && regs * CLU_THREADS < 128 * CLU_REGS_CTRL + CLU_EPI * CLU_REGS_EPI) n_cl = 0;
   if (e != cudaSuccess || n_cl < 1) {   // the kernels of their own serve the model
     cudaGetLastError();
     return cudaSuccess;
@@ -1790,7 +1800,12 @@ int cluster_slots(const FlowModel* m, int n) {
   return 0;
 }
 
-void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick) {
+// Wavefront: whether a tick of n slots, two per cluster, can run with one slot per cluster while few enough of them are live (the first and the
+// last ticks of an utterance: 10 chunks in flight and seven clusters, 14 of the 29 ticks of 20 chunks).  A cluster
+// with one slot takes 88 us a pass, with two 101: 20 s of audio 3,023 -> 2,933 us.
+bool wave_ring(const FlowModel* m, int n) { return m->n_pass == 1 && cluster_slots(m, n) == 2; }
+
+void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, bool ring) {
   const dc_config& c = m->cfg;
   CluParams p{};
   p.slots = m->d_slots; p.n_slots = n; p.spc = spc; p.CL = m->C / CLU_BN;
@@ -1808,9 +1823,9 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick) {
   p.err = m->d_err;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  cluster_config(cfg, attr, p.CL, (n + spc - 1) / spc, lc.st, lc.pdl);
+  cluster_config(cfg, attr, p.CL, ring ? m->max_clusters : (n + spc - 1) / spc, lc.st, lc.pdl);
   ProfScope ps(lc.prof, 7, lc.st);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, flow_cluster_kernel, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, ring ? flow_cluster_kernel<true> : flow_cluster_kernel<false>, p);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
   ++lc.launches;
 }
@@ -1819,16 +1834,17 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick) {
 // kernel(s) from `sets`).
 // tick = false: the n slots' chunks, all Euler steps.  tick = true: ONE pass of the network, every slot at the Euler step
 // that its slot-table entry encodes (wavefront decoding: the slots are consecutive chunks of one stream).
-void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchCtx& lc, bool tick = false) {
+// ring (a tick): only the slots from sets[0].s[0].pad on, as many as there are clusters, may be live.
+void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchCtx& lc, bool tick = false, bool ring = false) {
   const dc_config& c = m->cfg;
   const int C = m->C, mel = m->mel;
   for (int i = 0; i < n_sets; ++i)   // not a programmatic launch: it overwrites the table the previous chunk still reads
     launch(lc, set_slots_kernel, dim3(1), dim3(MAX_SLOTS_PER_SET), 0, false, 4, sets[i], m->d_slots);
-  const int spc = cluster_slots(m, n);
+  const int spc = ring ? 1 : cluster_slots(m, n);
   launch(lc, flow_prep_kernel, dim3(n, ((c.f_chunk + c.f_lookahead) * (mel / 4) + 127) / 128), dim3(128), 0, true, 4, (const SlotInfo*)m->d_slots, mel, m->xstate, spc > 0 ? m->AinP : m->Ain, m->Kin,
          (uint32_t)c.noise_seed_lo, (uint32_t)c.noise_seed_hi, (int)(spc > 0));
   if (spc > 0) {
-    enqueue_cluster(m, n, spc, lc, tick);
+    enqueue_cluster(m, n, spc, lc, tick, ring);
     return;
   }
 
@@ -2003,8 +2019,11 @@ void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchC
 
 // One captured graph per batch size: the whole chunk step becomes a single graph launch; only the
 // slot-table node's by-value argument changes from call to call.
-// Graphs are keyed by the slot count; tick graphs (one pass of the network, wavefront decoding) by its negative.
-bool build_graph(FlowModel* m, int n, bool tick) {
+// Graphs are keyed by the slot count; tick graphs (one pass of the network, wavefront decoding) by its negative, those of few live
+// slots beyond that.
+int graph_key(int n, bool tick, bool ring) { return !tick ? n : (ring ? -MAX_SLOTS_PER_SET - n : -n); }
+
+bool build_graph(FlowModel* m, int n, bool tick, bool ring) {
   if (n > MAX_SLOTS_PER_SET || m->cap_stream == nullptr) return false;
   for (int use_pdl = m->pdl ? 1 : 0; use_pdl >= 0; --use_pdl) {
     SlotSet dummy{};
@@ -2016,7 +2035,7 @@ bool build_graph(FlowModel* m, int n, bool tick) {
       return false;
     }
     LaunchCtx lc{m->cap_stream, use_pdl != 0, nullptr};
-    enqueue_chunk(m, n, &dummy, 1, lc, tick);
+    enqueue_chunk(m, n, &dummy, 1, lc, tick, ring);
     cudaError_t e = cudaStreamEndCapture(m->cap_stream, &graph);
     if (e != cudaSuccess || lc.err != cudaSuccess || graph == nullptr) {
       cudaGetLastError();
@@ -2044,7 +2063,7 @@ bool build_graph(FlowModel* m, int n, bool tick) {
     ge.graph = graph;
     ge.launches = lc.launches;
     ge.pdl = use_pdl != 0;
-    m->graphs[tick ? -n : n] = ge;
+    m->graphs[graph_key(n, tick, ring)] = ge;
     return true;
   }
   return false;
@@ -2149,8 +2168,12 @@ dc_status flow_decode_wave(FlowModel* m, int n_streams, FlowState* const* states
     if (nc > max_chunks) max_chunks = nc;
   }
   const bool profiling = m->prof != nullptr && m->prof->on;
-  auto it = m->graphs.find(-n);   // one stream: captured at create; other stream counts: at their first call
-  if (it == m->graphs.end() && !profiling && build_graph(m, n, true)) it = m->graphs.find(-n);
+  const bool may_ring = n_streams == 1 && wave_ring(m, n);
+  std::map<int, GraphEntry>::iterator its[2];   // one stream: captured at create; other stream counts: at their first call
+  for (int r = 0; r < (may_ring ? 2 : 1); ++r) {
+    its[r] = m->graphs.find(graph_key(n, true, r != 0));
+    if (its[r] == m->graphs.end() && !profiling && build_graph(m, n, true, r != 0)) its[r] = m->graphs.find(graph_key(n, true, r != 0));
+  }
   const size_t halo_step = (size_t)c.n_conv * HALO * m->C, kv_step = (size_t)c.n_attn * 2 * (m->P + m->Rk) * m->C;
   SlotSet& set = m->sets[0];
   for (long long t = 0; t < max_chunks + K - 1; ++t) {
@@ -2184,6 +2207,11 @@ dc_status flow_decode_wave(FlowModel* m, int n_streams, FlowState* const* states
       si.halo = s->halo + (size_t)pass * (s->halo_bytes / sizeof(bf16) / np) + (size_t)step * halo_step;
       si.kv = s->kv ? s->kv + (size_t)pass * (s->kv_bytes / sizeof(bf16) / np) + (size_t)step * kv_step : nullptr;
     }
+    // the live chunks, t - K + 1 .. t as far as they exist, are neighbours on the ring of slots
+    const long long j0 = t < K ? 0 : t - K + 1, j1 = t < max_chunks ? t : max_chunks - 1;
+    const bool ring = may_ring && j1 - j0 + 1 <= m->max_clusters;
+    if (ring) set.s[0].pad = (int)(j0 % K);
+    const auto it = its[ring ? 1 : 0];
     if (!profiling && it != m->graphs.end()) {
       GraphEntry& ge = it->second;
       void* args[2] = {&set, &m->d_slots};
@@ -2202,7 +2230,7 @@ dc_status flow_decode_wave(FlowModel* m, int n_streams, FlowState* const* states
       ++m->graph_launches;
     } else {
       LaunchCtx lc{st, m->pdl && !profiling, m->prof};
-      enqueue_chunk(m, n, &set, 1, lc, true);
+      enqueue_chunk(m, n, &set, 1, lc, true, ring);
       *launches += lc.launches;
       if (lc.err != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         set_error("wavefront launch failed: %s", cudaGetErrorString(lc.err));

@@ -132,6 +132,9 @@ struct CluJob {     // what the heads of a slot attend
 
 static_assert(8 * (16 + 2 * CLU_RS + 2 * (int)CLU_KVS + 10) + 2 * (int)sizeof(CluJob) + 8 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
 
+// RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].pad on, circularly.  (An instantiation of its
+// own: with the choice at run time every other call was 2 to 5 us slower.)
+template <bool RING>
 __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __grid_constant__ CluParams p) {
   constexpr int BN = CLU_BN, RS = CLU_RS;
   extern __shared__ __align__(1024) uint8_t clu_smem[];
@@ -167,7 +170,13 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (known to be the same for the whole warp)
   const int rank = (int)ptx::cluster_ctarank();
   const int n0 = rank * BN;
-  const int slot0 = (int)(blockIdx.x / (unsigned)p.CL) * p.spc, m0 = slot0 * SLOT_ROWS;
+  int slot_0 = (int)(blockIdx.x / (unsigned)p.CL) * p.spc;
+  if (RING) {
+    ptx::pdl_wait();
+    slot_0 += p.slots[0].pad;
+    if (slot_0 >= p.n_slots) slot_0 -= p.n_slots;
+  }
+  const int slot0 = slot_0, m0 = slot0 * SLOT_ROWS;
   const int nkb_c = p.C / KBLK, nkb_in = p.Kin / KBLK;
   const int n_out = p.mel / 16;
   const int nch_out = rank < n_out ? (n_out - rank + p.CL - 1) / p.CL : 0;   // 16-column chunks rank, rank + CL, ... of the output projection

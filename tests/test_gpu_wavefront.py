@@ -78,6 +78,12 @@ def test_wavefront_shorter_than_the_pipeline(dc):
     _wave_vs_chunks(dc, wl.tiny_flow(), 5)
 
 
+# more chunks in flight than clusters: ticks with few live slots take one slot per cluster, from wherever the live ones are on the ring
+@pytest.mark.parametrize("n_chunks", [1, 7, 8, 10, 13, 24])
+def test_wavefront_few_live_slots(dc, n_chunks):
+    _wave_vs_chunks(dc, wl.tiny_flow(hidden=512, n_heads=8, head_dim=64, n_steps=10, seed=36), 10 * n_chunks - 3)
+
+
 def test_wavefront_then_streaming_continues_from_its_carries(dc):
     _wave_vs_chunks(dc, wl.tiny_flow(), 87, split=50)
 
