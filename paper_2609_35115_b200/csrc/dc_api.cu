@@ -153,7 +153,7 @@ struct dc_model {
   dc_model* sub_voc = nullptr;
   // fp32 pipelines: dc_decode_batch runs every layer ONCE for all the streams of the batch (slot = grid plane); the slot
   // records live here and are rewritten per call by the first node of the captured batch step
-  dc::F32Batch*   d_batch = nullptr;
+  dc::F32BatchTable* d_batch = nullptr;
   struct BatchGraph {
     cudaGraph_t     graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -477,12 +477,8 @@ extern "C" dc_status dc_create(const float* w, size_t n_floats, const dc_config*
     if (e == cudaSuccess) e = pack_f32_weights(m);
     if (e == cudaSuccess) e = dc::prepare_f32_constants();
     if (e == cudaSuccess && cfg->max_batch > 1) {
-      dc::F32BatchTable* table = nullptr;
-      e = dc::dev_alloc(&table, sizeof(dc::F32BatchTable));
-      if (e == cudaSuccess) {
-        m->d_batch = &table->b;
-        e = cudaMemset(table, 0, sizeof(dc::F32BatchTable));
-      }
+      e = dc::dev_alloc(&m->d_batch, sizeof(dc::F32BatchTable));
+      if (e == cudaSuccess) e = cudaMemset(m->d_batch, 0, sizeof(dc::F32BatchTable));
     }
     if (e != cudaSuccess) {
       dc::set_error("weight upload failed: %s", cudaGetErrorString(e));
@@ -999,7 +995,7 @@ static dc_status decode_f32_batch(dc_model* m, int n, dc_stream* const* streams,
     it = m->gb.find(n);
   }
   if (it != m->gb.end() && !m->prof.on) {
-    dc::F32Batch* dst = m->d_batch;
+    dc::F32BatchTable* dst = m->d_batch;
     void* args[2] = {&hb, &dst};
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void*>(dc::set_f32_batch_func());

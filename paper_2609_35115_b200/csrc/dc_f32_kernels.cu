@@ -248,10 +248,9 @@ __global__ void __launch_bounds__(HT, 2) head_istft_f32_kernel(const HeadIstftF3
   ptx::pdl_wait();
   HeadIstftF32 p = p_in;
   if (p.batch != nullptr) {
-    if ((int)blockIdx.y >= p.batch->n) return;
-    const F32BatchSlot& bs = p.batch->s[blockIdx.y];
-    p.call = &bs.call;
-    const F32StreamPtrs& ptrs = reinterpret_cast<const F32BatchTable*>(p.batch)->ptrs[blockIdx.y];
+    if ((int)blockIdx.y >= p.batch->b.n) return;
+    p.call = &p.batch->b.s[blockIdx.y].call;
+    const F32StreamPtrs& ptrs = p.batch->ptrs[blockIdx.y];
     p.in_ring = ptrs.ring[p.layer];
     p.tails = ptrs.tails;
   }
@@ -422,14 +421,14 @@ __global__ void set_f32_call_kernel(const F32Call v, F32Call* dst) {
   if (threadIdx.x == 0) *dst = v;
 }
 
-__global__ void set_f32_batch_kernel(const __grid_constant__ F32Batch v, F32Batch* dst) {
+__global__ void set_f32_batch_kernel(const __grid_constant__ F32Batch v, F32BatchTable* dst) {
   if (threadIdx.x == 0) {
-    dst->n = v.n;
-    dst->pad = 0;
+    dst->b.n = v.n;
+    dst->b.pad = 0;
   }
   if ((int)threadIdx.x < v.n) {
-    dst->s[threadIdx.x] = v.s[threadIdx.x];
-    reinterpret_cast<F32BatchTable*>(dst)->ptrs[threadIdx.x] = *v.s[threadIdx.x].ptrs;
+    dst->b.s[threadIdx.x] = v.s[threadIdx.x];
+    dst->ptrs[threadIdx.x] = *v.s[threadIdx.x].ptrs;
   }
 }
 
@@ -476,7 +475,7 @@ void launch_set_f32_call(const F32Call& v, F32Call* dst, cudaStream_t st) {
   set_f32_call_kernel<<<1, 32, 0, st>>>(v, dst);
 }
 
-void launch_set_f32_batch(const F32Batch& v, F32Batch* dst, cudaStream_t st) {
+void launch_set_f32_batch(const F32Batch& v, F32BatchTable* dst, cudaStream_t st) {
   set_f32_batch_kernel<<<1, F32_MAX_BATCH, 0, st>>>(v, dst);
 }
 const void* set_f32_batch_func() { return (const void*)set_f32_batch_kernel; }

@@ -93,13 +93,12 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     TcSlot a{p.T_in, p.pos_in, p.in_direct, p.out_direct, p.in_ring, p.out_ring, p.save_ring, p.exc_rng_id};
     F32Call c{};
     if (p.batch != nullptr) {   // (the count, the call and the rings are requested together: two L2 latencies less in front of the rows: 8 streams 220 -> 217.5 us, 32 streams 645 -> 632)
-      const F32BatchSlot& bs = p.batch->s[slot];
-      const F32StreamPtrs& ptrs = reinterpret_cast<const F32BatchTable*>(p.batch)->ptrs[slot];
-      c = bs.call;
+      const F32StreamPtrs& ptrs = p.batch->ptrs[slot];
+      c = p.batch->b.s[slot].call;
       a.in_ring = ptrs.ring[p.layer];
       a.out_ring = p.last_layer ? nullptr : ptrs.ring[p.layer + 1];
       a.save_ring = p.first_layer ? ptrs.ring[p.layer] : nullptr;
-      if (slot >= p.batch->n) {
+      if (slot >= p.batch->b.n) {
         a.T = 0;
         return a;
       }

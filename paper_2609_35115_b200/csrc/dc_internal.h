@@ -31,8 +31,8 @@ struct F32Call {
 
 // Several streams of one fp32 model in ONE launch of every layer (multi-session serving): a record per slot in
 // device memory, rewritten per call by a setter kernel (its by-value argument), and - because every stream has
-// rings of its own - a per-stream table of ring addresses written once at dc_stream_open.  Slot i of the batch
-// is grid plane i of every layer kernel; the arithmetic of a slot is exactly that of a single-stream call.
+// rings of its own - a per-stream table of ring addresses written once at dc_stream_open, which the setter copies behind the
+// records.  Slot i of the batch is grid plane i of every layer kernel; the arithmetic of a slot is exactly that of a single-stream call.
 constexpr int F32_MAX_LAYERS = 24;
 constexpr int F32_MAX_BATCH = 64;
 struct F32StreamPtrs {
@@ -43,11 +43,11 @@ struct F32BatchSlot {
   F32Call              call;
   const F32StreamPtrs* ptrs;
 };
-struct F32Batch {
+struct F32Batch {            // the setter's argument
   int          n, pad;
   F32BatchSlot s[F32_MAX_BATCH];
 };
-// The record in device memory: the setter kernel copies the streams' tables behind it, so that a layer's CTAs find the rings' addresses
+// What lies in device memory and every layer reads: with the streams' tables behind the records a layer's CTAs find the rings' addresses
 // beside the call and not one latency behind it.
 struct F32BatchTable {
   F32Batch      b;
@@ -55,8 +55,8 @@ struct F32BatchTable {
 };
 
 struct TapConvF32 {
-  const F32Batch* batch;   // if set: slot = blockIdx.z / n_phase; per-call values and ring addresses come from batch->s[slot]
-  int          layer;      // ... ring[layer] is this layer's input ring, ring[layer + 1] its output ring
+  const F32BatchTable* batch; // if set: slot = blockIdx.z / n_phase; per-call values come from batch->b.s[slot], ring addresses from batch->ptrs[slot]
+  int          layer;      // ... whose ring[layer] is this layer's input ring, ring[layer + 1] its output ring
   const F32Call* call;     // if set: T_in, pos_in, pos_out, in_direct, out_direct come from *call
   int          rate_in;    // ... scaled by this layer's frames per chunk frame
   int          first_layer, last_layer;
@@ -111,13 +111,13 @@ void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc, cudaStream_t st
 void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st);
 void launch_set_f32_call(const F32Call& v, F32Call* dst, cudaStream_t st);
 const void* set_f32_call_func();
-void launch_set_f32_batch(const F32Batch& v, F32Batch* dst, cudaStream_t st);
+void launch_set_f32_batch(const F32Batch& v, F32BatchTable* dst, cudaStream_t st);
 const void* set_f32_batch_func();
 
 // Head conv (k = 3, input already SiLU-activated) + magnitude/phase -> inverse real DFT (n_fft = 16)
 // -> synthesis window -> overlap-add (hop 4) with the 12-sample tail carried across chunks.
 struct HeadIstftF32 {
-  const F32Batch* batch;      // if set: slot = blockIdx.y; per-call values, ring and tails come from batch->s[slot]
+  const F32BatchTable* batch; // if set: slot = blockIdx.y; per-call values come from batch->b.s[slot], ring and tails from batch->ptrs[slot]
   int          layer;
   const F32Call* call;        // if set: pos, T, tails and pcm come from *call
   int          rate_in;
