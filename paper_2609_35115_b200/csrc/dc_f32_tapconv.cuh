@@ -166,43 +166,29 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
       }
     }
   };
-  // The set-up beside the first latencies: the converting warps request their rows, warp 9 the first weights, warp 8 does the rest.
-  // (Behind the block's barrier both came one latency later: one stream of the vocoder 107.0 -> 99.6 us per chunk, 8 streams 234 -> 220, 32 streams 698 -> 645.)
-  auto weights = [&](int i, int st) {             // tile i of n_blocks x n_taps: three planes
-    const uint8_t* src = tc.W + ((size_t)((phase * tc.n_blocks * p.n_taps + i) * 3) * tc.C_pad + (size_t)n0) * 128;
-    ptx::mbar_expect_tx(&full_b[st], B_TILE);
-#pragma unroll 1
-    for (int q = 0; q < 3; ++q) ptx::bulk_load(sB + st * B_TILE + q * BN * 128, src + (size_t)q * tc.C_pad * 128, BN * 128, &full_b[st]);
-  };
+  // The set-up beside the first latency: the converting warps request their rows while another makes the barriers.  (Rows behind the block's barrier: one
+  // stream of the vocoder 101.6 us per chunk, so 97.5.  The first weights in front of it as well, which only hold the rows up: 99.6, 32 streams 630 against
+  // 624, and a layer of few frames slower than without either.)
   if (warp < 8) {
     load(0);
-  } else if (lane == 0) {
-    if (warp == 9) {
+  } else if (warp == 9 && lane == 0) {
 #pragma unroll 1
-      for (int i = 0; i < TC_MAX_B; ++i) {
-        ptx::mbar_init(&full_b[i], 1);
-        ptx::mbar_init(&empty_b[i], 1);
-      }
-    } else {
-#pragma unroll 1
-      for (int i = 0; i < TC_MAX_A; ++i) {
-        ptx::mbar_init(&full_a[i], TC_CONV);
-        ptx::mbar_init(&empty_a[i], 1);
-      }
-#pragma unroll 1
-      for (int i = 0; i < 2; ++i) {
-        ptx::mbar_init(&accum[i], 1);
-        ptx::mbar_init(&drained[i], TC_CONV);
-      }
-      *s_fail = 0;
+    for (int i = 0; i < TC_MAX_A; ++i) {
+      ptx::mbar_init(&full_a[i], TC_CONV);
+      ptx::mbar_init(&empty_a[i], 1);
     }
-    ptx::fence_barrier_init();
-    ptx::fence_proxy_async_smem();
-  }
-  __syncwarp();
-  if (warp == 9 && ptx::elect_one()) {
 #pragma unroll 1
-    for (int i = 0; i < tc.n_b && i < tc.n_blocks * p.n_taps; ++i) weights(i, i);
+    for (int i = 0; i < TC_MAX_B; ++i) {
+      ptx::mbar_init(&full_b[i], 1);
+      ptx::mbar_init(&empty_b[i], 1);
+    }
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&accum[i], 1);
+      ptx::mbar_init(&drained[i], TC_CONV);
+    }
+    *s_fail = 0;
+    ptx::fence_barrier_init();
   }
   __syncwarp();
   // columns: leading term (see above), then the 2^-8 and the 2^-16 terms
@@ -219,13 +205,20 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
 
   if (warp == 9) {
     // ---------------- weight stream: one tile of three planes per (block, tap) ----------------
+    const size_t plane = (size_t)tc.C_pad * 128;
+    const uint8_t* src = tc.W + (size_t)phase * tc.n_blocks * p.n_taps * 3 * plane + (size_t)n0 * 128;
+    const int n = tc.n_blocks * p.n_taps;
     int st = 0;
-    uint32_t ph = 0;
+    uint32_t ph = 1;
     bool ok = true;
 #pragma unroll 1
-    for (int i = tc.n_b; i < tc.n_blocks * p.n_taps && ok; ++i) {   // (the first n_b have been requested)
-      ok = tc_wait(&empty_b[st], ph, s_fail, tc.err, 0x201);
-      if (ok && ptx::elect_one()) weights(i, st);
+    for (int i = 0; i < n && ok; ++i, src += 3 * plane) {
+      if (i >= tc.n_b) ok = tc_wait(&empty_b[st], ph, s_fail, tc.err, 0x201);
+      if (ok && ptx::elect_one()) {
+        ptx::mbar_expect_tx(&full_b[st], B_TILE);
+#pragma unroll 1
+        for (int q = 0; q < 3; ++q) ptx::bulk_load(sB + st * B_TILE + q * BN * 128, src + q * plane, BN * 128, &full_b[st]);
+      }
       __syncwarp();
       if (++st == tc.n_b) { st = 0; ph ^= 1u; }
     }
