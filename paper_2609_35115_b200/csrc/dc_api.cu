@@ -1000,7 +1000,7 @@ static dc_status decode_f32_batch(dc_model* m, int n, dc_stream* const* streams,
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void*>(dc::set_f32_batch_func());
     kp.gridDim = dim3(1);
-    kp.blockDim = dim3(dc::F32_MAX_BATCH);
+    kp.blockDim = dim3(dc::F32_SET_THREADS);
     kp.kernelParams = args;
     DC_CUDA(cudaGraphExecKernelNodeSetParams(it->second.exec, it->second.set_node, &kp));
     DC_CUDA(cudaGraphLaunch(it->second.exec, cs));

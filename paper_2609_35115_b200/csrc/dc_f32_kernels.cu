@@ -421,14 +421,19 @@ __global__ void set_f32_call_kernel(const F32Call v, F32Call* dst) {
   if (threadIdx.x == 0) *dst = v;
 }
 
+// A warp per slot, a lane per 8-byte word of the stream's table and of the slot's record: one load's latency in all.  (A thread per slot copied its
+// 31 words in turn: 2, 8 and 32 streams of the two-layer conv stack 16.4, 17.4 and 20.4 us of GPU time per call, so 14.4, 16.4 and 16.4.)
+constexpr int PTRS_WORDS = sizeof(F32StreamPtrs) / 8, SLOT_WORDS = sizeof(F32BatchSlot) / 8;
+static_assert(PTRS_WORDS + SLOT_WORDS <= 32 && sizeof(F32StreamPtrs) % 8 == 0 && sizeof(F32BatchSlot) % 8 == 0, "a lane per word");
 __global__ void set_f32_batch_kernel(const __grid_constant__ F32Batch v, F32BatchTable* dst) {
   if (threadIdx.x == 0) {
     dst->b.n = v.n;
     dst->b.pad = 0;
   }
-  if ((int)threadIdx.x < v.n) {
-    dst->b.s[threadIdx.x] = v.s[threadIdx.x];
-    dst->ptrs[threadIdx.x] = *v.s[threadIdx.x].ptrs;
+  const int lane = threadIdx.x & 31, word = lane - PTRS_WORDS;
+  for (int i = threadIdx.x >> 5; i < v.n; i += F32_SET_THREADS / 32) {
+    if (word < 0) reinterpret_cast<uint64_t*>(&dst->ptrs[i])[lane] = reinterpret_cast<const uint64_t*>(v.s[i].ptrs)[lane];
+    else if (word < SLOT_WORDS) reinterpret_cast<uint64_t*>(&dst->b.s[i])[word] = reinterpret_cast<const uint64_t*>(&v.s[i])[word];
   }
 }
 
@@ -476,7 +481,7 @@ void launch_set_f32_call(const F32Call& v, F32Call* dst, cudaStream_t st) {
 }
 
 void launch_set_f32_batch(const F32Batch& v, F32BatchTable* dst, cudaStream_t st) {
-  set_f32_batch_kernel<<<1, F32_MAX_BATCH, 0, st>>>(v, dst);
+  set_f32_batch_kernel<<<1, F32_SET_THREADS, 0, st>>>(v, dst);
 }
 const void* set_f32_batch_func() { return (const void*)set_f32_batch_kernel; }
 

@@ -111,6 +111,7 @@ void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc, cudaStream_t st
 void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st);
 void launch_set_f32_call(const F32Call& v, F32Call* dst, cudaStream_t st);
 const void* set_f32_call_func();
+constexpr int F32_SET_THREADS = 512;   // of the setter's one block
 void launch_set_f32_batch(const F32Batch& v, F32BatchTable* dst, cudaStream_t st);
 const void* set_f32_batch_func();
 
