@@ -1736,6 +1736,11 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int CL, 
   }
 }
 
+auto cluster_fn(const FlowModel* m, bool ring) {
+  return m->U != nullptr ? (ring ? flow_cluster_kernel<true, true> : flow_cluster_kernel<false, true>)
+                         : (ring ? flow_cluster_kernel<true, false> : flow_cluster_kernel<false, false>);
+}
+
 // Which models the one-kernel step serves: hidden 64 .. 512 in powers of two (the activation panel of two slots is 128 rows of
 // `hidden` bf16 in shared memory, a cluster has at most 16 CTAs of 32 columns).  The measurement options and the CTA-pair option ask
 // for the kernels of their own.
@@ -1748,7 +1753,7 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   cudaError_t e = cudaSuccess;
   cudaFuncAttributes fa{};
   int regs = 1 << 16;
-  for (auto fn : {flow_cluster_kernel<false>, flow_cluster_kernel<true>}) {
+  for (auto fn : {cluster_fn(m, false), cluster_fn(m, true)}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
     if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
@@ -1758,7 +1763,7 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, CL, 1, nullptr, false);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, flow_cluster_kernel<false>, &cfg);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, cluster_fn(m, false), &cfg);
   // (the kernel redistributes the registers that it was launched with: they have to cover the split)
   if (e == cudaSuccess && regs * CLU_THREADS < 128 * CLU_REGS_CTRL + CLU_EPI * CLU_REGS_EPI) n_cl = 0;
   if (e != cudaSuccess || n_cl < 1) {   // the kernels of their own serve the model
@@ -1817,7 +1822,6 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, boo
   p.X[0] = m->Xa; p.X[1] = m->Xb; p.Q = m->Q; p.O = m->O; p.Ain = m->AinP;
   p.xstate = m->xstate; p.ssq = m->ssq;
   p.inv_C = 1.0f / (float)m->C; p.eps = c.rms_eps; p.inv_n = 1.0f / c.n_steps; p.cfg_w = c.cfg_scale;
-  p.rounded = m->U != nullptr;
   p.P = m->P; p.Rk = m->Rk; p.kv_hs = m->kv_hs; p.dh_shift = m->dh_shift;
   p.scale_log2e = c.n_attn > 0 ? (float)(1.4426950408889634 / sqrt((double)c.head_dim)) : 0.f;
   p.err = m->d_err;
@@ -1825,7 +1829,7 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, boo
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, p.CL, ring ? m->max_clusters : (n + spc - 1) / spc, lc.st, lc.pdl);
   ProfScope ps(lc.prof, 7, lc.st);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ring ? flow_cluster_kernel<true> : flow_cluster_kernel<false>, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_fn(m, ring), p);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
   ++lc.launches;
 }

@@ -56,7 +56,6 @@ struct CluParams {
   float*          xstate;
   float*          ssq;                 // [slot][C / 16][SLOT_ROWS] partial sums of squares of the rows that feed an RMS norm
   float           inv_C, eps, inv_n, cfg_w;
-  int             rounded;             // DC_OPT_ROUNDED_NORM
   int             P, Rk, kv_hs, dh_shift;
   float           scale_log2e;
   int*            err;
@@ -134,7 +133,10 @@ static_assert(8 * (16 + 2 * CLU_RS + 2 * (int)CLU_KVS + 10) + 2 * (int)sizeof(Cl
 
 // RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].pad on, circularly.  (An instantiation of its
 // own: with the choice at run time every other call was 2 to 5 us slower.)
-template <bool RING>
+// ROUNDED (DC_OPT_ROUNDED_NORM): the normalised activations are rounded to bf16 before the GEMM that reads them.  (As a choice at run time its code, which
+// grew with the rewrite by all threads, cost the models without it 2 % and hidden 64, the shortest stages, 4 %: one stream 854 us against 837, fourteen
+// 975 against 956, hidden 64 260 against 249.)
+template <bool RING, bool ROUNDED>
 __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __grid_constant__ CluParams p) {
   constexpr int BN = CLU_BN, RS = CLU_RS;
   extern __shared__ __align__(1024) uint8_t clu_smem[];
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         if (skip || warp == 0) {
         } else {
           const int n_iss = issuers(nkb);
-          const bool norm = p.rounded && (st.kind == CLU_QKV || st.kind == CLU_OUT);
+          const bool norm = ROUNDED && (st.kind == CLU_QKV || st.kind == CLU_OUT);
           if (me < n_iss) {
             const int N = st.kind == CLU_CONV || st.kind == CLU_QKV ? 3 * BN : (st.kind == CLU_OUT ? 16 * nch_out : BN);
             const uint32_t idesc = ptx::umma_idesc_bf16(TILE_M, N, 0, 0);
@@ -562,7 +564,6 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       if (kv_row >= p.Rk) kv_row -= p.Rk;
       kv_row += p.P;
     }
-    const int T0 = p.slots[slot0].T, T1 = p.spc == 2 && slot0 + 1 < p.n_slots ? p.slots[slot0 + 1].T : 0;
     uint32_t xr[8];                               // the residual stream: this thread's row and columns, bf16 pairs
 #pragma unroll
     for (int i = 0; i < 8; ++i) xr[i] = 0u;
@@ -695,33 +696,35 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         }
         rs = rsqrtf(ss * p.inv_C + p.eps);
       }
-      if (norm && p.rounded && cg == 0) s_x[row_t] = rs;
+      if (ROUNDED && norm && cg == 0) s_x[row_t] = chunk_row ? rs : -1.f;   // (-1: a row that stays as it is)
       ptx::named_bar_sync(1, CLU_EPI);               // constants are in place; every carried row has been read
-      if (norm && p.rounded) {
-        // The normalised activations as rounded bf16 values: the panel is rewritten in place, block by block ahead of the issuer, 32 bytes of a row by every
-        // thread.  (64 bytes by the threads that own rows, half of them with one slot: 1,125 us for the whole decoder, so 1,104.)
+      if (ROUNDED && norm) {
+        // The normalised activations as rounded bf16 values: the panel is rewritten in place, block by block ahead of the issuer, 16 bytes of every 32nd
+        // row by a thread (a warp's accesses are whole rows: no bank conflicts), all of them requested before the first is used.
+        // (32 bytes of each slot's row in turn, with a wait in between: 14 streams 1,138 us against 1,112, one guided stream 1,105 against 1,083, one
+        // stream 959 against 956.)
+        float k[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) k[i] = i < 2 * p.spc ? s_x[(et >> 3) + 32 * i] : -1.f;
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
           clu_wait(&full_a[kb], ((kb < nkb_c ? n_gc : 0u) + (kb < nkb_in ? n_gi : 0u)) & 1u, s_fail, p.err, 0x114);
-#pragma unroll 1
-          for (int h = 0; h < p.spc; ++h) {
-            const int row = h * SLOT_ROWS + (et >> 2), fr = (et >> 2) - HALO;
-            if (fr < 0 || fr >= (h ? T1 : T0)) continue;
-            uint8_t* prow = panel + kb * kb_bytes + row * 128 + (et & 3) * 32;
-            const float k = s_x[row];
+          uint4* px = reinterpret_cast<uint4*>(panel + kb * kb_bytes) + et;
+          uint4 x[4];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              uint4* px = reinterpret_cast<uint4*>(prow + 16 * c);
-              const uint4 x = *px;
-              const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-              uint32_t o[4];
+          for (int i = 0; i < 4; ++i)
+            if (!(k[i] < 0.f)) x[i] = px[256 * i];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(w[i] << 16) * k, __uint_as_float(w[i] & 0xFFFF0000u) * k);
-                o[i] = *reinterpret_cast<const uint32_t*>(&b2);
-              }
-              *px = make_uint4(o[0], o[1], o[2], o[3]);
+          for (int i = 0; i < 4; ++i) {
+            if (k[i] < 0.f) continue;
+            const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+            uint32_t o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(w[j] << 16) * k[i], __uint_as_float(w[j] & 0xFFFF0000u) * k[i]);
+              o[j] = *reinterpret_cast<const uint32_t*>(&b2);
             }
+            px[256 * i] = make_uint4(o[0], o[1], o[2], o[3]);
           }
           ptx::fence_proxy_async_smem();
           ptx::mbar_arrive(&normed[kb]);

@@ -116,6 +116,17 @@ def test_flow_cluster_odd_full_batch(dc, hidden, n):
     assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
 
 
+# the rounded norm rewrites the panel of one slot or of two: full batches of an odd and an even number, guided passes; the bytes of single calls and of the
+# kernels of their own (the option keeps them apart)
+@pytest.mark.parametrize("n,kw", [(7, {}), (9, {}), (14, {}), (1, dict(cfg_scale=0.7)), (3, dict(cfg_scale=0.7))])
+def test_flow_cluster_rounded_norm(dc, n, kw):
+    gu = _util()
+    cfg = wl.tiny_flow(hidden=512, n_heads=8, head_dim=64, mel_dim=80, n_steps=2, seed=40, **kw)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM)
+    assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
+    assert np.array_equal(got, _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM | dc.OPT_CTA_PAIRS)[3])
+
+
 # one reduction block per conv product (hidden 64): 32- and 64-column tiles, whose epilogue exchanges more rows than one pipeline stage holds
 @pytest.mark.parametrize("n", [76, 150])
 def test_conv_exchange_of_one_reduction_block(dc, n):
