@@ -402,6 +402,11 @@ dc_status dc_stream_check_guards(dc_stream* stream, int* n_damaged);
  * everything they had allocated released. */
 dc_status dc_test_fail_allocation(int nth);
 
+/* For tests of the wavefront (the paper has no counterpart): how many clusters of the one-kernel chunk step the device keeps
+ * resident for this model (0: the kernels of their own serve it), and how many wavefront passes have run with one slot per
+ * cluster so far.  DC_ERR_CONFIG for a model without a flow decoder. */
+dc_status dc_test_wavefront_form(const dc_model* model, int* resident_clusters, uint64_t* one_slot_passes);
+
 /* Self-test of the bounded device-side wait that every pipeline barrier in the kernels uses (the
  * fail-closed discipline of paper Section 3.3, applied to the device): launches a one-CTA kernel
  * that waits, for at most max_polls polls (1 .. 1,000,000), on a barrier that nothing ever

@@ -22,7 +22,7 @@ EXPORTS = ["dc_weights_count", "dc_create", "dc_destroy", "dc_stream_open", "dc_
            "dc_stream_carry_info", "dc_get_counters", "dc_status_str", "dc_last_error",
            "dc_decode_batch_host", "dc_profile_begin", "dc_profile_end", "dc_conv_stack_noalloc",
            "dc_selftest_bounded_wait", "dc_stream_snapshot", "dc_stream_restore", "dc_snapshot_free",
-           "dc_decode_wavefront", "dc_decode_wavefront_batch", "dc_stream_check_guards", "dc_test_fail_allocation", "dc_measure_fp32_peak"]
+           "dc_decode_wavefront", "dc_decode_wavefront_batch", "dc_stream_check_guards", "dc_test_fail_allocation", "dc_test_wavefront_form", "dc_measure_fp32_peak"]
 
 
 class dc_config(C.Structure):
@@ -81,6 +81,7 @@ def load_library():
     lib.dc_selftest_bounded_wait.argtypes = [C.c_int]
     lib.dc_stream_check_guards.argtypes = [vp, cp(C.c_int)]
     lib.dc_test_fail_allocation.argtypes = [C.c_int]
+    lib.dc_test_wavefront_form.argtypes = [vp, cp(C.c_int), cp(C.c_uint64)]
     lib.dc_measure_fp32_peak.argtypes = [cp(C.c_double)]
     lib.dc_stream_carry_info.argtypes = [vp, cp(C.c_uint64), C.c_int, cp(C.c_int)]
     lib.dc_get_counters.argtypes = [vp, cp(C.c_uint64)]
@@ -195,6 +196,12 @@ class Model:
         pairs = bool(self.c_cfg.options & OPT_CTA_PAIRS)      # class 7 is one or the other
         names += ["gemm_pair", "flow_cluster"] if pairs else ["flow_cluster", "gemm_pair"]
         return ({k: ms[i] if i < 8 else 0.0 for i, k in enumerate(names)}, {k: n[i] if i < 8 else 0 for i, k in enumerate(names)})
+
+    def wavefront_form(self):
+        """dc_test_wavefront_form: (clusters resident, wavefront passes with one slot per cluster so far)."""
+        n, passes = C.c_int(0), C.c_uint64(0)
+        _check(self.lib.dc_test_wavefront_form(self.handle, C.byref(n), C.byref(passes)), "dc_test_wavefront_form")
+        return n.value, passes.value
 
     def destroy(self):
         if self.handle:

@@ -1469,6 +1469,14 @@ extern "C" dc_status dc_profile_end(dc_model* m, double ms[8], uint64_t launches
   return DC_OK;
 }
 
+extern "C" dc_status dc_test_wavefront_form(const dc_model* m, int* resident_clusters, uint64_t* one_slot_passes) {
+  if (!m || !resident_clusters || !one_slot_passes) return DC_ERR_ARG;
+  const dc_model* q = m->sub_flow ? m->sub_flow : m;
+  if (!q->flow) return DC_ERR_CONFIG;
+  dc::flow_wave_form(q->flow, resident_clusters, one_slot_passes);
+  return DC_OK;
+}
+
 extern "C" dc_status dc_get_counters(const dc_model* m, uint64_t counters[8]) {
   if (!m || !counters) return DC_ERR_ARG;
   if (m->flow || m->f32_err) {   // synchronous read of the device error word (asynchronous decode calls cannot see it)

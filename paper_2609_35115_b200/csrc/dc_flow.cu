@@ -71,7 +71,7 @@ struct SlotInfo {
   // is folded into its halo / kv pointers by the host; what remains per slot is the timestep-bias row and two flags.
   int          tau_off;   // float offset of the slot's Euler step inside the timestep-bias table (0 when the launch's own step applies)
   int          flags;     // SLOT_FIRST: the prep kernel loads x_0 and mu; SLOT_LAST: the output projection also writes `out`
-  int          pad;       // slot 0, wavefront: where the live slots begin (flow_cluster_kernel)
+  int          first_live;  // of slot 0, in a wavefront pass with one slot per cluster: the slot at which the live ones begin
 };
 constexpr int SLOT_FIRST = 1, SLOT_LAST = 2;
 
@@ -1333,6 +1333,7 @@ struct FlowModel {
   cudaStream_t cap_stream = nullptr;     // used only to capture graphs at create
   std::map<int, GraphEntry> graphs;      // batch size -> captured chunk step
   uint64_t graph_launches = 0;           // graph launches issued by decode calls
+  uint64_t ring_passes = 0;              // wavefront passes with one slot per cluster so far
   std::vector<SlotSet> sets;
   // one-kernel chunk steps (flow_cluster_kernel): resident clusters (0: not for this model) and the packed weights
   int       max_clusters = 0;
@@ -1636,6 +1637,7 @@ dc_status flow_state_reset(FlowModel* m, FlowState* s, cudaStream_t st) {
 
 const int* flow_error_word(const FlowModel* m) { return m->d_err; }
 uint64_t flow_graph_launches(const FlowModel* m) { return m->graph_launches; }
+void flow_wave_form(const FlowModel* m, int* clusters, uint64_t* passes) { *clusters = m->max_clusters; *passes = m->ring_passes; }
 
 dc_status flow_selftest_bounded_wait(int max_polls) {
   if (max_polls < 1 || max_polls > 1000000) return DC_ERR_ARG;
@@ -1838,7 +1840,7 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, boo
 // kernel(s) from `sets`).
 // tick = false: the n slots' chunks, all Euler steps.  tick = true: ONE pass of the network, every slot at the Euler step
 // that its slot-table entry encodes (wavefront decoding: the slots are consecutive chunks of one stream).
-// ring (a tick): only the slots from sets[0].s[0].pad on, as many as there are clusters, may be live.
+// ring (a tick): only the slots from sets[0].s[0].first_live on, as many as there are clusters, may be live.
 void enqueue_chunk(FlowModel* m, int n, const SlotSet* sets, int n_sets, LaunchCtx& lc, bool tick = false, bool ring = false) {
   const dc_config& c = m->cfg;
   const int C = m->C, mel = m->mel;
@@ -2103,7 +2105,7 @@ dc_status flow_decode(FlowModel* m, int n, FlowState* const* states, const float
       si.rng_id = s->rng_id;
       si.tau_off = 0;
       si.flags = SLOT_FIRST;
-      si.pad = 0;
+      si.first_live = 0;
       si.pass = pass;
       si.feats = feats[stream];
       si.out = pass == 0 ? outp[stream] : nullptr;
@@ -2214,7 +2216,10 @@ dc_status flow_decode_wave(FlowModel* m, int n_streams, FlowState* const* states
     // the live chunks, t - K + 1 .. t as far as they exist, are neighbours on the ring of slots
     const long long j0 = t < K ? 0 : t - K + 1, j1 = t < max_chunks ? t : max_chunks - 1;
     const bool ring = may_ring && j1 - j0 + 1 <= m->max_clusters;
-    if (ring) set.s[0].pad = (int)(j0 % K);
+    if (ring) {
+      set.s[0].first_live = (int)(j0 % K);
+      ++m->ring_passes;
+    }
     const auto it = its[ring ? 1 : 0];
     if (!profiling && it != m->graphs.end()) {
       GraphEntry& ge = it->second;

@@ -131,7 +131,7 @@ struct CluJob {     // what the heads of a slot attend
 
 static_assert(8 * (16 + 2 * CLU_RS + 2 * (int)CLU_KVS + 10) + 2 * (int)sizeof(CluJob) + 8 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
 
-// RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].pad on, circularly.  (An instantiation of its
+// RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].first_live on, circularly.  (An instantiation of its
 // own: with the choice at run time every other call was 2 to 5 us slower.)
 // ROUNDED (DC_OPT_ROUNDED_NORM): the normalised activations are rounded to bf16 before the GEMM that reads them.  (As a choice at run time its code, which
 // grew with the rewrite by all threads, cost the models without it 2 % and hidden 64, the shortest stages, 4 %: one stream 854 us against 837, fourteen
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   int slot_0 = (int)(blockIdx.x / (unsigned)p.CL) * p.spc;
   if (RING) {
     ptx::pdl_wait();
-    slot_0 += p.slots[0].pad;
+    slot_0 += p.slots[0].first_live;
     if (slot_0 >= p.n_slots) slot_0 -= p.n_slots;
   }
   const int slot0 = slot_0, m0 = slot0 * SLOT_ROWS;

@@ -84,6 +84,54 @@ def test_wavefront_few_live_slots(dc, n_chunks):
     _wave_vs_chunks(dc, wl.tiny_flow(hidden=512, n_heads=8, head_dim=64, n_steps=10, seed=36), 10 * n_chunks - 3)
 
 
+def _one_slot_passes(m, n_chunks):
+    """Passes of a call that may run with one slot per cluster: the live chunks have a cluster each, all n_steps of them would not."""
+    clusters, _ = m.wavefront_form()
+    K = m.cfg.n_steps
+    if not clusters < K <= 2 * clusters:
+        pytest.skip(f"{clusters} clusters resident, {K} chunks in flight: no pass has a choice")
+    return sum(min(t, n_chunks - 1) - max(t - K + 1, 0) + 1 <= clusters for t in range(n_chunks + K - 1))
+
+
+# ... as a graph, as direct launches and under the profiler, with the folded and the rounded norm: the bytes of chunk-by-chunk decoding, the passes counted
+@pytest.mark.parametrize("n_chunks", [3, 13])
+@pytest.mark.parametrize("rounded", [False, True])
+@pytest.mark.parametrize("form", ["graph", "direct", "profiled"])
+def test_wavefront_one_slot_per_cluster_runs(dc, n_chunks, rounded, form):
+    cfg = wl.tiny_flow(hidden=512, n_heads=8, head_dim=64, n_steps=10, seed=41)
+    n = cfg.f_chunk * n_chunks - 3
+    w = wl.make_workload(cfg.replace(n_chunks=n_chunks), boundaries=[_uniform(n, cfg.f_chunk)])
+    options = (dc.OPT_ROUNDED_NORM if rounded else 0) | (dc.OPT_NO_GRAPH if form == "direct" else 0)
+    m = dc.Model(cfg, w.weights, max_batch=cfg.n_steps, options=options)
+    want = _one_slot_passes(m, n_chunks)
+    ref = _gu().run_gpu_stream(m, w.streams[0].feats, _uniform(n, cfg.f_chunk))
+    st = m.open_stream()
+    if form == "profiled":
+        m.profile_begin(4096)
+    got = st.decode_wavefront(torch.from_numpy(w.streams[0].feats).cuda()).cpu().numpy()
+    if form == "profiled":
+        assert m.profile_end()[1]["flow_cluster"] == n_chunks + cfg.n_steps - 1
+    assert m.wavefront_form()[1] == want > 0 and m.counters()[4] == 0
+    st.close()
+    m.destroy()
+    assert np.array_equal(got, ref)
+
+
+def test_wavefront_one_slot_per_cluster_token2wav(dc):
+    cfg = wl.tiny_token2wav().replace(hidden=512, n_heads=8, head_dim=64, n_steps=10, seed=42)
+    n_chunks, n = 9, 87
+    w = wl.make_workload(cfg.replace(n_chunks=n_chunks), boundaries=[_uniform(n, cfg.f_chunk)])
+    m = dc.Model(cfg, w.weights, max_batch=cfg.n_steps, max_wave_frames=n)
+    want = _one_slot_passes(m, n_chunks)
+    ref = _gu().run_gpu_stream(m, w.streams[0].feats, _uniform(n, cfg.f_chunk))
+    st = m.open_stream()
+    got = st.decode_wavefront(torch.from_numpy(w.streams[0].feats).cuda()).cpu().numpy()
+    assert m.wavefront_form()[1] == want > 0 and m.counters()[4] == 0
+    st.close()
+    m.destroy()
+    assert np.array_equal(got, ref)
+
+
 def test_wavefront_then_streaming_continues_from_its_carries(dc):
     _wave_vs_chunks(dc, wl.tiny_flow(), 87, split=50)
 
