@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -217,6 +218,7 @@ class Stream:
         self.lib = model.lib
         self.handle = C.c_void_p()
         _check(self.lib.dc_stream_open(model.handle, C.byref(self.handle)), "dc_stream_open")
+        self.address = self.handle.value or 0    # the handle as a plain number: batch calls make an array of them
 
     def decode_chunk(self, feats, out=None, stream=None):
         """feats: CUDA float32 tensor [T, in_dim]; returns a CUDA float32 tensor."""
@@ -297,7 +299,7 @@ class Stream:
     def close(self):
         if self.handle:
             _check(self.lib.dc_stream_close(self.handle), "dc_stream_close")
-            self.handle = C.c_void_p()
+            self.handle, self.address = C.c_void_p(), 0
 
 
 def _ptr_array(items, n):
@@ -312,11 +314,7 @@ def _ptr_array(items, n):
 
 def _batch_args(model: Model, streams: Sequence[Stream], feats, outs):
     n = len(streams)
-    key = tuple(id(s) for s in streams)
-    cache = model.__dict__.setdefault("_handle_cache", {})
-    hs = cache.get(key)
-    if hs is None:
-        hs = cache[key] = (C.c_void_p * n)(*[s.handle for s in streams])
+    hs = (C.c_void_p * n).from_buffer(array("Q", [s.address for s in streams]))
     fp, T = _ptr_array(feats, n)
     op, _ = _ptr_array(outs, n)
     nf = (C.c_int * n)(*([T] * n if T is not None else [f.shape[0] for f in feats]))
