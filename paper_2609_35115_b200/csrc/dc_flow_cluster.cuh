@@ -700,23 +700,26 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       ptx::named_bar_sync(1, CLU_EPI);               // constants are in place; every carried row has been read
       if (ROUNDED && norm) {
         // The normalised activations as rounded bf16 values: the panel is rewritten in place, block by block ahead of the issuer, 16 bytes of every 32nd
-        // row by a thread (a warp's accesses are whole rows: no bank conflicts), all of them requested before the first is used.
-        // (32 bytes of each slot's row in turn, with a wait in between: 14 streams 1,138 us against 1,112, one guided stream 1,105 against 1,083, one
-        // stream 959 against 956.)
+        // row by a thread (a warp's accesses are whole rows: no bank conflicts), all of them requested before the first is used.  Rows outside the chunk are
+        // read and not written: a branch around every piece cost more than the pieces.
+        // (32 bytes of each slot's row in turn, with a wait in between: 14 streams 1,140 us, one guided stream 1,105, one stream 960; pieces in branches of
+        // their own 1,110, 1,079 and 956; so 1,086, 1,054 and 934.)
+        const bool two = p.spc == 2;
         float k[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) k[i] = i < 2 * p.spc ? s_x[(et >> 3) + 32 * i] : -1.f;
+        for (int i = 0; i < 4; ++i) k[i] = i < 2 || two ? s_x[(et >> 3) + 32 * i] : -1.f;
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
           clu_wait(&full_a[kb], ((kb < nkb_c ? n_gc : 0u) + (kb < nkb_in ? n_gi : 0u)) & 1u, s_fail, p.err, 0x114);
           uint4* px = reinterpret_cast<uint4*>(panel + kb * kb_bytes) + et;
           uint4 x[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (!(k[i] < 0.f)) x[i] = px[256 * i];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (k[i] < 0.f) continue;
+          x[0] = px[0];
+          x[1] = px[256];
+          if (two) {
+            x[2] = px[512];
+            x[3] = px[768];
+          }
+          auto put = [&](int i) {
             const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
             uint32_t o[4];
 #pragma unroll
@@ -724,7 +727,13 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(w[j] << 16) * k[i], __uint_as_float(w[j] & 0xFFFF0000u) * k[i]);
               o[j] = *reinterpret_cast<const uint32_t*>(&b2);
             }
-            px[256 * i] = make_uint4(o[0], o[1], o[2], o[3]);
+            if (!(k[i] < 0.f)) px[256 * i] = make_uint4(o[0], o[1], o[2], o[3]);
+          };
+          put(0);
+          put(1);
+          if (two) {
+            put(2);
+            put(3);
           }
           ptx::fence_proxy_async_smem();
           ptx::mbar_arrive(&normed[kb]);
