@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(HT, 2) head_istft_f32_kernel(const HeadIstftF3
     p.tail_out = p.tails + 12 * (c.parity ^ 1);
     p.pcm = c.out;
   }
+  if ((int)blockIdx.x * HF >= p.T) return;
   float* Ws = smem;                              // [3][C / 4] blocks of four channels
   float* g = smem + 3 * (p.C / 4) * HWP;         // [HFR][NFFT] windowed frame signals
   const int tid = threadIdx.x;
@@ -272,7 +273,6 @@ __global__ void __launch_bounds__(HT, 2) head_istft_f32_kernel(const HeadIstftF3
     d[0] = make_float2(w.x, w.y);
     d[1] = make_float2(w.z, w.w);
   }
-  if ((int)blockIdx.x * HF >= p.T) return;       // (here: the call record's latency passes under the weights')
   __syncthreads();
   // a CTA takes every gridDim.x-th run of HF frames: the weights are laid out once for all of them
 #pragma unroll 1

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
   auto record = [&](int slot) {
     TcSlot a{p.T_in, p.pos_in, p.in_direct, p.out_direct, p.in_ring, p.out_ring, p.save_ring, p.exc_rng_id};
     F32Call c{};
-    if (p.batch != nullptr) {   // (the count, the call and the rings are requested together: two L2 latencies less in front of the rows: 8 streams 220 -> 217.5 us, 32 streams 645 -> 632)
+    if (p.batch != nullptr) {   // (the count, the call and the rings are requested together: two L2 latencies less in front of the rows.  Through the slot's pointer to its table: 8 streams 219 us against 212, 32 streams 641 against 622)
       const F32StreamPtrs& ptrs = p.batch->ptrs[slot];
       c = p.batch->b.s[slot].call;
       a.in_ring = ptrs.ring[p.layer];
@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
   };
   // The set-up beside the first latency: the converting warps request their rows while another makes the barriers.  (Rows behind the block's barrier: one
-  // stream of the vocoder 101.6 us per chunk, so 97.5.  The first weights in front of it as well, which only hold the rows up: 99.6, 32 streams 630 against
-  // 624, and a layer of few frames slower than without either.)
+  // stream of the vocoder 99.7 us per chunk against 97.5, 8 streams 218 against 212, 32 streams 641 against 622.  The first weights in front of it as well,
+  // which only hold the rows up: 99.6, 32 streams 630 against 624, and a layer of few frames slower than without either.)
   if (warp < 8) {
     load(0);
   } else if (warp == 9 && lane == 0) {

@@ -1808,8 +1808,8 @@ int cluster_slots(const FlowModel* m, int n) {
 }
 
 // Wavefront: whether a tick of n slots, two per cluster, can run with one slot per cluster while few enough of them are live (the first and the
-// last ticks of an utterance: 10 chunks in flight and seven clusters, 14 of the 29 ticks of 20 chunks).  A cluster
-// with one slot takes 88 us a pass, with two 101: 20 s of audio 3,023 -> 2,933 us.
+// last ticks of an utterance: 10 chunks in flight and seven clusters, 14 of the 29 ticks of 20 chunks).  A pass with its launches takes 85 us with one live
+// slot and 88 with up to seven, with two slots per cluster 87 and 94 (a full one 107): 20 s of audio 2,974 -> 2,867 us.
 bool wave_ring(const FlowModel* m, int n) { return m->n_pass == 1 && cluster_slots(m, n) == 2; }
 
 void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, bool ring) {
