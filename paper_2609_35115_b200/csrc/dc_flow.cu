@@ -1738,9 +1738,10 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int CL, 
   }
 }
 
-auto cluster_fn(const FlowModel* m, bool ring) {
-  return m->U != nullptr ? (ring ? flow_cluster_kernel<true, true> : flow_cluster_kernel<false, true>)
-                         : (ring ? flow_cluster_kernel<true, false> : flow_cluster_kernel<false, false>);
+auto cluster_fn(const FlowModel* m, int spc, bool ring) {
+  if (spc == 2) return m->U != nullptr ? flow_cluster_kernel<false, true, 2> : flow_cluster_kernel<false, false, 2>;
+  return m->U != nullptr ? (ring ? flow_cluster_kernel<true, true, 1> : flow_cluster_kernel<false, true, 1>)
+                         : (ring ? flow_cluster_kernel<true, false, 1> : flow_cluster_kernel<false, false, 1>);
 }
 
 // Which models the one-kernel step serves: hidden 64 .. 512 in powers of two (the activation panel of two slots is 128 rows of
@@ -1755,7 +1756,7 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   cudaError_t e = cudaSuccess;
   cudaFuncAttributes fa{};
   int regs = 1 << 16;
-  for (auto fn : {cluster_fn(m, false), cluster_fn(m, true)}) {
+  for (auto fn : {cluster_fn(m, 1, false), cluster_fn(m, 1, true), cluster_fn(m, 2, false)}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
     if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
@@ -1765,7 +1766,7 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, CL, 1, nullptr, false);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, cluster_fn(m, false), &cfg);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n_cl, cluster_fn(m, 2, false), &cfg);
   // (the kernel redistributes the registers that it was launched with: they have to cover the split)
   if (e == cudaSuccess && regs * CLU_THREADS < 128 * CLU_REGS_CTRL + CLU_EPI * CLU_REGS_EPI) n_cl = 0;
   if (e != cudaSuccess || n_cl < 1) {   // the kernels of their own serve the model
@@ -1815,7 +1816,7 @@ bool wave_ring(const FlowModel* m, int n) { return m->n_pass == 1 && cluster_slo
 void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, bool ring) {
   const dc_config& c = m->cfg;
   CluParams p{};
-  p.slots = m->d_slots; p.n_slots = n; p.spc = spc; p.CL = m->C / CLU_BN;
+  p.slots = m->d_slots; p.n_slots = n; p.CL = m->C / CLU_BN;
   p.C = m->C; p.mel = m->mel; p.Kin = m->Kin; p.n_heads = c.n_heads;
   p.n_conv = c.n_conv; p.n_attn = c.n_attn; p.cpa = m->cpa; p.n_steps = tick ? 1 : c.n_steps; p.tick = tick;
   for (int l = 0; l < c.n_conv; ++l) p.dil[l] = c.dilations[l];
@@ -1831,7 +1832,7 @@ void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, boo
   cudaLaunchAttribute attr[2];
   cluster_config(cfg, attr, p.CL, ring ? m->max_clusters : (n + spc - 1) / spc, lc.st, lc.pdl);
   ProfScope ps(lc.prof, 7, lc.st);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_fn(m, ring), p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_fn(m, spc, ring), p);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
   ++lc.launches;
 }

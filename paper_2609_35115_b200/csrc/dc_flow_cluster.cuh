@@ -42,7 +42,7 @@ static_assert(CLU_SMEM <= 227 * 1024, "one CTA's shared memory");
 
 struct CluParams {
   const SlotInfo* slots;
-  int             n_slots, spc;        // slots of the launch; slots per cluster (1 or 2)
+  int             n_slots;             // slots of the launch
   int             CL;                  // CTAs of a cluster
   int             C, mel, Kin, n_heads;
   int             n_conv, n_attn, cpa, n_steps;
@@ -82,8 +82,17 @@ struct CluStage {
 // at the positions c ^ (row & 7) that they take in the swizzled shared-memory tile, so that a block of a slot is one untiled
 // bulk copy of 8 KB (no tensor map to fetch: 800 cycles less until the first tile is there).
 constexpr int CLU_SLOT_KB = SLOT_ROWS * KBLK;
+__device__ __forceinline__ int clu_row16(int rho, int c) { return rho * KBLK + ((((c >> 3) ^ (rho & 7)) & ~1) << 3); }   // the 32 bytes of columns c .. c + 15
+template <int NC>
+__device__ __forceinline__ void pack_row(const float* v, uint32_t* w) {
+#pragma unroll
+  for (int i = 0; i < NC / 2; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    w[i] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+}
 __device__ __forceinline__ void clu_store16(bf16* blk, int rho, int c, const uint4& a, const uint4& b) {   // columns c .. c + 15 of a block
-  bf16* d = blk + rho * KBLK + ((((c >> 3) ^ (rho & 7)) & ~1) << 3);
+  bf16* d = blk + clu_row16(rho, c);
   store16(d, (rho & 1) ? b : a, (rho & 1) ? a : b);
 }
 
@@ -136,15 +145,23 @@ static_assert(8 * (16 + 2 * CLU_RS + 2 * (int)CLU_KVS + 10) + 2 * (int)sizeof(Cl
 // ROUNDED (DC_OPT_ROUNDED_NORM): the normalised activations are rounded to bf16 before the GEMM that reads them.  (As a choice at run time its code, which
 // grew with the rewrite by all threads, cost the models without it 2 % and hidden 64, the shortest stages, 4 %: one stream 854 us against 837, fourteen
 // 975 against 956, hidden 64 260 against 249.)
-template <bool RING, bool ROUNDED>
+// SPC: slots per cluster.  With one slot the products have 64 rows, which tensor memory holds in sixteen lanes of each quarter: all eight epilogue warps
+// have rows and a thread has 8 columns of one (lane l of a quarter: row l & 15, columns 8 (l >> 4) ..), where products of 128 rows leave the warps of
+// the upper quarters idle and give the others 16 - and an epilogue is a chain of instructions, five cycles each.  The products get shorter, too: 48.5
+// cycles for 64 x 96 x 16 against 56.5 for 128 x 96 x 16.  One stream 862 -> 801 us per chunk, hidden 256 317 -> 298, seven streams 872 -> 813, prompt and
+// look-ahead 832 -> 762; the same bytes.
+template <bool RING, bool ROUNDED, int SPC>
 __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __grid_constant__ CluParams p) {
   constexpr int BN = CLU_BN, RS = CLU_RS;
+  constexpr bool ONE = SPC == 1;
+  constexpr int NC = ONE ? 8 : 16;         // columns of a thread's row piece
+  constexpr int ROWS = SLOT_ROWS * SPC;    // rows of a GEMM stage's products
   extern __shared__ __align__(1024) uint8_t clu_smem[];
   uint8_t* panel = clu_smem;
   uint8_t* wring = panel + CLU_PANEL;
   // attention's share of the panel.  With one slot per cluster the activations take only its first half, and the K/V ring has
   // the other half to itself: the carried key blocks of the next attention stage are fetched stages ahead.
-  const int kb_bytes = p.spc * 8192;
+  constexpr int kb_bytes = SPC * 8192;
   uint8_t* sQ = panel;
   uint8_t* sP = sQ + ATT_Q_BYTES;
   uint8_t* kvring = panel + CLU_PANEL - CLU_KVS * CLU_KV_BYTES;
@@ -172,7 +189,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (known to be the same for the whole warp)
   const int rank = (int)ptx::cluster_ctarank();
   const int n0 = rank * BN;
-  int slot_0 = (int)(blockIdx.x / (unsigned)p.CL) * p.spc;
+  int slot_0 = (int)(blockIdx.x / (unsigned)p.CL) * SPC;
   if (RING) {
     ptx::pdl_wait();
     slot_0 += p.slots[0].first_live;
@@ -191,7 +208,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     ptx::pdl_wait();
     bool any = false;
 #pragma unroll 1
-    for (int i = 0; i < p.spc; ++i) any |= slot0 + i < p.n_slots && p.slots[slot0 + i].T > 0;
+    for (int i = 0; i < SPC; ++i) any |= slot0 + i < p.n_slots && p.slots[slot0 + i].T > 0;
     if (!any) return;
   }
   if (tid == 0) {
@@ -229,7 +246,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   auto issuers = [&](int nkb) { return nkb >= 2 ? 2 : 1; };
-  const int n_jobs = p.spc * p.n_heads;            // (slot, head) pairs of the cluster; CTA r takes r, r + CL, ...
+  const int n_jobs = SPC * p.n_heads;            // (slot, head) pairs of the cluster; CTA r takes r, r + CL, ...
   const long long kv_plane = (long long)(p.P + p.Rk) * p.C;
   const int dh = 1 << p.dh_shift;
 
@@ -280,7 +297,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     uint32_t wt = 0;                               // weight tiles of earlier stages
     uint32_t it0 = 0, pre = 0, n_q = 0;            // K/V items of earlier jobs; items of the next job already requested; Q tiles so far
     uint32_t n_s0 = 0, n_s1 = 0;                   // key blocks of the two streams in earlier jobs
-    const bool two = p.spc == 2 && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
+    const bool two = !ONE && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
     auto request = [&](const bf16* src, int nkb) {
       ptx::fence_proxy_async_global();
       if (ptx::elect_one()) {
@@ -306,7 +323,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           const bool norm = ROUNDED && (st.kind == CLU_QKV || st.kind == CLU_OUT);
           if (me < n_iss) {
             const int N = st.kind == CLU_CONV || st.kind == CLU_QKV ? 3 * BN : (st.kind == CLU_OUT ? 16 * nch_out : BN);
-            const uint32_t idesc = ptx::umma_idesc_bf16(TILE_M, N, 0, 0);
+            const uint32_t idesc = ptx::umma_idesc_bf16(ROWS, N, 0, 0);
             const uint32_t d_acc = tmem_base + (uint32_t)me * CLU_ACC2;
             // The loop is a chain of instructions of one thread, and every address it has to make costs as much as a product: ring
             // slot, phases and descriptors advance incrementally on 32-bit values, and the next block's barriers are polled ahead
@@ -359,8 +376,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         }
         // one slot per cluster: the K/V ring is its own, the next attention's carried blocks are requested in the first conv block
         // (s_job is there from the second stage on); two: the panel is free once the projection's products are done
-        fetch = p.n_attn > 0 && (p.spc == 1 ? st.kind == CLU_CONV : st.kind == CLU_QKV);
-        if (fetch && warp == 0 && p.spc == 2 && !clu_wait(accum, n_g & 1u, s_fail, p.err, 0x106)) fetch = false;
+        fetch = p.n_attn > 0 && (ONE ? st.kind == CLU_CONV : st.kind == CLU_QKV);
+        if (fetch && warp == 0 && !ONE && !clu_wait(accum, n_g & 1u, s_fail, p.err, 0x106)) fetch = false;
         ++n_g;
         if (st.kind == CLU_IN) { ++n_gi; xi = 0; } else if (!skip) ++n_gc;
         if (!skip && (st.kind == CLU_QKV || st.kind == CLU_OUT)) ++n_norm;
@@ -532,11 +549,12 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     ptx::pdl_wait();
     const int et = tid - 128;
     const int q = warp & 3, cg = (warp - 4) >> 2;
-    const int row_t = q * 32 + lane, r = m0 + row_t;
+    const int row_t = ONE ? q * 16 + (lane & 15) : q * 32 + lane, r = m0 + row_t;
+    const int c0 = 16 * cg + (ONE ? 8 * (lane >> 4) : 0);   // the thread's first column of the CTA's 32
     const int slot = r / SLOT_ROWS, rho = r % SLOT_ROWS, f = rho - HALO;
-    const bool own = row_t < p.spc * SLOT_ROWS && slot < p.n_slots;
+    const bool own = slot < p.n_slots;
     const SlotInfo si = own ? p.slots[slot] : SlotInfo{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0};
-    if (et < p.spc) {                               // (read by the control warps behind the first cluster barrier)
+    if (et < SPC) {                               // (read by the control warps behind the first cluster barrier)
       const SlotInfo sj = slot0 + et < p.n_slots ? p.slots[slot0 + et] : SlotInfo{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0};
       CluJob jb;
       jb.kv = sj.kv;
@@ -547,13 +565,13 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     bf16* const s_halo = si.halo;
     bf16* const s_kv = si.kv;
     const bool is_out = si.pass == 0;
-    const int tau0 = p.slots[slot0].tau_off, tau1 = slot0 + 1 < p.n_slots ? p.slots[slot0 + 1].tau_off : 0;
+    const int tau0 = p.slots[slot0].tau_off, tau1 = !ONE && slot0 + 1 < p.n_slots ? p.slots[slot0 + 1].tau_off : 0;
     const bool in_range = si.T > 0;
     const bool halo_row = in_range && rho < HALO, chunk_row = in_range && f >= 0 && f < si.T;
     const int new_row = rho - si.Tc;                // carry row this thread's value moves to
     const bool moves = (halo_row || chunk_row) && new_row >= 0 && new_row < HALO;
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
-    const float* tau_s = s_tau + ((q >> 1) & 1) * 64;
+    const float* tau_s = s_tau + (ONE ? 0 : (q >> 1) & 1) * 64;
     const int aq = q & 1, ah = q >> 1;              // softmax: query quarter, key half
     const int tp = min(si.T, p.P - si.n_prompt0);   // the chunk's first tp frames complete the prompt
     int kv_row = 0;                                 // K/V plane row of this thread's frame
@@ -564,9 +582,9 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       if (kv_row >= p.Rk) kv_row -= p.Rk;
       kv_row += p.P;
     }
-    uint32_t xr[8];                               // the residual stream: this thread's row and columns, bf16 pairs
+    uint32_t xr[NC / 2];                          // the residual stream: this thread's row and columns, bf16 pairs
 #pragma unroll
-    for (int i = 0; i < 8; ++i) xr[i] = 0u;
+    for (int i = 0; i < NC / 2; ++i) xr[i] = 0u;
     int xi = 0;
     uint32_t n_g = 0, n_gc = 0, n_gi = 0;
     uint32_t n_blk = 0;                             // key blocks of this thread's stream so far
@@ -675,16 +693,16 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           const int nb = kind == CLU_QKV ? 3 * BN : BN;
           if (et < nb) s_bias[et] = p.fc[ob + (et / BN) * p.C + n0 + et % BN];
         }
-        if (kind == CLU_CONV && et < 2 * BN) {
+        if (kind == CLU_CONV && et < SPC * BN) {
           const int sl = et / BN, c = et % BN;
-          s_tau[sl * 64 + c] = sl < p.spc ? p.fc[p.o_tau + (st.s * p.n_conv + st.l) * p.C + (sl ? tau1 : tau0) + n0 + c] : 0.f;
+          s_tau[sl * 64 + c] = p.fc[p.o_tau + (st.s * p.n_conv + st.l) * p.C + (sl ? tau1 : tau0) + n0 + c];
         }
       }
-      uint4 hr[2];                                   // the carried row for the next conv block
+      uint4 hr[NC / 8];                              // the carried row for the next conv block
       if (carry != nullptr && halo_row) {
-        const uint4* src = reinterpret_cast<const uint4*>(carry + rho * p.C + n0 + 16 * cg);
-        hr[0] = src[0];
-        hr[1] = src[1];
+        const uint4* src = reinterpret_cast<const uint4*>(carry + rho * p.C + n0 + c0);
+#pragma unroll
+        for (int i = 0; i < NC / 8; ++i) hr[i] = src[i];
       }
       float rs = 1.f;
       if (norm) {
@@ -696,7 +714,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         }
         rs = rsqrtf(ss * p.inv_C + p.eps);
       }
-      if (ROUNDED && norm && cg == 0) s_x[row_t] = chunk_row ? rs : -1.f;   // (-1: a row that stays as it is)
+      if (ROUNDED && norm && c0 == 0) s_x[row_t] = chunk_row ? rs : -1.f;   // (-1: a row that stays as it is)
       ptx::named_bar_sync(1, CLU_EPI);               // constants are in place; every carried row has been read
       if (ROUNDED && norm) {
         // The normalised activations as rounded bf16 values: the panel is rewritten in place, block by block ahead of the issuer, 16 bytes of every 32nd
@@ -704,7 +722,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         // read and not written: a branch around every piece cost more than the pieces.
         // (32 bytes of each slot's row in turn, with a wait in between: 14 streams 1,140 us, one guided stream 1,105, one stream 960; pieces in branches of
         // their own 1,110, 1,079 and 956; so 1,086, 1,054 and 934.)
-        const bool two = p.spc == 2;
+        constexpr bool two = !ONE;
         float k[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) k[i] = i < 2 || two ? s_x[(et >> 3) + 32 * i] : -1.f;
@@ -745,36 +763,57 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       const bool ok = got && *reinterpret_cast<volatile int*>(s_fail) == 0;
       const bool is_chunk = chunk_row && ok, is_halo = halo_row && ok;
 
-      auto load_pair = [&](uint32_t col, float* v) {  // even blocks + odd blocks, always in this order
+      auto load_pair = [&](uint32_t col, float* v) {  // NC columns of the 16 from `col` on; even blocks + odd blocks, always in this order
         if (n_iss == 2) {
-          float t[16];
-          ptx::tmem_ld16x2(lanes + col, lanes + CLU_ACC2 + col, v, t);
+          uint32_t t[2 * NC];
+          ptx::tmem_ld_rows_issue<NC>(lanes + col, t);
+          ptx::tmem_ld_rows_issue<NC>(lanes + CLU_ACC2 + col, t + NC);
+          ptx::tmem_ld_wait<2 * NC>(t);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] += t[i];
+          for (int i = 0; i < NC; ++i) v[i] = __uint_as_float(t[i]) + __uint_as_float(t[NC + i]);
         } else {
-          ptx::tmem_ld16(lanes + col, v);
+          uint32_t t[NC];
+          ptx::tmem_ld_rows_issue<NC>(lanes + col, t);
+          ptx::tmem_ld_wait<NC>(t);
+#pragma unroll
+          for (int i = 0; i < NC; ++i) v[i] = __uint_as_float(t[i]);
         }
+      };
+      // A row's 16 columns as one 32-byte store, the halves swapped where the row's place in the swizzle is odd.  (ONE: the two lanes of a row bring
+      // them together in the lower one.)
+      auto put_row = [&](bool pred, bf16* d, bool swap, const uint32_t* w) {
+        uint4 a = make_uint4(w[0], w[1], w[2], w[3]), b;
+        if (ONE) {
+          b.x = __shfl_xor_sync(0xffffffffu, a.x, 16);
+          b.y = __shfl_xor_sync(0xffffffffu, a.y, 16);
+          b.z = __shfl_xor_sync(0xffffffffu, a.z, 16);
+          b.w = __shfl_xor_sync(0xffffffffu, a.w, 16);
+          pred = pred && lane < 16;
+        } else {
+          b = make_uint4(w[NC / 2 - 4], w[NC / 2 - 3], w[NC / 2 - 2], w[NC / 2 - 1]);
+        }
+        if (pred) store16(d, swap ? b : a, swap ? a : b);
       };
 
       if (kind == CLU_OUT) {
 #pragma unroll 1
         for (int k = cg; k < nch_out; k += 2) {
-          const int n = (rank + k * p.CL) * 16;
-          float acc[16];
+          const int n = (rank + k * p.CL) * 16 + c0 - 16 * cg;
+          float acc[NC];
           load_pair((uint32_t)(16 * k), acc);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) acc[i] = fmaf(acc[i], rs, s_bias[16 * k + i]);
-          if (p.cfg_w > 0.f) {
+          for (int i = 0; i < NC; ++i) acc[i] = fmaf(acc[i], rs, s_bias[16 * k + c0 - 16 * cg + i]);
+          if (!ONE && p.cfg_w > 0.f) {
             // guided step: rows 64.. are the unconditional pass; they hand their velocity over through shared memory
             float4* xv4 = reinterpret_cast<float4*>(panel) + k * 256;
             if (q >= 2) {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) xv4[j * 64 + (q - 2) * 32 + lane] = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+              for (int j = 0; j < NC / 4; ++j) xv4[j * 64 + (q - 2) * 32 + lane] = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
             }
             ptx::named_bar_sync(2 + cg, 128);
             if (q < 2) {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
+              for (int j = 0; j < NC / 4; ++j) {
                 const float4 u = xv4[j * 64 + q * 32 + lane];
                 acc[4 * j] = fmaf(1.f + p.cfg_w, acc[4 * j], -p.cfg_w * u.x);
                 acc[4 * j + 1] = fmaf(1.f + p.cfg_w, acc[4 * j + 1], -p.cfg_w * u.y);
@@ -783,32 +822,35 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               }
             }
           }
-          if (is_chunk && is_out) {
-            float* xs = p.xstate + (long long)r * p.mel + n;
-            float xv[16];
+          const bool advances = is_chunk && is_out;
+          uint32_t w[NC / 2];
 #pragma unroll
-            for (int i = 0; i < 16; i += 4) {
+          for (int i = 0; i < NC / 2; ++i) w[i] = 0u;
+          if (advances) {
+            float* xs = p.xstate + (long long)r * p.mel + n;
+            float xv[NC];
+#pragma unroll
+            for (int i = 0; i < NC; i += 4) {
               const float4 t = *reinterpret_cast<const float4*>(xs + i);
               xv[i] = t.x; xv[i + 1] = t.y; xv[i + 2] = t.z; xv[i + 3] = t.w;
             }
 #pragma unroll
-            for (int i = 0; i < 16; ++i) xv[i] = xv[i] + acc[i] * p.inv_n;
+            for (int i = 0; i < NC; ++i) xv[i] = xv[i] + acc[i] * p.inv_n;
 #pragma unroll
-            for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(xs + i) = make_float4(xv[i], xv[i + 1], xv[i + 2], xv[i + 3]);
-            uint4 a, b;
-            pack16_bf16(xv, a, b);
-            bf16* blk = p.Ain + ((long long)slot * nkb_in + (n >> 6)) * CLU_SLOT_KB;
-            clu_store16(blk, rho, n & 63, a, b);
-            if (p.cfg_w > 0.f) clu_store16(blk + (long long)nkb_in * CLU_SLOT_KB, rho, n & 63, a, b);   // the unconditional pass starts from the same x
+            for (int i = 0; i < NC; i += 4) *reinterpret_cast<float4*>(xs + i) = make_float4(xv[i], xv[i + 1], xv[i + 2], xv[i + 3]);
+            pack_row<NC>(xv, w);
             const SlotInfo& so = p.slots[slot];      // (read again: only here, once per chunk)
             if ((p.tick ? (so.flags & SLOT_LAST) != 0 : st.s == p.n_steps - 1) && f < so.Tc) {
               float* o = so.out + (long long)f * p.mel + n;
 #pragma unroll
-              for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(xv[i], xv[i + 1], xv[i + 2], xv[i + 3]);
+              for (int i = 0; i < NC; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(xv[i], xv[i + 1], xv[i + 2], xv[i + 3]);
             }
           }
+          bf16* d = p.Ain + ((long long)slot * nkb_in + (n >> 6)) * CLU_SLOT_KB + clu_row16(rho, n & 63);
+          put_row(advances, d, rho & 1, w);
+          if (!ONE && p.cfg_w > 0.f) put_row(advances, d + (long long)nkb_in * CLU_SLOT_KB, rho & 1, w);   // the unconditional pass starts from the same x
         }
-        if (p.cfg_w > 0.f) ptx::fence_proxy_async_smem();   // (the exchange above: the next stage's bulk copies overwrite it)
+        if (!ONE && p.cfg_w > 0.f) ptx::fence_proxy_async_smem();   // (the exchange above: the next stage's bulk copies overwrite it)
         ptx::tc_fence_before();
         clu_arrive_release(warp);
       } else if (kind == CLU_QKV) {
@@ -819,68 +861,82 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         bf16* kvp = s_kv + kv_off + (long long)hh * p.kv_hs + ((long long)kv_row << p.dh_shift) + ((((wi >> 3) ^ perm) & ~1) << 3);
 #pragma unroll
         for (int which = 0; which < 3; ++which) {
-          float acc[16];
+          float acc[NC];
           load_pair((uint32_t)(which * BN + 16 * cg), acc);
-          const float4* bias4 = reinterpret_cast<const float4*>(s_bias + which * BN + 16 * cg);
+          const float4* bias4 = reinterpret_cast<const float4*>(s_bias + which * BN + c0);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int i = 0; i < NC / 4; ++i) {
             const float4 b4 = bias4[i];
             acc[4 * i] = fmaf(acc[4 * i], rs, b4.x);
             acc[4 * i + 1] = fmaf(acc[4 * i + 1], rs, b4.y);
             acc[4 * i + 2] = fmaf(acc[4 * i + 2], rs, b4.z);
             acc[4 * i + 3] = fmaf(acc[4 * i + 3], rs, b4.w);
           }
-          uint4 a, b;
-          pack16_bf16(acc, a, b);
-          if (is_chunk) {
-            if (which == 0) clu_store16(p.Q + ((long long)slot * nkb_c + (col >> 6)) * CLU_SLOT_KB, rho, col & 63, a, b);
-            else store16(kvp + (which - 1) * kv_plane, (perm & 1) ? b : a, (perm & 1) ? a : b);
-          }
+          uint32_t w[NC / 2];
+          pack_row<NC>(acc, w);
+          if (which == 0) put_row(is_chunk, p.Q + ((long long)slot * nkb_c + (col >> 6)) * CLU_SLOT_KB + clu_row16(rho, col & 63), rho & 1, w);
+          else put_row(is_chunk, kvp + (which - 1) * kv_plane, perm & 1, w);
         }
         ptx::tc_fence_before();
         clu_arrive_release(warp);
       } else {
         // ---- a new residual row: input projection, conv block, attention output projection ----
         bf16* out = p.X[kind == CLU_IN ? 0 : xi ^ 1];
-        uint4 va, vb;
-        const int c0 = 16 * cg, n = n0 + c0;
-        float2 acc[8];
+        const int n = n0 + c0;
+        float2 acc[NC / 2];
         if (kind == CLU_CONV) {
           // y[r] = Z_0[r - 2 d] + Z_1[r - d] + Z_2[r]: rows change lanes through shared memory (the panel is idle by now)
-          float2 z[8], z2[8];
+          float2 z[NC / 2], z2[NC / 2];
+          const uint32_t col = lanes + (uint32_t)(16 * cg);
+          auto sum = [&](const uint32_t* t, float2* v) {
+#pragma unroll
+            for (int i = 0; i < NC / 2; ++i) v[i] = add2(pair2(t[2 * i], t[2 * i + 1]), pair2(t[NC + 2 * i], t[NC + 2 * i + 1]));
+          };
           if (n_iss == 2) {
-            uint32_t ra[32], rb[32];             // even blocks + odd blocks, two taps behind one wait
-            ptx::tmem_ld16x2_issue(lanes + (uint32_t)c0, lanes + CLU_ACC2 + (uint32_t)c0, ra);
-            ptx::tmem_ld16x2_issue(lanes + (uint32_t)(BN + c0), lanes + CLU_ACC2 + (uint32_t)(BN + c0), rb);
-            ptx::tmem_ld_wait32(ra);
-            ptx::tmem_ld_wait32(rb);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              acc[i] = add2(pair2(ra[2 * i], ra[2 * i + 1]), pair2(ra[16 + 2 * i], ra[17 + 2 * i]));
-              z[i] = add2(pair2(rb[2 * i], rb[2 * i + 1]), pair2(rb[16 + 2 * i], rb[17 + 2 * i]));
+            uint32_t ra[2 * NC], rb[2 * NC];     // even blocks + odd blocks, two taps behind one wait (ONE: all three)
+            ptx::tmem_ld_rows_issue<NC>(col, ra);
+            ptx::tmem_ld_rows_issue<NC>(col + CLU_ACC2, ra + NC);
+            ptx::tmem_ld_rows_issue<NC>(col + BN, rb);
+            ptx::tmem_ld_rows_issue<NC>(col + CLU_ACC2 + BN, rb + NC);
+            if (ONE) {
+              uint32_t rc[2 * NC];
+              ptx::tmem_ld_rows_issue<NC>(col + 2 * BN, rc);
+              ptx::tmem_ld_rows_issue<NC>(col + CLU_ACC2 + 2 * BN, rc + NC);
+              ptx::tmem_ld_wait<2 * NC>(ra);
+              ptx::tmem_ld_wait<2 * NC>(rb);
+              ptx::tmem_ld_wait<2 * NC>(rc);
+              sum(ra, acc);
+              sum(rb, z);
+              sum(rc, z2);
+            } else {
+              ptx::tmem_ld_wait<2 * NC>(ra);
+              ptx::tmem_ld_wait<2 * NC>(rb);
+              sum(ra, acc);
+              sum(rb, z);
+              ptx::tmem_ld_rows_issue<NC>(col + 2 * BN, ra);
+              ptx::tmem_ld_rows_issue<NC>(col + CLU_ACC2 + 2 * BN, ra + NC);
+              ptx::tmem_ld_wait<2 * NC>(ra);
+              sum(ra, z2);
             }
-            ptx::tmem_ld16x2_issue(lanes + (uint32_t)(2 * BN + c0), lanes + CLU_ACC2 + (uint32_t)(2 * BN + c0), ra);
-            ptx::tmem_ld_wait32(ra);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) z2[i] = add2(pair2(ra[2 * i], ra[2 * i + 1]), pair2(ra[16 + 2 * i], ra[17 + 2 * i]));
           } else {
-            ptx::tmem_ld16(lanes + (uint32_t)c0, reinterpret_cast<float*>(acc));
-            ptx::tmem_ld16(lanes + (uint32_t)(BN + c0), reinterpret_cast<float*>(z));
-            ptx::tmem_ld16(lanes + (uint32_t)(2 * BN + c0), reinterpret_cast<float*>(z2));
+            load_pair((uint32_t)(16 * cg), reinterpret_cast<float*>(acc));
+            load_pair((uint32_t)(BN + 16 * cg), reinterpret_cast<float*>(z));
+            load_pair((uint32_t)(2 * BN + 16 * cg), reinterpret_cast<float*>(z2));
           }
-          float4* xz = reinterpret_cast<float4*>(panel) + cg * (2 * 4 * TILE_M);
+          // [column group][tap][four columns][row]
+          float4* xz = reinterpret_cast<float4*>(panel) + (c0 / NC) * (2 * (NC / 4) * ROWS);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            xz[j * TILE_M + row_t] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
-            xz[(4 + j) * TILE_M + row_t] = make_float4(z[2 * j].x, z[2 * j].y, z[2 * j + 1].x, z[2 * j + 1].y);
+          for (int j = 0; j < NC / 4; ++j) {
+            xz[j * ROWS + row_t] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
+            xz[(NC / 4 + j) * ROWS + row_t] = make_float4(z[2 * j].x, z[2 * j].y, z[2 * j + 1].x, z[2 * j + 1].y);
           }
           ptx::named_bar_sync(2 + cg, 128);
           const int d = p.dil[st.l], r0 = max(row_t - 2 * d, 0), r1 = max(row_t - d, 0);
           const float4* bias4 = reinterpret_cast<const float4*>(s_bias + c0);
           const float4* tau4 = reinterpret_cast<const float4*>(tau_s + c0);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 a0 = xz[j * TILE_M + r0], a1 = xz[(4 + j) * TILE_M + r1], b4 = bias4[j], t4 = tau4[j];
+          for (int j = 0; j < NC / 4; ++j) {
+            const float4 a0 = xz[j * ROWS + r0], a1 = xz[(NC / 4 + j) * ROWS + r1], b4 = bias4[j], t4 = tau4[j];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const float2 q0 = h ? make_float2(a0.z, a0.w) : make_float2(a0.x, a0.y), q1 = h ? make_float2(a1.z, a1.w) : make_float2(a1.x, a1.y);
@@ -891,36 +947,43 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             }
           }
         } else {
-          load_pair((uint32_t)c0, reinterpret_cast<float*>(acc));
+          load_pair((uint32_t)(16 * cg), reinterpret_cast<float*>(acc));
           const float4* bias4 = reinterpret_cast<const float4*>(s_bias + c0);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < NC / 4; ++j) {
             const float4 b4 = bias4[j];
             acc[2 * j] = add2(acc[2 * j], make_float2(b4.x, b4.y));
             acc[2 * j + 1] = add2(acc[2 * j + 1], make_float2(b4.z, b4.w));
           }
           if (kind == CLU_OPROJ) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] = add2(acc[i], unpack2(xr[i]));
+            for (int i = 0; i < NC / 2; ++i) acc[i] = add2(acc[i], unpack2(xr[i]));
           }
         }
-        pack16_bf16(reinterpret_cast<const float*>(acc), va, vb);
-        xr[0] = va.x; xr[1] = va.y; xr[2] = va.z; xr[3] = va.w;
-        xr[4] = vb.x; xr[5] = vb.y; xr[6] = vb.z; xr[7] = vb.w;
-        if (rho < HALO) { va = hr[0]; vb = hr[1]; }   // a left-context row hands the carried row on
-        if (is_chunk || (is_halo && next_conv))
-          clu_store16(out + ((long long)slot * nkb_c + (n >> 6)) * CLU_SLOT_KB, rho, n & 63, va, vb);
-        if (feeds_norm && in_range) {              // sum of squares of the 16 stored values, fixed order
-          float ss = 0.f;
-          if (is_chunk) {
+        pack_row<NC>(reinterpret_cast<const float*>(acc), xr);
+        uint32_t w[NC / 2];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float lo = __uint_as_float(xr[i] << 16), hi = __uint_as_float(xr[i] & 0xFFFF0000u);
-              ss = fmaf(lo, lo, ss);
-              ss = fmaf(hi, hi, ss);
+        for (int i = 0; i < NC / 2; ++i) w[i] = xr[i];
+        if (rho < HALO) {                            // a left-context row hands the carried row on
+#pragma unroll
+          for (int i = 0; i < NC / 8; ++i) { w[4 * i] = hr[i].x; w[4 * i + 1] = hr[i].y; w[4 * i + 2] = hr[i].z; w[4 * i + 3] = hr[i].w; }
+        }
+        put_row(is_chunk || (is_halo && next_conv), out + ((long long)slot * nkb_c + (n >> 6)) * CLU_SLOT_KB + clu_row16(rho, n & 63), rho & 1, w);
+        if (feeds_norm && in_range) {              // sum of squares of the row's 16 stored values, fixed order (ONE: the upper lane goes on from the lower one's)
+          float ss = 0.f;
+#pragma unroll
+          for (int part16 = 0; part16 < 16 / NC; ++part16) {
+            if (part16) ss = __shfl_xor_sync(0xffffffffu, ss, 16);
+            if (is_chunk) {
+#pragma unroll
+              for (int i = 0; i < NC / 2; ++i) {
+                const float lo = __uint_as_float(xr[i] << 16), hi = __uint_as_float(xr[i] & 0xFFFF0000u);
+                ss = fmaf(lo, lo, ss);
+                ss = fmaf(hi, hi, ss);
+              }
             }
           }
-          p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
+          if (!ONE || lane >= 16) p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
         }
         // The next stage's bulk copies overwrite the exchange of the taps: the writers' fence.  (One stream 909 -> 919 us; right behind the writes
         // 925, behind the barrier of clu_arrive_release 918.)
@@ -928,7 +991,11 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         ptx::tc_fence_before();
         clu_arrive_release(warp);
         // shift the carry by the committed frames: nobody in this launch reads it again
-        if (carry != nullptr && moves && ok) store16(carry + new_row * p.C + n0 + 16 * cg, va, vb);
+        if (carry != nullptr && moves && ok) {
+          bf16* d = carry + new_row * p.C + n0 + c0;
+          if (ONE) *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+          else store16(d, make_uint4(w[0], w[1], w[2], w[3]), make_uint4(w[NC / 2 - 4], w[NC / 2 - 3], w[NC / 2 - 2], w[NC / 2 - 1]));
+        }
       }
       ++n_g;
       if (kind == CLU_IN) { ++n_gi; xi = 0; } else if (!skip) ++n_gc;

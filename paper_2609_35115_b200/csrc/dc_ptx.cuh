@@ -266,6 +266,33 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t* r) {
                :
                : "memory");
 }
+// A warp's share of an accumulator, in two halves like the pair above.  N = 16: 16 columns of each of the 32 lanes (a thread has a whole row piece);
+// N = 8: 16 columns of lanes 0..15 of the quarter, where the rows of a 64-row product are: thread l has lane l & 15, columns 8 (l >> 4) ... + 7.
+template <int N>
+__device__ __forceinline__ void tmem_ld_rows_issue(uint32_t taddr, uint32_t* r) {
+  static_assert(N == 8 || N == 16, "columns per thread");
+  if (N == 16)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[N - 8]), "=r"(r[N - 7]),
+                   "=r"(r[N - 6]), "=r"(r[N - 5]), "=r"(r[N - 4]), "=r"(r[N - 3]), "=r"(r[N - 2]), "=r"(r[N - 1])
+                 : "r"(taddr)
+                 : "memory");
+  else
+    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 8;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
+  if (N > 8)     // (no use of these may be scheduled ahead of the wait either)
+#pragma unroll
+    for (int i = 8; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"

@@ -116,6 +116,28 @@ def test_flow_cluster_odd_full_batch(dc, hidden, n):
     assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
 
 
+# one slot per cluster has products of 64 rows, sixteen of a quarter of tensor memory each (eight of them left context): chunks that end at, in front of and
+# behind a quarter's last row; the bytes of two slots per cluster
+@pytest.mark.parametrize("hidden,rounded", [(64, False), (128, True), (512, False)])
+def test_flow_cluster_one_slot_rows(dc, hidden, rounded):
+    cfg = wl.tiny_flow(hidden=hidden, n_heads=hidden // 32, head_dim=32, mel_dim=80, n_steps=2, f_chunk=56, seed=41)
+    w = wl.make_workload(cfg)
+    n = {64: 80, 128: 40, 512: 9}[hidden]      # more than the resident clusters
+    m = dc.Model(cfg, w.weights, max_batch=n, options=dc.OPT_ROUNDED_NORM if rounded else 0)
+    one, many = m.open_stream(), [m.open_stream() for _ in range(n)]
+    gen = torch.Generator(device="cuda").manual_seed(hidden)
+    for T in (56, 1, 7, 8, 9, 23, 24, 25, 39, 40, 41, 55):
+        x = torch.randn(T, cfg.in_dim, generator=gen, device="cuda")
+        outs = [torch.zeros(T, cfg.mel_dim, device="cuda") for _ in range(n)]
+        dc.decode_batch(m, many, [x] * n, outs)
+        got = one.decode_chunk(x)
+        assert got.isfinite().all() and all(torch.equal(got, o) for o in outs), T
+    assert m.counters()[4] == 0
+    for s in [one] + many:
+        s.close()
+    m.destroy()
+
+
 # the rounded norm rewrites the panel of one slot or of two: full batches of an odd and an even number, guided passes; the bytes of single calls and of the
 # kernels of their own (the option keeps them apart)
 @pytest.mark.parametrize("n,kw", [(7, {}), (9, {}), (14, {}), (1, dict(cfg_scale=0.7)), (3, dict(cfg_scale=0.7))])
