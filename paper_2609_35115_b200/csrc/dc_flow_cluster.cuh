@@ -105,6 +105,34 @@ __device__ __forceinline__ void clu_arrive_release(int warp) {
   ptx::cluster_arrive_relaxed();
 }
 
+// One slot per cluster: a stage's rows leave the CTA as one piece, [64 rows][32 channels] (clu_at32), which one thread copies out of shared memory in bulk.
+// The copy has completed - its bytes are in L2, where the other CTAs' bulk copies read them - 480 cycles after the staging; the fence behind stores of the
+// threads took 1,040.  (16 CTAs hand 4 KB each to one another: the first operand block is there after 1,150 cycles instead of 1,790.  With a fence behind the
+// copy, which has nothing left to wait for, 2,010.)  One stream 801 -> 748 us per chunk, hidden 256 298 -> 275, seven streams 813 -> 755, prompt and
+// look-ahead 762 -> 704.
+__device__ __forceinline__ int clu_at32(int rho, int c) { return rho * 32 + (((c >> 3) ^ ((rho >> 1) & 3)) << 3); }   // element of channel c of a block: the 64-byte swizzle
+struct CluPiece {
+  void*       dst;
+  const void* src;
+  uint32_t    bytes;
+};
+template <int N>
+__device__ __forceinline__ void clu_arrive_bulk(int warp, const CluPiece (&piece)[N]) {
+  ptx::fence_proxy_async_smem();
+  ptx::named_bar_sync(1, CLU_EPI);
+  if (warp == 4) {
+    if (ptx::elect_one()) {
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (piece[i].bytes > 0) ptx::bulk_store(piece[i].dst, piece[i].src, piece[i].bytes);
+      ptx::bulk_store_wait();
+    }
+    __syncwarp();
+    ptx::fence_proxy_async_global();
+  }
+  ptx::cluster_arrive_relaxed();
+}
+
 // Bounded wait of a whole warp that gives up at once after any wait of this CTA has given up: the step then runs through without
 // waiting, the copying warps request nothing more, and the CTA pauses before it exits.  The vote keeps the warp together: lanes that leave a polling loop one by one go on as separate groups, and everything
 // up to the next warp-wide instruction is then executed several times (an issue loop took 600 cycles per block instead of 260).
@@ -329,6 +357,10 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             // slot, phases and descriptors advance incrementally on 32-bit values, and the next block's barriers are polled ahead
             // of this block's products (a wait that finds its barrier complete costs as much as a product, too).
             constexpr uint32_t DESC_HI = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61)) >> 32);
+            // one slot: blocks of 32 channels in the 64-byte swizzle (the input projection's operand comes from another kernel)
+            const bool b32 = ONE && st.kind != CLU_IN;
+            const uint32_t a_hi = b32 ? (uint32_t)((((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61)) >> 32) : DESC_HI;
+            const uint32_t a_k2 = b32 ? 4096u >> 4 : 4u;
             const uint32_t w_lo = ((ptx::smem_u32(wring) & 0x3FFFF) >> 4) | (1u << 16), a_step = (uint32_t)(n_iss * (kb_bytes >> 4));
             const uint32_t bar_w0 = ptx::smem_u32(full_w), bar_e0 = ptx::smem_u32(empty_w), a_bstep = 8u * (uint32_t)n_iss;
             uint32_t slot = (wt + (uint32_t)me) % RS, pw = ((wt + (uint32_t)me) / RS) & 1u, acc = 0;
@@ -347,7 +379,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
                 clu_wait(&full_w[slot], pw, s_fail, p.err, 0x103);
                 clu_wait(&(norm ? normed : full_a)[kb], pa & 1u, s_fail, p.err, 0x105);
               }
-              const uint64_t da = ((uint64_t)DESC_HI << 32) | a_lo, db = ((uint64_t)DESC_HI << 32) | (w_lo + slot * (uint32_t)(CLU_SLOT >> 4));
+              const uint64_t da = ((uint64_t)a_hi << 32) | a_lo, da2 = ((uint64_t)a_hi << 32) | (a_lo + a_k2), db = ((uint64_t)DESC_HI << 32) | (w_lo + slot * (uint32_t)(CLU_SLOT >> 4));
               const uint32_t empty = bar_e0 + 8u * slot;
               slot += (uint32_t)n_iss;
               if (slot >= RS) { slot -= RS; pw ^= 1u; }
@@ -360,8 +392,9 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               }
               if (ptx::elect_one()) {
                 ptx::umma_bf16(d_acc, da, db, idesc, acc);
-#pragma unroll
-                for (int k = 1; k < 4; ++k) ptx::umma_bf16(d_acc, da + 2 * k, db + 2 * k, idesc, 1);
+                ptx::umma_bf16(d_acc, da + 2, db + 2, idesc, 1);
+                ptx::umma_bf16(d_acc, da2, db + 4, idesc, 1);
+                ptx::umma_bf16(d_acc, da2 + 2, db + 6, idesc, 1);
                 ptx::umma_commit_s(empty);
               }
               __syncwarp();
@@ -654,14 +687,29 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
                 for (int i = 0; i < 16; ++i) o16[i] = nkb > 1 ? fmaf(q16[i], c1, o16[i] * c0) : o16[i] * c0;
                 uint4 a, bq;
                 pack16_bf16(o16, a, bq);
-                clu_store16(oblk, row + HALO, ((head << p.dh_shift) & 63) + c, a, bq);
+                if (ONE) {                         // (the queries' tile is idle by now)
+                  bf16* d = reinterpret_cast<bf16*>(sQ) + (c >> 5) * (SLOT_ROWS * 32);
+                  *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, c & 31)) = a;
+                  *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, (c & 31) + 8)) = bq;
+                } else {
+                  clu_store16(oblk, row + HALO, ((head << p.dh_shift) & 63) + c, a, bq);
+                }
               }
             }
           }
           ptx::tc_fence_before();
-          ptx::named_bar_sync(1, CLU_EPI);         // (the next job overwrites the exchange and the accumulators)
+          if (!ONE) ptx::named_bar_sync(1, CLU_EPI);   // (the next job overwrites the exchange and the accumulators; with one slot a CTA has at most one)
         }
-        clu_arrive_release(warp);
+        if (ONE) {
+          // the rows of the head's one or two blocks of 32 channels
+          const uint32_t bytes = rank < n_jobs && s_job[0].T > 0 ? (SLOT_ROWS - HALO) * 64u : 0u;
+          bf16* dst = p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + ((rank << p.dh_shift) >> 5) * (SLOT_ROWS * 32) + HALO * 32;
+          const uint8_t* src = sQ + HALO * 64;
+          const CluPiece piece[2] = {{dst, src, bytes}, {dst + SLOT_ROWS * 32, src + SLOT_ROWS * 64, p.dh_shift == 6 ? bytes : 0u}};
+          clu_arrive_bulk(warp, piece);
+        } else {
+          clu_arrive_release(warp);
+        }
         ptx::cluster_wait();
         continue;
       }
@@ -725,7 +773,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         constexpr bool two = !ONE;
         float k[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) k[i] = i < 2 || two ? s_x[(et >> 3) + 32 * i] : -1.f;
+        for (int i = 0; i < 4; ++i) k[i] = ONE ? s_x[et >> 2] : s_x[(et >> 3) + 32 * i];   // (one slot: 16 bytes of its row in either block of 32 channels)
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
           clu_wait(&full_a[kb], ((kb < nkb_c ? n_gc : 0u) + (kb < nkb_in ? n_gi : 0u)) & 1u, s_fail, p.err, 0x114);
@@ -968,7 +1016,11 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
 #pragma unroll
           for (int i = 0; i < NC / 8; ++i) { w[4 * i] = hr[i].x; w[4 * i + 1] = hr[i].y; w[4 * i + 2] = hr[i].z; w[4 * i + 3] = hr[i].w; }
         }
-        put_row(is_chunk || (is_halo && next_conv), out + ((long long)slot * nkb_c + (n >> 6)) * CLU_SLOT_KB + clu_row16(rho, n & 63), rho & 1, w);
+        // One slot: staged in the panel behind the taps' exchange.  (Rows that are neither the chunk's nor its left context go along; no row reads one behind it.)
+        bf16* const rows_out = reinterpret_cast<bf16*>(panel + 16384);
+        float* const ssq_out = reinterpret_cast<float*>(panel + 16384 + SLOT_ROWS * 64);
+        if (ONE) *reinterpret_cast<uint4*>(rows_out + clu_at32(rho, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
+        else put_row(is_chunk || (is_halo && next_conv), out + ((long long)slot * nkb_c + (n >> 6)) * CLU_SLOT_KB + clu_row16(rho, n & 63), rho & 1, w);
         if (feeds_norm && in_range) {              // sum of squares of the row's 16 stored values, fixed order (ONE: the upper lane goes on from the lower one's)
           float ss = 0.f;
 #pragma unroll
@@ -983,13 +1035,20 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               }
             }
           }
-          if (!ONE || lane >= 16) p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
+          if (!ONE) p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
+          else if (lane >= 16) ssq_out[cg * SLOT_ROWS + rho] = ss;
         }
         // The next stage's bulk copies overwrite the exchange of the taps: the writers' fence.  (One stream 909 -> 919 us; right behind the writes
         // 925, behind the barrier of clu_arrive_release 918.)
-        if (kind == CLU_CONV) ptx::fence_proxy_async_smem();
+        if (!ONE && kind == CLU_CONV) ptx::fence_proxy_async_smem();
         ptx::tc_fence_before();
-        clu_arrive_release(warp);
+        if (ONE) {
+          const CluPiece piece[2] = {{out + (long long)slot0 * nkb_c * CLU_SLOT_KB + rank * (SLOT_ROWS * 32), rows_out, SLOT_ROWS * 64u},
+                                     {p.ssq + ((long long)slot0 * (p.C >> 4) + 2 * rank) * SLOT_ROWS, ssq_out, feeds_norm && in_range ? 2u * SLOT_ROWS * 4u : 0u}};
+          clu_arrive_bulk(warp, piece);
+        } else {
+          clu_arrive_release(warp);
+        }
         // shift the carry by the committed frames: nobody in this launch reads it again
         if (carry != nullptr && moves && ok) {
           bf16* d = carry + new_row * p.C + n0 + c0;
