@@ -469,9 +469,10 @@ void launch_tile(const TapConvF32& p, int KS, cudaStream_t st) {
   launch_ex(tapconv_f32_kernel<BM, BN>, grid, dim3(KS * TT::NTG), (size_t)KS * TT::GROUP_FLOATS * sizeof(float), st, false, p, KS);
 }
 
-constexpr size_t tc_smem_bytes(int BN, int n_a, int n_b) { return (size_t)n_a * TC_PANEL + (size_t)n_b * 3 * BN * 128 + TC_BARS; }
-static_assert(tc_smem_bytes(64, 1, 2) <= 113 * 1024 && tc_smem_bytes(32, 1, TC_MAX_B) <= 113 * 1024, "a single panel: two CTAs per SM");
-static_assert(tc_smem_bytes(64, 2, 3) <= 227 * 1024 && tc_smem_bytes(32, 2, TC_MAX_B) <= 227 * 1024, "several panels: one");
+constexpr size_t tc_smem_bytes(int M, int BN, int n_a, int n_b) { return (size_t)n_a * tc_panel(M) + (size_t)n_b * 3 * BN * 128 + TC_BARS; }
+static_assert(tc_smem_bytes(128, 64, 1, 2) <= 113 * 1024 && tc_smem_bytes(128, 32, 1, TC_MAX_B) <= 113 * 1024, "a single panel: two CTAs per SM");
+static_assert(tc_smem_bytes(64, 32, 2, TC_MAX_B) <= 113 * 1024 && tc_smem_bytes(64, 64, 2, 2) <= 113 * 1024, "tiles of 64 frames: two");
+static_assert(tc_smem_bytes(128, 64, 2, 3) <= 227 * 1024 && tc_smem_bytes(128, 32, 2, TC_MAX_B) <= 227 * 1024, "several panels: one");
 }  // namespace
 
 const void* set_f32_call_func() { return (const void*)set_f32_call_kernel; }
@@ -501,8 +502,9 @@ void pack_tapconv(const TapConvF32& p, uint8_t* dst, TapConvTc* tc) {
 
 cudaError_t prepare_tapconv() {
   cudaError_t e = cudaSuccess;
-  for (auto fn : {tapconv_tc_kernel<32, false, false>, tapconv_tc_kernel<64, false, false>, tapconv_tc_kernel<32, true, false>, tapconv_tc_kernel<64, true, false>,
-                  tapconv_tc_kernel<64, true, true>})
+  for (auto fn : {tapconv_tc_kernel<32, false, false, 128>, tapconv_tc_kernel<64, false, false, 128>, tapconv_tc_kernel<32, true, false, 128>,
+                  tapconv_tc_kernel<64, true, false, 128>, tapconv_tc_kernel<64, true, true, 128>, tapconv_tc_kernel<32, false, false, 64>,
+                  tapconv_tc_kernel<32, true, false, 64>, tapconv_tc_kernel<64, true, false, 64>, tapconv_tc_kernel<64, false, false, 64>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(head_istft_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
@@ -510,23 +512,34 @@ cudaError_t prepare_tapconv() {
 
 void launch_tapconv_tc(const TapConvF32& p, const TapConvTc& tc_in, cudaStream_t st, int T_grid, int n_batch) {
   TapConvTc tc = tc_in;
-  const int planes = p.n_phase * (n_batch > 0 ? n_batch : 1), m_tiles = (T_grid + TC_M - 1) / TC_M;
+  const int planes = p.n_phase * (n_batch > 0 ? n_batch : 1);
   const bool drain = tc.n_blocks * (tc.per_tap ? p.n_taps : 1) > 1;   // (of the layer, not of the batch: it decides the order of the sum)
-  // 64 columns per CTA once that fills the GPU (a reduction step costs 209 cycles of the tensor pipe at 64 columns, 134 at 32), else 32
+  auto tiles = [&](int frames, int cols) { return (long long)((T_grid + frames - 1) / frames) * (tc.C_pad / cols) * planes; };
+  // 64 frames per tile while every tile has an SM of its own: a layer is then the latency of one tile, whose rows, products (114 cycles of the tensor pipe per
+  // reduction step, 178 for 128 frames, both at 32 columns) and epilogue are shorter.  One stream of the vocoder 98.3 -> 85.1 us per chunk, of one frame 95.0 ->
+  // 81.0.  With 64 columns where 32 give too many tiles of either height: 2, 3 and 5 streams 117.9 -> 102.9, 138.3 -> 135.3 and 175.1 -> 156.9 us.  Beyond one
+  // wave 128 frames cost less (64 x 64 tiles take 194 cycles, 128 x 64 ones 226): two of the small tiles per SM at every size took 188 us instead of 180 at
+  // 6 streams and 680 instead of 621 at 32.
+  const bool small32 = tiles(64, 32) <= tc.n_sm;
+  const bool small64 = !small32 && tc.C_pad % 64 == 0 && tiles(64, 64) <= tc.n_sm && tiles(128, 32) > tc.n_sm;
+  const bool small = small32 || small64;
+  // Tiles of 128 frames: 64 columns per CTA once that fills the GPU (a reduction step costs 226 cycles of the tensor pipe at 64 columns, 178 at 32), else 32
   // over twice the SMs.  A column's sum is the same either way.  A single panel leaves room for two CTAs per SM, which overlap one's
   // conversion and epilogue with the other's products; several panels overlap inside the CTA.
-  const bool wide0 = tc.C_pad % 64 == 0 && (long long)m_tiles * (tc.C_pad / 64) * planes >= tc.n_sm;
+  const bool wide0 = !small && tc.C_pad % 64 == 0 && tiles(128, 64) >= tc.n_sm;
   // two slots per tile where that saves a wave: several panels (one CTA per SM), chunks of at most half a tile
-  const bool pack = drain && n_batch > 1 && T_grid <= TC_PACK && tc.C_pad % 64 == 0 && (long long)(tc.C_pad / (wide0 ? 64 : 32)) * planes > tc.n_sm;
-  const bool wide = wide0 || pack;
+  const bool pack = !small && drain && n_batch > 1 && T_grid <= TC_PACK && tc.C_pad % 64 == 0 && (long long)(tc.C_pad / (wide0 ? 64 : 32)) * planes > tc.n_sm;
+  const bool wide = small64 || wide0 || pack;
+  const int bn = wide ? 64 : 32, M = small ? 64 : 128;
   tc.n_a = drain ? 2 : 1;
-  tc.n_b = wide ? (drain ? 3 : 2) : TC_MAX_B;
-  const int bn = wide ? 64 : 32;
-  const dim3 grid(m_tiles, tc.C_pad / bn, pack ? p.n_phase * ((n_batch + 1) / 2) : planes);
-  auto fn = pack ? tapconv_tc_kernel<64, true, true>
-                 : wide ? (drain ? tapconv_tc_kernel<64, true, false> : tapconv_tc_kernel<64, false, false>)
-                        : (drain ? tapconv_tc_kernel<32, true, false> : tapconv_tc_kernel<32, false, false>);
-  launch_ex(fn, grid, dim3(TC_THREADS), tc_smem_bytes(bn, tc.n_a, tc.n_b), st, false, p, tc);
+  tc.n_b = wide ? (small ? (drain ? 2 : 3) : (drain ? 3 : 2)) : TC_MAX_B;
+  const dim3 grid(pack ? 1 : (T_grid + M - 1) / M, tc.C_pad / bn, pack ? p.n_phase * ((n_batch + 1) / 2) : planes);
+  auto fn = small32 ? (drain ? tapconv_tc_kernel<32, true, false, 64> : tapconv_tc_kernel<32, false, false, 64>)
+            : small64 ? (drain ? tapconv_tc_kernel<64, true, false, 64> : tapconv_tc_kernel<64, false, false, 64>)
+            : pack ? tapconv_tc_kernel<64, true, true, 128>
+            : wide ? (drain ? tapconv_tc_kernel<64, true, false, 128> : tapconv_tc_kernel<64, false, false, 128>)
+                   : (drain ? tapconv_tc_kernel<32, true, false, 128> : tapconv_tc_kernel<32, false, false, 128>);
+  launch_ex(fn, grid, dim3(TC_THREADS), tc_smem_bytes(M, bn, tc.n_a, tc.n_b), st, false, p, tc);
 }
 
 void launch_tapconv_f32(const TapConvF32& p, cudaStream_t st) {

@@ -9,19 +9,16 @@
 // block of the vocoder (192,000 frames) went from 213 us, 22 TFLOP/s, on FFMA tiles (4 x 4 per thread, bound by shared-memory
 // operand latency) to what the conversion and the fp32 rows' traffic cost.
 //
-// One CTA: 128 frames x BN channels of one phase.  Ten warps: 0..7 read the fp32 input rows (ring, or the caller's chunk), split
+// One CTA: M (128 or 64) frames x BN channels of one phase.  Ten warps: 0..7 read the fp32 input rows (ring, or the caller's chunk), split
 // them and write the three bf16 planes as swizzled operand tiles, and later run the epilogue; 8 issues the products; 9 streams the
 // weights, split and packed as swizzled tiles at create.
-// A panel holds 64 channels of the 128 frames and of the up to 8 in front of them: a tap is a row offset of the operand
+// A panel holds 64 channels of the tile's frames and of the up to 8 in front of them: a tap is a row offset of the operand
 // descriptor, so a row is read and split once for all its taps.  (Dilations above 4 fill the panel once per tap.)
 // Per 64 channels and tap: 4 reduction steps of ah x bh, ah x [bm bl], am x [bh bm], al x bh.
 
-constexpr int TC_M = 128, TC_H = 8;               // frames per tile; left-context rows in front of them
-constexpr int TC_ROWS = TC_M + TC_H;
-constexpr int TC_PLANE = TC_ROWS * 128;            // bytes of one bf16 plane of a panel (64 channels)
-constexpr int TC_PANEL = 3 * TC_PLANE;
+constexpr int TC_H = 8;                           // left-context rows in front of a tile's frames
+constexpr int tc_panel(int M) { return 3 * (M + TC_H) * 128; }   // bytes of a panel (64 channels): three bf16 planes
 constexpr int TC_THREADS = 320, TC_CONV = 256;     // converting / epilogue threads
-constexpr int TC_ITEMS = (TC_ROWS * 8 + TC_CONV - 1) / TC_CONV;   // 8-channel pieces per thread and panel
 constexpr int TC_MAX_A = 2, TC_MAX_B = 4;
 constexpr int TC_BARS = 1024;                      // barriers (and alignment slack: the base is declared 1024-byte aligned)
 
@@ -66,8 +63,8 @@ __device__ __noinline__ float4 excite4(float4 v, long long t, int n, int rng_id,
 // The tensor cores truncate when they add to an accumulator, which over a long reduction is a bias (7.6e-5 of RMS at the vocoder's end
 // with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel, tap) - four additions - has an accumulator of
 // its own, which the epilogue threads add up in registers, rounded to nearest.  DRAIN (inputs of more than one panel): two sets of three, a
-// panel's taps each, one set added up while the next panel is multiplied.  One panel: one set; at 64 columns, where two CTAs share the SM's
-// tensor memory, two accumulators that the taps take in turn (TURN).  (A single one for the three taps, twelve additions: ten layers of 64 channels
+// panel's taps each, one set added up while the next panel is multiplied.  One panel: one set.  At 64 columns, where two CTAs share the SM's
+// tensor memory: two accumulators that the taps take in turn (TURN).  (A single one for the three taps, twelve additions: ten layers of 64 channels
 // end at 4.3e-6 of their norm, against 2.0e-6 for sums of the FP32 pipe.)
 //
 // PACK (batches; chunks of up to TC_PACK frames at the layer's rate): a tile holds two slots, the second one's rows 64 behind the
@@ -85,8 +82,11 @@ struct TcSlot {       // one stream's share of a launch
   int          rng_id;
 };
 
-template <int BN, bool DRAIN, bool PACK>
-__global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(const __grid_constant__ TapConvF32 p, const __grid_constant__ TapConvTc tc) {
+//
+// M: frames of a tile.  64 where tiles of 128 would leave SMs without one (launch_tapconv_tc has the rule and the figures).  A 64-row product lies in sixteen
+// TMEM lanes of each quarter, so that the epilogue's eight warps all have rows: a thread holds 8 columns of each 16.
+template <int BN, bool DRAIN, bool PACK, int M>
+__global__ void __launch_bounds__(TC_THREADS, DRAIN && M == 128 ? 1 : 2) tapconv_tc_kernel(const __grid_constant__ TapConvF32 p, const __grid_constant__ TapConvTc tc) {
   // per-call values: from the device-side call record of the stream or of the slot (captured graphs), or by value
   const int plane = (p.batch != nullptr ? blockIdx.z / p.n_phase : 0), phase = blockIdx.z - plane * p.n_phase;
   auto record = [&](int slot) {
@@ -114,16 +114,19 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     }
     return a;
   };
+  static_assert(M == 128 || (M == 64 && !PACK), "frames of a tile");
+  constexpr int ROWS = M + TC_H, PLANE = ROWS * 128, PANEL = 3 * PLANE;
+  constexpr int ITEMS = (ROWS * 8 + TC_CONV - 1) / TC_CONV;   // 8-channel pieces per thread and panel
   const TcSlot s0 = record(PACK ? 2 * plane : plane);
   TcSlot s1 = s0;
   if (PACK) s1 = record(2 * plane + 1);
-  const int m0 = PACK ? 0 : blockIdx.x * TC_M, n0 = blockIdx.y * BN;
+  const int m0 = PACK ? 0 : blockIdx.x * M, n0 = blockIdx.y * BN;
   if (PACK ? s0.T <= 0 : m0 >= s0.T) return;   // the grid is sized for the longest chunk
 
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   constexpr int B_TILE = 3 * BN * 128;
   uint8_t* sA = tc_smem;
-  uint8_t* sB = sA + tc.n_a * TC_PANEL;
+  uint8_t* sB = sA + tc.n_a * PANEL;
   uint64_t* full_a = reinterpret_cast<uint64_t*>(sB + tc.n_b * B_TILE);
   uint64_t* empty_a = full_a + TC_MAX_A;
   uint64_t* full_b = empty_a + TC_MAX_A;
@@ -148,18 +151,18 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     return (direct ? a.in_direct : a.in_ring) + (size_t)r * (uint32_t)C_in;
   };
   const int c8 = (tid & 7) * 8, row0 = tid >> 3;          // this thread's pieces: channels c8 .. c8 + 7 of rows row0, row0 + 32, ...
-  float4 xa[TC_ITEMS], xb[TC_ITEMS];
+  float4 xa[ITEMS], xb[ITEMS];
   auto load = [&](int u) {
     const int blk = tc.per_tap ? u / p.n_taps : u, tap = tc.per_tap ? u - blk * p.n_taps : 0;
     const int c = blk * 64 + c8;
     const int i0 = m0 - TC_H - (tc.per_tap ? p.shift[tap] : 0);
 #pragma unroll
-    for (int i = 0; i < TC_ITEMS; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
       const int row = row0 + 32 * i, seg = PACK && i >= TC_SEG / 32 ? TC_SEG : 0;   // (with PACK the tile starts at frame 0)
       const TcSlot& a = seg ? s1 : s0;
       xa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       xb[i] = xa[i];
-      if (row < TC_ROWS && m0 + row - seg - TC_H < a.T && c < C_in && (!PACK || a.T > 0)) {   // (an odd batch's last tile has no second slot)
+      if (row < ROWS && m0 + row - seg - TC_H < a.T && c < C_in && (!PACK || a.T > 0)) {   // (an odd batch's last tile has no second slot)
         const float* src = in_row(a, i0 + row - seg) + c;
         xa[i] = *reinterpret_cast<const float4*>(src);
         if (c + 4 < C_in) xb[i] = *reinterpret_cast<const float4*>(src + 4);
@@ -192,8 +195,8 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
   }
   __syncwarp();
   // columns: leading term (see above), then the 2^-8 and the 2^-16 terms
-  constexpr bool TURN = !DRAIN && BN > 32;
-  constexpr uint32_t S_COL = DRAIN ? 6 * BN : (TURN ? 2 * BN : 3 * BN);
+  constexpr bool TURN = BN > 32 && (!DRAIN || M == 64);
+  constexpr uint32_t S_COL = TURN ? 2 * BN : (DRAIN ? 6 * BN : 3 * BN);
   constexpr uint32_t TMEM_COLS = S_COL + 2 * BN <= 128 ? 128 : (S_COL + 2 * BN <= 256 ? 256 : 512);
   if (warp == 8) ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   ptx::tc_fence_before();
@@ -227,29 +230,30 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     // One (panel, tap) after the other; the loop is a chain of one thread's instructions, so addresses advance on 32-bit values and
     // the next barriers are polled ahead of this step's products (with a wait in front of every step it took 1,700 cycles, the
     // products alone 900).
-    const uint32_t id2 = ptx::umma_idesc_bf16(TC_M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(TC_M, BN, 0, 0);
+    const uint32_t id2 = ptx::umma_idesc_bf16(M, 2 * BN, 0, 0), id1 = ptx::umma_idesc_bf16(M, BN, 0, 0);
     constexpr uint32_t DESC_HI = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61)) >> 32);
     const uint32_t a_lo = ((ptx::smem_u32(sA) & 0x3FFFF) >> 4) | (1u << 16), b_lo = ((ptx::smem_u32(sB) & 0x3FFFF) >> 4) | (1u << 16);
     const uint32_t bar_b = ptx::smem_u32(full_b), bar_eb = ptx::smem_u32(empty_b), bar_a = ptx::smem_u32(full_a), bar_ea = ptx::smem_u32(empty_a);
     const uint32_t off0 = (uint32_t)(tc.per_tap ? TC_H : TC_H - p.shift[0]) * 8u, off1 = (uint32_t)(TC_H - p.shift[1]) * 8u, off2 = (uint32_t)(TC_H - p.shift[2]) * 8u;
     uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
     bool ok = true, ready_a = ptx::mbar_try_wait_s(bar_a, 0), ready_b = ptx::mbar_try_wait_s(bar_b, 0);
-    int u = 0, j = 0;
+    int u = 0, j = 0, v = 0;                       // panel, its tap, taps so far
 #pragma unroll 1
     while (u < n_units && ok) {
       if (j == 0) {
-        if (DRAIN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
+        if (DRAIN && !TURN && u >= 2) ok = tc_wait(&drained[u & 1], ((u >> 1) - 1) & 1, s_fail, tc.err, 0x206);
         if (!__all_sync(0xffffffffu, ready_a)) ok &= tc_wait(&full_a[sa], pa, s_fail, tc.err, 0x202);
       }
-      if (TURN && j >= 2) ok = tc_wait(&drained[j & 1], ((j >> 1) - 1) & 1, s_fail, tc.err, 0x206);
+      if (TURN && v >= 2) ok &= tc_wait(&drained[v & 1], ((v >> 1) - 1) & 1, s_fail, tc.err, 0x206);
       if (!__all_sync(0xffffffffu, ready_b)) ok &= tc_wait(&full_b[sb], pb, s_fail, tc.err, 0x203);
       if (!ok) break;
       ptx::tc_fence_after();
       const bool last = j + 1 == taps_u, first = u == 0 && j == 0;
-      const uint32_t al0 = a_lo + sa * (uint32_t)(TC_PANEL >> 4) + (j == 0 ? off0 : (j == 1 ? off1 : off2)), bl0 = b_lo + sb * (uint32_t)(B_TILE >> 4);
-      const uint64_t ah = ((uint64_t)DESC_HI << 32) | al0, am = ah + (TC_PLANE >> 4), al = am + (TC_PLANE >> 4), b = ((uint64_t)DESC_HI << 32) | bl0;
-      const uint32_t eb = bar_eb + 8u * sb, ea = bar_ea + 8u * sa, d_main = tmem_base + (uint32_t)(TURN ? j & 1 : (u & 1) * 3 + j) * BN;
-      uint64_t* done = &accum[(TURN ? j : u) & 1];
+      const uint32_t al0 = a_lo + sa * (uint32_t)(PANEL >> 4) + (j == 0 ? off0 : (j == 1 ? off1 : off2)), bl0 = b_lo + sb * (uint32_t)(B_TILE >> 4);
+      const uint64_t ah = ((uint64_t)DESC_HI << 32) | al0, am = ah + (PLANE >> 4), al = am + (PLANE >> 4), b = ((uint64_t)DESC_HI << 32) | bl0;
+      const uint32_t eb = bar_eb + 8u * sb, ea = bar_ea + 8u * sa, d_main = tmem_base + (uint32_t)(TURN ? v & 1 : (u & 1) * 3 + j) * BN;
+      uint64_t* done = &accum[(TURN ? v : u) & 1];
+      ++v;
       if (++sb == (uint32_t)tc.n_b) { sb = 0; pb ^= 1u; }
       if (last) {
         if (++sa == (uint32_t)tc.n_a) { sa = 0; pa ^= 1u; }
@@ -278,33 +282,45 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     // ---------------- input rows -> bf16 planes ----------------
     const int q = warp & 3, col0 = (warp >> 2) * (BN / 2);   // epilogue: TMEM lane quarter; columns col0 .. col0 + BN / 2 - 1
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
-    constexpr int NC = BN / 32;
-    float sum[NC][16];
+    constexpr int NC = BN / 32, W = M / 8;                   // a thread's columns: W of each 16
+    float sum[NC][W], panel_sum[TURN ? NC : 1][W];
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
-      for (int i = 0; i < 16; ++i) sum[c][i] = 0.f;
-    auto drain = [&](int u) {                                // panel u (with TURN: tap u)
+      for (int i = 0; i < W; ++i) sum[c][i] = 0.f;
+    auto drain = [&](int u, int j) {                         // panel u (with TURN: the u-th tap, tap j of its panel)
       const bool got = tc_wait(&accum[u & 1], (u >> 1) & 1, s_fail, tc.err, 0x205);
       ptx::tc_fence_after();
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const uint32_t col = lanes + (uint32_t)((u & 1) * (TURN ? 1 : 3) * BN + col0 + 16 * c);
-        float z[16], y[16];
+        uint32_t z[2 * W];
+        float s[W];
+        ptx::tmem_ld_rows_issue<W>(col, z);
         if (TURN || taps_u == 1) {
-          ptx::tmem_ld16(col, z);
+          ptx::tmem_ld_wait<W>(z);
+#pragma unroll
+          for (int i = 0; i < W; ++i) s[i] = __uint_as_float(z[i]);
         } else {
-          ptx::tmem_ld16x2(col, col + BN, z, y);
+          ptx::tmem_ld_rows_issue<W>(col + BN, z + W);
+          ptx::tmem_ld_wait<2 * W>(z);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) z[i] += y[i];
+          for (int i = 0; i < W; ++i) s[i] = __uint_as_float(z[i]) + __uint_as_float(z[W + i]);
           if (taps_u == 3) {
-            ptx::tmem_ld16(col + 2 * BN, y);
+            ptx::tmem_ld_rows_issue<W>(col + 2 * BN, z);
+            ptx::tmem_ld_wait<W>(z);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) z[i] += y[i];
+            for (int i = 0; i < W; ++i) s[i] += __uint_as_float(z[i]);
           }
         }
+        if (TURN) {                                          // (a panel's taps are added up first, as below)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum[c][i] += z[i];
+          for (int i = 0; i < W; ++i) panel_sum[c][i] = s[i] = j == 0 ? s[i] : panel_sum[c][i] + s[i];
+        }
+        if (!TURN || j + 1 == taps_u) {
+#pragma unroll
+          for (int i = 0; i < W; ++i) sum[c][i] += s[i];
+        }
       }
       ptx::tc_fence_before();
       ptx::mbar_arrive(&drained[u & 1]);
@@ -316,11 +332,11 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
 #pragma unroll 1
     for (int u = 0; u < n_units; ++u) {
       if (u >= tc.n_a) ok &= tc_wait(&empty_a[sa], ph, s_fail, tc.err, 0x204);
-      uint8_t* dst = sA + sa * TC_PANEL;
+      uint8_t* dst = sA + sa * PANEL;
 #pragma unroll
-      for (int i = 0; i < TC_ITEMS; ++i) {
+      for (int i = 0; i < ITEMS; ++i) {
         const int row = row0 + 32 * i;
-        if (row < TC_ROWS) {
+        if (row < ROWS) {
           uint4 h, m, l;
           split2(xa[i].x, xa[i].y, h.x, m.x, l.x);
           split2(xa[i].z, xa[i].w, h.y, m.y, l.y);
@@ -328,15 +344,22 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
           split2(xb[i].z, xb[i].w, h.w, m.w, l.w);
           uint8_t* d = dst + row * 128 + (((tid & 7) ^ (row & 7)) << 4);
           *reinterpret_cast<uint4*>(d) = h;
-          *reinterpret_cast<uint4*>(d + TC_PLANE) = m;
-          *reinterpret_cast<uint4*>(d + 2 * TC_PLANE) = l;
+          *reinterpret_cast<uint4*>(d + PLANE) = m;
+          *reinterpret_cast<uint4*>(d + 2 * PLANE) = l;
         }
       }
       ptx::fence_proxy_async_smem();
       ptx::mbar_arrive(&full_a[sa]);
       if (++sa == tc.n_a) { sa = 0; ph ^= 1u; }
       if (u + 1 < n_units) load(u + 1);
-      if (DRAIN && u > 0) ok &= drain(u - 1);
+      if (DRAIN && u > 0) {
+        if (TURN) {
+#pragma unroll 1
+          for (int j = 0; j < taps_u; ++j) ok &= drain((u - 1) * taps_u + j, j);
+        } else {
+          ok &= drain(u - 1, 0);
+        }
+      }
     }
 
     // Carry update of the first layer: its left context for the next chunk is the tail of the caller's chunk, written into ring
@@ -362,70 +385,73 @@ __global__ void __launch_bounds__(TC_THREADS, DRAIN ? 1 : 2) tapconv_tc_kernel(c
     // of the load/store pipe's time.
     constexpr int LPR = BN / 8;                    // lanes that share a row, 4 channels each
     constexpr int LD = BN / 2 + 4;                 // floats between rows of the staging tile (no bank conflicts)
-    float* stage = reinterpret_cast<float*>(sA) + warp * 32 * LD;
+    constexpr int RW = M / 4, NP = RW * LPR / 32;   // rows of a warp; pieces of a thread
+    float* stage = reinterpret_cast<float*>(sA) + warp * RW * LD;
     const int g = lane % LPR, rr = lane / LPR, n = n0 + col0 + 4 * g;
     const bool n_ok = n < p.C_out;
     // the warp's slot and its first frame there
     const TcSlot& a = PACK && q >= TC_SEG / 32 ? s1 : s0;
-    const int first = m0 + q * 32 + rr - (PACK && q >= TC_SEG / 32 ? TC_SEG : 0);
+    const int first = m0 + q * RW + rr - (PACK && q >= TC_SEG / 32 ? TC_SEG : 0);
     const bool direct = a.out_direct != nullptr;
     float* const out = direct ? a.out_direct : a.out_ring;
     const uint32_t out0 = direct ? 0u : (uint32_t)(p.n_phase * a.pos), out_mask = direct ? ~0u : (uint32_t)p.out_mask;
     const int T_out = PACK ? min(a.T, TC_SEG) : a.T;
-    const int n_sums = TURN ? p.n_taps : n_units;
     if (TURN) {
 #pragma unroll 1
-      for (int j = 0; j + 1 < n_sums; ++j) ok &= drain(j);
+      for (int j = 0; j + 1 < taps_u; ++j) ok &= drain((n_units - 1) * taps_u + j, j);
     }
-    float4 x[LPR];                                 // the residual rows, fetched under the products (with TURN half of them: registers)
+    float4 x[NP];                                 // the residual rows, fetched under the products (with TURN half of them: registers)
     auto residual = [&](int i) {
       const int row = first + i * (32 / LPR);
       x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p.residual_silu && row < T_out && n_ok) x[i] = *reinterpret_cast<const float4*>(in_row(a, row) + n);
     };
-    constexpr int X_EARLY = TURN ? LPR / 2 : LPR;
+    constexpr int X_EARLY = TURN ? NP / 2 : NP;
 #pragma unroll
     for (int i = 0; i < X_EARLY; ++i) residual(i);
     const float4 bias = n_ok ? *reinterpret_cast<const float4*>(p.bias + n) : make_float4(0.f, 0.f, 0.f, 0.f);
-    ok &= drain(n_sums - 1);
+    ok &= TURN ? drain(n_units * taps_u - 1, taps_u - 1) : drain(n_units - 1, 0);
     ok = ok && *reinterpret_cast<volatile int*>(s_fail) == 0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      float z0[16], z1[16], z2[16];
-      ptx::tmem_ld16x2(lanes + (uint32_t)(S_COL + col0 + 16 * c), lanes + (uint32_t)(S_COL + BN + col0 + 16 * c), z1, z2);
+      uint32_t z[2 * W];
+      float z0[W];
+      ptx::tmem_ld_rows_issue<W>(lanes + (uint32_t)(S_COL + col0 + 16 * c), z);
+      ptx::tmem_ld_rows_issue<W>(lanes + (uint32_t)(S_COL + BN + col0 + 16 * c), z + W);
+      ptx::tmem_ld_wait<2 * W>(z);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) z0[i] = sum[c][i] + (z1[i] + z2[i]);
+      for (int i = 0; i < W; ++i) z0[i] = sum[c][i] + (__uint_as_float(z[i]) + __uint_as_float(z[W + i]));
+      float* d = stage + (M == 64 ? lane & 15 : lane) * LD + 16 * c + (M == 64 ? 8 * (lane >> 4) : 0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4*>(stage + lane * LD + 16 * c + 4 * i) = make_float4(z0[4 * i], z0[4 * i + 1], z0[4 * i + 2], z0[4 * i + 3]);
+      for (int i = 0; i < W / 4; ++i) *reinterpret_cast<float4*>(d + 4 * i) = make_float4(z0[4 * i], z0[4 * i + 1], z0[4 * i + 2], z0[4 * i + 3]);
     }
 #pragma unroll
-    for (int i = X_EARLY; i < LPR; ++i) residual(i);
+    for (int i = X_EARLY; i < NP; ++i) residual(i);
     __syncwarp();
     // (one pass per step over all of the thread's pieces: the options cost one branch each, and the pieces' latencies overlap)
-    float4 v[LPR];
+    float4 v[NP];
 #pragma unroll
-    for (int i = 0; i < LPR; ++i) {
+    for (int i = 0; i < NP; ++i) {
       v[i] = *reinterpret_cast<const float4*>(stage + (rr + i * (32 / LPR)) * LD + 4 * g);
       v[i] = make_float4(v[i].x + bias.x, v[i].y + bias.y, v[i].z + bias.z, v[i].w + bias.w);
     }
     if (p.residual_silu) {
 #pragma unroll
-      for (int i = 0; i < LPR; ++i)
+      for (int i = 0; i < NP; ++i)
         v[i] = make_float4(x[i].x + silu_f(v[i].x), x[i].y + silu_f(v[i].y), x[i].z + silu_f(v[i].z), x[i].w + silu_f(v[i].w));
     }
     if (p.post_silu) {
 #pragma unroll
-      for (int i = 0; i < LPR; ++i) v[i] = make_float4(silu_f(v[i].x), silu_f(v[i].y), silu_f(v[i].z), silu_f(v[i].w));
+      for (int i = 0; i < NP; ++i) v[i] = make_float4(silu_f(v[i].x), silu_f(v[i].y), silu_f(v[i].z), silu_f(v[i].w));
     }
     if (p.exc_std != 0.f) {   // the stream's clock at this layer's output rate is the generator's offset
 #pragma unroll
-      for (int i = 0; i < LPR; ++i)
+      for (int i = 0; i < NP; ++i)
         v[i] = excite4(v[i], (long long)p.n_phase * (a.pos + first + i * (32 / LPR)) + phase, n, a.rng_id, p.exc_std, p.exc_seed_lo, p.exc_seed_hi);
     }
     if (n_ok && ok) {
 #pragma unroll
-      for (int i = 0; i < LPR; ++i) {
+      for (int i = 0; i < NP; ++i) {
         const int row = first + i * (32 / LPR);
         const uint32_t ro = (out0 + (uint32_t)(p.n_phase * row + phase)) & out_mask;
         if (row < T_out) *reinterpret_cast<float4*>(out + (size_t)ro * (uint32_t)p.C_out + n) = v[i];

@@ -70,6 +70,16 @@ def test_vocoder_batch_tiles(dc, mel, channels, f_chunk, n):
     assert gu.rel_err(got, orc.run_offline(cfg, weights, x, bounds).reshape(-1)) <= 1e-4
 
 
+# tiles of 64 frames: alone (32 columns each) and in batches whose layers take 64 columns, with one panel of input channels and with several; the last frames of
+# a tile, a second tile of one frame; the bytes of single calls, which take other tiles
+@pytest.mark.parametrize("mel,channels,f_chunk,n", [(8, (512, 64, 64), 56, 12), (80, (512, 256, 64), 50, 3), (80, (256, 128, 132), 33, 2), (80, (512, 128, 64), 65, 5)])
+def test_vocoder_small_tiles(dc, mel, channels, f_chunk, n):
+    gu = _util()
+    cfg = wl.tiny_vocoder(mel_dim=mel, up_channels=channels, f_chunk=f_chunk, n_chunks=3, seed=42)
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n)
+    assert gu.rel_err(got, orc.run_offline(cfg, weights, x, bounds).reshape(-1)) <= 1e-4
+
+
 # batches on both sides of one and two slots per cluster and of the kernels of their own; every cluster size; keys with a gap between
 # prompt and history, one block and several
 @pytest.mark.parametrize("hidden,heads,n,kw", [
