@@ -105,11 +105,11 @@ __device__ __forceinline__ void clu_arrive_release(int warp) {
   ptx::cluster_arrive_relaxed();
 }
 
-// One slot per cluster: a stage's rows leave the CTA as one piece, [64 rows][32 channels] (clu_at32), which one thread copies out of shared memory in bulk.
+// A stage's rows leave the CTA as one piece, [64 or 128 rows][32 channels] (clu_at32), which one thread copies out of shared memory in bulk.
 // The copy has completed - its bytes are in L2, where the other CTAs' bulk copies read them - 480 cycles after the staging; the fence behind stores of the
 // threads took 1,040.  (16 CTAs hand 4 KB each to one another: the first operand block is there after 1,150 cycles instead of 1,790.  With a fence behind the
 // copy, which has nothing left to wait for, 2,010.)  One stream 801 -> 748 us per chunk, hidden 256 298 -> 275, seven streams 813 -> 755, prompt and
-// look-ahead 762 -> 704.
+// look-ahead 762 -> 704; two slots per cluster: fourteen streams 990 -> 933, one guided stream 967 -> 913.
 __device__ __forceinline__ int clu_at32(int rho, int c) { return rho * 32 + (((c >> 3) ^ ((rho >> 1) & 3)) << 3); }   // element of channel c of a block: the 64-byte swizzle
 struct CluPiece {
   void*       dst;
@@ -274,6 +274,10 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   auto issuers = [&](int nkb) { return nkb >= 2 ? 2 : 1; };
+  // Descriptor of K/V slot ks.  With two slots per cluster made anew for every block: fourteen streams 995 -> 938 us against one made in front of the loop and
+  // advanced, which keeps it out of the uniform registers that a product takes it from; with one slot 745 -> 751.
+  auto kv_base = [&](uint32_t a) { return p.dh_shift == 6 ? att_kv_desc<64>(a) : att_kv_desc<32>(a); };
+  auto kv_desc = [&](uint64_t first, uint32_t ks) { return ONE ? first + (uint64_t)(ks * (CLU_KV_BYTES >> 4)) : kv_base(ptx::smem_u32(kvring + ks * CLU_KV_BYTES)); };
   const int n_jobs = SPC * p.n_heads;            // (slot, head) pairs of the cluster; CTA r takes r, r + CL, ...
   const long long kv_plane = (long long)(p.P + p.Rk) * p.C;
   const int dh = 1 << p.dh_shift;
@@ -326,19 +330,24 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     uint32_t it0 = 0, pre = 0, n_q = 0;            // K/V items of earlier jobs; items of the next job already requested; Q tiles so far
     uint32_t n_s0 = 0, n_s1 = 0;                   // key blocks of the two streams in earlier jobs
     const bool two = !ONE && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
-    auto request = [&](const bf16* src, int nkb) {
+    // (the input projection's operand comes from another kernel: a slot's blocks are its own)
+    auto request = [&](const bf16* src, int nkb, bool in) {
       ptx::fence_proxy_async_global();
       if (ptx::elect_one()) {
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
           ptx::mbar_expect_tx(&full_a[kb], two ? 16384u : 8192u);
-          ptx::bulk_load(panel + kb * kb_bytes, src + kb * CLU_SLOT_KB, 8192u, &full_a[kb]);
-          if (two) ptx::bulk_load(panel + kb * kb_bytes + 8192, src + (nkb + kb) * CLU_SLOT_KB, 8192u, &full_a[kb]);
+          if (!ONE && in) {
+            ptx::bulk_load(panel + kb * kb_bytes, src + kb * CLU_SLOT_KB, 8192u, &full_a[kb]);
+            if (two) ptx::bulk_load(panel + kb * kb_bytes + 8192, src + (nkb + kb) * CLU_SLOT_KB, 8192u, &full_a[kb]);
+          } else {
+            ptx::bulk_load(panel + kb * kb_bytes, src + kb * (two ? 2 : 1) * CLU_SLOT_KB, two ? 16384u : 8192u, &full_a[kb]);
+          }
         }
       }
       __syncwarp();
     };
-    if (warp == 0) request(p.Ain + (long long)slot0 * nkb_in * CLU_SLOT_KB, nkb_in);
+    if (warp == 0) request(p.Ain + (long long)slot0 * nkb_in * CLU_SLOT_KB, nkb_in, true);
 #pragma unroll 1
     for (CluStage st; st.s < p.n_steps; st.next(p)) {
       bool fetch = false;
@@ -357,10 +366,9 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             // slot, phases and descriptors advance incrementally on 32-bit values, and the next block's barriers are polled ahead
             // of this block's products (a wait that finds its barrier complete costs as much as a product, too).
             constexpr uint32_t DESC_HI = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61)) >> 32);
-            // one slot: blocks of 32 channels in the 64-byte swizzle (the input projection's operand comes from another kernel)
-            const bool b32 = ONE && st.kind != CLU_IN;
+            const bool b32 = st.kind != CLU_IN;    // blocks of 32 channels in the 64-byte swizzle
             const uint32_t a_hi = b32 ? (uint32_t)((((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61)) >> 32) : DESC_HI;
-            const uint32_t a_k2 = b32 ? 4096u >> 4 : 4u;
+            const uint32_t a_k2 = b32 ? (two ? 8192u : 4096u) >> 4 : 4u;
             const uint32_t w_lo = ((ptx::smem_u32(wring) & 0x3FFFF) >> 4) | (1u << 16), a_step = (uint32_t)(n_iss * (kb_bytes >> 4));
             const uint32_t bar_w0 = ptx::smem_u32(full_w), bar_e0 = ptx::smem_u32(empty_w), a_bstep = 8u * (uint32_t)n_iss;
             uint32_t slot = (wt + (uint32_t)me) % RS, pw = ((wt + (uint32_t)me) / RS) & 1u, acc = 0;
@@ -492,7 +500,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         // ---- scores: S(b) as soon as its stream's previous scores have been read.  (Scores and P V from one warp: 2,000 cycles of
         // waits and issue per block, which paced the sweep; a warp for each halves that.) ----
         const uint32_t idesc_s = ptx::umma_idesc_bf16(128, ATT_KB, 0, 0);
-        const uint64_t dkv = p.dh_shift == 6 ? att_kv_desc<64>(ptx::smem_u32(kvring)) : att_kv_desc<32>(ptx::smem_u32(kvring));
+        const uint64_t dkv = ONE ? kv_base(ptx::smem_u32(kvring)) : 0ull;
 #pragma unroll 1
         for (int jid = rank; jid < n_jobs; jid += p.CL) {
           const int nkb = s_job[jid / p.n_heads].k.nkb, head = jid % p.n_heads;
@@ -507,7 +515,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             const uint32_t k = w ? n_s1++ : n_s0++;
             if (k > 0) clu_wait(&bar_sfree[w], (k - 1) & 1u, s_fail, p.err, 0x109);   // the stream's previous scores have been read
             ptx::tc_fence_after();
-            const uint64_t dk = dkv + (uint64_t)(ks * (CLU_KV_BYTES >> 4));
+            const uint64_t dk = kv_desc(dkv, ks);
             const uint32_t d_s = tmem_base + (uint32_t)w * ATT_KB;
             if (ptx::elect_one()) {
               ptx::umma_bf16(d_s, dq, dk, idesc_s, 0);
@@ -527,7 +535,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         // ---- O_w += P(b) V(b) ----
         const uint32_t idesc_pv = ptx::umma_idesc_bf16(128, dh, 0, 1);   // B = V, MN-major
         const uint64_t dp = ptx::umma_desc_sw128(ptx::smem_u32(sP));
-        const uint64_t dkv = p.dh_shift == 6 ? att_kv_desc<64>(ptx::smem_u32(kvring)) : att_kv_desc<32>(ptx::smem_u32(kvring));
+        const uint64_t dkv = ONE ? kv_base(ptx::smem_u32(kvring)) : 0ull;
         const uint32_t v_step = 2u << p.dh_shift;
 #pragma unroll 1
         for (int jid = rank; jid < n_jobs; jid += p.CL) {
@@ -540,7 +548,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             clu_wait(&full_kv[vs], (gi / CLU_KVS) & 1u, s_fail, p.err, 0x10d);
             clu_wait(&bar_p[w], (w ? n_s1++ : n_s0++) & 1u, s_fail, p.err, 0x10c);
             ptx::tc_fence_after();
-            const uint64_t dpb = dp + (uint64_t)(w * (ATT_P_BYTES >> 4)), dv = dkv + (uint64_t)(vs * (CLU_KV_BYTES >> 4));
+            const uint64_t dpb = dp + (uint64_t)(w * (ATT_P_BYTES >> 4)), dv = kv_desc(dkv, vs);
             const uint32_t d_o = tmem_base + CLU_O_COL + (uint32_t)w * 64u;
             const int ksteps = min(ATT_KB / 16, (L - b * ATT_KB + 15) >> 4);
             if (ptx::elect_one()) {
@@ -567,7 +575,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       // (read here, where nobody waits for it: a wait takes so long to give up that what it left behind one stage earlier has landed)
       const bool failed = warp == 0 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0);
       ptx::cluster_wait();
-      if (wants && !failed) request(nx_src, nx_nkb);
+      if (wants && !failed) request(nx_src, nx_nkb, nx.kind == CLU_IN);
       if (failed) {
 #pragma unroll 1
         for (st.next(p); st.s < p.n_steps; st.next(p)) {
@@ -599,6 +607,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     bf16* const s_kv = si.kv;
     const bool is_out = si.pass == 0;
     const int tau0 = p.slots[slot0].tau_off, tau1 = !ONE && slot0 + 1 < p.n_slots ? p.slots[slot0 + 1].tau_off : 0;
+    const int rows = !ONE && slot0 + 1 < p.n_slots ? 2 * SLOT_ROWS : SLOT_ROWS;   // of the cluster's blocks (an odd batch's last cluster has one slot)
     const bool in_range = si.T > 0;
     const bool halo_row = in_range && rho < HALO, chunk_row = in_range && f >= 0 && f < si.T;
     const int new_row = rho - si.Tc;                // carry row this thread's value moves to
@@ -624,11 +633,12 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
 #pragma unroll 1
     for (CluStage st; st.s < p.n_steps; st.next(p)) {
       if (st.kind == CLU_ATT) {
+        const bool one_job = ONE || n_jobs <= p.CL;  // of this CTA: its rows leave in bulk
 #pragma unroll 1
         for (int jid = rank; jid < n_jobs; jid += p.CL) {
           const CluJob jb = s_job[jid / p.n_heads];
           if (jb.T == 0) continue;
-          const int nkb = jb.k.nkb, head = jid % p.n_heads, aslot = slot0 + jid / p.n_heads;
+          const int nkb = jb.k.nkb, head = jid % p.n_heads;
           const int row = aq * 32 + lane, w = cg;
           float* sx = s_x + w * 128;
           float m_ref = -INFINITY, lsum = 0.f;
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           if (ah == 0) {                           // O rows 0..63 live in lanes 0..63; each group of warps stores half of the columns
             float c0, c1;
             att_combine(nkb, s_m[row], s_x[row] + s_x[64 + row], s_m[64 + row], s_x[128 + row] + s_x[192 + row], &c0, &c1);
-            bf16* oblk = p.O + ((long long)aslot * nkb_c + (head << p.dh_shift >> 6)) * CLU_SLOT_KB;
+            const int orow = (ONE ? 0 : (jid / p.n_heads) * SLOT_ROWS) + HALO + row;
 #pragma unroll 1
             for (int c = w * (dh >> 1); c < (w + 1) * (dh >> 1); c += 16) {
               float o16[16], q16[16];
@@ -687,25 +697,29 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
                 for (int i = 0; i < 16; ++i) o16[i] = nkb > 1 ? fmaf(q16[i], c1, o16[i] * c0) : o16[i] * c0;
                 uint4 a, bq;
                 pack16_bf16(o16, a, bq);
-                if (ONE) {                         // (the queries' tile is idle by now)
+                if (one_job) {                     // (the queries' tile is idle by now)
                   bf16* d = reinterpret_cast<bf16*>(sQ) + (c >> 5) * (SLOT_ROWS * 32);
                   *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, c & 31)) = a;
                   *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, (c & 31) + 8)) = bq;
                 } else {
-                  clu_store16(oblk, row + HALO, ((head << p.dh_shift) & 63) + c, a, bq);
+                  const int ch = (head << p.dh_shift) + c, perm = (orow >> 1) & 3;
+                  store16(p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + (long long)(ch >> 5) * (rows * 32) + orow * 32 + ((((ch & 31) >> 3) ^ perm) & ~1) * 8,
+                          (perm & 1) ? bq : a, (perm & 1) ? a : bq);
                 }
               }
             }
           }
           ptx::tc_fence_before();
-          if (!ONE) ptx::named_bar_sync(1, CLU_EPI);   // (the next job overwrites the exchange and the accumulators; with one slot a CTA has at most one)
+          if (!one_job) ptx::named_bar_sync(1, CLU_EPI);   // (the next job overwrites the exchange and the accumulators)
         }
-        if (ONE) {
-          // the rows of the head's one or two blocks of 32 channels
-          const uint32_t bytes = rank < n_jobs && s_job[0].T > 0 ? (SLOT_ROWS - HALO) * 64u : 0u;
-          bf16* dst = p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + ((rank << p.dh_shift) >> 5) * (SLOT_ROWS * 32) + HALO * 32;
+        if (one_job) {
+          // the 56 rows of its slot in the head's one or two blocks of 32 channels
+          const int head = ONE ? rank : rank % p.n_heads, sl = ONE ? 0 : rank / p.n_heads;
+          const bool has = rank < n_jobs && slot0 + sl < p.n_slots && s_job[sl].T > 0;
+          const uint32_t bytes = has ? (SLOT_ROWS - HALO) * 64u : 0u;
+          bf16* dst = p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + ((head << p.dh_shift) >> 5) * (rows * 32) + (sl * SLOT_ROWS + HALO) * 32;
           const uint8_t* src = sQ + HALO * 64;
-          const CluPiece piece[2] = {{dst, src, bytes}, {dst + SLOT_ROWS * 32, src + SLOT_ROWS * 64, p.dh_shift == 6 ? bytes : 0u}};
+          const CluPiece piece[2] = {{dst, src, bytes}, {dst + rows * 32, src + SLOT_ROWS * 64, p.dh_shift == 6 ? bytes : 0u}};
           clu_arrive_bulk(warp, piece);
         } else {
           clu_arrive_release(warp);
@@ -770,10 +784,10 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         // read and not written: a branch around every piece cost more than the pieces.
         // (32 bytes of each slot's row in turn, with a wait in between: 14 streams 1,140 us, one guided stream 1,105, one stream 960; pieces in branches of
         // their own 1,110, 1,079 and 956; so 1,086, 1,054 and 934.)
-        constexpr bool two = !ONE;
+        const bool two = !ONE && rows == 2 * SLOT_ROWS;
         float k[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) k[i] = ONE ? s_x[et >> 2] : s_x[(et >> 3) + 32 * i];   // (one slot: 16 bytes of its row in either block of 32 channels)
+        for (int i = 0; i < 4; ++i) k[i] = s_x[(rows == SLOT_ROWS ? 0 : (i & 1) * SLOT_ROWS) + (et >> 2)];   // (16 bytes of a slot's row in either block of 32 channels)
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
           clu_wait(&full_a[kb], ((kb < nkb_c ? n_gc : 0u) + (kb < nkb_in ? n_gi : 0u)) & 1u, s_fail, p.err, 0x114);
@@ -809,7 +823,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       const bool got = clu_wait(accum, n_g & 1u, s_fail, p.err, 0x113);
       ptx::tc_fence_after();
       const bool ok = got && *reinterpret_cast<volatile int*>(s_fail) == 0;
-      const bool is_chunk = chunk_row && ok, is_halo = halo_row && ok;
+      const bool is_chunk = chunk_row && ok;
 
       auto load_pair = [&](uint32_t col, float* v) {  // NC columns of the 16 from `col` on; even blocks + odd blocks, always in this order
         if (n_iss == 2) {
@@ -930,7 +944,6 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       } else {
         // ---- a new residual row: input projection, conv block, attention output projection ----
         bf16* out = p.X[kind == CLU_IN ? 0 : xi ^ 1];
-        const int n = n0 + c0;
         float2 acc[NC / 2];
         if (kind == CLU_CONV) {
           // y[r] = Z_0[r - 2 d] + Z_1[r - d] + Z_2[r]: rows change lanes through shared memory (the panel is idle by now)
@@ -1016,11 +1029,12 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
 #pragma unroll
           for (int i = 0; i < NC / 8; ++i) { w[4 * i] = hr[i].x; w[4 * i + 1] = hr[i].y; w[4 * i + 2] = hr[i].z; w[4 * i + 3] = hr[i].w; }
         }
-        // One slot: staged in the panel behind the taps' exchange.  (Rows that are neither the chunk's nor its left context go along; no row reads one behind it.)
-        bf16* const rows_out = reinterpret_cast<bf16*>(panel + 16384);
-        float* const ssq_out = reinterpret_cast<float*>(panel + 16384 + SLOT_ROWS * 64);
-        if (ONE) *reinterpret_cast<uint4*>(rows_out + clu_at32(rho, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
-        else put_row(is_chunk || (is_halo && next_conv), out + ((long long)slot * nkb_c + (n >> 6)) * CLU_SLOT_KB + clu_row16(rho, n & 63), rho & 1, w);
+        // Staged in the panel behind the taps' exchange.  (Rows that are neither the chunk's nor its left context go along; no row reads one behind it.)
+        bf16* const rows_out = reinterpret_cast<bf16*>(panel + SPC * 16384);
+        float* const ssq_out = reinterpret_cast<float*>(panel + SPC * 16384 + ROWS * 64);   // [slot][2][SLOT_ROWS]
+#pragma unroll
+        for (int i = 0; i < NC / 8; ++i)
+          *reinterpret_cast<uint4*>(rows_out + clu_at32(row_t, c0 + 8 * i)) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         if (feeds_norm && in_range) {              // sum of squares of the row's 16 stored values, fixed order (ONE: the upper lane goes on from the lower one's)
           float ss = 0.f;
 #pragma unroll
@@ -1035,19 +1049,19 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               }
             }
           }
-          if (!ONE) p.ssq[((long long)slot * (p.C >> 4) + (n >> 4)) * SLOT_ROWS + rho] = ss;
-          else if (lane >= 16) ssq_out[cg * SLOT_ROWS + rho] = ss;
+          if (!ONE || lane >= 16) ssq_out[(row_t >> 6) * 2 * SLOT_ROWS + cg * SLOT_ROWS + rho] = ss;
         }
-        // The next stage's bulk copies overwrite the exchange of the taps: the writers' fence.  (One stream 909 -> 919 us; right behind the writes
-        // 925, behind the barrier of clu_arrive_release 918.)
-        if (!ONE && kind == CLU_CONV) ptx::fence_proxy_async_smem();
         ptx::tc_fence_before();
+        const long long ssq_slot = (long long)(p.C >> 4) * SLOT_ROWS;
+        float* const ssq = p.ssq + (long long)slot0 * ssq_slot + 2 * rank * SLOT_ROWS;
+        const uint32_t ssq_bytes = feeds_norm ? 2u * SLOT_ROWS * 4u : 0u;
+        const CluPiece rows_piece = {out + (long long)slot0 * nkb_c * CLU_SLOT_KB + rank * (rows * 32), rows_out, (uint32_t)rows * 64u};
         if (ONE) {
-          const CluPiece piece[2] = {{out + (long long)slot0 * nkb_c * CLU_SLOT_KB + rank * (SLOT_ROWS * 32), rows_out, SLOT_ROWS * 64u},
-                                     {p.ssq + ((long long)slot0 * (p.C >> 4) + 2 * rank) * SLOT_ROWS, ssq_out, feeds_norm && in_range ? 2u * SLOT_ROWS * 4u : 0u}};
+          const CluPiece piece[2] = {rows_piece, {ssq, ssq_out, ssq_bytes}};
           clu_arrive_bulk(warp, piece);
         } else {
-          clu_arrive_release(warp);
+          const CluPiece piece[3] = {rows_piece, {ssq, ssq_out, ssq_bytes}, {ssq + ssq_slot, ssq_out + 2 * SLOT_ROWS, rows == 2 * SLOT_ROWS ? ssq_bytes : 0u}};
+          clu_arrive_bulk(warp, piece);
         }
         // shift the carry by the committed frames: nobody in this launch reads it again
         if (carry != nullptr && moves && ok) {
