@@ -159,6 +159,20 @@ def test_flow_cluster_rounded_norm(dc, n, kw):
     assert np.array_equal(got, _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM | dc.OPT_CTA_PAIRS)[3])
 
 
+# three and four slots per cluster, in tiles of two: an odd slot, a last cluster of one, two and three, the smallest and the largest batch and those beside them; both
+# head widths, a gap between prompt and history, one key block and several, guided passes, look-ahead, the rounded norm
+@pytest.mark.parametrize("hidden,heads,n,kw", [
+    (512, 8, 18, {}), (512, 8, 19, {}), (512, 8, 21, dict(kv_cap=300)), (512, 8, 22, {}), (512, 8, 27, {}), (512, 8, 28, {}), (512, 8, 29, {}),
+    (512, 16, 20, dict(f_prompt=13, kv_cap=150)), (512, 8, 23, dict(f_prompt=130)), (512, 16, 25, dict(f_lookahead=6)), (512, 8, 10, dict(cfg_scale=0.7)),
+    (512, 8, 13, dict(cfg_scale=0.7)), (512, 8, 20, dict(rounded=True)), (512, 8, 26, dict(rounded=True))])
+def test_flow_tiles(dc, hidden, heads, n, kw):
+    gu = _util()
+    cfg = wl.tiny_flow(hidden=hidden, n_heads=heads, head_dim=hidden // heads, mel_dim=80, n_steps=2, seed=43, **{k: v for k, v in kw.items() if k != "rounded"})
+    weights, x, bounds, got = _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM if "rounded" in kw else 0)
+    if not cfg.f_lookahead:      # (a call's look-ahead frames are presented again by the next one: other tests compare those)
+        assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
+
+
 # one reduction block per conv product (hidden 64): 32- and 64-column tiles, whose epilogue exchanges more rows than one pipeline stage holds
 @pytest.mark.parametrize("n", [76, 150])
 def test_conv_exchange_of_one_reduction_block(dc, n):
