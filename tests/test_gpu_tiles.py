@@ -173,6 +173,37 @@ def test_flow_tiles(dc, hidden, heads, n, kw):
         assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
 
 
+# large scores: a later key block's maximum exceeds the reference by more than 2^8 and the accumulated output is rescaled.  One and two slots per cluster, tiles, kernels
+# of their own: each has its own rows in tensor memory, and all give the same bytes
+@pytest.mark.parametrize("heads", [8, 16])
+def test_attention_rescale_in_every_form(dc, heads):
+    cfg = wl.tiny_flow(hidden=512, n_heads=heads, head_dim=512 // heads, mel_dim=80, n_steps=2, kv_cap=500, f_chunk=50, seed=44)
+    w, at = wl.make_workload(cfg).weights.copy(), 0
+    for name, shape, _ in wl.blob_layout(cfg):
+        n = int(np.prod(shape))
+        if "q" in name.lower() and len(shape) == 2:
+            w[at:at + n] *= 10.0          # scores of 14 binary orders, the largest of 128 some 30 above their mean
+        at += n
+    m = dc.Model(cfg, w, max_batch=29)
+    streams = [m.open_stream() for _ in range(29)]
+    gen = torch.Generator(device="cuda").manual_seed(44)
+    x = [torch.randn(cfg.f_chunk, cfg.in_dim, generator=gen, device="cuda") for _ in range(12)]
+    outs = {}
+    for n in (1, 9, 20, 29):
+        for s in streams:
+            s.reset()
+        for c in x:
+            out = torch.zeros(n, cfg.f_chunk, cfg.mel_dim, device="cuda")
+            dc.decode_batch(m, streams[:n], c.expand(n, -1, -1).contiguous(), out)
+        outs[n] = out
+    assert m.counters()[4] == 0 and outs[1].isfinite().all()
+    for n in (9, 20, 29):
+        assert torch.equal(outs[n], outs[1].expand(n, -1, -1)), n
+    for s in streams:
+        s.close()
+    m.destroy()
+
+
 # one reduction block per conv product (hidden 64): 32- and 64-column tiles, whose epilogue exchanges more rows than one pipeline stage holds
 @pytest.mark.parametrize("n", [76, 150])
 def test_conv_exchange_of_one_reduction_block(dc, n):
