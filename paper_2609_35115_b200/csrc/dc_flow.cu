@@ -1237,7 +1237,6 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) flow_attn_kernel(const AttnPar
 }
 
 #include "dc_flow_cluster.cuh"
-#include "dc_flow_tiles.cuh"
 
 // ---- host helpers ----------------------------------------------------------------------------
 
@@ -1740,7 +1739,6 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int CL, 
 }
 
 auto cluster_fn(const FlowModel* m, int spc, bool ring) {
-  if (spc > 2) return m->U != nullptr ? flow_tiles_kernel<true> : flow_tiles_kernel<false>;
   if (spc == 2) return m->U != nullptr ? flow_cluster_kernel<false, true, 2> : flow_cluster_kernel<false, false, 2>;
   return m->U != nullptr ? (ring ? flow_cluster_kernel<true, true, 1> : flow_cluster_kernel<false, true, 1>)
                          : (ring ? flow_cluster_kernel<true, false, 1> : flow_cluster_kernel<false, false, 1>);
@@ -1758,7 +1756,7 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
   cudaError_t e = cudaSuccess;
   cudaFuncAttributes fa{};
   int regs = 1 << 16;
-  for (auto fn : {cluster_fn(m, 1, false), cluster_fn(m, 1, true), cluster_fn(m, 2, false), cluster_fn(m, 3, false)}) {
+  for (auto fn : {cluster_fn(m, 1, false), cluster_fn(m, 1, true), cluster_fn(m, 2, false)}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CLU_SMEM);
     if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
@@ -1804,16 +1802,9 @@ cudaError_t cluster_create(FlowModel* m, size_t w_in, const std::vector<size_t>&
 // Slots per cluster of the one-kernel step for a batch of n slots, 0 if its clusters would not all be resident at once (a second
 // wave doubles the step: the kernels of their own serve the batch).  One slot per cluster where that fits, else two; the two passes
 // of a guided stream share a cluster.
-// Three or four (flow_tiles_kernel) at hidden 512 where the kernels of their own would need 64-column tiles, i.e. from 19 slots on: 20 streams 1,526 -> 1,358 us, 24
-// 1,531 -> 1,408, 28 1,584 -> 1,411, 14 guided ones 1,587 -> 1,410.  Below, their 32-column tiles are as fast (16 streams 1,350 against 1,355); beyond, a third tile
-// costs more than it brings (32 streams 1,875 against 1,635), and so does the second one at hidden 256, whose stages are shorter (32 streams 534 against 490).
 int cluster_slots(const FlowModel* m, int n) {
   for (int spc = m->n_pass; spc <= 2; ++spc)
     if ((n + spc - 1) / spc <= m->max_clusters) return spc;
-  const bool wide = (n + 1) / 2 * (m->C / 32) > m->n_sm, fits = (m->mel / 16 + m->C / CLU_BN - 1) / (m->C / CLU_BN) * 16 <= TIL_ACC;
-  if (m->C == 512 && wide && fits)
-    for (int spc = m->n_pass == 2 ? 4 : 3; spc <= 2 * TIL_MAX; spc += m->n_pass)
-      if ((n + spc - 1) / spc <= m->max_clusters) return spc;
   return 0;
 }
 
@@ -1825,7 +1816,7 @@ bool wave_ring(const FlowModel* m, int n) { return m->n_pass == 1 && cluster_slo
 void enqueue_cluster(FlowModel* m, int n, int spc, LaunchCtx& lc, bool tick, bool ring) {
   const dc_config& c = m->cfg;
   CluParams p{};
-  p.slots = m->d_slots; p.n_slots = n; p.spc = spc; p.CL = m->C / CLU_BN;
+  p.slots = m->d_slots; p.n_slots = n; p.CL = m->C / CLU_BN;
   p.C = m->C; p.mel = m->mel; p.Kin = m->Kin; p.n_heads = c.n_heads;
   p.n_conv = c.n_conv; p.n_attn = c.n_attn; p.cpa = m->cpa; p.n_steps = tick ? 1 : c.n_steps; p.tick = tick;
   for (int l = 0; l < c.n_conv; ++l) p.dil[l] = c.dilations[l];

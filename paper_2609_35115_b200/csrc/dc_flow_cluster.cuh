@@ -42,7 +42,7 @@ static_assert(CLU_SMEM <= 227 * 1024, "one CTA's shared memory");
 
 struct CluParams {
   const SlotInfo* slots;
-  int             n_slots, spc;        // slots of the launch; slots per cluster
+  int             n_slots;             // slots of the launch
   int             CL;                  // CTAs of a cluster
   int             C, mel, Kin, n_heads;
   int             n_conv, n_attn, cpa, n_steps;

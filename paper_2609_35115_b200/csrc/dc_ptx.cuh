@@ -54,38 +54,6 @@ __device__ __forceinline__ bool mbar_try_wait_s(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// ... on a barrier that other CTAs of the cluster arrive at, and an arrival there (at a shared::cluster address; the arriving thread has made its
-// stores visible by a fence of its own).
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One look, without the time that try_wait may block for: a warp that polls several barriers.
-__device__ __forceinline__ bool mbar_test_wait_s(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // Bounded wait.  Returns false after kMaxPolls failed polls (each poll blocks in hardware for a
 // short, implementation-defined time), which is orders of magnitude beyond any legitimate wait here: whatever was in flight when
 // the wait began has landed when it gives up.
@@ -165,7 +133,6 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)), "r"(smem_u32(src)), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;" ::: "memory"); }   // ... have been read
 __device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // Asks `bytes` (a multiple of 16) from a 16-byte aligned address into L2.
@@ -318,19 +285,6 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t* r) {
                :
                : "memory");
 }
-// 8 columns of this thread's lane, 32 bits each.
-__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t* r) {   // (tmem_ld_wait<8>)
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\ntcgen05.wait::st.sync.aligned;" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
-               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-
 // A warp's share of an accumulator, in two halves like the pair above.  N = 16: 16 columns of each of the 32 lanes (a thread has a whole row piece);
 // N = 8: 16 columns of lanes 0..15 of the quarter, where the rows of a 64-row product are: thread l has lane l & 15, columns 8 (l >> 4) ... + 7.
 template <int N>

@@ -159,22 +159,8 @@ def test_flow_cluster_rounded_norm(dc, n, kw):
     assert np.array_equal(got, _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM | dc.OPT_CTA_PAIRS)[3])
 
 
-# three and four slots per cluster, in tiles of two: an odd slot, a last cluster of one, two and three, the smallest and the largest batch and those beside them; both
-# head widths, a gap between prompt and history, one key block and several, guided passes, look-ahead, the rounded norm
-@pytest.mark.parametrize("hidden,heads,n,kw", [
-    (512, 8, 18, {}), (512, 8, 19, {}), (512, 8, 21, dict(kv_cap=300)), (512, 8, 22, {}), (512, 8, 27, {}), (512, 8, 28, {}), (512, 8, 29, {}),
-    (512, 16, 20, dict(f_prompt=13, kv_cap=150)), (512, 8, 23, dict(f_prompt=130)), (512, 16, 25, dict(f_lookahead=6)), (512, 8, 10, dict(cfg_scale=0.7)),
-    (512, 8, 13, dict(cfg_scale=0.7)), (512, 8, 20, dict(rounded=True)), (512, 8, 26, dict(rounded=True))])
-def test_flow_tiles(dc, hidden, heads, n, kw):
-    gu = _util()
-    cfg = wl.tiny_flow(hidden=hidden, n_heads=heads, head_dim=hidden // heads, mel_dim=80, n_steps=2, seed=43, **{k: v for k, v in kw.items() if k != "rounded"})
-    weights, x, bounds, got = _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM if "rounded" in kw else 0)
-    if not cfg.f_lookahead:      # (a call's look-ahead frames are presented again by the next one: other tests compare those)
-        assert gu.rel_err(got.reshape(-1, cfg.out_per_frame), orc.run_offline(cfg, weights, x, bounds)) <= 2e-2
-
-
-# large scores: a later key block's maximum exceeds the reference by more than 2^8 and the accumulated output is rescaled.  One and two slots per cluster, tiles, kernels
-# of their own: each has its own rows in tensor memory, and all give the same bytes
+# large scores: a later key block's maximum exceeds the reference by more than 2^8 and the accumulated output is rescaled.  One and two slots per cluster and kernels of
+# their own: each has its own rows in tensor memory, and all give the same bytes
 @pytest.mark.parametrize("heads", [8, 16])
 def test_attention_rescale_in_every_form(dc, heads):
     cfg = wl.tiny_flow(hidden=512, n_heads=heads, head_dim=512 // heads, mel_dim=80, n_steps=2, kv_cap=500, f_chunk=50, seed=44)
@@ -184,12 +170,12 @@ def test_attention_rescale_in_every_form(dc, heads):
         if "q" in name.lower() and len(shape) == 2:
             w[at:at + n] *= 10.0          # scores of 14 binary orders, the largest of 128 some 30 above their mean
         at += n
-    m = dc.Model(cfg, w, max_batch=29)
-    streams = [m.open_stream() for _ in range(29)]
+    m = dc.Model(cfg, w, max_batch=20)
+    streams = [m.open_stream() for _ in range(20)]
     gen = torch.Generator(device="cuda").manual_seed(44)
     x = [torch.randn(cfg.f_chunk, cfg.in_dim, generator=gen, device="cuda") for _ in range(12)]
     outs = {}
-    for n in (1, 9, 20, 29):
+    for n in (1, 9, 20):
         for s in streams:
             s.reset()
         for c in x:
@@ -197,7 +183,7 @@ def test_attention_rescale_in_every_form(dc, heads):
             dc.decode_batch(m, streams[:n], c.expand(n, -1, -1).contiguous(), out)
         outs[n] = out
     assert m.counters()[4] == 0 and outs[1].isfinite().all()
-    for n in (9, 20, 29):
+    for n in (9, 20):
         assert torch.equal(outs[n], outs[1].expand(n, -1, -1)), n
     for s in streams:
         s.close()
