@@ -149,19 +149,6 @@ __device__ __forceinline__ bool clu_wait(uint64_t* bar, uint32_t parity, int* s_
   return false;
 }
 
-// O rows of a 64-row product (16 lanes of the warp's quarter) scaled by alpha, the same in both lanes of a row.  A rare call: see att_rescale.
-__device__ __noinline__ void clu_rescale(uint32_t addr, float alpha, int cols) {
-#pragma unroll 1
-  for (int c = 0; c < cols; c += 16) {
-    uint32_t o[8];
-    ptx::tmem_ld_rows_issue<8>(addr + (uint32_t)c, o);
-    ptx::tmem_ld_wait<8>(o);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-    ptx::tmem_st_rows8(addr + (uint32_t)c, o);
-  }
-}
-
 // ---- K/V items of one attention job, in the order in which the products consume them: K0 K1 K2 V0 K3 V1 ... V(n-1) ----
 __device__ __forceinline__ int clu_item_k(int b) { return b < 2 ? b : 2 * b - 2; }
 __device__ __forceinline__ int clu_item_v(int b, int n) { return b + 2 < n ? 2 * b + 3 : 2 * n - (n - b); }
@@ -457,11 +444,12 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             // have all been waited for when it was filled)
             if (!first && !clu_wait(&empty_kv[last_k % CLU_KVS], (last_k / CLU_KVS) & 1u, s_fail, p.err, 0x107)) break;
             // the slot's 56 chunk rows of the head's 64-column block (rows T.. are never stored; with head_dim 32 the block
-            // holds two heads)
+            // holds two heads), twice: see flow_attn_kernel
             if (ptx::elect_one()) {
               const bf16* src = p.Q + ((long long)slot * nkb_c + (head << p.dh_shift >> 6)) * CLU_SLOT_KB + HALO * 64;
-              ptx::mbar_expect_tx(bar_q, (SLOT_ROWS - HALO) * 128u);
+              ptx::mbar_expect_tx(bar_q, 2u * (SLOT_ROWS - HALO) * 128u);
               ptx::bulk_load(sQ, src, (SLOT_ROWS - HALO) * 128u, bar_q);
+              ptx::bulk_load(sQ + 8192, src, (SLOT_ROWS - HALO) * 128u, bar_q);
             }
             __syncwarp();
           }
@@ -511,7 +499,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       } else if (att && warp == 1) {
         // ---- scores: S(b) as soon as its stream's previous scores have been read.  (Scores and P V from one warp: 2,000 cycles of
         // waits and issue per block, which paced the sweep; a warp for each halves that.) ----
-        const uint32_t idesc_s = ptx::umma_idesc_bf16(SLOT_ROWS, ATT_KB, 0, 0);
+        const uint32_t idesc_s = ptx::umma_idesc_bf16(128, ATT_KB, 0, 0);
         const uint64_t dkv = ONE ? kv_base(ptx::smem_u32(kvring)) : 0ull;
 #pragma unroll 1
         for (int jid = rank; jid < n_jobs; jid += p.CL) {
@@ -545,7 +533,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         }
       } else if (att && warp == 3) {
         // ---- O_w += P(b) V(b) ----
-        const uint32_t idesc_pv = ptx::umma_idesc_bf16(SLOT_ROWS, dh, 0, 1);   // B = V, MN-major
+        const uint32_t idesc_pv = ptx::umma_idesc_bf16(128, dh, 0, 1);   // B = V, MN-major
         const uint64_t dp = ptx::umma_desc_sw128(ptx::smem_u32(sP));
         const uint64_t dkv = ONE ? kv_base(ptx::smem_u32(kvring)) : 0ull;
         const uint32_t v_step = 2u << p.dh_shift;
@@ -626,6 +614,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     const bool moves = (halo_row || chunk_row) && new_row >= 0 && new_row < HALO;
     const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16);
     const float* tau_s = s_tau + (ONE ? 0 : (q >> 1) & 1) * 64;
+    const int aq = q & 1, ah = q >> 1;              // softmax: query quarter, key half
     const int tp = min(si.T, p.P - si.n_prompt0);   // the chunk's first tp frames complete the prompt
     int kv_row = 0;                                 // K/V plane row of this thread's frame
     if (f < tp) {
@@ -650,10 +639,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           const CluJob jb = s_job[jid / p.n_heads];
           if (jb.T == 0) continue;
           const int nkb = jb.k.nkb, head = jid % p.n_heads;
-          // Products of 64 rows: a quarter of tensor memory holds 16 of them, and the two lanes of a row take half of a block's key columns each, so that a
-          // row's statistics stay in its warp.  (128 rows, every query twice, a thread's partner in another warp: maxima through shared memory and two
-          // barriers per block, 48.5 cycles per 16 keys of P V instead of 32.5, and O in the lanes of half of the warps: one stream 727 us per chunk against 743, fourteen 918 against 930.)
-          const int row = q * 16 + (lane & 15), half = lane >> 4, w = cg;
+          const int row = aq * 32 + lane, w = cg;
+          float* sx = s_x + w * 128;
           float m_ref = -INFINITY, lsum = 0.f;
           bool ok = true;
 #pragma unroll 1
@@ -662,12 +649,15 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
             ok &= clu_wait(&bar_s[w], k & 1u, s_fail, p.err, 0x10e);
             ptx::tc_fence_after();
             float v[64];
-            ptx::tmem_ld64x2(lanes + (uint32_t)(w * ATT_KB), v);
+            ptx::tmem_ld64(lanes + (uint32_t)(w * ATT_KB + ah * 64), v);
             ptx::tc_fence_before();
             ptx::mbar_arrive(&bar_sfree[w]);       // S(b) has been read: the stream's next scores may overwrite it
-            const int col0 = b * ATT_KB + half * 64;
-            float mx = att_mask_max(v, jb.k.L - col0, jb.k.g0 - col0, jb.k.g1 - col0) * p.scale_log2e;
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+            const int col0 = b * ATT_KB + ah * 64;
+            float mx = att_mask_max(v, jb.k.L - col0, jb.k.g0 - col0, jb.k.g1 - col0);
+            sx[ah * 64 + row] = mx * p.scale_log2e;
+            ptx::named_bar_sync(4 + w, 128);
+            mx = fmaxf(sx[row], sx[64 + row]);
+            ptx::named_bar_sync(4 + w, 128);
             if (b >= 2) ok &= clu_wait(&bar_pv[w], (k - 1) & 1u, s_fail, p.err, 0x110);   // the stream's P buffer and O are quiescent
             if (b < 2) {
               m_ref = mx;
@@ -678,48 +668,43 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
                 const float alpha = need ? exp2f(m_ref - mx) : 1.0f;
                 if (need) m_ref = mx;
                 lsum *= alpha;
-                clu_rescale(lanes + (uint32_t)(CLU_O_COL + w * 64), alpha, dh);
+                if (ah == 0) att_rescale(lanes + (uint32_t)(CLU_O_COL + w * 64), alpha, dh);
                 ptx::tc_fence_before();
               }
             }
-            lsum += att_exp_store(v, p.scale_log2e, m_ref, sP + w * ATT_P_BYTES + half * 8192 + row * 128, row);
+            lsum += att_exp_store(v, p.scale_log2e, m_ref, sP + w * ATT_P_BYTES + ah * 8192 + row * 128, row);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
             ptx::mbar_arrive(&bar_p[w]);
           }
-          const float upper = __shfl_xor_sync(0xffffffffu, lsum, 16);
-          if (half == 0) {
-            s_x[w * 64 + row] = lsum + upper;
-            s_m[w * 64 + row] = m_ref;
-          }
+          sx[ah * 64 + row] = lsum;
+          if (ah == 0) s_m[w * 64 + row] = m_ref;
           // (each group waits for its own stream, whose phases it has followed; the barrier tells the other group)
           if (w < nkb) ok &= clu_wait(&bar_pv[w], (n_blk - 1) & 1u, s_fail, p.err, 0x111);
           ptx::named_bar_sync(1, CLU_EPI);
           ptx::tc_fence_after();
           ok = ok && *reinterpret_cast<volatile int*>(s_fail) == 0;
-          {                                        // each group of warps stores half of the columns
+          if (ah == 0) {                           // O rows 0..63 live in lanes 0..63; each group of warps stores half of the columns
             float c0, c1;
-            att_combine(nkb, s_m[row], s_x[row], s_m[64 + row], s_x[64 + row], &c0, &c1);
+            att_combine(nkb, s_m[row], s_x[row] + s_x[64 + row], s_m[64 + row], s_x[128 + row] + s_x[192 + row], &c0, &c1);
             const int orow = (ONE ? 0 : (jid / p.n_heads) * SLOT_ROWS) + HALO + row;
 #pragma unroll 1
             for (int c = w * (dh >> 1); c < (w + 1) * (dh >> 1); c += 16) {
-              uint32_t o[16];                      // O_0, O_1 (anything with one block)
-              ptx::tmem_ld_rows_issue<8>(lanes + (uint32_t)(CLU_O_COL + c), o);
-              ptx::tmem_ld_rows_issue<8>(lanes + (uint32_t)(CLU_O_COL + 64 + c), o + 8);
-              ptx::tmem_ld_wait<16>(o);
+              float o16[16], q16[16];
+              ptx::tmem_ld16x2(lanes + (uint32_t)(CLU_O_COL + c), lanes + (uint32_t)(CLU_O_COL + 64 + c), o16, q16);   // (O_1 is anything with one block)
               if (row < jb.T && ok) {
-                float o8[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) o8[i] = nkb > 1 ? fmaf(__uint_as_float(o[8 + i]), c1, __uint_as_float(o[i]) * c0) : __uint_as_float(o[i]) * c0;
-                uint32_t pk[4];
-                pack_row<8>(o8, pk);
-                const uint4 a = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                const int ch = c + 8 * half;
+                for (int i = 0; i < 16; ++i) o16[i] = nkb > 1 ? fmaf(q16[i], c1, o16[i] * c0) : o16[i] * c0;
+                uint4 a, bq;
+                pack16_bf16(o16, a, bq);
                 if (one_job) {                     // (the queries' tile is idle by now)
-                  *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(sQ) + (ch >> 5) * (SLOT_ROWS * 32) + clu_at32(row + HALO, ch & 31)) = a;
+                  bf16* d = reinterpret_cast<bf16*>(sQ) + (c >> 5) * (SLOT_ROWS * 32);
+                  *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, c & 31)) = a;
+                  *reinterpret_cast<uint4*>(d + clu_at32(row + HALO, (c & 31) + 8)) = bq;
                 } else {
-                  const int hc = (head << p.dh_shift) + ch;
-                  *reinterpret_cast<uint4*>(p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + (long long)(hc >> 5) * (rows * 32) + clu_at32(orow, hc & 31)) = a;
+                  const int ch = (head << p.dh_shift) + c, perm = (orow >> 1) & 3;
+                  store16(p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + (long long)(ch >> 5) * (rows * 32) + orow * 32 + ((((ch & 31) >> 3) ^ perm) & ~1) * 8,
+                          (perm & 1) ? bq : a, (perm & 1) ? a : bq);
                 }
               }
             }
