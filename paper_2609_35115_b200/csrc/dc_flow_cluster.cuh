@@ -23,7 +23,6 @@ constexpr int CLU_EPI = 256;
 constexpr int CLU_REGS_CTRL = 104, CLU_REGS_EPI = 200;
 constexpr int CLU_PANEL = 128 * 1024;                // activations [block][64 spc rows][128 B] (hidden <= 512); attention: Q, two P buffers, K/V ring
 constexpr int CLU_KV_BYTES = ATT_KB * 128;           // one K or V block
-constexpr uint32_t CLU_KVS = 4;                      // K/V ring slots
 constexpr int CLU_ACC2 = 256;                        // TMEM column of the odd issuer's accumulator
 constexpr int CLU_O_COL = 256;                       // attention: S of even / odd blocks at columns 0 / 128, O of the two streams at 256 / 320
 constexpr int CLU_TAIL = 3072;                       // barriers and constants behind the rings
@@ -149,24 +148,13 @@ __device__ __forceinline__ bool clu_wait(uint64_t* bar, uint32_t parity, int* s_
   return false;
 }
 
-// ---- K/V items of one attention job, in the order in which the products consume them: K0 K1 K2 V0 K3 V1 ... V(n-1) ----
-__device__ __forceinline__ int clu_item_k(int b) { return b < 2 ? b : 2 * b - 2; }
-__device__ __forceinline__ int clu_item_v(int b, int n) { return b + 2 < n ? 2 * b + 3 : 2 * n - (n - b); }
-__device__ __forceinline__ void clu_item(int i, int n, bool* is_v, int* b) {
-  if (i == 2 * n - 1) { *is_v = true; *b = n - 1; }
-  else if (n >= 2 && i == 2 * n - 2) { *is_v = true; *b = n - 2; }
-  else if (i < 2) { *is_v = false; *b = i; }
-  else if (i & 1) { *is_v = true; *b = (i - 3) >> 1; }
-  else { *is_v = false; *b = (i >> 1) + 1; }
-}
-
 struct CluJob {     // what the heads of a slot attend
   const bf16* kv;
   int         T;
   AttKeys     k;
 };
 
-static_assert(8 * (16 + 2 * CLU_RS + 2 * (int)CLU_KVS + 10) + 2 * (int)sizeof(CluJob) + 8 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
+static_assert(8 * (16 + 2 * CLU_RS + 3 * (int)CLU_KVS + 10) + 2 * (int)sizeof(CluJob) + 8 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
 
 // RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].first_live on, circularly.  (An instantiation of its
 // own: with the choice at run time every other call was 2 to 5 us slower.)
@@ -197,8 +185,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   uint64_t* normed = full_a + 8;         // [8]
   uint64_t* full_w = normed + 8;         // [RS]
   uint64_t* empty_w = full_w + RS;       // [RS]
-  uint64_t* full_kv = empty_w + RS;      // [CLU_KVS]
-  uint64_t* empty_kv = full_kv + CLU_KVS;
+  uint64_t* full_kv = empty_w + RS;      // [2 CLU_KVS]: clu_kv_full
+  uint64_t* empty_kv = full_kv + 2 * CLU_KVS;
   uint64_t* accum = empty_kv + CLU_KVS;
   uint64_t* bar_q = accum + 1;
   uint64_t* bar_s = bar_q + 1;           // [2] each, by stream (key block parity)
@@ -252,7 +240,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     }
 #pragma unroll 1
     for (int i = 0; i < (int)CLU_KVS; ++i) {
-      ptx::mbar_init(&full_kv[i], 1);
+      ptx::mbar_init(&full_kv[clu_kv_full(false, i)], 1);
+      ptx::mbar_init(&full_kv[clu_kv_full(true, i)], 1);
       ptx::mbar_init(&empty_kv[i], 1);
     }
     ptx::mbar_init(accum, 2);
@@ -329,6 +318,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     uint32_t wt = 0;                               // weight tiles of earlier stages
     uint32_t it0 = 0, pre = 0, n_q = 0;            // K/V items of earlier jobs; items of the next job already requested; Q tiles so far
     uint32_t n_s0 = 0, n_s1 = 0;                   // key blocks of the two streams in earlier jobs
+    CluKvPhases kv_phases;                         // warp 1: of the K barriers, warp 3: of the V barriers
     const bool two = !ONE && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
     // (the input projection's operand comes from another kernel: a slot's blocks are its own)
     auto request = [&](const bf16* src, int nkb, bool in) {
@@ -472,7 +462,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
               ptx::fence_proxy_async_smem();
               __syncwarp();
             }
-            if (ptx::elect_one()) jb.k.fetch(planes + (is_v ? kv_plane : 0), b, n, p.P, p.Rk, p.dh_shift, dst, &full_kv[ks]);
+            if (ptx::elect_one()) jb.k.fetch(planes + (is_v ? kv_plane : 0), b, n, p.P, p.Rk, p.dh_shift, dst, &full_kv[clu_kv_full(is_v, ks)]);
             __syncwarp();
           }
           if (!att) {
@@ -510,7 +500,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           for (int b = 0; b < nkb; ++b) {
             const int w = b & 1;
             const uint32_t gi = it0 + (uint32_t)clu_item_k(b), ks = gi % CLU_KVS;
-            clu_wait(&full_kv[ks], (gi / CLU_KVS) & 1u, s_fail, p.err, 0x108);
+            clu_wait(&full_kv[clu_kv_full(false, ks)], kv_phases.next(ks), s_fail, p.err, 0x108);
             if (b == 0) clu_wait(bar_q, n_q++ & 1u, s_fail, p.err, 0x10a);
             const uint32_t k = w ? n_s1++ : n_s0++;
             if (k > 0) clu_wait(&bar_sfree[w], (k - 1) & 1u, s_fail, p.err, 0x109);   // the stream's previous scores have been read
@@ -545,7 +535,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           for (int b = 0; b < nkb; ++b) {
             const int w = b & 1;
             const uint32_t gi = it0 + (uint32_t)clu_item_v(b, nkb), vs = gi % CLU_KVS;
-            clu_wait(&full_kv[vs], (gi / CLU_KVS) & 1u, s_fail, p.err, 0x10d);
+            clu_wait(&full_kv[clu_kv_full(true, vs)], kv_phases.next(vs), s_fail, p.err, 0x10d);
             clu_wait(&bar_p[w], (w ? n_s1++ : n_s0++) & 1u, s_fail, p.err, 0x10c);
             ptx::tc_fence_after();
             const uint64_t dpb = dp + (uint64_t)(w * (ATT_P_BYTES >> 4)), dv = kv_desc(dkv, vs);
