@@ -1,4 +1,5 @@
-// The K/V ring of the flow decoder's cluster step: the order of its items and the phases of its barriers.  Plain C++, so that the host can walk it as well.
+// Barriers of the flow decoder's cluster step whose phases more than one warp or CTA has to agree on: the K/V ring and the hand-over of a stage's rows.
+// Plain C++, so that the host can walk them as well.
 #pragma once
 #include <stdint.h>
 
@@ -36,5 +37,10 @@ struct CluKvPhases {              // a waiting warp's count of its barriers' pha
     return parity;
   }
 };
+
+// The barrier on which the CTAs of a cluster signal that their rows of the n-th stage handed over in bulk are there, and its phase.  Two in turn: a CTA may
+// signal stage n + 1 while another still waits for a signal of stage n, but none stage n + 2, because every CTA has passed a cluster barrier behind its wait.
+DC_HD uint32_t clu_hand(uint32_t n) { return n & 1u; }
+DC_HD uint32_t clu_hand_parity(uint32_t n) { return (n >> 1) & 1u; }
 
 }  // namespace dc

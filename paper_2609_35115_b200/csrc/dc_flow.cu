@@ -28,7 +28,7 @@
 #include <vector>
 
 #include "dc_internal.h"
-#include "dc_kv_ring.h"
+#include "dc_cluster_sync.h"
 #include "dc_ptx.cuh"
 #include "dc_rng.cuh"
 

@@ -104,11 +104,15 @@ __device__ __forceinline__ void clu_arrive_release(int warp) {
   ptx::cluster_arrive_relaxed();
 }
 
-// A stage's rows leave the CTA as one piece, [64 or 128 rows][32 channels] (clu_at32), which one thread copies out of shared memory in bulk.
-// The copy has completed - its bytes are in L2, where the other CTAs' bulk copies read them - 480 cycles after the staging; the fence behind stores of the
-// threads took 1,040.  (16 CTAs hand 4 KB each to one another: the first operand block is there after 1,150 cycles instead of 1,790.  With a fence behind the
-// copy, which has nothing left to wait for, 2,010.)  One stream 801 -> 748 us per chunk, hidden 256 298 -> 275, seven streams 813 -> 755, prompt and
-// look-ahead 762 -> 704; two slots per cluster: fourteen streams 990 -> 933, one guided stream 967 -> 913.
+// A stage's rows leave the CTA as one piece, [64 or 128 rows][32 channels] (clu_at32), which one thread copies out of shared memory in bulk, and a signal to every
+// CTA of the cluster tells that they are there.  What orders the rows in front of the other CTAs' reads: the copying thread waits for its copies to
+// complete, which makes their writes visible to it; behind that its warp stores one word into every CTA with st.async, whose complete-tx on the CTA's `hand`
+// barrier has release semantics at cluster scope; who reads the rows or the row statistics has waited on `hand` with acquire at cluster scope.  The cluster
+// barrier, whose arrivals are relaxed here, orders no rows: it tells that the buffers are free again.
+// Measured for the hand-over alone (16 CTAs, 4 KB each, cycles from the staging until it is released / until the first operand block is there): behind thread stores and a
+// fence 1,385 / 1,945, the copies with a fence behind them 1,670 / 2,228, with the signals 948 / 1,500, with nothing but the relaxed barrier, which orders nothing,
+// 828 / 1,387.  One stream 764 us per chunk (thread stores and a fence 801, a fence behind the copies 829, the relaxed barrier alone 743), hidden 256 289 (298, -,
+// 275), fourteen streams 944 (990, -, 931).  The request of the next operand behind the cluster barrier AND the signals: 771, hidden 256 286, fourteen 949.
 __device__ __forceinline__ int clu_at32(int rho, int c) { return rho * 32 + (((c >> 3) ^ ((rho >> 1) & 3)) << 3); }   // element of channel c of a block: the 64-byte swizzle
 struct CluPiece {
   void*       dst;
@@ -116,10 +120,11 @@ struct CluPiece {
   uint32_t    bytes;
 };
 template <int N>
-__device__ __forceinline__ void clu_arrive_bulk(int warp, const CluPiece (&piece)[N]) {
+__device__ __forceinline__ void clu_arrive_bulk(int warp, int lane, const CluPiece (&piece)[N], uint32_t hand, uint32_t word, int CL) {
   ptx::fence_proxy_async_smem();
   ptx::named_bar_sync(1, CLU_EPI);
   if (warp == 4) {
+    const uint32_t to = lane < CL ? lane : 0, bar_to = ptx::map_to_cta(hand, to), word_to = ptx::map_to_cta(word, to);
     if (ptx::elect_one()) {
 #pragma unroll
       for (int i = 0; i < N; ++i)
@@ -128,6 +133,8 @@ __device__ __forceinline__ void clu_arrive_bulk(int warp, const CluPiece (&piece
     }
     __syncwarp();
     ptx::fence_proxy_async_global();
+    if (lane < CL) ptx::st_async(word_to, 0u, bar_to);
+    __syncwarp();
   }
   ptx::cluster_arrive_relaxed();
 }
@@ -135,11 +142,12 @@ __device__ __forceinline__ void clu_arrive_bulk(int warp, const CluPiece (&piece
 // Bounded wait of a whole warp that gives up at once after any wait of this CTA has given up: the step then runs through without
 // waiting, the copying warps request nothing more, and the CTA pauses before it exits.  The vote keeps the warp together: lanes that leave a polling loop one by one go on as separate groups, and everything
 // up to the next warp-wide instruction is then executed several times (an issue loop took 600 cycles per block instead of 260).
+template <bool CLUSTER = false>   // phases that other CTAs complete: acquire at cluster scope
 __device__ __forceinline__ bool clu_wait(uint64_t* bar, uint32_t parity, int* s_fail, int* err, int code) {
   const uint32_t a = ptx::smem_u32(bar);
 #pragma unroll 1
   for (uint32_t i = 0; i < (1u << 20); ++i) {
-    if (__all_sync(0xffffffffu, ptx::mbar_try_wait_s(a, parity))) return true;
+    if (__all_sync(0xffffffffu, CLUSTER ? ptx::mbar_try_wait_cluster_s(a, parity) : ptx::mbar_try_wait_s(a, parity))) return true;
     if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0)) return false;
   }
   *reinterpret_cast<volatile int*>(s_fail) = 1;
@@ -154,7 +162,7 @@ struct CluJob {     // what the heads of a slot attend
   AttKeys     k;
 };
 
-static_assert(8 * (16 + 2 * CLU_RS + 3 * (int)CLU_KVS + 10) + 2 * (int)sizeof(CluJob) + 8 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
+static_assert(8 * (16 + 2 * CLU_RS + 3 * (int)CLU_KVS + 12) + 2 * (int)sizeof(CluJob) + 12 + 4 * CLU_CONST_FLOATS <= CLU_TAIL, "barriers and constants");
 
 // RING (a wavefront pass): fewer clusters than slots, the live slots are those from slot slots[0].first_live on, circularly.  (An instantiation of its
 // own: with the choice at run time every other call was 2 to 5 us slower.)
@@ -193,9 +201,11 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   uint64_t* bar_sfree = bar_s + 2;
   uint64_t* bar_p = bar_sfree + 2;
   uint64_t* bar_pv = bar_p + 2;
-  CluJob* s_job = reinterpret_cast<CluJob*>(bar_pv + 2);                  // [2], one per slot
+  uint64_t* hand = bar_pv + 2;           // [2], in turn: a stage's rows of every CTA of the cluster are there
+  CluJob* s_job = reinterpret_cast<CluJob*>(hand + 2);                    // [2], one per slot
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_job + 2);
   int* s_fail = reinterpret_cast<int*>(tmem_slot + 1);
+  uint32_t* s_word = tmem_slot + 2;      // what the signals store: nobody reads it
   float* s_bias = reinterpret_cast<float*>(wring + RS * CLU_SLOT + CLU_TAIL - 4 * CLU_CONST_FLOATS);   // [3 BN], 16-byte aligned
   float* s_tau = s_bias + 3 * 64;                          // [2][64]
   float* s_x = s_tau + 128;                                // [2][2][64]: per stream, exchange between the column halves
@@ -252,6 +262,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       ptx::mbar_init(&bar_sfree[i], 128);
       ptx::mbar_init(&bar_p[i], 128);
       ptx::mbar_init(&bar_pv[i], 1);
+      ptx::mbar_init(&hand[i], 1);
     }
     *s_fail = 0;
     ptx::fence_barrier_init();
@@ -260,6 +271,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
+  ptx::cluster_arrive_relaxed();         // (the other CTAs signal on this one's barriers; fence_barrier_init is the release)
+  ptx::cluster_wait();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   auto issuers = [&](int nkb) { return nkb >= 2 ? 2 : 1; };
@@ -268,6 +281,8 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
   auto kv_base = [&](uint32_t a) { return p.dh_shift == 6 ? att_kv_desc<64>(a) : att_kv_desc<32>(a); };
   auto kv_desc = [&](uint64_t first, uint32_t ks) { return ONE ? first + (uint64_t)(ks * (CLU_KV_BYTES >> 4)) : kv_base(ptx::smem_u32(kvring + ks * CLU_KV_BYTES)); };
   const int n_jobs = SPC * p.n_heads;            // (slot, head) pairs of the cluster; CTA r takes r, r + CL, ...
+  const bool one_job = ONE || n_jobs <= p.CL;    // at most one of a CTA: its rows leave in bulk
+  auto in_bulk = [&](int kind) { return kind == CLU_ATT ? one_job : kind != CLU_QKV && kind != CLU_OUT; };
   const long long kv_plane = (long long)(p.P + p.Rk) * p.C;
   const int dh = 1 << p.dh_shift;
 
@@ -319,6 +334,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     uint32_t it0 = 0, pre = 0, n_q = 0;            // K/V items of earlier jobs; items of the next job already requested; Q tiles so far
     uint32_t n_s0 = 0, n_s1 = 0;                   // key blocks of the two streams in earlier jobs
     CluKvPhases kv_phases;                         // warp 1: of the K barriers, warp 3: of the V barriers
+    uint32_t n_hand = 0;                           // warp 0: stages whose rows left in bulk so far
     const bool two = !ONE && slot0 + 1 < p.n_slots;   // (an odd batch's last cluster has one slot: the other's rows are anything)
     // (the input projection's operand comes from another kernel: a slot's blocks are its own)
     auto request = [&](const bf16* src, int nkb, bool in) {
@@ -561,11 +577,23 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       const bool wants = warp == 0 && nx.s < p.n_steps && nx.kind != CLU_ATT && !(nx.kind == CLU_OUT && nch_out == 0);
       const int nx_nkb = nx.kind == CLU_IN ? nkb_in : nkb_c;
       const bf16* nx_src = (nx.kind == CLU_IN ? p.Ain : (nx.kind == CLU_OPROJ ? p.O : p.X[xi])) + (long long)slot0 * nx_nkb * CLU_SLOT_KB;
+      // (this barrier's previous phase is complete: warp 0 has waited for it, two stages in bulk ago)
+      const bool bulk = warp == 0 && in_bulk(st.kind);
+      uint64_t* const bar_h = &hand[clu_hand(n_hand)];
+      const uint32_t ph_h = clu_hand_parity(n_hand);
+      if (bulk) {
+        if (ptx::elect_one()) ptx::mbar_expect_tx(bar_h, 4u * (uint32_t)p.CL);
+        __syncwarp();
+        ++n_hand;
+      }
       ptx::cluster_arrive_relaxed();
       // (read here, where nobody waits for it: a wait takes so long to give up that what it left behind one stage earlier has landed)
-      const bool failed = warp == 0 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0);
-      ptx::cluster_wait();
+      bool failed = warp == 0 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(s_fail) != 0);
+      // The rows of a stage in bulk: this CTA's own signal tells that its panel is free, so the request need not wait for the cluster barrier as well.
+      if (bulk && !failed) failed = !clu_wait<true>(bar_h, ph_h, s_fail, p.err, 0x115);
+      if (!bulk) ptx::cluster_wait();
       if (wants && !failed) request(nx_src, nx_nkb, nx.kind == CLU_IN);
+      if (bulk) ptx::cluster_wait();
       if (failed) {
 #pragma unroll 1
         for (st.next(p); st.s < p.n_steps; st.next(p)) {
@@ -619,11 +647,11 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
     for (int i = 0; i < NC / 2; ++i) xr[i] = 0u;
     int xi = 0;
     uint32_t n_g = 0, n_gc = 0, n_gi = 0;
+    uint32_t n_hand = 0;                            // stages whose rows left in bulk so far
     uint32_t n_blk = 0;                             // key blocks of this thread's stream so far
 #pragma unroll 1
     for (CluStage st; st.s < p.n_steps; st.next(p)) {
       if (st.kind == CLU_ATT) {
-        const bool one_job = ONE || n_jobs <= p.CL;  // of this CTA: its rows leave in bulk
 #pragma unroll 1
         for (int jid = rank; jid < n_jobs; jid += p.CL) {
           const CluJob jb = s_job[jid / p.n_heads];
@@ -710,7 +738,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
           bf16* dst = p.O + (long long)slot0 * nkb_c * CLU_SLOT_KB + ((head << p.dh_shift) >> 5) * (rows * 32) + (sl * SLOT_ROWS + HALO) * 32;
           const uint8_t* src = sQ + HALO * 64;
           const CluPiece piece[2] = {{dst, src, bytes}, {dst + rows * 32, src + SLOT_ROWS * 64, p.dh_shift == 6 ? bytes : 0u}};
-          clu_arrive_bulk(warp, piece);
+          clu_arrive_bulk(warp, lane, piece, ptx::smem_u32(&hand[clu_hand(n_hand++)]), ptx::smem_u32(s_word), p.CL);
         } else {
           clu_arrive_release(warp);
         }
@@ -729,6 +757,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
 
       // ---- what does not depend on the accumulator, under the main loop ----
       float4 part[8];                                // partial sums of squares of the row, 16 channels each (first: their loads take longest)
+      if (norm) clu_wait<true>(&hand[clu_hand(n_hand - 1u)], clu_hand_parity(n_hand - 1u), s_fail, p.err, 0x116);   // (the statistics of the stage before, of every CTA)
       if (norm && chunk_row) {
         const float* src = p.ssq + (long long)slot * (p.C >> 4) * SLOT_ROWS + rho;
 #pragma unroll
@@ -1046,12 +1075,13 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
         float* const ssq = p.ssq + (long long)slot0 * ssq_slot + 2 * rank * SLOT_ROWS;
         const uint32_t ssq_bytes = feeds_norm ? 2u * SLOT_ROWS * 4u : 0u;
         const CluPiece rows_piece = {out + (long long)slot0 * nkb_c * CLU_SLOT_KB + rank * (rows * 32), rows_out, (uint32_t)rows * 64u};
+        const uint32_t hand_now = ptx::smem_u32(&hand[clu_hand(n_hand++)]);
         if (ONE) {
           const CluPiece piece[2] = {rows_piece, {ssq, ssq_out, ssq_bytes}};
-          clu_arrive_bulk(warp, piece);
+          clu_arrive_bulk(warp, lane, piece, hand_now, ptx::smem_u32(s_word), p.CL);
         } else {
           const CluPiece piece[3] = {rows_piece, {ssq, ssq_out, ssq_bytes}, {ssq + ssq_slot, ssq_out + 2 * SLOT_ROWS, rows == 2 * SLOT_ROWS ? ssq_bytes : 0u}};
-          clu_arrive_bulk(warp, piece);
+          clu_arrive_bulk(warp, lane, piece, hand_now, ptx::smem_u32(s_word), p.CL);
         }
         // shift the carry by the committed frames: nobody in this launch reads it again
         if (carry != nullptr && moves && ok) {

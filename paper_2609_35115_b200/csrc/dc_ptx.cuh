@@ -54,6 +54,20 @@ __device__ __forceinline__ bool mbar_try_wait_s(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// ... of a phase that other CTAs of the cluster complete.
+__device__ __forceinline__ bool mbar_try_wait_cluster_s(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait.  Returns false after kMaxPolls failed polls (each poll blocks in hardware for a
 // short, implementation-defined time), which is orders of magnitude beyond any legitimate wait here: whatever was in flight when
 // the wait began has landed when it gives up.
@@ -134,6 +148,11 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)), "r"(smem_u32(src)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// Stores a word to a shared::cluster address; 4 bytes are then counted on the barrier at `bar` in the same CTA, with release semantics at cluster scope.
+__device__ __forceinline__ void st_async(uint32_t dst, uint32_t v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(dst), "r"(v), "r"(bar) : "memory");
+}
 
 // Asks `bytes` (a multiple of 16) from a 16-byte aligned address into L2.
 __device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
