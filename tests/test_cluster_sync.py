@@ -1,5 +1,5 @@
-"""The K/V ring of the flow decoder's cluster step (csrc/dc_kv_ring.h, compiled for the host): however late its loads land and however its warps are
-interleaved, no warp passes a wait for a block that has not landed."""
+"""The barriers of the flow decoder's cluster step (csrc/dc_cluster_sync.h, compiled for the host): however late loads and signals land and however warps and
+CTAs are interleaved, no warp passes a wait for a K/V block that has not landed, and no CTA reads a row before the signal of the CTA that wrote it."""
 import ctypes
 import os
 import random
@@ -10,13 +10,15 @@ import pytest
 import paper_2609_35115_b200 as dc
 
 SRC = """
-#include "dc_kv_ring.h"
+#include "dc_cluster_sync.h"
 extern "C" {
 unsigned kv_slots() { return dc::CLU_KVS; }
 int kv_item(int i, int n) { bool v; int b; dc::clu_item(i, n, &v, &b); return 2 * b + v; }
 int kv_item_k(int b) { return dc::clu_item_k(b); }
 int kv_item_v(int b, int n) { return dc::clu_item_v(b, n); }
 unsigned kv_full(int is_v, unsigned slot) { return dc::clu_kv_full(is_v != 0, slot); }
+unsigned hand(unsigned n) { return dc::clu_hand(n); }
+unsigned hand_parity(unsigned n) { return dc::clu_hand_parity(n); }
 unsigned kv_next(unsigned* bits, unsigned slot) { dc::CluKvPhases p; p.bits = *bits; const unsigned r = p.next(slot); *bits = p.bits; return r; }
 }
 """
@@ -24,7 +26,7 @@ unsigned kv_next(unsigned* bits, unsigned slot) { dc::CluKvPhases p; p.bits = *b
 
 @pytest.fixture(scope="module")
 def ring(tmp_path_factory):
-    d = tmp_path_factory.mktemp("kv_ring")
+    d = tmp_path_factory.mktemp("cluster_sync")
     (d / "ring.cpp").write_text(SRC)
     csrc = os.path.join(os.path.dirname(dc.__file__), "csrc")
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", csrc, "-o", str(d / "ring.so"), str(d / "ring.cpp")], check=True)
@@ -155,3 +157,109 @@ def test_the_walk_finds_one_barrier_for_both_kinds(ring):
 
     assert [early([n]) for n in range(1, 7)] == [False, False, False, True, True, True]
     assert early([5, 5])
+
+
+def walk_hand(ring, stages, ctas, rng, form="two"):
+    """One interleaving of the loaders' and the epilogues' warps of a cluster over stages that hand over in bulk ("b"), in bulk with row statistics for the next
+    stage ("s"), or behind a fence ("f").  A row is visible to a CTA from the writer's signal on; "two": as in the kernel, "one": a single barrier,
+    "none": only the cluster barrier between a stage and the next."""
+    nth, n = [], 0                                   # of a stage: how many in bulk came before it
+    for kind in stages:
+        nth.append(n)
+        n += kind != "f"
+    index = (lambda j: 0) if form == "one" else ring.hand
+    parity = (lambda j: j & 1) if form == "one" else ring.hand_parity
+    phase = [[0, 0] for _ in range(ctas)]            # completed phases of a CTA's barriers
+    armed, tx = [[False, False] for _ in range(ctas)], [[0, 0] for _ in range(ctas)]
+    seen = [set() for _ in range(ctas)]              # (stage, writer) of the signals that have landed
+    flying = []
+    arrived = [0] * len(stages)                      # at the cluster barrier behind a stage; two warps of every CTA
+
+    def settle(c, i):
+        if armed[c][i] and tx[c][i] == 0:
+            phase[c][i] += 1
+            armed[c][i] = False
+
+    def passes(c, j):
+        return (phase[c][index(j)] & 1) != parity(j)
+
+    def check(c, k):
+        if any((k, w) not in seen[c] for w in range(ctas)):
+            raise Early((c, k))
+
+    requested = [0] * ctas                           # operands: of the stages before this number
+
+    def loader(c):
+        requested[c] = 1
+        for k, kind in enumerate(stages):
+            if kind != "f" and form != "none":
+                i = index(nth[k])
+                assert not armed[c][i], "the phase before is still open"
+                tx[c][i] += ctas
+                armed[c][i] = True
+                settle(c, i)
+            arrived[k] += 1
+            yield lambda: True
+            if kind != "f" and form != "none":
+                yield lambda: passes(c, nth[k])
+            else:
+                yield lambda: arrived[k] == 2 * ctas
+            if kind != "f":
+                check(c, k)
+            requested[c] = k + 2
+            yield lambda: arrived[k] == 2 * ctas
+
+    def epilogue(c):
+        for k, kind in enumerate(stages):
+            yield lambda: requested[c] > k
+            if k > 0 and stages[k - 1] == "s":
+                if form != "none":
+                    yield lambda: passes(c, nth[k - 1])
+                check(c, k - 1)
+            yield lambda: True                       # the products
+            if kind != "f":
+                flying.extend((k, c, d) for d in range(ctas))
+            arrived[k] += 1
+            yield lambda: arrived[k] == 2 * ctas
+
+    warps = [w(c) for c in range(ctas) for w in (loader, epilogue)]
+    ready = [next(w) for w in warps]
+    slow = rng.choice([0.02, 0.2, 0.6])
+    while warps:
+        can = [i for i, r in enumerate(ready) if r()]
+        if flying and (not can or rng.random() < slow):
+            k, c, d = flying.pop(rng.randrange(len(flying)))
+            seen[d].add((k, c))
+            if form != "none":
+                i = index(nth[k])
+                tx[d][i] -= 1
+                settle(d, i)
+            continue
+        assert can, "no move is left"
+        i = rng.choice(can)
+        try:
+            ready[i] = next(warps[i])
+        except StopIteration:
+            del warps[i], ready[i]
+
+
+# input, conv blocks, projections, attention (in bulk or behind a fence), output projection, output
+HAND_STAGES = {"one job": "bbsfbbbsfbsf" * 3, "several jobs": "bbsffbbsffsf" * 3, "short": "bsfbsf" * 4}
+
+
+@pytest.mark.parametrize("stages", HAND_STAGES.values(), ids=HAND_STAGES.keys())
+@pytest.mark.parametrize("ctas", [2, 5])
+def test_no_row_is_read_before_its_writers_signal(ring, stages, ctas):
+    for seed in range(60):
+        walk_hand(ring, stages, ctas, random.Random(seed))
+
+
+@pytest.mark.parametrize("form", ["none", "one"])
+def test_the_walk_finds_the_cluster_barrier_alone_and_a_single_barrier(ring, form):
+    found = 0
+    for seed in range(60):
+        try:
+            walk_hand(ring, HAND_STAGES["one job"], 4, random.Random(seed), form)
+        except (Early, AssertionError):
+            found += 1
+    assert found > 0
