@@ -70,9 +70,10 @@ def test_vocoder_batch_tiles(dc, mel, channels, f_chunk, n):
     assert gu.rel_err(got, orc.run_offline(cfg, weights, x, bounds).reshape(-1)) <= 1e-4
 
 
-# tiles of 64 frames: alone (32 columns each) and in batches whose layers take 64 columns, with one panel of input channels and with several; the last frames of
-# a tile, a second tile of one frame; the bytes of single calls, which take other tiles
-@pytest.mark.parametrize("mel,channels,f_chunk,n", [(8, (512, 64, 64), 56, 12), (80, (512, 256, 64), 50, 3), (80, (256, 128, 132), 33, 2), (80, (512, 128, 64), 65, 5)])
+# tiles of 64 frames: alone (32 columns each) and in batches; the first layer of the first case takes 64 columns with one panel of input channels, that of the last
+# 64 columns with two panels (at 148 SMs); the last frames of a tile, a second and a third tile of one frame; the bytes of single calls, which take other tiles
+@pytest.mark.parametrize("mel,channels,f_chunk,n", [(8, (512, 64, 64), 56, 12), (80, (512, 256, 64), 50, 3), (80, (256, 128, 132), 33, 2), (80, (512, 128, 64), 65, 5),
+                                                    (80, (512, 128, 64), 129, 5)])
 def test_vocoder_small_tiles(dc, mel, channels, f_chunk, n):
     gu = _util()
     cfg = wl.tiny_vocoder(mel_dim=mel, up_channels=channels, f_chunk=f_chunk, n_chunks=3, seed=42)
@@ -159,10 +160,13 @@ def test_flow_cluster_rounded_norm(dc, n, kw):
     assert np.array_equal(got, _batch_equals_single(dc, cfg, n, options=dc.OPT_ROUNDED_NORM | dc.OPT_CTA_PAIRS)[3])
 
 
-# large scores: a later key block's maximum exceeds the reference by more than 2^8 and the accumulated output is rescaled.  One and two slots per cluster and kernels of
-# their own: each has its own rows in tensor memory, and all give the same bytes
+# large scores: a later key block's maximum exceeds the reference by more than 2^8 and the accumulated output is rescaled (counted in the oracle's scores, wherever
+# the blocks begin).  One and two slots per cluster and kernels of their own: each has its own rows in tensor memory, and all give the same bytes.
+# The bound: scores of 14 binary orders turn last bits of a product into percents of a weight.  The oracle differs from itself by 3.2e-2 of RMS with scores in fp32,
+# by 3.8e-2 with its weights rounded against another reference, by 3.4e-2 with two accumulators rescaled as on the device; twice the largest.  Without the rescaling
+# of the row sums it differs by 0.64, without that of the accumulated output by 2.1, with half of the columns rescaled twice by 1.9.
 @pytest.mark.parametrize("heads", [8, 16])
-def test_attention_rescale_in_every_form(dc, heads):
+def test_attention_rescale_in_every_form(dc, heads, monkeypatch):
     cfg = wl.tiny_flow(hidden=512, n_heads=heads, head_dim=512 // heads, mel_dim=80, n_steps=2, kv_cap=500, f_chunk=50, seed=44)
     w, at = wl.make_workload(cfg).weights.copy(), 0
     for name, shape, _ in wl.blob_layout(cfg):
@@ -185,6 +189,23 @@ def test_attention_rescale_in_every_form(dc, heads):
     assert m.counters()[4] == 0 and outs[1].isfinite().all()
     for n in (9, 20):
         assert torch.equal(outs[n], outs[1].expand(n, -1, -1)), n
+    rescaled, attend = [], orc._attend
+
+    def counting(cfg, q, k, v, rb):
+        dh = cfg.head_dim
+        for e in range(cfg.n_heads if k.shape[0] > 300 else 0):
+            s = (q[:, e * dh:(e + 1) * dh] @ k[:, e * dh:(e + 1) * dh].T) * (np.log2(np.e) / np.sqrt(dh))
+            count = []
+            for phi in range(8):          # the first block holds 128 - phi keys; block b follows block b - 2 into its accumulator
+                top = [s[:, max(0, 128 * i - phi):128 * (i + 1) - phi].max(axis=1) for i in range((k.shape[0] + phi + 127) // 128)]
+                count.append(sum(int((top[i] > top[i - 2] + 8.0).sum()) for i in range(2, min(4, len(top)))))
+            rescaled.append(min(count))
+        return attend(cfg, q, k, v, rb)
+
+    monkeypatch.setattr(orc, "_attend", counting)
+    ref = orc.run_stream(cfg, w, torch.cat(x).cpu().numpy(), list(range(0, 12 * cfg.f_chunk + 1, cfg.f_chunk)))
+    assert sum(rescaled) >= 100
+    assert _util().rel_err(outs[1][0].cpu().numpy(), ref[-cfg.f_chunk:]) <= 8e-2
     for s in streams:
         s.close()
     m.destroy()
