@@ -64,7 +64,9 @@ __device__ __noinline__ float4 excite4(float4 v, long long t, int n, int rng_id,
 // with one accumulator, 2.1e-5 with one per panel).  So the leading term of every (panel, tap) - four additions - has an accumulator of
 // its own, which the epilogue threads add up in registers, rounded to nearest.  DRAIN (inputs of more than one panel): two sets of three, a
 // panel's taps each, one set added up while the next panel is multiplied.  One panel: one set.  At 64 columns, where two CTAs share the SM's
-// tensor memory: two accumulators that the taps take in turn (TURN).  (A single one for the three taps, twelve additions: ten layers of 64 channels
+// tensor memory: two accumulators that the taps take in turn (TURN).  (64 frames and several panels as well: a launch alone has one such tile per SM at most, but
+// launches of other sessions lie beside it.  Three models of 2, 3 and 5 streams each 182, 272 and 325 us, with room for one CTA per SM 190, 275 and 331; one
+// model 101.5, 133.5 and 155.3 against 101.1, 133.4 and 153.8.)  (A single one for the three taps, twelve additions: ten layers of 64 channels
 // end at 4.3e-6 of their norm, against 2.0e-6 for sums of the FP32 pipe.)
 //
 // PACK (batches; chunks of up to TC_PACK frames at the layer's rate): a tile holds two slots, the second one's rows 64 behind the

@@ -4,11 +4,12 @@
 // A stage of the network (one GEMM, or attention) for a few slots is far too little work to fill the GPU; what it costs as
 // a kernel of its own is latency: launch boundary, set-up, the wait for the whole previous grid, the first operand tiles
 // through L2.  Here a cluster of CL CTAs keeps one or two slots (64 or 128 rows) for the whole step: CTA r owns the columns
-// [32 r, 32 r + 32) of every layer, the activations pass from stage to stage through L2, and the hardware cluster barrier
-// stands where the launch boundary was.
-//   * Measured for the hand-over alone (16 CTAs write 4 KB each, everybody reads the 64 KB): 1,500 cycles until the barrier
-//     releases, 2,570 until the first operand tile has landed, 3,140 for all of them; through global counters instead of the
-//     barrier 3,460 / 4,940 / 5,660; pushed through distributed shared memory 4,020 (17 bytes per cycle and SM).
+// [32 r, 32 r + 32) of every layer, the activations pass from stage to stage through L2, and the hardware cluster barrier and
+// signals from CTA to CTA stand where the launch boundary was.
+//   * Measured for the hand-over alone (16 CTAs write 4 KB each, everybody reads the 64 KB; cycles until it is released / the
+//     first operand block has landed / all of them): bulk copies and signals (clu_arrive_bulk) 950 / 1,500 / 2,020, thread stores
+//     and a fence (clu_arrive_release) 1,380 / 1,940 / 2,460; through global counters instead of the barrier 3,460 / 4,940 /
+//     5,660; pushed through distributed shared memory 3,760 for all (17 bytes per cycle and SM).
 //   * Weights do not depend on the activations: one warp streams the CTA's share of every layer (packed at create in the
 //     order and the shared-memory image in which it is consumed) through a ring that runs up to RS reduction blocks ahead,
 //     across stage and step boundaries.
@@ -51,7 +52,8 @@ struct CluParams {
   int             o_bout, o_tau;
   const uint8_t*  wstream;             // [CL] streams of wstream_bytes
   long long       wstream_bytes;
-  bf16 *          X[2], *Q, *O, *Ain;  // activations in block layout (CLU_SLOT_KB)
+  bf16 *          X[2], *O;            // activations between GEMMs, blocks of 32 channels (clu_at32): [cluster][C / 32][rows of its slots][32]
+  bf16 *          Q, *Ain;             // queries, input of the network: blocks of 64 channels (clu_row16): [slot][C or Kin / 64][64 rows][64]
   float*          xstate;
   float*          ssq;                 // [slot][C / 16][SLOT_ROWS] partial sums of squares of the rows that feed an RMS norm
   float           inv_C, eps, inv_n, cfg_w;
@@ -77,9 +79,8 @@ struct CluStage {
   }
 };
 
-// The activations that pass from stage to stage: [slot][64-channel block][64 rows][64 channels], a row's eight 16-byte chunks
-// at the positions c ^ (row & 7) that they take in the swizzled shared-memory tile, so that a block of a slot is one untiled
-// bulk copy of 8 KB (no tensor map to fetch: 800 cycles less until the first tile is there).
+// A row's 16-byte chunks lie in global memory where the swizzled shared-memory tile has them, so that a block of a slot is one untiled bulk copy (no tensor
+// map to fetch: 800 cycles less until the first tile is there): in blocks of 64 channels chunk c of a row at c ^ (row & 7), in blocks of 32 at c ^ ((row >> 1) & 3).
 constexpr int CLU_SLOT_KB = SLOT_ROWS * KBLK;
 __device__ __forceinline__ int clu_row16(int rho, int c) { return rho * KBLK + ((((c >> 3) ^ (rho & 7)) & ~1) << 3); }   // the 32 bytes of columns c .. c + 15
 template <int NC>
@@ -89,10 +90,6 @@ __device__ __forceinline__ void pack_row(const float* v, uint32_t* w) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     w[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
-}
-__device__ __forceinline__ void clu_store16(bf16* blk, int rho, int c, const uint4& a, const uint4& b) {   // columns c .. c + 15 of a block
-  bf16* d = blk + clu_row16(rho, c);
-  store16(d, (rho & 1) ? b : a, (rho & 1) ? a : b);
 }
 
 // The stage's stores become visible to the cluster, then the epilogue's threads arrive: a barrier among them and ONE warp's fence,
@@ -111,7 +108,7 @@ __device__ __forceinline__ void clu_arrive_release(int warp) {
 // barrier, whose arrivals are relaxed here, orders no rows: it tells that the buffers are free again.
 // Measured for the hand-over alone (16 CTAs, 4 KB each, cycles from the staging until it is released / until the first operand block is there): behind thread stores and a
 // fence 1,385 / 1,945, the copies with a fence behind them 1,670 / 2,228, with the signals 948 / 1,500, with nothing but the relaxed barrier, which orders nothing,
-// 828 / 1,387.  One stream 764 us per chunk (thread stores and a fence 801, a fence behind the copies 829, the relaxed barrier alone 743), hidden 256 289 (298, -,
+// 828 / 1,387.  One stream 764 us per chunk at the time, 747 now (thread stores and a fence 801, a fence behind the copies 829, the relaxed barrier alone 743), hidden 256 289 (298, -,
 // 275), fourteen streams 944 (990, -, 931).  The request of the next operand behind the cluster barrier AND the signals: 771, hidden 256 286, fourteen 949.
 __device__ __forceinline__ int clu_at32(int rho, int c) { return rho * 32 + (((c >> 3) ^ ((rho >> 1) & 3)) << 3); }   // element of channel c of a block: the 64-byte swizzle
 struct CluPiece {
@@ -604,7 +601,7 @@ __global__ void __launch_bounds__(CLU_THREADS, 1) flow_cluster_kernel(const __gr
       }
     }
   } else {
-    // ---------------- epilogue: a thread owns one row and 16 columns; attention: warps 4..7 even, 8..11 odd key blocks ----------------
+    // ---------------- epilogue: a thread owns one row and NC columns; attention: warps 4..7 even, 8..11 odd key blocks ----------------
     ptx::pdl_wait();
     const int et = tid - 128;
     const int q = warp & 3, cg = (warp - 4) >> 2;
