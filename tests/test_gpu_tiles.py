@@ -306,7 +306,8 @@ def test_profile_brackets_the_launches_of_a_call(dc, n, cluster):
 
 
 # two slots per cluster (fourteen streams, seven guided ones) and one, from the empty window to the full one, one to five key blocks, beside copies that
-# hold up the loads of carried rows: the same bytes every time.  (A wait of the K/V ring that passed early showed in 2 of 8,700 such rounds.)
+# hold up the loads of carried rows: the same bytes every time.  (A wait of the K/V ring that passed early showed in 2 of 8,700 such rounds, and only in an attention
+# with a shorter softmax: the walk of the ring on the host is what tests the wait.)
 @pytest.mark.parametrize("net,n", [("cfg3", 14), ("cfg3_guided", 7), ("cfg3", 1)])
 def test_cluster_step_repeats_beside_copies(dc, net, n):
     cfg = {**wl.CONFIGS, **wl.EXTRA_CONFIGS}[net]
